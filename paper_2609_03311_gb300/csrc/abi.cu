@@ -156,6 +156,7 @@ void free_workspace(Workspace& w) {
   host_free(w.h_tok_off); host_free(w.h_sorted_slot); host_free(w.h_err); host_free(w.h_items);
   host_free(w.h_tiles);
   dev_free(w.sel_A); dev_free(w.sel_a_off); dev_free(w.sel_u); dev_free(w.sel_pos); dev_free(w.sel_x);
+  dev_free(w.sel_units); dev_free(w.sel_stats);
   if (w.sel_empty) {
     free_store(w.sel_empty);
     delete static_cast<dopr_store*>(w.sel_empty);
@@ -589,10 +590,17 @@ struct SelectState {
   int top_k, top_p;
   float* A;        // device, the largest chunk's sum of n^2
   int64_t a_elems;  // floats in A
-  int64_t* a_off;  // device, per chunk document
+  const int64_t* a_off;  // device, per document: its matrix's offset within its chunk's
   float* u;        // device, [all tokens]
   int32_t* positions;
   bf16* x;
+  const SelUnit* units;  // device, per chunk its row tiles then its column tiles
+  float2* stats;         // device, [Hq][rows of the largest chunk]
+  struct Chunk {
+    int64_t first;  // of units
+    int n_row_tiles, n_tiles, max_n;
+  };
+  std::vector<Chunk> chunks;
 };
 
 dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cudaStream_t st,
@@ -712,9 +720,11 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
         if (final_layer) continue;
       }
       if (sel && final_layer) {  // rank the chunk's tokens on this layer's q and k
+        CUtensorMap tm_rows{};
+        if (!make_tmap_16b_2d(&tm_rows, w.qkv, m->qkv_dim, Tc, (uint64_t)m->qkv_dim * 2, 64, SEL_TILE, true, true))
+          return fail(DOPR_ERR_CUDA, "cuTensorMapEncodeTiled failed for the QKV buffer");
+        const SelectState::Chunk& sc = sel->chunks[ci];
         SelectArgs sa{};
-        sa.qkv = w.qkv;
-        sa.ld_qkv = m->qkv_dim;
         sa.Hq = Hq;
         sa.Hkv = Hkv;
         sa.tok_pair = w.tok_pair;
@@ -723,23 +733,20 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
         sa.p0 = s0;
         sa.n_docs = s1 - s0;
         sa.n_rows = Tc;
-        sa.a_off = sel->a_off;
+        sa.a_off = sel->a_off + s0;
         sa.A = sel->A;
+        sa.row_tiles = sel->units + sc.first;
+        sa.n_row_tiles = sc.n_row_tiles;
+        sa.n_tiles = sc.n_tiles;
+        sa.max_n = sc.max_n;
+        sa.stats = sel->stats;
         sa.top_p = sel->top_p;
         sa.top_k = sel->top_k;
         sa.u = sel->u + t0;
         sa.positions = sel->positions;
         sa.x = sel->x;
         sa.ext = ext;
-        std::vector<int64_t> aoff(s1 - s0);
-        int64_t acc = 0;
-        for (int32_t d = s0; d < s1; ++d) {
-          const int64_t nd = w.h_tok_off[d + 1] - w.h_tok_off[d];
-          aoff[d - s0] = acc;
-          acc += nd * nd;
-        }
-        CUDA_TRY(cudaMemcpyAsync(sel->a_off, aoff.data(), sizeof(int64_t) * aoff.size(), cudaMemcpyHostToDevice, st));
-        CUDA_TRY(launch_select(sa, st));
+        CUDA_TRY(launch_select(tm_rows, sa, sms, st));
       }
       AttnArgs aa{};
       aa.items = w.items + (last ? plan.chunk_item[ci] : li0);
@@ -1394,16 +1401,35 @@ dopr_status dopr_select_prefix_inputs(dopr_model* m, int32_t n_docs, const int32
   plan.chunk_litem.assign(1, 0);
   plan.chunk_tile.assign(1, 0);
   plan.chunk_ltile.assign(1, 0);
-  int64_t a_max = 0;
-  int32_t docs_max = 0;
+  int64_t a_max = 0, rows_max = 0;
+  std::vector<int64_t> a_off(n_docs);
+  std::vector<SelUnit> units;
+  std::vector<SelectState::Chunk> chunks;
   for (int32_t s0 = 0; s0 < n_docs;) {
     int32_t s1 = s0 + 1;
     while (s1 < n_docs && w.h_tok_off[s1 + 1] - w.h_tok_off[s0] <= w.chunk_cap) ++s1;
     ap.add(w.h_tok_off, w.h_tok_off[s0], s0, s1, 0, 0, 0);
+    // the chunk's score tiles: row tiles with the most key tiles first, then the column tiles
+    SelectState::Chunk sc{(int64_t)units.size(), 0, 0, 0};
     int64_t a = 0;
-    for (int32_t d = s0; d < s1; ++d) a += (int64_t)(doc_offsets[d + 1] - doc_offsets[d]) * (doc_offsets[d + 1] - doc_offsets[d]);
+    for (int32_t d = s0; d < s1; ++d) {
+      const int32_t nd = doc_offsets[d + 1] - doc_offsets[d];
+      a_off[d] = a;
+      for (int32_t rt = 0; rt * SEL_TILE < nd; ++rt)
+        units.push_back(SelUnit{doc_offsets[d] - doc_offsets[s0], nd, rt, 0, a});
+      a += (int64_t)nd * nd;
+      sc.max_n = std::max(sc.max_n, nd);
+    }
+    sc.n_row_tiles = (int)((int64_t)units.size() - sc.first);
+    std::stable_sort(units.begin() + sc.first, units.end(), [](const SelUnit& x, const SelUnit& y) { return x.rt > y.rt; });
+    for (int i = 0; i < sc.n_row_tiles; ++i) {
+      SelUnit u = units[sc.first + i];
+      for (u.ct = 0; u.ct <= u.rt; ++u.ct) units.push_back(u);
+    }
+    sc.n_tiles = (int)((int64_t)units.size() - sc.first - sc.n_row_tiles);
+    chunks.push_back(sc);
     a_max = std::max(a_max, a);
-    docs_max = std::max(docs_max, s1 - s0);
+    rows_max = std::max<int64_t>(rows_max, w.h_tok_off[s1] - w.h_tok_off[s0]);
     plan.chunk_pair.push_back(s1);
     plan.chunk_item.push_back(0);
     ap.close_chunk(plan);
@@ -1412,11 +1438,16 @@ dopr_status dopr_select_prefix_inputs(dopr_model* m, int32_t n_docs, const int32
   STATUS_TRY(ap.upload(w, plan, 0, st));
   // selection buffers, grown on demand and kept for the next call
   STATUS_TRY(grow_dev(&w.sel_A, w.sel_a_cap, a_max));
-  STATUS_TRY(grow_dev(&w.sel_a_off, w.sel_doc_cap, docs_max));
+  STATUS_TRY(grow_dev(&w.sel_a_off, w.sel_doc_cap, n_docs));
+  STATUS_TRY(grow_dev(&w.sel_units, w.sel_unit_cap, (int64_t)units.size()));
+  STATUS_TRY(grow_dev(&w.sel_stats, w.sel_stat_cap, rows_max * c.n_q_heads));
   STATUS_TRY(grow_dev(&w.sel_u, w.sel_tok_cap, T));
   STATUS_TRY(grow_dev(&w.sel_pos, w.sel_pos_cap, (int64_t)n_docs * top_k));
   STATUS_TRY(grow_dev(&w.sel_x, w.sel_x_cap, (int64_t)n_docs * top_k * H));
-  SelectState sel{top_k, top_p, w.sel_A, a_max, w.sel_a_off, w.sel_u, w.sel_pos, w.sel_x};
+  CUDA_TRY(cudaMemcpyAsync(w.sel_a_off, a_off.data(), sizeof(int64_t) * n_docs, cudaMemcpyHostToDevice, st));
+  CUDA_TRY(cudaMemcpyAsync(w.sel_units, units.data(), sizeof(SelUnit) * units.size(), cudaMemcpyHostToDevice, st));
+  SelectState sel{top_k, top_p, w.sel_A, a_max, w.sel_a_off, w.sel_u, w.sel_pos, w.sel_x, w.sel_units, w.sel_stats,
+                  std::move(chunks)};
   cudaError_t e = cudaMemsetAsync(w.err, 0, sizeof(int), st);
   rs = e == cudaSuccess ? run_layers(m, w.sel_empty, plan, nullptr, st, nullptr, &sel)
                          : fail(DOPR_ERR_CUDA, "memset failed");

@@ -84,6 +84,16 @@ struct Store {
   bool tm_pool_ok = false;
 };
 
+// Key token selection (k_select.cu).
+constexpr int SEL_MAX_N = 2048;  // longest document the selection takes
+constexpr int SEL_TILE = 128;    // rows and key columns of a score tile
+// A 128-row tile (row tile rt of a document at chunk rows [ts, ts + n)) or one 128-column tile ct
+// of it; the document's A-bar, transposed ([column][row]), starts at float a_off of A.
+struct SelUnit {
+  int32_t ts, n, rt, ct;
+  int64_t a_off;
+};
+
 struct Workspace {
   int chunk_cap = 0;  // tokens per chunk
   float* r = nullptr;          // [chunk][H] fp32 residual stream
@@ -129,6 +139,9 @@ struct Workspace {
   float* sel_u = nullptr;      // salience of every token
   int32_t* sel_pos = nullptr;  // [docs][top_k]
   bf16* sel_x = nullptr;       // [docs][top_k][H]
+  SelUnit* sel_units = nullptr;  // score tiles of every chunk
+  float2* sel_stats = nullptr;   // [Hq][rows of the largest chunk]
+  int64_t sel_unit_cap = 0, sel_stat_cap = 0;
   int64_t sel_a_cap = 0, sel_doc_cap = 0, sel_tok_cap = 0, sel_pos_cap = 0, sel_x_cap = 0;
 };
 
@@ -331,15 +344,16 @@ void set_last_error_message(const std::string& msg);
 // Debug kernel: bounded wait on a barrier nothing completes.
 // Key token selection (k_select.cu), per chunk of whole documents (pairs p0 ..
 // p0 + n_docs - 1, chunk rows 0 .. n_rows - 1).
-constexpr int SEL_MAX_N = 2048;  // longest document the selection takes
 struct SelectArgs {
-  const f16* qkv;  // the chunk's q | k | v rows after the last layer's projection
-  int ld_qkv, Hq, Hkv;
+  int Hq, Hkv;
   const int32_t* tok_pair;  // packed token -> document (pair) index
   const int32_t* tok_off;   // document -> first packed token
   int t0, p0, n_docs, n_rows;
   const int64_t* a_off;     // chunk document -> offset of its n x n A-bar in A
   float* A;
+  const SelUnit* row_tiles;  // the chunk's n_row_tiles row tiles, then its n_tiles column tiles
+  int n_row_tiles, n_tiles, max_n;  // max_n: tokens of its longest document
+  float2* stats;            // [Hq][chunk rows]: softmax maximum and 1 / (sum * Hq)
   int top_p, top_k;
   float* u;                 // salience of chunk row t at u[t]
   int32_t* positions;       // [all documents][top_k]
@@ -347,7 +361,9 @@ struct SelectArgs {
   Extents ext;
 };
 cudaError_t select_setup();
-cudaError_t launch_select(const SelectArgs& a, cudaStream_t st);
+// tm_rows: the chunk's packed q | k | v rows after the last layer's projection, box 64 columns x
+// SEL_TILE rows (fp16, 128-byte swizzle).
+cudaError_t launch_select(const CUtensorMap& tm_rows, const SelectArgs& a, int num_sms, cudaStream_t st);
 cudaError_t launch_select_gather(const SelectArgs& a, const float* r, int H, const bf16* gain, float eps,
                                  cudaStream_t st);
 // Prefix build: K/V rows of chunk tokens [0, T) (packed tokens t0 + t) into the store pool.

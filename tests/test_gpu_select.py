@@ -171,3 +171,40 @@ def test_selection_workspace_is_reused_across_calls():
         assert torch.equal(got[1].view(torch.int16), want[1].view(torch.int16)), f"call {i}: states"
         np.testing.assert_array_equal(got[2], want[2], err_msg=f"call {i}: salience")
     model.close()
+
+
+SHAPE_G1 = synth.ModelShape("sel-g1", n_layers=1, hidden=256, n_q_heads=2, n_kv_heads=2, head_dim=128, ffn=128,
+                            vocab=500)
+SHAPE_G16 = synth.ModelShape("sel-g16", n_layers=1, hidden=256, n_q_heads=32, n_kv_heads=2, head_dim=128, ffn=128,
+                             vocab=500)
+
+
+@pytest.mark.parametrize("shape,lens,top_p", [
+    (SHAPE_G1, [127, 128, 129, 1, 2], 10 ** 6), (SHAPE_G1, [255, 256, 257], 31), (SHAPE_G16, [33, 128, 385], 10 ** 6),
+    (SHAPE_G16, [511, 512, 513], 512), (SHAPE_G1, [1023, 1024, 1025, 31, 32], 10 ** 6),
+    (SHAPE_G2, [1024, 130, 7], 1023), (SHAPE_G1, [2047, 2048], 2047)])
+def test_selection_at_tile_and_register_edges(shape, lens, top_p):
+    # Document lengths around the 128-token score tiles and the 512 / 1,024 / 2,048-entry column kernels.
+    # The column mean has a closed form: every row of A-bar sums to 1, so the column sums u_i (n - i) add up to n.
+    # Its fp32 error: the weights' own (ex2 and scale, under 1e-5 relative) and that of the sums; 1e-4 bounds both.
+    w = synth.make_weights(shape, seed=46, norms="random")
+    model = dopr.Model(dopr.make_config(shape, max_position=2048), w)
+    off, tok, docs = _docs(shape, lens, seed=46)
+    K = 100
+    pos, _, u = dopr.select_prefix_inputs(model, off, tok, K, top_p)
+    _, _, mean = dopr.select_prefix_inputs(model, off, tok, K, 10 ** 6)
+    om = oracle.OracleModel(oshape(shape), w)
+    for d, ids in enumerate(docs):
+        n = len(ids)
+        got, mu = (v[off[d]:off[d + 1]].astype(np.float64) for v in (u, mean))
+        assert abs(np.sum(mu * np.arange(n, 0, -1)) - n) <= 1e-4 * n, (d, np.sum(mu * np.arange(n, 0, -1)))
+        want = oracle.select_topk(got, K)  # the ranking of the returned salience, ties to the lower position
+        np.testing.assert_array_equal(pos[d, :min(K, n)], want[:min(K, n)])
+        assert np.all(pos[d, min(K, n):] == -1)
+        if n <= 600:
+            ref = oracle.salience(om.forward(om.embed(ids), 0, want_probs=True)["probs"], top_p)
+            assert np.all(np.abs(got - ref) <= _u_tol(ref)), (d, float(np.max(np.abs(got - ref))))
+        whole = np.arange(n, 0, -1) <= top_p  # columns whose top-p mean is their mean
+        np.testing.assert_allclose(got[whole], mu[whole], rtol=1e-6)
+        assert np.all(got >= mu * (1 - 1e-6))  # the largest entries' mean is no smaller than all entries'
+    model.close()
