@@ -426,6 +426,18 @@ __device__ __forceinline__ void pair_tile_coords(int t, int m_tiles, int n_tiles
   }
 }
 
+// A bounded wait of the whole warp: all lanes go on or give up together.
+__device__ __forceinline__ bool wait_all_lanes(uint32_t bar, uint32_t parity, const GemmParams& p) {
+  return __all_sync(0xffffffffu, mbar_wait_cluster(bar, parity, p.err, p.timeout_ns)) != 0;
+}
+// A producer that gave up: its copies in flight land within microseconds; give them that long
+// before the CTA can reach its exit (no barrier to wait on: they count on the leader's).
+__device__ __forceinline__ void let_copies_land() {
+  const uint64_t t0 = globaltimer_ns();
+  while (globaltimer_ns() - t0 < 20000ull) {
+  }
+}
+
 template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmParams p) {
@@ -486,74 +498,69 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   }
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer (both CTAs): own A rows and own half of B's rows
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int t = pair; t < total && ok; t += n_pairs) {
-        int mb, nb;
-        pair_tile_coords(t, m_tiles, n_tiles, order, mb, nb);
-        for (int kb = 0; kb < k_blocks; ++kb) {
-          if (!mbar_wait_cluster(empty_bar(stage), phase ^ 1u, p.err, p.timeout_ns)) {
-            ok = false;
-            break;
-          }
+    // ---------------- TMA producer (both CTAs): own A rows and own half of B's rows.  Here and
+    // in the issuer the whole warp runs the loop and one lane issues: with the loop's state
+    // warp-uniform an MMA or a copy costs its thread far fewer instructions (in a loop of one
+    // diverged lane an MMA took about 78 clocks to issue).  16,000 rows: N 4,096 K 12,288
+    // 993 -> 967 us, N 6,144 K 4,096 453 -> 443; 4,100 rows, gate/up N 6,144 K 1,024 44.2 -> 40.5.
+    const bool one = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int t = pair; t < total && ok; t += n_pairs) {
+      int mb, nb;
+      pair_tile_coords(t, m_tiles, n_tiles, order, mb, nb);
+      for (int kb = 0; kb < k_blocks; ++kb) {
+        ok = wait_all_lanes(empty_bar(stage), phase ^ 1u, p);
+        if (!ok) break;
+        if (one) {
           if (leader) mbar_arrive_expect_tx(full_bar(stage), 2 * PAIR_STAGE_BYTES);
           const uint32_t fb = mapa_shared(full_bar(stage), 0);
           tma_load_2d_pair(sA + stage * A_BYTES, &tmA, fb, kb * BK, mb * PAIR_BM + static_cast<int>(rank) * BM);
           tma_load_2d_pair(sB + stage * PAIR_B_BYTES, &tmB, fb, kb * BK, nb * BN + static_cast<int>(rank) * BM);
-          if (++stage == PAIR_STAGES) {
-            stage = 0;
-            phase ^= 1u;
-          }
         }
-      }
-      if (!ok) {
-        // copies in flight land within microseconds; give them that long before the
-        // CTA can reach its exit (no barrier to wait on: they count on the leader's)
-        const uint64_t t0 = globaltimer_ns();
-        while (globaltimer_ns() - t0 < 20000ull) {
+        if (++stage == PAIR_STAGES) {
+          stage = 0;
+          phase ^= 1u;
         }
       }
     }
+    if (!ok) let_copies_land();
   } else if (warp == 1) {
-    if (lane == 0 && leader) {
+    if (leader) {
       // ---------------- MMA issuer (leader only)
+      const bool one = elect_one();
       int stage = 0;
       uint32_t phase = 0;
       int local = 0;
       bool ok = true;
       for (int t = pair; t < total && ok; t += n_pairs, ++local) {
         const int acc = local % PAIR_ACCS;
-        const uint32_t acc_phase = (local / PAIR_ACCS) & 1;
-        if (!mbar_wait_cluster(tempty_bar(acc), acc_phase ^ 1u, p.err, p.timeout_ns)) {
-          ok = false;
-          break;
-        }
+        ok = wait_all_lanes(tempty_bar(acc), ((local / PAIR_ACCS) & 1) ^ 1u, p);
+        if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * BN;
         for (int kb = 0; kb < k_blocks; ++kb) {
-          if (!mbar_wait_cluster(full_bar(stage), phase, p.err, p.timeout_ns)) {
-            ok = false;
-            break;
-          }
+          ok = wait_all_lanes(full_bar(stage), phase, p);
+          if (!ok) break;
           tc_fence_after();
-          const uint64_t ad = umma_desc_sw128(sA + stage * A_BYTES);
-          const uint64_t bd = umma_desc_sw128(sB + stage * PAIR_B_BYTES);
+          if (one) {
+            const uint64_t ad = umma_desc_sw128(sA + stage * A_BYTES);
+            const uint64_t bd = umma_desc_sw128(sB + stage * PAIR_B_BYTES);
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k)  // +32 bytes along K per step, in 16-byte units
-            umma_f16_pair(d_tmem, ad + 2 * k, bd + 2 * k, PAIR_IDESC, (kb | k) != 0);
-          umma_commit_pair_mc(empty_bar(stage), 3);  // both CTAs' stage is free once these MMAs end
+            for (int k = 0; k < BK / 16; ++k)  // +32 bytes along K per step, in 16-byte units
+              umma_f16_pair(d_tmem, ad + 2 * k, bd + 2 * k, PAIR_IDESC, (kb | k) != 0);
+            umma_commit_pair_mc(empty_bar(stage), 3);  // both CTAs' stage is free once these MMAs end
+          }
           if (++stage == PAIR_STAGES) {
             stage = 0;
             phase ^= 1u;
           }
         }
-        if (ok) umma_commit_pair_mc(tfull_bar(acc), 3);
+        if (ok && one) umma_commit_pair_mc(tfull_bar(acc), 3);
       }
       // All MMAs this thread issued are complete once drain_bar flips.
-      umma_commit_pair_mc(drain_bar, 1);
+      if (one) umma_commit_pair_mc(drain_bar, 1);
       mbar_wait(drain_bar, 0, p.err, ok ? p.timeout_ns : 100000000ull);
     }
   } else {
