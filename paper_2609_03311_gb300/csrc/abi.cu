@@ -179,14 +179,10 @@ dopr_status build_weight_maps(Model* m) {
   const int H = c.hidden, F = c.ffn, L = c.n_layers;
   m->tm_qkv.resize(L); m->tm_o.resize(L); m->tm_gu.resize(L); m->tm_down.resize(L);
   for (int l = 0; l < L; ++l) {
-    bool ok = make_tmap_16b_2d(&m->tm_qkv[l], m->w_qkv + (size_t)l * m->qkv_dim * H, H, m->qkv_dim, (uint64_t)H * 2,
-                               GEMM_BK, GEMM_B_BOX, true, true) &&
-              make_tmap_16b_2d(&m->tm_o[l], m->w_o + (size_t)l * H * m->o_dim, m->o_dim, H, (uint64_t)m->o_dim * 2,
-                               GEMM_BK, GEMM_B_BOX, true, true) &&
-              make_tmap_16b_2d(&m->tm_gu[l], m->w_gu + (size_t)l * 2 * F * H, H, 2 * F, (uint64_t)H * 2, GEMM_BK,
-                               GEMM_B_BOX, true, true) &&
-              make_tmap_16b_2d(&m->tm_down[l], m->w_down + (size_t)l * H * F, F, H, (uint64_t)F * 2, GEMM_BK,
-                               GEMM_B_BOX, true, true);
+    const bool ok = make_gemm_operand_b(&m->tm_qkv[l], m->w_qkv + (size_t)l * m->qkv_dim * H, H, m->qkv_dim) &&
+                    make_gemm_operand_b(&m->tm_o[l], m->w_o + (size_t)l * H * m->o_dim, m->o_dim, H) &&
+                    make_gemm_operand_b(&m->tm_gu[l], m->w_gu + (size_t)l * 2 * F * H, H, 2 * F) &&
+                    make_gemm_operand_b(&m->tm_down[l], m->w_down + (size_t)l * H * F, F, H);
     if (!ok) return fail(DOPR_ERR_CUDA, "cuTensorMapEncodeTiled failed for layer %d weights", l);
   }
   m->maps_ok = true;
@@ -203,16 +199,17 @@ dopr_status alloc_chunk_buffers(Model* m, int cap) {
   STATUS_TRY(dev_alloc(&w.o, (size_t)cap * m->o_dim));
   STATUS_TRY(dev_alloc(&w.act, (size_t)cap * c.ffn));
   STATUS_TRY(dev_alloc(&w.ss_e, (size_t)cap));
-  const size_t parts = (size_t)(c.hidden / GEMM_BN) * GEMM_SS_PER_TILE;
-  STATUS_TRY(dev_alloc(&w.ss_a, (size_t)cap * parts));
-  STATUS_TRY(dev_alloc(&w.ss_m, (size_t)cap * parts));
+  // partial sums of squares: H / 128 a row, or H / 32 for launches of few rows
+  const size_t sums = std::max((size_t)cap * (c.hidden / GEMM_BN) * GEMM_SS_PER_TILE,
+                               (size_t)GEMM_FEW_MAX_ROWS * (c.hidden / GEMM_FEW_SS_COLS));
+  STATUS_TRY(dev_alloc(&w.ss_a, sums));
+  STATUS_TRY(dev_alloc(&w.ss_m, sums));
   STATUS_TRY(dev_alloc(&w.r_s, (size_t)cap * c.hidden));
-  STATUS_TRY(dev_alloc(&w.ss_s, (size_t)cap * parts));
+  STATUS_TRY(dev_alloc(&w.ss_s, sums));
   STATUS_TRY(dev_alloc(&w.err, 1));
   STATUS_TRY(host_alloc(&w.h_err, 1));
-  bool ok = make_tmap_16b_2d(&w.tm_xn, w.xn, c.hidden, cap, (uint64_t)c.hidden * 2, GEMM_BK, GEMM_BM, true, true) &&
-            make_tmap_16b_2d(&w.tm_o, w.o, m->o_dim, cap, (uint64_t)m->o_dim * 2, GEMM_BK, GEMM_BM, true, true) &&
-            make_tmap_16b_2d(&w.tm_act, w.act, c.ffn, cap, (uint64_t)c.ffn * 2, GEMM_BK, GEMM_BM, true, true);
+  const bool ok = make_gemm_operand_a(&w.tm_xn, w.xn, c.hidden, cap) &&
+                  make_gemm_operand_a(&w.tm_o, w.o, m->o_dim, cap) && make_gemm_operand_a(&w.tm_act, w.act, c.ffn, cap);
   if (!ok) return fail(DOPR_ERR_CUDA, "cuTensorMapEncodeTiled failed for activation buffers");
   return DOPR_OK;
 }
@@ -608,7 +605,10 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
   Workspace& w = m->ws;
   const auto& c = m->cfg;
   const int H = c.hidden, F = c.ffn, L = c.n_layers, Hq = c.n_q_heads, Hkv = c.n_kv_heads;
-  const int parts = H / GEMM_BN * GEMM_SS_PER_TILE;  // partial sums of squares per row from a residual epilogue
+  // partial sums of squares per row from the residual epilogue of a launch of M rows
+  auto parts_of = [&](int M, int K) {
+    return gemm_plan(EPI_RESID_ADD, M, H, K, m->num_sms).few ? H / GEMM_FEW_SS_COLS : H / GEMM_BN * GEMM_SS_PER_TILE;
+  };
   const int mpad = ((s->max_m + 63) / 64) * 64;
   const int sms = m->num_sms;
   const bool scoring = !build && !sel;
@@ -686,6 +686,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
     const auto op_last = gemm_cost(np, H, m->o_dim, np * H * 10.0);
     const auto gu_last = gemm_cost(np, 2.0 * F, H, np * F * 2.0);
     const auto dn_last = gemm_cost(np, H, F, np * H * 8.0);
+    const int parts_a = parts_of(Tc, F);  // of every layer's attention norm but the first's
     for (int l = 0; l < L; ++l) {
       NvtxRange layer_range("dopr layer %d", l);
       // In the last layer only the score-token rows reach the score: after the full QKV
@@ -700,9 +701,9 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
       pq.ld_out = m->qkv_dim;
       if (l > 0) {  // layer 0's operand comes from the embedding, already normalised
         pq.ss_in = w.ss_a;
-        pq.ss_parts = parts;
+        pq.ss_parts = parts_a;
         pq.ss_pre = w.ss_m;
-        pq.ss_pre_parts = parts;
+        pq.ss_pre_parts = parts_of(Tc, m->o_dim);
       }
       pq.tok_pos = w.tok_pos + t0;
       pq.rope = m->rope;
@@ -787,7 +788,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
                              return e;
                            }));
       const float* ss_pre = l == 0 ? w.ss_e : w.ss_a;  // the attention norm of this layer
-      const int ss_pre_parts = l == 0 ? 1 : parts;
+      const int ss_pre_parts = l == 0 ? 1 : parts_a;
       float* resid = w.r;
       int rows = Tc;
       if (last) {
@@ -799,6 +800,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
         resid = w.r_s;
         rows = np;
       }
+      const int parts_m = parts_of(rows, m->o_dim);
       GemmParams po = base;  // O projection + residual, emits the MLP norm's operand
       po.M = rows;
       po.N = H;
@@ -808,7 +810,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
       po.xn_out = w.xn;
       po.xn_gain = m->mlp_norm + (size_t)l * H;
       po.ss_out = w.ss_m;
-      po.ss_out_parts = parts;
+      po.ss_out_parts = parts_m;
       po.ss_pre = ss_pre;
       po.ss_pre_parts = ss_pre_parts;
       CUDA_TRY(prof_launch(m, K_GEMM_O, 1, last ? op_last.first : op.first, last ? op_last.second : op.second, st,
@@ -820,7 +822,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
       pg.out = w.act;
       pg.ld_out = F;
       pg.ss_in = w.ss_m;
-      pg.ss_parts = parts;
+      pg.ss_parts = parts_m;
       pg.ss_pre = ss_pre;
       pg.ss_pre_parts = ss_pre_parts;
       CUDA_TRY(prof_launch(m, K_GEMM_GATE_UP, 1, last ? gu_last.first : gu.first, last ? gu_last.second : gu.second,
@@ -835,9 +837,9 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
         pd.xn_out = w.xn;
         pd.xn_gain = m->attn_norm + (size_t)(l + 1) * H;
         pd.ss_out = w.ss_a;
-        pd.ss_out_parts = parts;
+        pd.ss_out_parts = parts_a;
         pd.ss_pre = w.ss_m;  // the MLP norm of this layer
-        pd.ss_pre_parts = parts;
+        pd.ss_pre_parts = parts_m;
       }
       CUDA_TRY(prof_launch(m, K_GEMM_DOWN, 1, last ? dn_last.first : dn.first, last ? dn_last.second : dn.second, st,
                            [&] { return launch_gemm(EPI_RESID_ADD, w.tm_act, m->tm_down[l], pd, sms, st); }));
@@ -945,6 +947,34 @@ bool make_tmap_16b_2d(CUtensorMap* map, const void* base, uint64_t cols, uint64_
                   swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
+}
+
+// The K-major operand [rows][k] as the 3-D tensor (64 elements, rows, k / 64).
+static bool make_tmap_k_blocks(CUtensorMap* map, const void* base, uint64_t k, uint64_t rows, uint32_t box_rows,
+                               uint32_t box_blocks) {
+  auto fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {GEMM_BK, rows, k / GEMM_BK};
+  cuuint64_t strides[2] = {k * 2, GEMM_BK * 2};
+  cuuint32_t box[3] = {GEMM_BK, box_rows, box_blocks};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
+bool make_gemm_operand_a(GemmOperandA* a, const void* base, uint64_t k, uint64_t rows) {
+  bool ok = make_tmap_16b_2d(&a->wide, base, k, rows, k * 2, GEMM_BK, GEMM_BM, true, true);
+  for (int i = 0; i < 3; ++i) ok = ok && make_tmap_k_blocks(&a->few[i], base, k, rows, 32u << i, GEMM_FEW_KB(32 << i));
+  return ok;
+}
+
+bool make_gemm_operand_b(GemmOperandB* b, const void* base, uint64_t k, uint64_t rows) {
+  bool ok = make_tmap_16b_2d(&b->wide, base, k, rows, k * 2, GEMM_BK, GEMM_B_BOX, true, true);
+  for (int n = 0; n < 2; ++n)
+    for (int kb = 0; kb < 2; ++kb) ok = ok && make_tmap_k_blocks(&b->few[n][kb], base, k, rows, 32u << n, 2u << kb);
+  return ok;
 }
 
 // The Q columns of a packed QKV buffer [rows][cols] as a 3-D tensor: 128 elements of a head
@@ -1626,9 +1656,9 @@ dopr_status dopr_debug_gemm(int32_t M, int32_t N, int32_t K, const void* A, cons
   if (epilogue < 0 || epilogue > 2) return fail(DOPR_ERR_INVALID_ARG, "bad epilogue %d", epilogue);
   if (M == 0) return DOPR_OK;
   if (gemm_setup() != cudaSuccess) return fail(DOPR_ERR_CUDA, "gemm setup failed");
-  CUtensorMap ta, tb;
-  if (!make_tmap_16b_2d(&ta, A, K, M, (uint64_t)K * 2, GEMM_BK, GEMM_BM, true, true) ||
-      !make_tmap_16b_2d(&tb, B, K, N, (uint64_t)K * 2, GEMM_BK, GEMM_B_BOX, true, true))
+  GemmOperandA ta;
+  GemmOperandB tb;
+  if (!make_gemm_operand_a(&ta, A, K, M) || !make_gemm_operand_b(&tb, B, K, N))
     return fail(DOPR_ERR_CUDA, "cuTensorMapEncodeTiled failed (pointers must be 16-byte aligned)");
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);

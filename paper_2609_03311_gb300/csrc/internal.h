@@ -84,6 +84,26 @@ struct Store {
   bool tm_pool_ok = false;
 };
 
+// GEMM epilogues.
+enum GemmEpi : int { EPI_STORE = 0, EPI_RESID_ADD = 1, EPI_SWIGLU = 2, EPI_QKV = 3 };
+constexpr int GEMM_BM = 128, GEMM_BN = 256, GEMM_BK = 64;
+// Rows of a B (weight) tensor-map box: each CTA of a pair stages 128 of a tile's 256 B rows.
+constexpr int GEMM_B_BOX = 128;
+constexpr int GEMM_SS_PER_TILE = 2;  // partial sums of squares a residual epilogue writes per row and n-tile
+constexpr int GEMM_FEW_MAX_ROWS = 1024;  // launches of more rows always take the wide tiles
+constexpr int GEMM_FEW_SS_COLS = 32;     // columns per partial sum of squares k_gemm_few writes (wide: 128)
+__host__ __device__ constexpr int GEMM_FEW_KB(int rows) { return rows == 32 ? 4 : 2; }  // 64-wide k-blocks to a stage of k_gemm_few
+// Tensor maps of a GEMM operand (fp16, 128-byte swizzle): `wide` 2-D boxes of 64 elements x 128
+// rows; `few` 3-D (64 elements, rows, k-blocks of 64) boxes of 64 x R rows x GEMM_FEW_KB(R).
+struct GemmOperandA {
+  CUtensorMap wide{}, few[3]{};  // R = 32, 64, 128
+};
+struct GemmOperandB {
+  CUtensorMap wide{}, few[2][2]{};  // [64 or 128 tile columns: 32 or 64 rows a CTA][2 or 4 k-blocks]
+};
+bool make_gemm_operand_a(GemmOperandA* a, const void* base, uint64_t k, uint64_t rows);
+bool make_gemm_operand_b(GemmOperandB* b, const void* base, uint64_t k, uint64_t rows);
+
 // Key token selection (k_select.cu).
 constexpr int SEL_MAX_N = 2048;  // longest document the selection takes
 constexpr int SEL_TILE = 128;    // rows and key columns of a score tile
@@ -102,11 +122,11 @@ struct Workspace {
   f16* o = nullptr;            // [chunk][Hq*128] attention output
   f16* act = nullptr;          // [chunk][F] SwiGLU output
   float* ss_e = nullptr;       // [chunk] sum of squares of the embedded rows
-  float* ss_a = nullptr;       // [chunk][2H/256] partial sums of squares for the attention norm
+  float* ss_a = nullptr;       // [chunk][H/128] (few rows: [rows][H/32]) partial sums of squares for the attention norm
   float* ss_m = nullptr;       // [chunk][2H/256] partial sums of squares for the MLP norm
   float* r_s = nullptr;        // [chunk][H] score-token rows of the last layer (compact)
   float* ss_s = nullptr;       // [chunk][2H/256] their attention-norm partial sums
-  CUtensorMap tm_xn{}, tm_o{}, tm_act{};
+  GemmOperandA tm_xn, tm_o, tm_act;
   // per call, grown on demand
   int64_t pair_cap = 0, tok_cap = 0, qtok_cap = 0, doc_cap = 0, item_cap = 0;
   int32_t* q_off = nullptr;
@@ -188,7 +208,7 @@ struct Model {
   float mlp_b2 = 0.f;
   float2* rope = nullptr;      // [max_position][64] (cos, sin)
   std::vector<uint8_t> have;   // [kind * L + layer]
-  std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
+  std::vector<GemmOperandB> tm_qkv, tm_o, tm_gu, tm_down;
   bool maps_ok = false;
   Workspace ws;
 };
@@ -201,19 +221,13 @@ bool make_tmap_16b_2d(CUtensorMap* map, const void* base, uint64_t cols, uint64_
 bool make_tmap_q_heads(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint32_t box_rows,
                        uint32_t box_heads);
 
-// GEMM epilogues.
-enum GemmEpi : int { EPI_STORE = 0, EPI_RESID_ADD = 1, EPI_SWIGLU = 2, EPI_QKV = 3 };
-constexpr int GEMM_BM = 128, GEMM_BN = 256, GEMM_BK = 64;
-// Rows of a B (weight) tensor-map box: each CTA of a pair stages 128 of a tile's 256 B rows.
-constexpr int GEMM_B_BOX = 128;
-constexpr int GEMM_SS_PER_TILE = 2;  // partial sums of squares a residual epilogue writes per row and n-tile
 struct GemmParams {
   int M, N, K;
   void* out;          // fp16 [M][ld_out] (store, QKV, SwiGLU: ld_out = N/2) or fp32 residual [M][ld_out]
   int64_t ld_out;
   // Fused RMSNorm.  rs(ss, parts) = rsqrt(sum_i ss[row*parts + i] / norm_dim + eps); a null
   // array means 1.  Producer (residual epilogue): xn_out = f16(r' * xn_gain * rs(ss_pre)) and
-  // ss_out[row*ss_out_parts + n-tile] = partial sum of r'^2.  Consumer: accumulator rows are
+  // ss_out[row*ss_out_parts + i] = partial sums of r'^2 (128 columns each, 32 from k_gemm_few).  Consumer: accumulator rows are
   // scaled by rs(ss_in) / rs(ss_pre), so the operand stays near unit scale in fp16.
   const float* ss_in;
   int ss_parts;
@@ -235,8 +249,15 @@ struct GemmParams {
   uint64_t timeout_ns;
 };
 cudaError_t gemm_setup();
+// The tile a launch of M rows takes: wide (k_gemm_pair, 2 x 128 rows, 256 columns) or, for few
+// rows, 2 x 32, 64 or 128 rows and 64 or 128 columns (k_gemm_few).
+struct GemmPlan {
+  bool few;
+  int rows, cols;  // A rows per CTA of the pair, columns
+};
+GemmPlan gemm_plan(int epi, int M, int N, int K, int num_sms);
 // C[M][N] = A[M][K] * B[N][K]^T followed by the epilogue `epi`.
-cudaError_t launch_gemm(int epi, const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, int num_sms,
+cudaError_t launch_gemm(int epi, const GemmOperandA& A, const GemmOperandB& B, const GemmParams& p, int num_sms,
                         cudaStream_t st);
 
 // Row kernels.

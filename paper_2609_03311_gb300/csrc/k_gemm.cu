@@ -65,14 +65,26 @@ constexpr int BAR_BYTES = 256;
 // sequence made the SwiGLU epilogue outlast short main loops (K = 1,024).
 __device__ __forceinline__ float silu_f(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
 
-// RMSNorm factor of a row from its partial sums of squares, added in index
-// order.  When the count allows, the partials arrive as independent 16-byte
+// RMSNorm factor of a row from its partial sums of squares: one per 128 columns, added in
+// index order, or (from k_gemm_few) one per 32 columns, added by fours first -- the order in
+// which the residual epilogue of a wide tile adds them up itself, so the factor is the same
+// bit for bit.  When the count allows, the partials arrive as independent 16-byte
 // loads (up to 32 in flight) instead of one dependent load per partial.
 __device__ __forceinline__ float norm_factor(const float* ss, int parts, const GemmParams& p, int row) {
   if (!ss) return 1.f;
   const float* s = ss + static_cast<int64_t>(min(row, p.M - 1)) * parts;
   float t = 0.f;
-  if ((parts & 3) == 0) {
+  if (parts * 32 == p.norm_dim) {
+    for (int i = 0; i < parts; i += 32) {  // norm_dim is a multiple of 256, so parts is one of 8
+      float4 v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        v[q] = i + 4 * q < parts ? __ldg(reinterpret_cast<const float4*>(s + i) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (i + 4 * q < parts) t += ((v[q].x + v[q].y) + v[q].z) + v[q].w;
+    }
+  } else if ((parts & 3) == 0) {
     for (int i = 0; i < parts; i += 32) {
       float4 v[8];
 #pragma unroll
@@ -97,17 +109,31 @@ __device__ __forceinline__ float row_scale(const GemmParams& p, int row) {
   return norm_factor(p.ss_in, p.ss_parts, p, row) / norm_factor(p.ss_pre, p.ss_pre_parts, p, row);
 }
 
-// The warp's 32 rows x 32 words sit in `xs` (row-per-lane layout, stride 33).
-// Write them out transposed: lane L covers rows i*4 + L/8 (i = 0..7) and words
-// (L%8)*4 .. +3, i.e. 8 lanes per 128-byte row segment.  Word w of row r goes to
-// dst_lo(r) + w for w < 16 and to dst_hi(r) + (w - 16) for w >= 16 (two 64-byte
-// segments; for one contiguous 128-byte segment pass dst_hi = dst_lo + 16).
-template <typename RowPtr>
-__device__ __forceinline__ void store_words_transposed(const uint32_t* xs, int lane, int row0, int M, RowPtr dst) {
+// Sums over a group of 8 consecutive lanes of the lanes' s[0..7]: lane i of the group gets the
+// sum of the s[i] (7 shuffles).
+__device__ __forceinline__ float group8_sums(const float (&s)[8], int lane) {
+  float a[4], b[2];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int r = i * 4 + (lane >> 3);
-    const int w = (lane & 7) * 4;
+  for (int i = 0; i < 4; ++i)
+    a[i] = (lane & 4 ? s[i + 4] : s[i]) + __shfl_xor_sync(0xffffffffu, lane & 4 ? s[i] : s[i + 4], 4);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    b[i] = (lane & 2 ? a[i + 2] : a[i]) + __shfl_xor_sync(0xffffffffu, lane & 2 ? a[i] : a[i + 2], 2);
+  return (lane & 1 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, lane & 1 ? b[0] : b[1], 1);
+}
+
+// The warp's 32 rows x 32 words sit in `xs` (row-per-lane layout, stride 33).
+// Write the first WORDS words of each row out transposed: with 32 words lane L covers rows
+// i*4 + L/8 (i = 0..7) and words (L%8)*4 .. +3, i.e. 8 lanes per 128-byte row segment
+// (16 words: 4 lanes per 64-byte segment).  dst(r, w) is where word w of row r goes.
+template <int WORDS, typename RowPtr>
+__device__ __forceinline__ void store_words_transposed(const uint32_t* xs, int lane, int row0, int M, RowPtr dst) {
+  constexpr int LANES = WORDS / 4;  // lanes to a row segment
+  static_assert(WORDS == 32 || WORDS == 16, "row segments of 128 or 64 bytes");
+#pragma unroll
+  for (int i = 0; i < LANES; ++i) {
+    const int r = i * (32 / LANES) + lane / LANES;
+    const int w = (lane % LANES) * 4;
     if (row0 + r < M) {
       uint4 v;
       v.x = xs[r * 33 + w + 0];
@@ -126,10 +152,9 @@ struct EpiPre {
   int pos[8];   // QKV: positions of the 8 rows a lane rotates in the transposed layout
 };
 
-template <int EPI>
-__device__ __forceinline__ void epilogue_prefetch(const GemmParams& p, int mb, int nb, int quarter, int part,
-                                                  int lane, EpiPre& pre) {
-  const int row0 = mb * BM + quarter * 32;
+template <int EPI, int BNT>
+__device__ __forceinline__ void epilogue_prefetch(const GemmParams& p, int row0, int nb, int part, int lane,
+                                                  EpiPre& pre) {
   if constexpr (EPI == EPI_RESID_ADD) {
     pre.scale = p.xn_out ? norm_factor(p.ss_pre, p.ss_pre_parts, p, row0 + lane) : 1.f;
   } else if constexpr (EPI == EPI_STORE) {
@@ -138,16 +163,18 @@ __device__ __forceinline__ void epilogue_prefetch(const GemmParams& p, int mb, i
     pre.scale = row_scale(p, row0 + lane);
   }
   if constexpr (EPI == EPI_QKV) {
-    if (nb * BN + part * 128 < p.q_cols + p.k_cols)
+    if (nb * BNT + (BNT == 256 ? part * 128 : 0) < p.q_cols + p.k_cols)
 #pragma unroll
       for (int i = 0; i < 8; ++i) pre.pos[i] = p.tok_pos[min(row0 + i * 4 + (lane >> 3), p.M - 1)];
   }
 }
 
-template <int EPI>
-__device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t taddr, int mb, int nb, int quarter,
-                                              int part, int lane, uint32_t* xs, const EpiPre& pre) {
-  const int row0 = mb * BM + quarter * 32;  // first row of this warp; lane = row - row0 = TMEM lane
+// BNT: columns of the tile, 256 (k_gemm_pair) or 64 / 128 (k_gemm_few).  The arithmetic on a row
+// is the same for every BNT, written with explicit fused operations so that it stays so.
+template <int EPI, int BNT>
+__device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t taddr, int row0, int nb, int part,
+                                              int lane, uint32_t* xs, const EpiPre& pre) {
+  // row0: first row of this warp; lane = row - row0 = TMEM lane
   bool bad = false;  // a value written as fp16 is not finite or beyond 65504 (reported once per tile)
   // this lane's row exists (rows past M hold whatever the operand buffers held there; never stored)
   const bool live = row0 + lane < p.M;
@@ -155,8 +182,10 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
     f16* out = reinterpret_cast<f16*>(p.out);
     const float rs = pre.scale;
     {
-      const int hh = part;                 // this warp's 128-column head of the tile
-      const int hc = nb * BN + hh * 128;  // first output column of this head
+      static_assert(BNT == 256 || BNT == 128, "whole 128-column heads");
+      constexpr bool ONE = BNT == 128;         // one head in the tile, its columns shared by the two parts
+      const int hh = ONE ? 0 : part;           // this warp's 128-column head of the tile
+      const int hc = nb * BNT + hh * 128;      // first output column of this head
       const bool rope = (EPI == EPI_QKV) && hc < p.q_cols + p.k_cols;
       if (rope) {
         // per-head RMSNorm of the row-scaled values: sum of squares in the row layout
@@ -167,9 +196,9 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
           tmem_ld32(taddr + hh * 128 + c, v);
           tmem_ld_wait();
 #pragma unroll
-          for (int j = 0; j < 32; ++j) ss += __uint_as_float(v[j]) * __uint_as_float(v[j]);
+          for (int j = 0; j < 32; ++j) ss = fmaf(__uint_as_float(v[j]), __uint_as_float(v[j]), ss);
         }
-        const float inv_row = rs * rsqrtf(ss * rs * rs * (1.f / 128.f) + p.eps);
+        const float inv_row = rs * rsqrtf(fmaf(ss * rs * rs, 1.f / 128.f, p.eps));
         const bf16* wgt = hc < p.q_cols ? p.q_norm : p.k_norm;
         // the rotation runs in the transposed layout: lane L owns rows i*4 + L/8 and
         // columns w4 .. w4+3 of each 32-column chunk, so RoPE-table reads and the
@@ -179,7 +208,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
 #pragma unroll
         for (int i = 0; i < 8; ++i) inv_i[i] = __shfl_sync(0xffffffffu, inv_row, i * 4 + (lane >> 3));
 #pragma unroll 1
-        for (int c = 0; c < 64; c += 32) {
+        for (int c = ONE ? part * 32 : 0; c < (ONE ? part * 32 + 32 : 64); c += 32) {
           // the rows' (cos, sin) for frequencies c+w4 .. +3 (rows past M read position
           // 0's entries and are not stored), ahead of the accumulator reads below
           float4 c01[8], c23[8];
@@ -227,8 +256,8 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
 #pragma unroll
               for (int k = 0; k < 4; ++k) {
                 const float u = a[k] * inv_i[i] * g1[k], w = b[k] * inv_i[i] * g2[k];
-                y1[k] = u * cosv[k] - w * sinv[k];
-                y2[k] = w * cosv[k] + u * sinv[k];
+                y1[k] = fmaf(u, cosv[k], -(w * sinv[k]));
+                y2[k] = fmaf(w, cosv[k], u * sinv[k]);
                 bad |= !(fp16_ok(y1[k]) && fp16_ok(y2[k]));
               }
               f16* orow = out + static_cast<int64_t>(row0 + r) * p.ld_out + hc + c + w4;
@@ -239,7 +268,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
         }
       } else {
 #pragma unroll 1
-        for (int c = 0; c < 128; c += 64) {
+        for (int c = ONE ? part * 64 : 0; c < (ONE ? part * 64 + 64 : 128); c += 64) {
           uint32_t a[32], b[32];
           tmem_ld32(taddr + hh * 128 + c, a);
           tmem_ld32(taddr + hh * 128 + c + 32, b);
@@ -253,7 +282,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
             xs[lane * 33 + 16 + j / 2] = pack_f16x2(b0, b1);
           }
           __syncwarp();
-          store_words_transposed(xs, lane, row0, p.M, [&](int r, int wd) {
+          store_words_transposed<32>(xs, lane, row0, p.M, [&](int r, int wd) {
             return out + static_cast<int64_t>(row0 + r) * p.ld_out + hc + c + 2 * wd;
           });
           __syncwarp();
@@ -266,18 +295,17 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
     // residual values of chunk c+1 are loaded while chunk c is processed.
     float* res = reinterpret_cast<float*>(p.out);
     const int w4 = (lane & 7) * 4;
-    float ss[8], prev[8];
+    float prev[8], ss128 = 0.f;
     // each lane fetched its own row's previous norm factor; the row layout below takes them by shuffle
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      ss[i] = 0.f;
       prev[i] = __shfl_sync(0xffffffffu, pre.scale, i * 4 + (lane >> 3));
     }
     auto rrow = [&](int i, int c) {
-      return reinterpret_cast<float4*>(res + static_cast<int64_t>(row0 + i * 4 + (lane >> 3)) * p.ld_out + nb * BN +
+      return reinterpret_cast<float4*>(res + static_cast<int64_t>(row0 + i * 4 + (lane >> 3)) * p.ld_out + nb * BNT +
                                        c + w4);
     };
-    const int cbeg = part * (BN / 2), cend = cbeg + BN / 2;  // this warp's half of the columns
+    const int cbeg = part * (BNT / 2), cend = cbeg + BNT / 2;  // this warp's half of the columns
     float4 cur[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
@@ -295,7 +323,8 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
 #pragma unroll
       for (int j = 0; j < 32; ++j) xs[lane * 33 + j] = v[j];
       __syncwarp();
-      const int col = nb * BN + c + w4;
+      const int col = nb * BNT + c + w4;
+      float ss[8];
       float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
       if (p.xn_out) {
         const uint2 gw = *reinterpret_cast<const uint2*>(p.xn_gain + col);
@@ -306,6 +335,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int r = i * 4 + (lane >> 3);
+        ss[i] = 0.f;
         if (row0 + r < p.M) {
           float4 x = cur[i];
           x.x += __uint_as_float(xs[r * 33 + w4 + 0]);
@@ -314,7 +344,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
           x.w += __uint_as_float(xs[r * 33 + w4 + 3]);
           *rrow(i, c) = x;
           if (p.xn_out) {
-            ss[i] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
+            ss[i] = fmaf(x.w, x.w, fmaf(x.z, x.z, fmaf(x.y, x.y, x.x * x.x)));
             const float sc = prev[i];
             const float n0 = x.x * g4.x * sc, n1 = x.y * g4.y * sc, n2 = x.z * g4.z * sc, n3 = x.w * g4.w * sc;
             bad |= !(fp16_ok(n0) && fp16_ok(n1) && fp16_ok(n2) && fp16_ok(n3));
@@ -327,29 +357,30 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
         cur[i] = nxt[i];
       }
       __syncwarp();
-    }
-    if (p.ss_out) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        float t = ss[i];
-        t += __shfl_xor_sync(0xffffffffu, t, 1);
-        t += __shfl_xor_sync(0xffffffffu, t, 2);
-        t += __shfl_xor_sync(0xffffffffu, t, 4);
-        const int r = i * 4 + (lane >> 3);
-        if ((lane & 7) == 0 && row0 + r < p.M)
-          p.ss_out[static_cast<int64_t>(row0 + r) * p.ss_out_parts + nb * GEMM_SS_PER_TILE + part] = t;
+      if (p.ss_out) {  // lane i of each 8 now takes row i * 4 + lane / 8 of these 32 columns
+        const float s32 = group8_sums(ss, lane);
+        ss128 += s32;
+        const int r = (lane & 7) * 4 + (lane >> 3);
+        if (row0 + r < p.M) {
+          if constexpr (BNT < 256)
+            p.ss_out[static_cast<int64_t>(row0 + r) * p.ss_out_parts + (nb * BNT + c) / 32] = s32;
+          else if (c + 32 == cend)
+            p.ss_out[static_cast<int64_t>(row0 + r) * p.ss_out_parts + nb * GEMM_SS_PER_TILE + part] = ss128;
+        }
       }
     }
-  } else {  // EPI_SWIGLU: columns 0..127 gate, 128..255 up of the same 128 outputs
+  } else {  // EPI_SWIGLU: the tile's first half of the columns gate, its second half up of the same outputs
     f16* out = reinterpret_cast<f16*>(p.out);
     const float rs = pre.scale;
-    {
-      const int c = part * 64;  // this warp's 64 of the tile's 128 outputs
+    constexpr int OUTS = BNT / 2;                  // outputs of the tile
+    constexpr int MINE = OUTS >= 64 ? OUTS / 2 : 32;  // of this warp (with 32 in all, part 0 takes them)
+    if (part * MINE < OUTS) {
+      const int c = part * MINE;
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
+      for (int half = 0; half < MINE / 32; ++half) {
         uint32_t g[32], u[32];
         tmem_ld32(taddr + c + 32 * half, g);
-        tmem_ld32(taddr + BN / 2 + c + 32 * half, u);
+        tmem_ld32(taddr + OUTS + c + 32 * half, u);
         tmem_ld_wait();
 #pragma unroll
         for (int j = 0; j < 32; j += 2) {
@@ -360,8 +391,8 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
         }
       }
       __syncwarp();
-      store_words_transposed(xs, lane, row0, p.M, [&](int r, int wd) {
-        return out + static_cast<int64_t>(row0 + r) * p.ld_out + nb * (BN / 2) + c + 2 * wd;
+      store_words_transposed<MINE / 2>(xs, lane, row0, p.M, [&](int r, int wd) {
+        return out + static_cast<int64_t>(row0 + r) * p.ld_out + nb * OUTS + c + 2 * wd;
       });
       __syncwarp();
     }
@@ -572,15 +603,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     for (int t = pair; t < total; t += n_pairs, ++local) {
       int mb2, nb;
       pair_tile_coords(t, m_tiles, n_tiles, order, mb2, nb);
-      const int mb = 2 * mb2 + static_cast<int>(rank);  // this CTA's 128-row block
+      const int row0 = (2 * mb2 + static_cast<int>(rank)) * BM + quarter * 32;  // in this CTA's 128-row block
       const int acc = local % PAIR_ACCS;
       const uint32_t acc_phase = (local / PAIR_ACCS) & 1;
       EpiPre pre;
-      epilogue_prefetch<EPI>(p, mb, nb, quarter, part, lane, pre);
+      epilogue_prefetch<EPI, BN>(p, row0, nb, part, lane, pre);
       if (!mbar_wait_cluster(tfull_bar(acc), acc_phase, p.err, p.timeout_ns)) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BN;
-      epilogue_tile<EPI>(p, taddr, mb, nb, quarter, part, lane, xs, pre);
+      epilogue_tile<EPI, BN>(p, taddr, row0, nb, part, lane, xs, pre);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
@@ -597,9 +628,227 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   }
 }
 
+// ============================================================================
+// Few rows (the last layer's score rows, small batches): the pair kernel with narrower tiles,
+// 64 or 128 columns, and R = 32, 64 or 128 A rows per CTA instead of 128.
+//
+// With few rows a launch is bound by streaming the weights, and 256-column tiles leave most
+// SMs without a tile (O and down of the 8B shape: 16 tiles on 32 of 152 SMs) while each SM
+// takes in operand bytes at no more than about 64 bytes a clock, of which half or more were A
+// rows that hold nothing.  Narrow tiles put 4 times as many SMs to work, and a CTA copies only
+// its R rows (the MMA still runs 128 rows a CTA; what it reads past the R rows is other shared
+// memory, in tile rows that are never stored).  A stage is KB 64-wide k-blocks, so that each
+// operand is one copy of at least 8 KB a stage (a 3-D map: 64 elements, rows, k-blocks).
+// The K order of a row's MMAs is the wide tiles', so its result is the same bit for bit.
+constexpr int FEW_RING = 192 * 1024;
+constexpr int FEW_MAX_STAGES = 12;
+constexpr int FEW_SMEM_BYTES = 1024 + FEW_RING + XPOSE_BYTES + BAR_BYTES;
+static_assert(FEW_SMEM_BYTES <= 227 * 1024, "shared memory budget");
+static_assert((2 * FEW_MAX_STAGES + 5) * 8 + 4 <= BAR_BYTES, "barrier area");
+// The B stages follow the A stages, so the 128 rows that an MMA reads from the start of the last
+// R-row A block (up to 12 KB past it) lie inside the ring.
+
+template <int EPI, int BNT, int R>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
+    k_gemm_few(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmParams p) {
+  constexpr int KB = GEMM_FEW_KB(R);
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  constexpr int a_blk = R * BK * 2, b_blk = BNT / 2 * BK * 2;  // one k-block of this CTA's A rows, of its B rows
+  constexpr int stage_bytes = KB * (a_blk + b_blk);
+  constexpr int stages = FEW_RING / stage_bytes < FEW_MAX_STAGES ? FEW_RING / stage_bytes : FEW_MAX_STAGES;
+  const uint32_t sA = smem_u32(smem);
+  const uint32_t sB = sA + stages * KB * a_blk;
+  uint32_t* xpose = reinterpret_cast<uint32_t*>(smem + FEW_RING);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + FEW_RING + XPOSE_BYTES);
+  const uint32_t bar0 = smem_u32(bars);
+  auto full_bar = [&](int s) { return bar0 + 8u * s; };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (FEW_MAX_STAGES + s); };
+  auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * FEW_MAX_STAGES + a); };
+  auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * FEW_MAX_STAGES + 2 + a); };
+  const uint32_t drain_bar = bar0 + 8u * (2 * FEW_MAX_STAGES + 4);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * FEW_MAX_STAGES + 5);
+  constexpr uint32_t TMEM_COLS = PAIR_ACCS * BNT;
+  constexpr uint32_t IDESC = umma_idesc_f16(PAIR_BM, BNT);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const bool leader = rank == 0;
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int m_tiles = (p.M + 2 * R - 1) / (2 * R), k_blocks = p.K / BK, k_steps = (k_blocks + KB - 1) / KB;
+  int total = m_tiles * (p.N / BNT);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(full_bar(s), 1);
+      mbar_init(empty_bar(s), 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(tfull_bar(a), 1);
+      mbar_init(tempty_bar(a), 2 * EPI_WARPS);
+    }
+    mbar_init(drain_bar, 1);
+    fence_mbar_init();
+    tma_prefetch_desc(&tmA);
+    tma_prefetch_desc(&tmB);
+  }
+  if (warp == 1) {
+    tmem_alloc_pair(smem_u32(tmem_slot), TMEM_COLS);
+    tmem_relinquish_pair();
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();  // both CTAs' barriers exist before either addresses the other's
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  {
+    uint32_t other;  // as in k_gemm_pair: both allocations must agree
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(other) : "r"(mapa_shared(smem_u32(tmem_slot), rank ^ 1u)));
+    if (other != tmem_base) {
+      if (threadIdx.x == 0) atomicOr(p.err, DEV_ERR_BOUNDS);
+      total = 0;  // no tile runs
+    }
+  }
+
+  if (warp == 0) {
+    // ---------------- TMA producer (both CTAs): own A rows and own half of B's rows
+    const bool one = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int t = pair; t < total && ok; t += n_pairs) {
+      const int nb = t / m_tiles, row = (t % m_tiles) * 2 * R + static_cast<int>(rank) * R;
+      // SwiGLU weights hold gate and up in alternating blocks of 128 rows: rank 0 takes gate rows, rank 1 up rows
+      const int o = nb * (BNT / 2);
+      const int brow = EPI == EPI_SWIGLU ? (o / 128) * 256 + o % 128 + static_cast<int>(rank) * 128
+                                         : nb * BNT + static_cast<int>(rank) * (BNT / 2);
+      for (int ks = 0; ks < k_steps; ++ks) {
+        ok = wait_all_lanes(empty_bar(stage), phase ^ 1u, p);
+        if (!ok) break;
+        if (one) {
+          // k-blocks past K are filled with zeros and count as copied
+          if (leader) mbar_arrive_expect_tx(full_bar(stage), 2 * stage_bytes);
+          const uint32_t fb = mapa_shared(full_bar(stage), 0);
+          tma_load_3d_pair(sB + stage * KB * b_blk, &tmB, fb, 0, brow, ks * KB);
+          tma_load_3d_pair(sA + stage * KB * a_blk, &tmA, fb, 0, row, ks * KB);
+        }
+        if (++stage == stages) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+    }
+    if (!ok) let_copies_land();
+  } else if (warp == 1) {
+    if (leader) {
+      // ---------------- MMA issuer (leader only): the whole warp runs the loop, so that its state
+      // and the operand descriptors stay warp-uniform; one lane issues
+      const bool one = elect_one();
+      int stage = 0;
+      uint32_t phase = 0;
+      int local = 0;
+      bool ok = true;
+      for (int t = pair; t < total && ok; t += n_pairs, ++local) {
+        const int acc = local % PAIR_ACCS;
+        ok = wait_all_lanes(tempty_bar(acc), ((local / PAIR_ACCS) & 1) ^ 1u, p);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d_tmem = tmem_base + acc * BNT;
+        for (int ks = 0; ks < k_steps; ++ks) {
+          ok = wait_all_lanes(full_bar(stage), phase, p);
+          if (!ok) break;
+          tc_fence_after();
+          if (one) {
+            const uint64_t ad = umma_desc_sw128(sA + stage * KB * a_blk);
+            const uint64_t bd = umma_desc_sw128(sB + stage * KB * b_blk);
+            const int left = k_blocks - ks * KB;
+#pragma unroll
+            for (int kb = 0; kb < KB; ++kb)
+              if (kb < left) {
+#pragma unroll
+                for (int k = 0; k < BK / 16; ++k)
+                  umma_f16_pair(d_tmem, ad + (kb * (a_blk / 16) + 2 * k), bd + (kb * (b_blk / 16) + 2 * k), IDESC,
+                                (ks | kb | k) != 0);
+              }
+            umma_commit_pair_mc(empty_bar(stage), 3);  // both CTAs' stage is free once these MMAs end
+          }
+          if (++stage == stages) {
+            stage = 0;
+            phase ^= 1u;
+          }
+        }
+        if (ok && one) umma_commit_pair_mc(tfull_bar(acc), 3);
+      }
+      if (one) umma_commit_pair_mc(drain_bar, 1);
+      mbar_wait(drain_bar, 0, p.err, ok ? p.timeout_ns : 100000000ull);
+    }
+  } else {
+    // ---------------- epilogue warps 2..9 (both CTAs) on this CTA's R rows of the tile
+    const int quarter = warp & 3;
+    const int part = (warp - 2) >> 2;
+    uint32_t* xs = xpose + (warp - 2) * XPOSE_WORDS;
+    int local = 0;
+    for (int t = pair; t < total; t += n_pairs, ++local) {
+      const int nb = t / m_tiles, row0 = (t % m_tiles) * 2 * R + static_cast<int>(rank) * R + quarter * 32;
+      const bool mine = quarter * 32 < R && row0 < p.M;  // a quarter with rows of the tile (R is a multiple of 32)
+      const int acc = local % PAIR_ACCS;
+      EpiPre pre;
+      if (mine) epilogue_prefetch<EPI, BNT>(p, row0, nb, part, lane, pre);
+      if (!mbar_wait_cluster(tfull_bar(acc), (local / PAIR_ACCS) & 1, p.err, p.timeout_ns)) break;
+      tc_fence_after();
+      const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BNT;
+      if (mine) epilogue_tile<EPI, BNT>(p, taddr, row0, nb, part, lane, xs, pre);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();  // neither CTA leaves while the other may still address its barriers or TMEM
+  tc_fence_after();
+  if (warp == 1) {
+    __syncwarp();
+    tmem_dealloc_pair(tmem_base, TMEM_COLS);
+  }
+}
+
+// f(kernel) for the few-rows kernel of a plan.
+template <int EPI, typename F>
+auto few_kernel(int rows, int cols, F&& f) {
+  if constexpr (EPI == EPI_RESID_ADD || EPI == EPI_SWIGLU)
+    if (cols == 64) return rows == 32 ? f(k_gemm_few<EPI, 64, 32>) : rows == 64 ? f(k_gemm_few<EPI, 64, 64>) : f(k_gemm_few<EPI, 64, 128>);
+  return rows == 32 ? f(k_gemm_few<EPI, 128, 32>) : rows == 64 ? f(k_gemm_few<EPI, 128, 64>) : f(k_gemm_few<EPI, 128, 128>);
+}
+
 template <int EPI>
 cudaError_t set_smem() {
-  return cudaFuncSetAttribute(k_gemm_pair<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, PAIR_SMEM_BYTES);
+  cudaError_t e = cudaFuncSetAttribute(k_gemm_pair<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, PAIR_SMEM_BYTES);
+  for (int rows = 32; rows <= BM; rows *= 2)
+    for (int cols = 64; cols <= 128; cols *= 2)
+      if (e == cudaSuccess)
+        e = few_kernel<EPI>(rows, cols, [](auto* k) {
+          return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, FEW_SMEM_BYTES);
+        });
+  return e;
+}
+
+template <int EPI>
+void launch_epi(const GemmOperandA& A, const GemmOperandB& B, const GemmParams& p, const GemmPlan& g, int num_sms,
+                cudaStream_t st) {
+  const int tiles = ((p.M + 2 * g.rows - 1) / (2 * g.rows)) * (p.N / g.cols);
+  const int grid = 2 * (tiles < num_sms / 2 ? tiles : num_sms / 2 > 0 ? num_sms / 2 : 1);
+  if (!g.few) {
+    k_gemm_pair<EPI><<<grid, THREADS, PAIR_SMEM_BYTES, st>>>(A.wide, B.wide, p);
+    return;
+  }
+  const CUtensorMap& ta = A.few[g.rows == 32 ? 0 : g.rows == 64 ? 1 : 2];
+  const CUtensorMap& tb = B.few[g.cols == 128][GEMM_FEW_KB(g.rows) == 4];
+  few_kernel<EPI>(g.rows, g.cols, [&](auto* k) {
+    k<<<grid, THREADS, FEW_SMEM_BYTES, st>>>(ta, tb, p);
+    return 0;
+  });
 }
 
 }  // namespace
@@ -612,27 +861,54 @@ cudaError_t gemm_setup() {
   return set_smem<EPI_QKV>();
 }
 
-cudaError_t launch_gemm(int epi, const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& params,
-                        int num_sms, cudaStream_t st) {
+// The clocks a CTA pair needs for a 64-wide k-block of a tile of 2 R rows and n columns: its SMs
+// take in R + n / 2 operand rows of 128 bytes at about 64 bytes a clock, and the four MMAs take
+// 512 at n = 256 but 288 at 128 and 192 at 64 (each reads 128 A rows a CTA, whatever R is).
+// Every tile adds a start and an epilogue that is not hidden, about 2,000 clocks.  The tile
+// with the least clocks over the launch's rounds is taken; the wide one unless a narrow one
+// saves a tenth (its L2 reuse is better).  Measured (cold cache, wide / taken): N 4,096
+// K 12,288, 25 rows 63.7 / 30.5 us, 180 rows 66.0 / 42.2 us; N 4,096 K 4,096, 25 rows
+// 28.0 / 14.5 us; gate/up N 24,576 K 4,096, 25 rows 59.0 / 47.6 us.
+GemmPlan gemm_plan(int epi, int M, int N, int K, int num_sms) {
+  const int64_t pairs = num_sms / 2 > 0 ? num_sms / 2 : 1;
+  auto clocks = [&](int R, int n) {
+    const int64_t tiles = static_cast<int64_t>((M + 2 * R - 1) / (2 * R)) * (N / n);
+    const int64_t in = 2 * (R + n / 2), mma = n == BN ? 2 * BN : 96 + 3 * n / 2;
+    return (tiles + pairs - 1) / pairs * (K / BK * (in > mma ? in : mma) + 2000);
+  };
+  GemmPlan best{false, BM, BN};
+  if (M > GEMM_FEW_MAX_ROWS) return best;
+  int64_t least = clocks(BM, BN) * 9 / 10;
+  const int cols[2] = {128, 64};
+  for (int n : cols) {
+    if (N % n || (n == 64 && epi != EPI_RESID_ADD && epi != EPI_SWIGLU)) continue;
+    for (int R = 32; R <= BM; R *= 2)
+      if (clocks(R, n) < least) {
+        least = clocks(R, n);
+        best = GemmPlan{true, R, n};
+      }
+  }
+  return best;
+}
+
+cudaError_t launch_gemm(int epi, const GemmOperandA& A, const GemmOperandB& B, const GemmParams& params, int num_sms,
+                        cudaStream_t st) {
   if (params.M <= 0) return cudaSuccess;
   GemmParams p = params;
   p.timeout_ns = WAIT_TIMEOUT_NS;
-  // one CTA pair per two SMs (persistent), never more pairs than 256-row tiles
-  const int tiles = ((p.M + PAIR_BM - 1) / PAIR_BM) * (p.N / BN);
-  const int pairs = tiles < num_sms / 2 ? tiles : num_sms / 2;
-  const int grid = 2 * (pairs > 0 ? pairs : 1);
+  const GemmPlan g = gemm_plan(epi, p.M, p.N, p.K, num_sms);
   switch (epi) {
     case EPI_STORE:
-      k_gemm_pair<EPI_STORE><<<grid, THREADS, PAIR_SMEM_BYTES, st>>>(tmA, tmB, p);
+      launch_epi<EPI_STORE>(A, B, p, g, num_sms, st);
       break;
     case EPI_RESID_ADD:
-      k_gemm_pair<EPI_RESID_ADD><<<grid, THREADS, PAIR_SMEM_BYTES, st>>>(tmA, tmB, p);
+      launch_epi<EPI_RESID_ADD>(A, B, p, g, num_sms, st);
       break;
     case EPI_SWIGLU:
-      k_gemm_pair<EPI_SWIGLU><<<grid, THREADS, PAIR_SMEM_BYTES, st>>>(tmA, tmB, p);
+      launch_epi<EPI_SWIGLU>(A, B, p, g, num_sms, st);
       break;
     default:
-      k_gemm_pair<EPI_QKV><<<grid, THREADS, PAIR_SMEM_BYTES, st>>>(tmA, tmB, p);
+      launch_epi<EPI_QKV>(A, B, p, g, num_sms, st);
       break;
   }
   return cudaGetLastError();

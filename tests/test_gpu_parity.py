@@ -371,3 +371,25 @@ def test_bounded_wait_gives_up_and_context_survives():
     out = dopr.gemm(A, B)
     torch.cuda.synchronize()
     assert torch.allclose(out.float(), (A.float() @ B.float().T), rtol=1e-2, atol=1e-1)
+
+
+@pytest.mark.parametrize("N,K", [(256, 64), (512, 320), (1024, 3072), (2560, 1024), (4096, 2048)])
+def test_gemm_few_rows_match_wide_tiles_bit_for_bit(N, K):
+    # Launches of few rows take narrow tiles (64 or 128 columns, 32 to 128 rows a CTA), chosen by size; more than
+    # 1,024 rows always take the wide ones.  A row's K order is the same in all, so its result is too.  K = 320 is not
+    # a whole number of the narrow kernel's 128- or 256-element stages.
+    g = torch.Generator(device="cuda").manual_seed(N + K)
+    A = torch.randn(1300, K, device="cuda", generator=g).to(torch.float16)
+    B = (0.05 * torch.randn(N, K, device="cuda", generator=g)).to(torch.float16)
+    R = torch.randn(1300, N, device="cuda", generator=g)
+
+    def run(M, epi):
+        return dopr.gemm(A[:M].contiguous(), B, epi, out=R[:M].clone() if epi == dopr.EPI_RESID_ADD else None)
+
+    for epi in (dopr.EPI_STORE, dopr.EPI_RESID_ADD, dopr.EPI_SWIGLU):
+        wide = run(1300, epi)
+        for M in (1, 31, 32, 33, 64, 65, 127, 128, 129, 255, 256, 257, 640, 1023, 1024):
+            assert torch.equal(run(M, epi), wide[:M]), (epi, M)
+    ref = _ref_gemm(A, B)
+    err = (run(33, dopr.EPI_STORE).double() - ref[:33]).abs()
+    assert torch.all(err <= ref[:33].abs() * 2 ** -10 + 1e-4 * ref.abs().max()), float(err.max())
