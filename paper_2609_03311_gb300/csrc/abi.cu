@@ -151,8 +151,8 @@ void free_workspace(Workspace& w) {
   dev_free(w.ss_e); dev_free(w.ss_a); dev_free(w.ss_m); dev_free(w.r_s); dev_free(w.ss_s);
   dev_free(w.q_off); dev_free(w.q_tok); dev_free(w.doc_ids); dev_free(w.scores);
   dev_free(w.pair_slot); dev_free(w.perm); dev_free(w.sorted_slot); dev_free(w.tok_off);
-  dev_free(w.tok_id); dev_free(w.tok_pos); dev_free(w.tok_pair); dev_free(w.doc_count);
-  dev_free(w.items); dev_free(w.tiles); dev_free(w.err);
+  dev_free(w.tok_id); dev_free(w.tok_pos); dev_free(w.tok_pair);
+  dev_free(w.items); dev_free(w.tiles); dev_free(w.err); dev_free(w.ss_chunks);
   host_free(w.h_tok_off); host_free(w.h_sorted_slot); host_free(w.h_err); host_free(w.h_items);
   host_free(w.h_tiles);
   dev_free(w.sel_A); dev_free(w.sel_a_off); dev_free(w.sel_u); dev_free(w.sel_pos); dev_free(w.sel_x);
@@ -199,14 +199,15 @@ dopr_status alloc_chunk_buffers(Model* m, int cap) {
   STATUS_TRY(dev_alloc(&w.o, (size_t)cap * m->o_dim));
   STATUS_TRY(dev_alloc(&w.act, (size_t)cap * c.ffn));
   STATUS_TRY(dev_alloc(&w.ss_e, (size_t)cap));
-  // partial sums of squares: H / 128 a row, or H / 32 for launches of few rows
-  const size_t sums = std::max((size_t)cap * (c.hidden / GEMM_BN) * GEMM_SS_PER_TILE,
-                               (size_t)GEMM_FEW_MAX_ROWS * (c.hidden / GEMM_FEW_SS_COLS));
+  const size_t sums = (size_t)cap * (c.hidden / GEMM_BN) * GEMM_SS_PER_TILE;
   STATUS_TRY(dev_alloc(&w.ss_a, sums));
   STATUS_TRY(dev_alloc(&w.ss_m, sums));
   STATUS_TRY(dev_alloc(&w.r_s, (size_t)cap * c.hidden));
   STATUS_TRY(dev_alloc(&w.ss_s, sums));
-  STATUS_TRY(dev_alloc(&w.err, 1));
+  const size_t few_groups = (size_t)GEMM_FEW_MAX_ROWS / 32 * (c.hidden / 128);
+  w.err_bytes = sizeof(int) * (64 + few_groups);
+  STATUS_TRY(dev_alloc(&w.err, 64 + few_groups));
+  STATUS_TRY(dev_alloc(&w.ss_chunks, few_groups * 1024));
   STATUS_TRY(host_alloc(&w.h_err, 1));
   const bool ok = make_gemm_operand_a(&w.tm_xn, w.xn, c.hidden, cap) &&
                   make_gemm_operand_a(&w.tm_o, w.o, m->o_dim, cap) && make_gemm_operand_a(&w.tm_act, w.act, c.ffn, cap);
@@ -521,7 +522,7 @@ struct AttnPlanner {
 dopr_status run_packer(Model* m, Store* s, int32_t n, const int32_t* dqo, const int32_t* dqt, const int64_t* ddoc,
                        cudaStream_t st, Plan& plan) {
   Workspace& w = m->ws;
-  CUDA_TRY(cudaMemsetAsync(w.err, 0, sizeof(int), st));
+  CUDA_TRY(cudaMemsetAsync(w.err, 0, w.err_bytes, st));
   PackArgs a = pack_args(m, s, n, dqo, dqt, ddoc);
   CUDA_TRY(prof_launch(m, K_PACK, 4, 0.0, 24.0 * n, st, [&] { return launch_pack_order(a, st); }));
   CUDA_TRY(cudaMemcpyAsync(w.h_tok_off, w.tok_off, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToHost, st));
@@ -605,10 +606,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
   Workspace& w = m->ws;
   const auto& c = m->cfg;
   const int H = c.hidden, F = c.ffn, L = c.n_layers, Hq = c.n_q_heads, Hkv = c.n_kv_heads;
-  // partial sums of squares per row from the residual epilogue of a launch of M rows
-  auto parts_of = [&](int M, int K) {
-    return gemm_plan(EPI_RESID_ADD, M, H, K, m->num_sms).few ? H / GEMM_FEW_SS_COLS : H / GEMM_BN * GEMM_SS_PER_TILE;
-  };
+  const int parts = H / GEMM_BN * GEMM_SS_PER_TILE;  // partial sums of squares per row from a residual epilogue
   const int mpad = ((s->max_m + 63) / 64) * 64;
   const int sms = m->num_sms;
   const bool scoring = !build && !sel;
@@ -643,6 +641,8 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
     ext.a_elems = sel ? sel->a_elems : 0;
     CUDA_TRY(prof_launch(m, K_EMBED_NORM, 1, 0.0, T * H * 8.0, st, [&] {
       return launch_embed(w.tok_id + t0, Tc, build ? build->x : m->embed, m->attn_norm, H, c.rms_eps, w.r, w.xn,
+    base.ss_chunks = w.ss_chunks;
+    base.ss_count = w.err + 64;
                           w.ss_e, ext, st);
     }));
     GemmParams base{};
@@ -686,7 +686,6 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
     const auto op_last = gemm_cost(np, H, m->o_dim, np * H * 10.0);
     const auto gu_last = gemm_cost(np, 2.0 * F, H, np * F * 2.0);
     const auto dn_last = gemm_cost(np, H, F, np * H * 8.0);
-    const int parts_a = parts_of(Tc, F);  // of every layer's attention norm but the first's
     for (int l = 0; l < L; ++l) {
       NvtxRange layer_range("dopr layer %d", l);
       // In the last layer only the score-token rows reach the score: after the full QKV
@@ -701,9 +700,9 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
       pq.ld_out = m->qkv_dim;
       if (l > 0) {  // layer 0's operand comes from the embedding, already normalised
         pq.ss_in = w.ss_a;
-        pq.ss_parts = parts_a;
+        pq.ss_parts = parts;
         pq.ss_pre = w.ss_m;
-        pq.ss_pre_parts = parts_of(Tc, m->o_dim);
+        pq.ss_pre_parts = parts;
       }
       pq.tok_pos = w.tok_pos + t0;
       pq.rope = m->rope;
@@ -788,7 +787,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
                              return e;
                            }));
       const float* ss_pre = l == 0 ? w.ss_e : w.ss_a;  // the attention norm of this layer
-      const int ss_pre_parts = l == 0 ? 1 : parts_a;
+      const int ss_pre_parts = l == 0 ? 1 : parts;
       float* resid = w.r;
       int rows = Tc;
       if (last) {
@@ -800,7 +799,6 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
         resid = w.r_s;
         rows = np;
       }
-      const int parts_m = parts_of(rows, m->o_dim);
       GemmParams po = base;  // O projection + residual, emits the MLP norm's operand
       po.M = rows;
       po.N = H;
@@ -810,7 +808,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
       po.xn_out = w.xn;
       po.xn_gain = m->mlp_norm + (size_t)l * H;
       po.ss_out = w.ss_m;
-      po.ss_out_parts = parts_m;
+      po.ss_out_parts = parts;
       po.ss_pre = ss_pre;
       po.ss_pre_parts = ss_pre_parts;
       CUDA_TRY(prof_launch(m, K_GEMM_O, 1, last ? op_last.first : op.first, last ? op_last.second : op.second, st,
@@ -822,7 +820,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
       pg.out = w.act;
       pg.ld_out = F;
       pg.ss_in = w.ss_m;
-      pg.ss_parts = parts_m;
+      pg.ss_parts = parts;
       pg.ss_pre = ss_pre;
       pg.ss_pre_parts = ss_pre_parts;
       CUDA_TRY(prof_launch(m, K_GEMM_GATE_UP, 1, last ? gu_last.first : gu.first, last ? gu_last.second : gu.second,
@@ -837,9 +835,9 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
         pd.xn_out = w.xn;
         pd.xn_gain = m->attn_norm + (size_t)(l + 1) * H;
         pd.ss_out = w.ss_a;
-        pd.ss_out_parts = parts_a;
+        pd.ss_out_parts = parts;
         pd.ss_pre = w.ss_m;  // the MLP norm of this layer
-        pd.ss_pre_parts = parts_m;
+        pd.ss_pre_parts = parts;
       }
       CUDA_TRY(prof_launch(m, K_GEMM_DOWN, 1, last ? dn_last.first : dn.first, last ? dn_last.second : dn.second, st,
                            [&] { return launch_gemm(EPI_RESID_ADD, w.tm_act, m->tm_down[l], pd, sms, st); }));
@@ -1354,7 +1352,7 @@ dopr_status dopr_build_prefixes(dopr_model* m, dopr_store* s, int32_t n_docs, co
       }
       dx = stage;
     }
-    CUDA_TRY(cudaMemsetAsync(w.err, 0, sizeof(int), st));
+    CUDA_TRY(cudaMemsetAsync(w.err, 0, w.err_bytes, st));
     BuildArgs b{dx, (int64_t)rows};
     const dopr_status rs = run_layers(m, s, plan, nullptr, st, &b);
     cudaError_t e = cudaMemcpyAsync(w.h_err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -1478,7 +1476,7 @@ dopr_status dopr_select_prefix_inputs(dopr_model* m, int32_t n_docs, const int32
   CUDA_TRY(cudaMemcpyAsync(w.sel_units, units.data(), sizeof(SelUnit) * units.size(), cudaMemcpyHostToDevice, st));
   SelectState sel{top_k, top_p, w.sel_A, a_max, w.sel_a_off, w.sel_u, w.sel_pos, w.sel_x, w.sel_units, w.sel_stats,
                   std::move(chunks)};
-  cudaError_t e = cudaMemsetAsync(w.err, 0, sizeof(int), st);
+  cudaError_t e = cudaMemsetAsync(w.err, 0, w.err_bytes, st);
   rs = e == cudaSuccess ? run_layers(m, w.sel_empty, plan, nullptr, st, nullptr, &sel)
                          : fail(DOPR_ERR_CUDA, "memset failed");
   if (rs == DOPR_OK) {

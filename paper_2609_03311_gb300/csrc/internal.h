@@ -91,7 +91,6 @@ constexpr int GEMM_BM = 128, GEMM_BN = 256, GEMM_BK = 64;
 constexpr int GEMM_B_BOX = 128;
 constexpr int GEMM_SS_PER_TILE = 2;  // partial sums of squares a residual epilogue writes per row and n-tile
 constexpr int GEMM_FEW_MAX_ROWS = 1024;  // launches of more rows always take the wide tiles
-constexpr int GEMM_FEW_SS_COLS = 32;     // columns per partial sum of squares k_gemm_few writes (wide: 128)
 __host__ __device__ constexpr int GEMM_FEW_KB(int rows) { return rows == 32 ? 4 : 2; }  // 64-wide k-blocks to a stage of k_gemm_few
 // Tensor maps of a GEMM operand (fp16, 128-byte swizzle): `wide` 2-D boxes of 64 elements x 128
 // rows; `few` 3-D (64 elements, rows, k-blocks of 64) boxes of 64 x R rows x GEMM_FEW_KB(R).
@@ -122,7 +121,7 @@ struct Workspace {
   f16* o = nullptr;            // [chunk][Hq*128] attention output
   f16* act = nullptr;          // [chunk][F] SwiGLU output
   float* ss_e = nullptr;       // [chunk] sum of squares of the embedded rows
-  float* ss_a = nullptr;       // [chunk][H/128] (few rows: [rows][H/32]) partial sums of squares for the attention norm
+  float* ss_a = nullptr;       // [chunk][H/128] partial sums of squares for the attention norm
   float* ss_m = nullptr;       // [chunk][2H/256] partial sums of squares for the MLP norm
   float* r_s = nullptr;        // [chunk][H] score-token rows of the last layer (compact)
   float* ss_s = nullptr;       // [chunk][2H/256] their attention-norm partial sums
@@ -145,6 +144,8 @@ struct Workspace {
   AttnTile* tiles = nullptr;     // tensor-core attention tiles of the call
   int64_t tile_cap = 0;
   int* err = nullptr;
+  size_t err_bytes = 0;
+  float* ss_chunks = nullptr;  // [GEMM_FEW_MAX_ROWS / 32][H/128][1024]
   // pinned host staging
   int32_t* h_tok_off = nullptr;
   int32_t* h_sorted_slot = nullptr;
@@ -227,7 +228,7 @@ struct GemmParams {
   int64_t ld_out;
   // Fused RMSNorm.  rs(ss, parts) = rsqrt(sum_i ss[row*parts + i] / norm_dim + eps); a null
   // array means 1.  Producer (residual epilogue): xn_out = f16(r' * xn_gain * rs(ss_pre)) and
-  // ss_out[row*ss_out_parts + i] = partial sums of r'^2 (128 columns each, 32 from k_gemm_few).  Consumer: accumulator rows are
+  // ss_out[row*ss_out_parts + i] = partial sums of r'^2, one per 128 columns.  Consumer: accumulator rows are
   // scaled by rs(ss_in) / rs(ss_pre), so the operand stays near unit scale in fp16.
   const float* ss_in;
   int ss_parts;
@@ -239,6 +240,10 @@ struct GemmParams {
   const bf16* xn_gain;
   float* ss_out;
   int ss_out_parts;
+  // k_gemm_few: per 32 rows and 128 columns, the four 32-column chunks' sums on their way to
+  // ss_out (1,024 floats) and how many are there (0 between launches)
+  float* ss_chunks;
+  int* ss_count;
   // QKV epilogue: per-head RMSNorm gains and RoPE at tok_pos[row]
   const int32_t* tok_pos;
   const float2* rope;

@@ -65,26 +65,14 @@ constexpr int BAR_BYTES = 256;
 // sequence made the SwiGLU epilogue outlast short main loops (K = 1,024).
 __device__ __forceinline__ float silu_f(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
 
-// RMSNorm factor of a row from its partial sums of squares: one per 128 columns, added in
-// index order, or (from k_gemm_few) one per 32 columns, added by fours first -- the order in
-// which the residual epilogue of a wide tile adds them up itself, so the factor is the same
-// bit for bit.  When the count allows, the partials arrive as independent 16-byte
+// RMSNorm factor of a row from its partial sums of squares (one per 128 columns), added in index
+// order.  When the count allows, the partials arrive as independent 16-byte
 // loads (up to 32 in flight) instead of one dependent load per partial.
 __device__ __forceinline__ float norm_factor(const float* ss, int parts, const GemmParams& p, int row) {
   if (!ss) return 1.f;
   const float* s = ss + static_cast<int64_t>(min(row, p.M - 1)) * parts;
   float t = 0.f;
-  if (parts * 32 == p.norm_dim) {
-    for (int i = 0; i < parts; i += 32) {  // norm_dim is a multiple of 256, so parts is one of 8
-      float4 v[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        v[q] = i + 4 * q < parts ? __ldg(reinterpret_cast<const float4*>(s + i) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (i + 4 * q < parts) t += ((v[q].x + v[q].y) + v[q].z) + v[q].w;
-    }
-  } else if ((parts & 3) == 0) {
+  if ((parts & 3) == 0) {
     for (int i = 0; i < parts; i += 32) {
       float4 v[8];
 #pragma unroll
@@ -109,17 +97,46 @@ __device__ __forceinline__ float row_scale(const GemmParams& p, int row) {
   return norm_factor(p.ss_in, p.ss_parts, p, row) / norm_factor(p.ss_pre, p.ss_pre_parts, p, row);
 }
 
-// Sums over a group of 8 consecutive lanes of the lanes' s[0..7]: lane i of the group gets the
-// sum of the s[i] (7 shuffles).
-__device__ __forceinline__ float group8_sums(const float (&s)[8], int lane) {
-  float a[4], b[2];
+// The partial sum of squares of 128 columns of rows row0 + i*4 + lane/8 (i = 0..7) from the lanes'
+// own sums over their columns.
+__device__ __forceinline__ void store_square_sums(const GemmParams& p, int row0, int lane, int group,
+                                                  const float (&ss)[8]) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-    a[i] = (lane & 4 ? s[i + 4] : s[i]) + __shfl_xor_sync(0xffffffffu, lane & 4 ? s[i] : s[i + 4], 4);
+  for (int i = 0; i < 8; ++i) {
+    float t = ss[i];
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+    t += __shfl_xor_sync(0xffffffffu, t, 4);
+    const int r = i * 4 + (lane >> 3);
+    if ((lane & 7) == 0 && row0 + r < p.M) p.ss_out[static_cast<int64_t>(row0 + r) * p.ss_out_parts + group] = t;
+  }
+}
+
+// A narrow tile's warp holds the lanes' sums over one 32-column chunk (of the group's four) for
+// its 32 rows.  The warps that hold the group's chunks may be in different CTAs: each leaves its
+// lanes' sums in global memory and counts itself in; the last to come adds the chunks up in
+// column order, exactly as a wide tile's warp does with its own, and clears the count.  Nothing
+// waits.
+__device__ __forceinline__ void publish_square_sums(const GemmParams& p, int row0, int lane, int group, int chunk,
+                                                    const float (&ss)[8]) {
+  const int64_t at = static_cast<int64_t>(row0 / 32) * p.ss_out_parts + group;
+  float* mine = p.ss_chunks + ((at * 4 + chunk) * 8) * 32 + lane;
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
-    b[i] = (lane & 2 ? a[i + 2] : a[i]) + __shfl_xor_sync(0xffffffffu, lane & 2 ? a[i] : a[i + 2], 2);
-  return (lane & 1 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, lane & 1 ? b[0] : b[1], 1);
+  for (int i = 0; i < 8; ++i) __stcg(mine + i * 32, ss[i]);
+  __threadfence();
+  __syncwarp();
+  int before = 0;
+  if (lane == 0) before = atomicAdd(p.ss_count + at, 1);
+  if (__shfl_sync(0xffffffffu, before, 0) != 3) return;
+  __threadfence();
+  if (lane == 0) p.ss_count[at] = 0;
+  float sum[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float* c = p.ss_chunks + (at * 32 + i) * 32 + lane;  // chunk k at + k * 256
+    sum[i] = ((__ldcg(c) + __ldcg(c + 256)) + __ldcg(c + 512)) + __ldcg(c + 768);
+  }
+  store_square_sums(p, row0, lane, group, sum);
 }
 
 // The warp's 32 rows x 32 words sit in `xs` (row-per-lane layout, stride 33).
@@ -170,7 +187,7 @@ __device__ __forceinline__ void epilogue_prefetch(const GemmParams& p, int row0,
 }
 
 // BNT: columns of the tile, 256 (k_gemm_pair) or 64 / 128 (k_gemm_few).  The arithmetic on a row
-// is the same for every BNT, written with explicit fused operations so that it stays so.
+// is the same for every BNT, operation for operation.
 template <int EPI, int BNT>
 __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t taddr, int row0, int nb, int part,
                                               int lane, uint32_t* xs, const EpiPre& pre) {
@@ -196,9 +213,9 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
           tmem_ld32(taddr + hh * 128 + c, v);
           tmem_ld_wait();
 #pragma unroll
-          for (int j = 0; j < 32; ++j) ss = fmaf(__uint_as_float(v[j]), __uint_as_float(v[j]), ss);
+          for (int j = 0; j < 32; ++j) ss += __uint_as_float(v[j]) * __uint_as_float(v[j]);
         }
-        const float inv_row = rs * rsqrtf(fmaf(ss * rs * rs, 1.f / 128.f, p.eps));
+        const float inv_row = rs * rsqrtf(ss * rs * rs * (1.f / 128.f) + p.eps);
         const bf16* wgt = hc < p.q_cols ? p.q_norm : p.k_norm;
         // the rotation runs in the transposed layout: lane L owns rows i*4 + L/8 and
         // columns w4 .. w4+3 of each 32-column chunk, so RoPE-table reads and the
@@ -256,8 +273,8 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
 #pragma unroll
               for (int k = 0; k < 4; ++k) {
                 const float u = a[k] * inv_i[i] * g1[k], w = b[k] * inv_i[i] * g2[k];
-                y1[k] = fmaf(u, cosv[k], -(w * sinv[k]));
-                y2[k] = fmaf(w, cosv[k], u * sinv[k]);
+                y1[k] = u * cosv[k] - w * sinv[k];
+                y2[k] = w * cosv[k] + u * sinv[k];
                 bad |= !(fp16_ok(y1[k]) && fp16_ok(y2[k]));
               }
               f16* orow = out + static_cast<int64_t>(row0 + r) * p.ld_out + hc + c + w4;
@@ -295,10 +312,11 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
     // residual values of chunk c+1 are loaded while chunk c is processed.
     float* res = reinterpret_cast<float*>(p.out);
     const int w4 = (lane & 7) * 4;
-    float prev[8], ss128 = 0.f;
+    float ss[8], prev[8];
     // each lane fetched its own row's previous norm factor; the row layout below takes them by shuffle
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
+      ss[i] = 0.f;
       prev[i] = __shfl_sync(0xffffffffu, pre.scale, i * 4 + (lane >> 3));
     }
     auto rrow = [&](int i, int c) {
@@ -324,7 +342,10 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
       for (int j = 0; j < 32; ++j) xs[lane * 33 + j] = v[j];
       __syncwarp();
       const int col = nb * BNT + c + w4;
-      float ss[8];
+      if (BNT < 256) {  // a chunk's sums stand alone here
+#pragma unroll
+        for (int i = 0; i < 8; ++i) ss[i] = 0.f;
+      }
       float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
       if (p.xn_out) {
         const uint2 gw = *reinterpret_cast<const uint2*>(p.xn_gain + col);
@@ -335,7 +356,6 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int r = i * 4 + (lane >> 3);
-        ss[i] = 0.f;
         if (row0 + r < p.M) {
           float4 x = cur[i];
           x.x += __uint_as_float(xs[r * 33 + w4 + 0]);
@@ -344,7 +364,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
           x.w += __uint_as_float(xs[r * 33 + w4 + 3]);
           *rrow(i, c) = x;
           if (p.xn_out) {
-            ss[i] = fmaf(x.w, x.w, fmaf(x.z, x.z, fmaf(x.y, x.y, x.x * x.x)));
+            ss[i] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
             const float sc = prev[i];
             const float n0 = x.x * g4.x * sc, n1 = x.y * g4.y * sc, n2 = x.z * g4.z * sc, n3 = x.w * g4.w * sc;
             bad |= !(fp16_ok(n0) && fp16_ok(n1) && fp16_ok(n2) && fp16_ok(n3));
@@ -357,18 +377,10 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
         cur[i] = nxt[i];
       }
       __syncwarp();
-      if (p.ss_out) {  // lane i of each 8 now takes row i * 4 + lane / 8 of these 32 columns
-        const float s32 = group8_sums(ss, lane);
-        ss128 += s32;
-        const int r = (lane & 7) * 4 + (lane >> 3);
-        if (row0 + r < p.M) {
-          if constexpr (BNT < 256)
-            p.ss_out[static_cast<int64_t>(row0 + r) * p.ss_out_parts + (nb * BNT + c) / 32] = s32;
-          else if (c + 32 == cend)
-            p.ss_out[static_cast<int64_t>(row0 + r) * p.ss_out_parts + nb * GEMM_SS_PER_TILE + part] = ss128;
-        }
-      }
+      if (BNT < 256 && p.ss_out)
+        publish_square_sums(p, row0, lane, (nb * BNT + c) / 128, (nb * BNT + c) / 32 % 4, ss);
     }
+    if (BNT == 256 && p.ss_out) store_square_sums(p, row0, lane, nb * GEMM_SS_PER_TILE + part, ss);
   } else {  // EPI_SWIGLU: the tile's first half of the columns gate, its second half up of the same outputs
     f16* out = reinterpret_cast<f16*>(p.out);
     const float rs = pre.scale;
