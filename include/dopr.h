@@ -350,7 +350,7 @@ DOPR_API dopr_status dopr_debug_wait_timeout(int32_t timeout_ms);
  * no buffer sizes: the caller guarantees the extents above.
  * Limits: n_pairs <= 32768 and store max_doc_id < 131072; larger requests
  * return DOPR_ERR_UNSUPPORTED with a message and launch nothing.  The scratch
- * array (about 768 KiB) is held by every GPU that loads the library until the
+ * array (about 256 KiB) is held by every GPU that loads the library until the
  * process exits.  The first call on a device looks the array's device address
  * up (cudaGetSymbolAddress) with that device current; make that first call
  * before any stream capture.  Every call shares the one array: calls that

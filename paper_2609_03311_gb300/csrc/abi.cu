@@ -230,7 +230,7 @@ dopr_status grow_dev(T** p, int64_t& cap, int64_t need) {
 }
 
 // Grow the per-call buffers.
-dopr_status ensure_call_buffers(Model* m, int64_t n_pairs, int64_t n_tokens, int64_t n_qtokens, int64_t n_docs) {
+dopr_status ensure_call_buffers(Model* m, int64_t n_pairs, int64_t n_tokens, int64_t n_qtokens) {
   Workspace& w = m->ws;
   if (n_pairs > w.pair_cap) {
     const int64_t cap = std::max<int64_t>(n_pairs, 2 * w.pair_cap);
@@ -282,12 +282,6 @@ dopr_status ensure_call_buffers(Model* m, int64_t n_pairs, int64_t n_tokens, int
     w.qtok_cap = 0;
     STATUS_TRY(dev_alloc(&w.q_tok, cap));
     w.qtok_cap = cap;
-  }
-  if (n_docs > w.doc_cap) {
-    dev_free(w.doc_count);
-    w.doc_cap = 0;
-    STATUS_TRY(dev_alloc(&w.doc_count, n_docs));
-    w.doc_cap = n_docs;
   }
   return DOPR_OK;
 }
@@ -395,7 +389,6 @@ PackArgs pack_args(Model* m, Store* s, int32_t n, const int32_t* dqo, const int3
   a.vocab = m->cfg.vocab;
   a.score_token = m->cfg.score_token_id;
   a.max_position = m->cfg.max_position;
-  a.doc_count = w.doc_count;
   a.pair_slot = w.pair_slot;
   a.perm = w.perm;
   a.sorted_slot = w.sorted_slot;
@@ -524,7 +517,7 @@ dopr_status run_packer(Model* m, Store* s, int32_t n, const int32_t* dqo, const 
   Workspace& w = m->ws;
   CUDA_TRY(cudaMemsetAsync(w.err, 0, w.err_bytes, st));
   PackArgs a = pack_args(m, s, n, dqo, dqt, ddoc);
-  CUDA_TRY(prof_launch(m, K_PACK, 4, 0.0, 24.0 * n, st, [&] { return launch_pack_order(a, st); }));
+  CUDA_TRY(prof_launch(m, K_PACK, 1, 0.0, 24.0 * n, st, [&] { return launch_pack_order(a, st); }));
   CUDA_TRY(cudaMemcpyAsync(w.h_tok_off, w.tok_off, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaMemcpyAsync(w.h_sorted_slot, w.sorted_slot, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaMemcpyAsync(w.h_err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -532,7 +525,7 @@ dopr_status run_packer(Model* m, Store* s, int32_t n, const int32_t* dqo, const 
   STATUS_TRY(map_device_error(*w.h_err));
   plan.n_tokens = w.h_tok_off[n];
   // token buffers sized from the packed total, then packer part 2
-  STATUS_TRY(ensure_call_buffers(m, n, plan.n_tokens, 0, 0));
+  STATUS_TRY(ensure_call_buffers(m, n, plan.n_tokens, 0));
   a = pack_args(m, s, n, dqo, dqt, ddoc);
   CUDA_TRY(prof_launch(m, K_PACK, 1, 0.0, 16.0 * plan.n_tokens, st, [&] { return launch_pack_tokens(a, st); }));
   // chunks of whole pairs, then attention items (runs of one doc, <= ATTN_MAX_PAIRS),
@@ -641,8 +634,6 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
     ext.a_elems = sel ? sel->a_elems : 0;
     CUDA_TRY(prof_launch(m, K_EMBED_NORM, 1, 0.0, T * H * 8.0, st, [&] {
       return launch_embed(w.tok_id + t0, Tc, build ? build->x : m->embed, m->attn_norm, H, c.rms_eps, w.r, w.xn,
-    base.ss_chunks = w.ss_chunks;
-    base.ss_count = w.err + 64;
                           w.ss_e, ext, st);
     }));
     GemmParams base{};
@@ -650,6 +641,8 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
     base.norm_dim = H;
     base.eps = c.rms_eps;
     base.err = w.err;
+    base.ss_chunks = w.ss_chunks;
+    base.ss_count = w.err + 64;
     const int32_t np = s1 - s0;
     double last_keys = 0.0;  // keys seen by the score-token rows alone
     for (int32_t sp = s0; sp < s1; ++sp)
@@ -1191,7 +1184,9 @@ dopr_status dopr_store_create(const dopr_model_config* cfg, int64_t max_doc_id, 
     if (x != DOPR_OK && st == DOPR_OK) st = x;
     return x == DOPR_OK;
   };
-  if (guard(dev_alloc(&s->pool, (size_t)std::max<int64_t>(s->pool_bytes, 256))) &&
+  if (pack_setup() != cudaSuccess)
+    guard(fail(DOPR_ERR_CUDA, "kernel attribute setup failed: %s", cudaGetErrorString(cudaGetLastError())));
+  if (st == DOPR_OK && guard(dev_alloc(&s->pool, (size_t)std::max<int64_t>(s->pool_bytes, 256))) &&
       guard(dev_alloc(&s->d_slot_of, nd)) && guard(dev_alloc(&s->d_slot_m, nd)) &&
       guard(dev_alloc(&s->d_slot_row, nd)) && guard(dev_alloc(&s->d_slot_ok, nd)) && guard(dev_alloc(&s->d_range, 1))) {
     if (cudaMemset(s->d_slot_of, 0xFF, nd * sizeof(int32_t)) != cudaSuccess ||
@@ -1300,7 +1295,7 @@ dopr_status dopr_build_prefixes(dopr_model* m, dopr_store* s, int32_t n_docs, co
     if (x_offsets[d + 1] > x_offsets[d]) pd.push_back(d);
   const int32_t n = (int32_t)pd.size();
   if (n > 0) {
-    STATUS_TRY(ensure_call_buffers(m, n, rows, 0, 0));
+    STATUS_TRY(ensure_call_buffers(m, n, rows, 0));
     std::vector<int32_t> tok_id(rows), tok_pos(rows), tok_pair(rows);
     w.h_tok_off[0] = 0;
     for (int32_t p = 0; p < n; ++p) {
@@ -1402,7 +1397,7 @@ dopr_status dopr_select_prefix_inputs(dopr_model* m, int32_t n_docs, const int32
     STATUS_TRY(dopr_store_create(&c, 0, 256, &empty));
     w.sel_empty = empty;
   }
-  dopr_status rs = ensure_call_buffers(m, n_docs, T, 0, 0);
+  dopr_status rs = ensure_call_buffers(m, n_docs, T, 0);
   if (rs != DOPR_OK) return rs;
   std::vector<int32_t> tok_pos(T), tok_pair(T);
   for (int32_t d = 0; d < n_docs; ++d) {
@@ -1547,7 +1542,7 @@ dopr_status dopr_score(dopr_model* m, dopr_store* s, int32_t n, const int32_t* q
     if (n > 0 && q_offsets[n] > 0 && !q_tokens) return fail(DOPR_ERR_INVALID_ARG, "q_tokens is NULL");
     STATUS_TRY(validate_host_inputs(m, s, n, q_offsets, q_tokens, doc_ids));
     const int64_t nq = q_offsets[n];
-    STATUS_TRY(ensure_call_buffers(m, n, 0, std::max<int64_t>(nq, 1), s->max_doc_id + 1));
+    STATUS_TRY(ensure_call_buffers(m, n, 0, std::max<int64_t>(nq, 1)));
     CUDA_TRY(cudaMemcpyAsync(w.q_off, q_offsets, sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, st));
     if (nq > 0) CUDA_TRY(cudaMemcpyAsync(w.q_tok, q_tokens, sizeof(int32_t) * nq, cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaMemcpyAsync(w.doc_ids, doc_ids, sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
@@ -1555,7 +1550,7 @@ dopr_status dopr_score(dopr_model* m, dopr_store* s, int32_t n, const int32_t* q
     dqt = w.q_tok;
     ddoc = w.doc_ids;
   } else {
-    STATUS_TRY(ensure_call_buffers(m, n, 0, 0, s->max_doc_id + 1));
+    STATUS_TRY(ensure_call_buffers(m, n, 0, 0));
   }
   Plan plan;
   STATUS_TRY(run_packer(m, s, n, dqo, dqt, ddoc, st, plan));
@@ -1587,7 +1582,7 @@ dopr_status dopr_debug_pack_plan(dopr_model* m, dopr_store* s, int32_t n, const 
   CUDA_TRY(cudaSetDevice(m->device));
   Workspace& w = m->ws;
   const int64_t nq = q_offsets[n];
-  STATUS_TRY(ensure_call_buffers(m, n, 0, std::max<int64_t>(nq, 1), s->max_doc_id + 1));
+  STATUS_TRY(ensure_call_buffers(m, n, 0, std::max<int64_t>(nq, 1)));
   cudaStream_t st = 0;
   CUDA_TRY(cudaMemcpy(w.q_off, q_offsets, sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice));
   if (nq > 0) CUDA_TRY(cudaMemcpy(w.q_tok, q_tokens, sizeof(int32_t) * nq, cudaMemcpyHostToDevice));

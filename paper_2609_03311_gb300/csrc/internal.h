@@ -127,7 +127,7 @@ struct Workspace {
   float* ss_s = nullptr;       // [chunk][2H/256] their attention-norm partial sums
   GemmOperandA tm_xn, tm_o, tm_act;
   // per call, grown on demand
-  int64_t pair_cap = 0, tok_cap = 0, qtok_cap = 0, doc_cap = 0, item_cap = 0;
+  int64_t pair_cap = 0, tok_cap = 0, qtok_cap = 0, item_cap = 0;
   int32_t* q_off = nullptr;
   int32_t* q_tok = nullptr;
   int64_t* doc_ids = nullptr;
@@ -139,10 +139,10 @@ struct Workspace {
   int32_t* tok_id = nullptr;
   int32_t* tok_pos = nullptr;
   int32_t* tok_pair = nullptr;
-  int32_t* doc_count = nullptr;  // [max_doc_id+1] counting-sort buckets
   AttnItem* items = nullptr;     // all items of the call, then the mma.sync kernel's items
   AttnTile* tiles = nullptr;     // tensor-core attention tiles of the call
   int64_t tile_cap = 0;
+  // the call's device error word, then the few-row GEMMs' chunk counts (cleared with it)
   int* err = nullptr;
   size_t err_bytes = 0;
   float* ss_chunks = nullptr;  // [GEMM_FEW_MAX_ROWS / 32][H/128][1024]
@@ -348,7 +348,6 @@ struct PackArgs {
   const int32_t* slot_m;
   const uint8_t* slot_ok;
   int vocab, score_token, max_position;
-  int32_t* doc_count;  // [max_doc_id+1], zeroed by the launcher
   int32_t* pair_slot;
   int32_t* perm;
   int32_t* sorted_slot;
@@ -358,8 +357,10 @@ struct PackArgs {
   int32_t* tok_pair;
   int* err;
 };
+// Shared memory of the ordering kernel, once per device (dopr_store_create).
+cudaError_t pack_setup();
 // Device packer, first part: validation, stable sort by doc id, packed token
-// offsets (tok_off).  Zeroes doc_count itself.
+// offsets (tok_off).  Writes perm, sorted_slot and tok_off only when every pair is valid.
 cudaError_t launch_pack_order(const PackArgs& a, cudaStream_t st);
 // Second part, once the token buffers are sized: token ids, positions, pair index.
 cudaError_t launch_pack_tokens(const PackArgs& a, cudaStream_t st);

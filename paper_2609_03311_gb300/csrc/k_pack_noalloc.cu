@@ -11,7 +11,7 @@
 // the call itself allocates nothing.
 //
 // The scratch array below lives in every GPU that loads the library, until
-// the process exits (NOALLOC_SCRATCH_INTS 32-bit words, about 768 KiB).
+// the process exits (NOALLOC_SCRATCH_INTS 32-bit words, about 256 KiB).
 #include <mutex>
 #include <string>
 
@@ -26,9 +26,9 @@ namespace {
 constexpr int NOALLOC_MAX_PAIRS = 32768;   // largest n_pairs accepted
 constexpr int NOALLOC_MAX_DOCS = 131072;   // largest store max_doc_id + 1 accepted
 constexpr int NOALLOC_ERR_WORDS = 64;
-constexpr int NOALLOC_SCRATCH_INTS = NOALLOC_MAX_DOCS + 2 * NOALLOC_MAX_PAIRS + NOALLOC_ERR_WORDS;
+constexpr int NOALLOC_SCRATCH_INTS = 2 * NOALLOC_MAX_PAIRS + NOALLOC_ERR_WORDS;
 
-// Layout: [doc histogram: MAX_DOCS][pair slot: MAX_PAIRS][sorted slot: MAX_PAIRS][error word ...]
+// Layout: [pair slot: MAX_PAIRS][sorted slot: MAX_PAIRS][error word ...]
 static __device__ __align__(256) int32_t g_pack_scratch[NOALLOC_SCRATCH_INTS];
 
 constexpr int MAX_DEVICES = 256;
@@ -110,7 +110,7 @@ extern "C" dopr_status dopr_pack_order_noalloc(const dopr_store* store, int32_t 
   dopr_status st = scratch_for_current_device(&scratch);
   if (st != DOPR_OK) return st;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  int32_t* err = scratch + NOALLOC_MAX_DOCS + 2 * NOALLOC_MAX_PAIRS;
+  int32_t* err = scratch + 2 * NOALLOC_MAX_PAIRS;
   if (n_pairs == 0) {
     e = cudaMemsetAsync(tok_off, 0, sizeof(int32_t), stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
@@ -132,10 +132,9 @@ extern "C" dopr_status dopr_pack_order_noalloc(const dopr_store* store, int32_t 
   a.vocab = store->cfg.vocab;
   a.score_token = store->cfg.score_token_id;
   a.max_position = store->cfg.max_position;
-  a.doc_count = scratch;  // zeroed by launch_pack_order before use
-  a.pair_slot = scratch + NOALLOC_MAX_DOCS;
+  a.pair_slot = scratch;
   a.perm = perm;
-  a.sorted_slot = scratch + NOALLOC_MAX_DOCS + NOALLOC_MAX_PAIRS;
+  a.sorted_slot = scratch + NOALLOC_MAX_PAIRS;
   a.tok_off = tok_off;
   a.err = err;
   int h_err = 0;

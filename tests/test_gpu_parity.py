@@ -393,3 +393,35 @@ def test_gemm_few_rows_match_wide_tiles_bit_for_bit(N, K):
     ref = _ref_gemm(A, B)
     err = (run(33, dopr.EPI_STORE).double() - ref[:33]).abs()
     assert torch.all(err <= ref[:33].abs() * 2 ** -10 + 1e-4 * ref.abs().max()), float(err.max())
+
+
+@pytest.mark.parametrize("max_doc,ids", [(0, 1), (1022, 300), (1023, 1024), (1024, 40), ((1 << 20) + 5, 200)])
+def test_pack_order_at_digit_and_block_edges(max_doc, ids):
+    # Document ids of 1, 10, 11 and 21 bits (one, one, two and three radix passes), batches around the warp, block and
+    # scan-tile sizes; few ids make long runs of equal digits.
+    shape = synth.ModelShape("pack-1l", n_layers=1, hidden=256, n_q_heads=2, n_kv_heads=1, head_dim=128, ffn=128,
+                             vocab=300)
+    cfg = dopr.make_config(shape, max_position=1024)
+    model = dopr.Model(cfg, synth.make_weights(shape, seed=3))
+    rng = np.random.default_rng(max_doc)
+    docs = np.unique(np.concatenate([[0, max_doc], rng.integers(0, max_doc + 1, size=ids)]))
+    store = dopr.Store(cfg, max_doc, len(docs) * dopr.prefix_bytes(cfg, 3))
+    m_of = {int(d): int(d) % 3 for d in docs}
+    for d, m in m_of.items():
+        store.put(d, *synth.make_prefix(shape, m, d, seed=3))
+    for n in (1, 31, 32, 33, 1023, 1025, 4096, 4097, 33000):
+        lens = rng.integers(0, 4, size=n)
+        qo = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        qt = rng.integers(0, shape.vocab, size=int(qo[-1])).astype(np.int32)
+        di = rng.choice(docs, size=n).astype(np.int64)
+        got = dopr.pack_plan(model, store, qo, qt, di)
+        perm = np.argsort(di, kind="stable")
+        np.testing.assert_array_equal(got["perm"], perm)
+        tok_off = np.concatenate([[0], np.cumsum(lens[perm] + 1)])
+        np.testing.assert_array_equal(got["tok_off"], tok_off)
+        pair = np.repeat(np.arange(n), lens[perm] + 1)
+        np.testing.assert_array_equal(got["tok_pair"], pair)
+        base = np.array([m_of[int(d)] for d in di[perm]])
+        np.testing.assert_array_equal(got["tok_pos"], np.arange(tok_off[-1]) - tok_off[pair] + base[pair])
+    model.close()
+    store.close()
