@@ -838,11 +838,13 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
     if (scoring) {
       if (m->mlp_width > 0) {
         const double wd = m->mlp_width;
-        CUDA_TRY(prof_launch(m, K_SCORE, 1, 2.0 * H * wd * (s1 - s0), (s1 - s0) * (H * 4.0 + 4.0) + wd * H * 2.0, st,
+        // the sums of the head's splits go to the residual buffer, which only r_s succeeds here
+        // (a row has H >= 256 = MLP_MAX_SPLITS floats)
+        CUDA_TRY(prof_launch(m, K_SCORE, 2, 2.0 * H * wd * (s1 - s0), (s1 - s0) * (H * 4.0 + 4.0) + wd * H * 2.0, st,
                              [&] {
                                return launch_score_mlp(w.r_s, H, w.tok_off, t0, s0, s1, 1, w.perm, m->final_norm,
                                                        c.rms_eps, m->mlp_width, m->mlp_act, m->mlp_w1, m->mlp_b1,
-                                                       m->mlp_w2, m->mlp_b2, d_scores, ext, st);
+                                                       m->mlp_w2, m->mlp_b2, w.r, d_scores, ext, st);
                              }));
       } else {
         CUDA_TRY(prof_launch(m, K_SCORE, 1, 4.0 * H * (s1 - s0), (s1 - s0) * (H * 4.0 + 4.0), st, [&] {

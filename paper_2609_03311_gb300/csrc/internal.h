@@ -278,12 +278,15 @@ cudaError_t launch_bf16_to_f16(void* buf, int64_t n, int* range, cudaStream_t st
 cudaError_t launch_score(const float* r, int H, const int32_t* tok_off, int tok0, int p_begin, int p_end, int compact,
                          const int32_t* perm, const bf16* gain, const bf16* head, float eps, float* scores,
                          const Extents& ext, cudaStream_t st);
-// Compact the score-token rows of sorted pairs [p_begin, p_end): dst_r[i] = r[row(i)] (H floats) and
-// dst_ss[i] = ss[row(i)] (parts floats), row(i) = tok_off[p_begin+i+1]-1-tok0.
+// The MLP scoring head instead; part: (p_end - p_begin) x mlp_splits(width) floats of scratch.
+constexpr int MLP_MAX_SPLITS = 256;
+int mlp_splits(int width);
 cudaError_t launch_score_mlp(const float* r, int H, const int32_t* tok_off, int tok0, int p_begin, int p_end,
                              int compact, const int32_t* perm, const bf16* gain, float eps, int width, int act,
-                             const bf16* w1, const bf16* b1, const bf16* w2, float b2, float* scores,
+                             const bf16* w1, const bf16* b1, const bf16* w2, float b2, float* part, float* scores,
                              const Extents& ext, cudaStream_t st);
+// Compact the score-token rows of sorted pairs [p_begin, p_end): dst_r[i] = r[row(i)] (H floats) and
+// dst_ss[i] = ss[row(i)] (parts floats), row(i) = tok_off[p_begin+i+1]-1-tok0.
 cudaError_t launch_gather_score_rows(const float* r, const float* ss, int H, int parts, const int32_t* tok_off,
                                      int tok0, int p_begin, int p_end, float* dst_r, float* dst_ss, const Extents& ext,
                                      cudaStream_t st);

@@ -2,7 +2,7 @@
 //   embedding gather (with the first RMSNorm's operand and sum of squares),
 //   the two-row score head, and the prefix-store layout transpose.  The other
 //   RMSNorms and the q/k norm + RoPE are fused into the GEMM epilogues.
-// One warp per row (or per head vector); 16-byte vector accesses.
+// 16-byte vector accesses; the kernels whose rows are few give a row a whole block.
 #include <algorithm>
 
 #include "device_common.cuh"
@@ -11,10 +11,33 @@
 namespace dopr {
 namespace {
 
-constexpr int ROW_WARPS = 8;  // warps per block for row kernels
+// Sum of v over the block's WARPS warps (every thread gets it); red: WARPS floats of shared memory.
+template <int WARPS>
+__device__ __forceinline__ float block_sum(float v, float* red) {
+  v = warp_sum(v);
+  __syncthreads();  // red is reused across calls
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  float t = 0.f;
+#pragma unroll
+  for (int w = 0; w < WARPS; ++w) t += red[w];
+  return t;
+}
+
+// Four consecutive bf16 values (8-byte aligned) as floats.
+__device__ __forceinline__ void bf16x4_to_float(const bf16* p, float (&v)[4]) {
+  const uint2 w = *reinterpret_cast<const uint2*>(p);
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.x));
+  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.y));
+  v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+}
 
 // One warp per row: r = E[id] widened to fp32, ss = sum(r^2),
-// xn = f16(r * rsqrt(ss/H + eps) * g).  The row is read twice (the second read hits L1).
+// xn = f16(r * rsqrt(ss/H + eps) * g).  Bound by its 8 H bytes a row, and in small calls by
+// latency: EMBED_AHEAD 16-byte loads are in flight per lane (one at a time took 16 rounds for a
+// 4,096-element row).  The row is read twice (the second read hits L1).  4,096 elements:
+// 25 rows 9.7 -> 7.6 us, 3,800 rows 29.3 -> 26.1 us, 32,768 rows 171 -> 158 us.
+constexpr int ROW_WARPS = 4, EMBED_AHEAD = 8;
 __global__ void __launch_bounds__(ROW_WARPS * 32)
     k_embed(const int32_t* __restrict__ tok_id, int T, const bf16* __restrict__ embed, const bf16* __restrict__ gain,
             int H, float eps, float* __restrict__ r, f16* __restrict__ xn, float* __restrict__ ss_out, Extents ext) {
@@ -26,24 +49,33 @@ __global__ void __launch_bounds__(ROW_WARPS * 32)
   float* rr = r + static_cast<int64_t>(row) * H;
   f16* xr = xn + static_cast<int64_t>(row) * H;
   float ss = 0.f;
-  for (int c = lane * 8; c < H; c += 256) {
-    const uint4 w = *reinterpret_cast<const uint4*>(e + c);
-    const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(&w);
-    float v[8];
+  for (int c0 = lane * 8; c0 < H; c0 += 256 * EMBED_AHEAD) {
+    uint4 w[EMBED_AHEAD];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float2 a = __bfloat1622float2(w2[k]);
-      v[2 * k] = a.x;
-      v[2 * k + 1] = a.y;
-    }
+    for (int q = 0; q < EMBED_AHEAD; ++q)
+      if (c0 + 256 * q < H) w[q] = *reinterpret_cast<const uint4*>(e + c0 + 256 * q);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) ss += v[k] * v[k];
-    *reinterpret_cast<float4*>(rr + c) = make_float4(v[0], v[1], v[2], v[3]);
-    *reinterpret_cast<float4*>(rr + c + 4) = make_float4(v[4], v[5], v[6], v[7]);
+    for (int q = 0; q < EMBED_AHEAD; ++q)
+      if (c0 + 256 * q < H) {
+        const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(&w[q]);
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float2 a = __bfloat1622float2(w2[k]);
+          v[2 * k] = a.x;
+          v[2 * k + 1] = a.y;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) ss = fmaf(v[k], v[k], ss);
+        float* dst = rr + c0 + 256 * q;
+        *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<float4*>(dst + 4) = make_float4(v[4], v[5], v[6], v[7]);
+      }
   }
   ss = warp_sum(ss);
   const float inv = rsqrtf(ss / static_cast<float>(H) + eps);
   bool bad = false;
+#pragma unroll 4
   for (int c = lane * 8; c < H; c += 256) {
     const uint4 w = *reinterpret_cast<const uint4*>(e + c);
     const uint4 gw = *reinterpret_cast<const uint4*>(gain + c);
@@ -74,43 +106,60 @@ __global__ void k_bf16_to_f16(uint32_t* __restrict__ buf, int64_t n_words, int* 
 }
 
 // Score head at the score-token row of each sorted pair in [p_begin, p_end):
-// s = <W[0] - W[1], RMSNorm(r_row) * g>, written to scores[perm[pair]].
-__global__ void __launch_bounds__(ROW_WARPS * 32)
-    k_score(const float* __restrict__ r, int H, const int32_t* __restrict__ tok_off, int tok0, int p_begin, int p_end,
-            int compact, const int32_t* __restrict__ perm, const bf16* __restrict__ gain,
-            const bf16* __restrict__ head, float eps, float* __restrict__ scores, Extents ext) {
-  const int s = p_begin + blockIdx.x * ROW_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (s >= p_end) return;
+// s = <W[0] - W[1], RMSNorm(r_row) * g>, written to scores[perm[pair]].  One CTA per pair: a
+// call has few pairs, so what counts is the latency of a row (4,096 elements: a warp per row
+// walked it in 192 dependent loads, 37-40 us; a block in four rounds, 6 us).
+constexpr int SCORE_THREADS = 256;
+__global__ void __launch_bounds__(SCORE_THREADS)
+    k_score(const float* __restrict__ r, int H, const int32_t* __restrict__ tok_off, int tok0, int p_begin, int compact,
+            const int32_t* __restrict__ perm, const bf16* __restrict__ gain, const bf16* __restrict__ head, float eps,
+            float* __restrict__ scores, Extents ext) {
+  __shared__ float red[SCORE_THREADS / 32];
+  const int s = p_begin + blockIdx.x;
   const int64_t row = compact ? s - p_begin : tok_off[s + 1] - 1 - tok0;
-  if (!index_ok(ext.err, row, ext.rows)) return;
+  if (!index_ok(ext.err, row, ext.rows)) return;  // uniform across the block
   const float* x = r + row * H;
   float ss = 0.f;
-  for (int c = lane * 4; c < H; c += 128) {
+#pragma unroll 4
+  for (int c = threadIdx.x * 4; c < H; c += SCORE_THREADS * 4) {
     const float4 v = *reinterpret_cast<const float4*>(x + c);
     ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
   }
-  const float inv = rsqrtf(warp_sum(ss) / static_cast<float>(H) + eps);
+  const float inv = rsqrtf(block_sum<SCORE_THREADS / 32>(ss, red) / static_cast<float>(H) + eps);
   float yes = 0.f, no = 0.f;
-  for (int c = lane * 2; c < H; c += 64) {
-    const float2 v = *reinterpret_cast<const float2*>(x + c);
-    const float2 g = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(gain + c));
-    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(head + c));
-    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(head + H + c));
-    const float h0 = v.x * inv * g.x, h1 = v.y * inv * g.y;
-    yes += h0 * a.x + h1 * a.y;
-    no += h0 * b.x + h1 * b.y;
+#pragma unroll 4
+  for (int c = threadIdx.x * 4; c < H; c += SCORE_THREADS * 4) {
+    const float4 v = *reinterpret_cast<const float4*>(x + c);
+    float g[4], a[4], b[4];
+    bf16x4_to_float(gain + c, g);
+    bf16x4_to_float(head + c, a);
+    bf16x4_to_float(head + H + c, b);
+    const float h[4] = {v.x * inv * g[0], v.y * inv * g[1], v.z * inv * g[2], v.w * inv * g[3]};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      yes += h[k] * a[k];
+      no += h[k] * b[k];
+    }
   }
-  yes = warp_sum(yes);
-  no = warp_sum(no);
+  yes = block_sum<SCORE_THREADS / 32>(yes, red);
+  no = block_sum<SCORE_THREADS / 32>(no, red);
   const float sc = yes - no;
-  report_range(ext.err, !isfinite(sc));
-  if (lane == 0) scores[perm[s]] = sc;
+  if (threadIdx.x == 0) {
+    if (!isfinite(sc) && ext.err) atomicOr(ext.err, DEV_ERR_RANGE);
+    scores[perm[s]] = sc;
+  }
 }
 
-// MLP scoring head (Sec. 3.2.3): one CTA per pair.  hn = RMSNorm(row) * g in
-// shared memory; each warp takes hidden units j = warp, warp + 8, ...: z = W1[j] . hn
-// + b1[j], act(z) * w2[j] summed; the block sum + b2 is the score.
-constexpr int MLP_THREADS = 256;
+// MLP scoring head (Sec. 3.2.3): act(W1 hn + b1) . w2 + b2 with hn = RMSNorm(row) * g.
+// A CTA takes MLP_PAIRS pairs and, 32 at a time, its share of the hidden units, four to a warp:
+// the elements of hn go through shared memory MLP_CHUNK at a time, a lane multiplies its
+// elements of four W1 rows into all eight pairs (fp32), so a W1 element is read from L2 once
+// for eight pairs, and not once a pair, and each pass over a pair's hn serves 32 units.  The
+// sums over a CTA's units go to part[pair][split]; k_score_mlp_sum adds them in split order.
+// 50 pairs, 1,024 units, 2,560 elements: one CTA per pair 508 us, these 29 us.
+constexpr int MLP_WARPS = 8, MLP_PAIRS = 8, MLP_UNITS = 4, MLP_CHUNK = 1024;
+constexpr int MLP_THREADS = 32 * MLP_WARPS;
+constexpr int MLP_PASS = MLP_WARPS * MLP_UNITS;  // hidden units of one pass
 __device__ __forceinline__ float head_act(float z, int act) {
   switch (act) {
     case 0: return fmaxf(z, 0.f);
@@ -121,60 +170,117 @@ __device__ __forceinline__ float head_act(float z, int act) {
 }
 __global__ void __launch_bounds__(MLP_THREADS)
     k_score_mlp(const float* __restrict__ r, int H, const int32_t* __restrict__ tok_off, int tok0, int p_begin,
-                int compact, const int32_t* __restrict__ perm, const bf16* __restrict__ gain, float eps, int width,
-                int act, const bf16* __restrict__ w1, const bf16* __restrict__ b1, const bf16* __restrict__ w2,
-                float b2, float* __restrict__ scores, Extents ext) {
-  extern __shared__ float hn[];  // [H], then 32 partial sums
-  float* red = hn + H;
-  const int s = p_begin + blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t row = compact ? s - p_begin : tok_off[s + 1] - 1 - tok0;
-  if (!index_ok(ext.err, row, ext.rows)) return;  // uniform across the block
-  const float* x = r + row * H;
-  float ss = 0.f;
-  for (int c = threadIdx.x; c < H; c += blockDim.x) ss += x[c] * x[c];
-  ss = warp_sum(ss);
-  if (lane == 0) red[warp] = ss;
-  __syncthreads();
-  float tot = 0.f;
-  for (int w = 0; w < MLP_THREADS / 32; ++w) tot += red[w];
-  const float inv = rsqrtf(tot / static_cast<float>(H) + eps);
-  for (int c = threadIdx.x; c < H; c += blockDim.x) hn[c] = x[c] * inv * __bfloat162float(gain[c]);
-  __syncthreads();
-  float part = 0.f;
-  for (int j = warp; j < width; j += MLP_THREADS / 32) {
-    const bf16* wr = w1 + static_cast<int64_t>(j) * H;
-    float z = 0.f;
-    for (int c = lane * 2; c < H; c += 64) {
-      const float2 wv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(wr + c));
-      z += wv.x * hn[c] + wv.y * hn[c + 1];
-    }
-    z = warp_sum(z) + __bfloat162float(b1[j]);
-    part += head_act(z, act) * __bfloat162float(w2[j]);
+                int p_end, int compact, const bf16* __restrict__ gain, float eps, int width, int act,
+                const bf16* __restrict__ w1, const bf16* __restrict__ b1, const bf16* __restrict__ w2, int passes,
+                float* __restrict__ part, Extents ext) {
+  __shared__ float hn[MLP_PAIRS][MLP_CHUNK];
+  __shared__ float red[MLP_WARPS][MLP_PAIRS];
+  const int s0 = p_begin + blockIdx.x * MLP_PAIRS, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  static_assert(MLP_WARPS == MLP_PAIRS, "a warp stages a pair");
+  // this warp's pair: its row and norm factor (pairs past p_end stage zeros)
+  const float* x = nullptr;
+  if (s0 + warp < p_end) {
+    const int64_t row = compact ? s0 + warp - p_begin : tok_off[s0 + warp + 1] - 1 - tok0;
+    if (index_ok(ext.err, row, ext.rows)) x = r + row * H;
   }
+  float ss = 0.f;
+  if (x) {
+#pragma unroll 8
+    for (int c = lane * 4; c < H; c += 128) {
+      const float4 v = *reinterpret_cast<const float4*>(x + c);
+      ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+    }
+  }
+  const float inv = rsqrtf(warp_sum(ss) / static_cast<float>(H) + eps);
+  float total = 0.f;  // lane i < MLP_PAIRS: pair i's sum over this warp's units
+  for (int q = 0; q < passes; ++q) {
+    const int j0 = (static_cast<int>(blockIdx.y) * passes + q) * MLP_PASS + warp * MLP_UNITS;
+    float z[MLP_UNITS][MLP_PAIRS];
+#pragma unroll
+    for (int u = 0; u < MLP_UNITS; ++u)
+#pragma unroll
+      for (int i = 0; i < MLP_PAIRS; ++i) z[u][i] = 0.f;
+    for (int c0 = 0; c0 < H; c0 += MLP_CHUNK) {
+      const int n = min(MLP_CHUNK, H - c0);  // a multiple of 256
+      __syncthreads();
+#pragma unroll 8
+      for (int c = lane * 4; c < n; c += 128) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (x) {
+          v = *reinterpret_cast<const float4*>(x + c0 + c);
+          float g[4];
+          bf16x4_to_float(gain + c0 + c, g);
+          v = make_float4(v.x * inv * g[0], v.y * inv * g[1], v.z * inv * g[2], v.w * inv * g[3]);
+        }
+        *reinterpret_cast<float4*>(&hn[warp][c]) = v;
+      }
+      __syncthreads();
+      if (j0 < width) {
+#pragma unroll 2
+        for (int c = lane * 4; c < n; c += 128) {
+          float w[MLP_UNITS][4];
+#pragma unroll
+          for (int u = 0; u < MLP_UNITS; ++u)  // units past the width read its last row and are dropped
+            bf16x4_to_float(w1 + static_cast<int64_t>(min(j0 + u, width - 1)) * H + c0 + c, w[u]);
+#pragma unroll
+          for (int i = 0; i < MLP_PAIRS; ++i) {
+            const float4 h = *reinterpret_cast<const float4*>(&hn[i][c]);
+#pragma unroll
+            for (int u = 0; u < MLP_UNITS; ++u)
+              z[u][i] += w[u][0] * h.x + w[u][1] * h.y + w[u][2] * h.z + w[u][3] * h.w;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < MLP_UNITS; ++u) {
+      float mine = 0.f;
+#pragma unroll
+      for (int i = 0; i < MLP_PAIRS; ++i) {
+        const float v = warp_sum(z[u][i]);
+        if (lane == i) mine = v;
+      }
+      if (j0 + u < width)
+        total += head_act(mine + __bfloat162float(b1[j0 + u]), act) * __bfloat162float(w2[j0 + u]);
+    }
+  }
+  if (lane < MLP_PAIRS) red[warp][lane] = total;
   __syncthreads();
-  if (lane == 0) red[warp] = part;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float sc = b2;
-    for (int w = 0; w < MLP_THREADS / 32; ++w) sc += red[w];
-    if (!isfinite(sc) && ext.err) atomicOr(ext.err, DEV_ERR_RANGE);
-    scores[perm[s]] = sc;
+  if (threadIdx.x < MLP_PAIRS && s0 + static_cast<int>(threadIdx.x) < p_end) {
+    float t = 0.f;
+    for (int w = 0; w < MLP_WARPS; ++w) t += red[w][threadIdx.x];
+    part[static_cast<int64_t>(s0 + threadIdx.x - p_begin) * gridDim.y + blockIdx.y] = t;
+  }
+}
+// One warp per pair: its splits' sums in order, and b2.
+__global__ void k_score_mlp_sum(const float* __restrict__ part, int splits, int n, const int32_t* __restrict__ perm, float b2,
+                                float* __restrict__ scores, int* err) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= n) return;
+  float t = 0.f;
+  for (int k = lane; k < splits; k += 32) t += part[static_cast<int64_t>(i) * splits + k];
+  const float sc = warp_sum(t) + b2;
+  if (lane == 0) {
+    if (!isfinite(sc) && err) atomicOr(err, DEV_ERR_RANGE);
+    scores[perm[i]] = sc;
   }
 }
 
-// One warp per pair: copy its score-token row of r (and of the partial sums) to row i.
-__global__ void __launch_bounds__(ROW_WARPS * 32)
+// One block per pair: copy its score-token row of r (and of the partial sums) to row i (8.1 ->
+// 4.5 us at 1-100 pairs of 4,096 elements: a latency, like the score head's).
+constexpr int GATHER_THREADS = 256;
+__global__ void __launch_bounds__(GATHER_THREADS)
     k_gather_score_rows(const float* __restrict__ r, const float* __restrict__ ss, int H, int parts,
-                        const int32_t* __restrict__ tok_off, int tok0, int p_begin, int p_end,
-                        float* __restrict__ dst_r, float* __restrict__ dst_ss, Extents ext) {
-  const int i = blockIdx.x * ROW_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (p_begin + i >= p_end) return;
+                        const int32_t* __restrict__ tok_off, int tok0, int p_begin, float* __restrict__ dst_r,
+                        float* __restrict__ dst_ss, Extents ext) {
+  const int i = blockIdx.x;
   const int64_t row = tok_off[p_begin + i + 1] - 1 - tok0;
   if (!index_ok(ext.err, row, ext.rows) || !index_ok(ext.err, i, ext.rows)) return;
   const float4* src = reinterpret_cast<const float4*>(r + row * H);
   float4* dst = reinterpret_cast<float4*>(dst_r + static_cast<int64_t>(i) * H);
-  for (int c = lane; c < H / 4; c += 32) dst[c] = src[c];
-  for (int c = lane; c < parts; c += 32) dst_ss[static_cast<int64_t>(i) * parts + c] = ss[row * parts + c];
+#pragma unroll 4
+  for (int c = threadIdx.x; c < H / 4; c += GATHER_THREADS) dst[c] = src[c];
+  for (int c = threadIdx.x; c < parts; c += GATHER_THREADS) dst_ss[static_cast<int64_t>(i) * parts + c] = ss[row * parts + c];
 }
 
 // [m][Hkv][128] bf16 -> [Hkv][m][128] fp16 for K and V (8 elements per thread).
@@ -242,14 +348,12 @@ __global__ void k_wait_timeout_probe(int* err, uint64_t timeout_ns) {
   __syncthreads();
 }
 
-inline int blocks_for(int64_t rows) { return static_cast<int>((rows + ROW_WARPS - 1) / ROW_WARPS); }
-
 }  // namespace
 
 cudaError_t launch_embed(const int32_t* tok_id, int T, const bf16* embed, const bf16* gain, int H, float eps, float* r,
                          f16* xn, float* ss, const Extents& ext, cudaStream_t st) {
   if (T <= 0) return cudaSuccess;
-  k_embed<<<blocks_for(T), ROW_WARPS * 32, 0, st>>>(tok_id, T, embed, gain, H, eps, r, xn, ss, ext);
+  k_embed<<<(T + ROW_WARPS - 1) / ROW_WARPS, ROW_WARPS * 32, 0, st>>>(tok_id, T, embed, gain, H, eps, r, xn, ss, ext);
   return cudaGetLastError();
 }
 
@@ -265,18 +369,28 @@ cudaError_t launch_score(const float* r, int H, const int32_t* tok_off, int tok0
                          const int32_t* perm, const bf16* gain, const bf16* head, float eps, float* scores,
                          const Extents& ext, cudaStream_t st) {
   if (p_end <= p_begin) return cudaSuccess;
-  k_score<<<blocks_for(p_end - p_begin), ROW_WARPS * 32, 0, st>>>(r, H, tok_off, tok0, p_begin, p_end, compact, perm,
-                                                                  gain, head, eps, scores, ext);
+  k_score<<<p_end - p_begin, SCORE_THREADS, 0, st>>>(r, H, tok_off, tok0, p_begin, compact, perm, gain, head, eps, scores,
+                                                     ext);
   return cudaGetLastError();
+}
+
+int mlp_splits(int width) {
+  const int passes = (width + MLP_PASS - 1) / MLP_PASS;
+  return passes <= MLP_MAX_SPLITS ? passes : (passes + 1) / 2;  // width <= 16,384: 512 passes
 }
 
 cudaError_t launch_score_mlp(const float* r, int H, const int32_t* tok_off, int tok0, int p_begin, int p_end,
                              int compact, const int32_t* perm, const bf16* gain, float eps, int width, int act,
-                             const bf16* w1, const bf16* b1, const bf16* w2, float b2, float* scores,
+                             const bf16* w1, const bf16* b1, const bf16* w2, float b2, float* part, float* scores,
                              const Extents& ext, cudaStream_t st) {
   if (p_end <= p_begin) return cudaSuccess;
-  k_score_mlp<<<p_end - p_begin, MLP_THREADS, (H + 32) * sizeof(float), st>>>(
-      r, H, tok_off, tok0, p_begin, compact, perm, gain, eps, width, act, w1, b1, w2, b2, scores, ext);
+  const int n = p_end - p_begin, splits = mlp_splits(width);
+  const int passes = (width + MLP_PASS * splits - 1) / (MLP_PASS * splits);
+  k_score_mlp<<<dim3((n + MLP_PAIRS - 1) / MLP_PAIRS, splits), MLP_THREADS, 0, st>>>(
+      r, H, tok_off, tok0, p_begin, p_end, compact, gain, eps, width, act, w1, b1, w2, passes, part, ext);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_score_mlp_sum<<<(n + 3) / 4, 128, 0, st>>>(part, splits, n, perm + p_begin, b2, scores, ext.err);
   return cudaGetLastError();
 }
 
@@ -284,8 +398,8 @@ cudaError_t launch_gather_score_rows(const float* r, const float* ss, int H, int
                                      int tok0, int p_begin, int p_end, float* dst_r, float* dst_ss,
                                      const Extents& ext, cudaStream_t st) {
   if (p_end <= p_begin) return cudaSuccess;
-  k_gather_score_rows<<<blocks_for(p_end - p_begin), ROW_WARPS * 32, 0, st>>>(r, ss, H, parts, tok_off, tok0, p_begin,
-                                                                              p_end, dst_r, dst_ss, ext);
+  k_gather_score_rows<<<p_end - p_begin, GATHER_THREADS, 0, st>>>(r, ss, H, parts, tok_off, tok0, p_begin, dst_r, dst_ss,
+                                                                  ext);
   return cudaGetLastError();
 }
 

@@ -61,3 +61,32 @@ def test_mlp_head_scores_match_oracle(act):
     assert np.max(np.abs(got2 - ref2)) <= TOL
     model.close()
     store.close()
+
+
+@pytest.mark.parametrize("width,n", [(1, 1), (31, 8), (33, 9), (1000, 7), (8225, 17)])
+def test_mlp_head_at_tile_edges(width, n):
+    # hidden units in passes of 32 (above 8,192 units two passes a block), pairs in blocks of eight
+    s = SHAPE
+    w = synth.make_weights(s, seed=52, norms="random")
+    cfg = dopr.make_config(s, max_position=1024)
+    model = dopr.Model(cfg, w)
+    om = oracle.OracleModel(oracle.Shape(s.n_layers, s.hidden, s.n_q_heads, s.n_kv_heads, s.head_dim, s.ffn,
+                                         s.vocab, s.rope_theta, s.rms_eps, s.score_token_id), w)
+    store = dopr.Store(cfg, 0, 4096)
+    k, v = synth.make_prefix(s, 0, 0, seed=52)
+    store.put(0, k, v)
+    head = _head(width, s.hidden, 52, 1)
+    head["w2"] = (head["w2"].float() * (96 / width) ** 0.5).to(torch.bfloat16)  # scores of the size of 96 units'
+    dopr.set_mlp_head(model, head)
+    rng = np.random.default_rng(52)
+    ql = rng.integers(0, 12, size=n)
+    qo = np.concatenate([[0], np.cumsum(ql)]).astype(np.int32)
+    qt = rng.integers(0, s.vocab, size=int(qo[-1])).astype(np.int32)
+    got = dopr.score(model, store, qo, qt, np.zeros(n, np.int64)).numpy()
+    ref = []
+    for p in range(n):
+        h = om.forward(om.embed(np.concatenate([qt[qo[p]:qo[p + 1]], [s.score_token_id]])), 0, None, None)["h"]
+        ref.append(om.mlp_head(h[-1], head))
+    assert np.max(np.abs(got - np.array(ref))) <= TOL, np.max(np.abs(got - np.array(ref)))
+    model.close()
+    store.close()
