@@ -133,6 +133,14 @@ __device__ __forceinline__ bool elect_one() {
   return ok != 0;
 }
 
+// The same by a whole converged warp: all lanes go on or give up together.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* err, uint64_t timeout_ns) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, timeout_ns)) != 0;
+}
+__device__ __forceinline__ bool mbar_test_warp(uint32_t bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_test(bar, parity)) != 0;
+}
+
 // --------------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");

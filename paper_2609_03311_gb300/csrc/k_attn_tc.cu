@@ -225,21 +225,22 @@ __global__ void __launch_bounds__(THREADS, 1)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
+    {
+      const bool one = elect_one();
       // ======================= TMA producer: Q, then K blocks, then V blocks, unit after unit
       Ring rq, rk, rv;
       uint32_t armed = 0, armed_par = 0;  // bit per barrier index: ever armed / parity of the last arm
       auto arm = [&](int b, uint32_t par, uint32_t bytes) {
-        mbar_arrive_expect_tx(bar(b), bytes);
+        if (one) mbar_arrive_expect_tx(bar(b), bytes);
         armed |= 1u << b;
         armed_par = (armed_par & ~(1u << b)) | (par << b);
       };
       // Q and K of unit i + 1 go out before V of unit i: the MMA issuer runs
       // S(i + 1) ahead of P V(i), so V(i) may wait for ring space behind P V(i).
       auto issue_q = [&](int tok_begin, int g) -> bool {
-        if (!mbar_wait(bar(BAR_Q_EMPTY + rq.stage), rq.phase ^ 1u, a.err, WAIT_TIMEOUT_NS)) return false;
+        if (!mbar_wait_warp(bar(BAR_Q_EMPTY + rq.stage), rq.phase ^ 1u, a.err, WAIT_TIMEOUT_NS)) return false;
         arm(BAR_Q_FULL + rq.stage, rq.phase, Q_BYTES);
-        for (int h = 0; h < 2; ++h)  // one box per 64-column half: TT rows of each of the group's G heads
+        for (int h = 0; one && h < 2; ++h)  // one box per 64-column half: TT rows of each of the group's G heads
           tma_load_3d(sQ + rq.stage * Q_BYTES + h * Q_HALF, &tm_q, bar(BAR_Q_FULL + rq.stage), h * 64, tok_begin,
                       g * G);
         rq.next(Q_STAGES);
@@ -262,20 +263,20 @@ __global__ void __launch_bounds__(THREADS, 1)
         int si = 0, k = 0, key = pre64;  // own-key cursor: segment, row within it, key column
         int sv = tp->seg[0];
         for (int j = 0; j < nb; ++j) {
-          if (!mbar_wait(bar(empty0 + r.stage), r.phase ^ 1u, a.err, WAIT_TIMEOUT_NS)) return false;
+          if (!mbar_wait_warp(bar(empty0 + r.stage), r.phase ^ 1u, a.err, WAIT_TIMEOUT_NS)) return false;
           // half h of the stage: K halves lie K_STAGES * 8 KB apart (see OFF_K), V halves 8 KB apart
           const uint32_t dst = kv ? ring + r.stage * KV_BYTES : ring + r.stage * KV_HALF;
           const uint32_t hstride = kv ? KV_HALF : K_STAGES * KV_HALF;
           const uint32_t fb = bar(full0 + r.stage);
           if (j * KBLK < pre64) {
             arm(full0 + r.stage, r.phase, KV_BYTES);
-            for (int h = 0; h < 2; ++h) tma_load_2d(dst + h * hstride, &tm_pool, fb, h * 64, pool_row + j * KBLK);
+            for (int h = 0; one && h < 2; ++h) tma_load_2d(dst + h * hstride, &tm_pool, fb, h * 64, pool_row + j * KBLK);
           } else {
             const int groups = min(KBLK, n_keys - j * KBLK) / GROUP_ROWS;
             arm(full0 + r.stage, r.phase, groups * GROUP_BYTES);
             if (groups * GROUP_ROWS == KBLK && key == j * KBLK && k + KBLK <= seg_len(sv)) {
               // the whole block is 64 consecutive tokens of one pair: one 64-row box per half
-              for (int h = 0; h < 2; ++h)
+              for (int h = 0; one && h < 2; ++h)
                 tma_load_2d(dst + h * hstride, &tm_kv64, fb, col0 + h * 64, tok_begin + seg_start(sv) + k);
               key += KBLK;
               k += KBLK;
@@ -289,7 +290,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 // two groups at once when both are 16 consecutive visible tokens of this pair
                 const int n = (q + 2 <= groups && k + 2 * GROUP_ROWS <= seg_len(sv)) ? 2 : 1;
                 if (off >= 0 && off + n * GROUP_ROWS <= KBLK)  // otherwise skipped and the wait times out
-                  for (int h = 0; h < 2; ++h)
+                  for (int h = 0; one && h < 2; ++h)
                     tma_load_2d(dst + off * 128 + h * hstride, n == 2 ? &tm_kv32 : &tm_kv, fb, col0 + h * 64,
                                 tok_begin + seg_start(sv) + k);
                 key += n * GROUP_ROWS;
@@ -321,11 +322,12 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       if (!ok) {  // every copy this thread started lands before the CTA can exit
         for (int b = 0; b < 32; ++b)
-          if (armed & (1u << b)) mbar_wait(bar(b), (armed_par >> b) & 1u, a.err, 100000000ull);
+          if (armed & (1u << b)) mbar_wait_warp(bar(b), (armed_par >> b) & 1u, a.err, 100000000ull);
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
+      const bool one = elect_one();
       // ======================= MMA issuer: an event loop over non-blocking barrier tests.
       // P V blocks of unit ip go in as soon as their P and V are there; S blocks of
       // unit is (at most one unit ahead) as soon as Q, the slot's region and K are.
@@ -350,28 +352,28 @@ __global__ void __launch_bounds__(THREADS, 1)
           const int n_keys = nk_p;
           const int nbp = (n_keys + KBLK - 1) / KBLK;
           auto p_ready = [&](int j) {
-            return mbar_test(bar(BAR_P_FULL + slot * MAX_BLOCKS + j), (ppar >> (slot * MAX_BLOCKS + j)) & 1u);
+            return mbar_test_warp(bar(BAR_P_FULL + slot * MAX_BLOCKS + j), (ppar >> (slot * MAX_BLOCKS + j)) & 1u);
           };
           while (jp < nbp) {
             bool ready = p_ready(jp);
             // O (columns 128..255) covers S blocks 2 and 3: with more than two blocks the
             // softmax must be past its last S read, i.e. the last block's P is in
             if (ready && jp == 0 && nbp > 2) ready = p_ready(nbp - 1);
-            if (!ready || !mbar_test(bar(BAR_V_FULL + rv.stage), rv.phase)) break;
+            if (!ready || !mbar_test_warp(bar(BAR_V_FULL + rv.stage), rv.phase)) break;
             tc_fence_after();
             const int steps = min(KBLK, n_keys - jp * KBLK) / 16;  // only rows the producer loaded
             const uint32_t pcol = tmem + slot * SLOT_COLS + 32 * jp;  // 16 keys = 8 columns per step
-            for (int kk = 0; kk < steps; ++kk)
+            for (int kk = 0; one && kk < steps; ++kk)
               umma_f16_ts(tmem + slot * SLOT_COLS + O_COL, pcol + 8 * kk,
                           umma_desc_sw128_mn(sV + rv.stage * KV_BYTES + kk * 2048, KV_HALF, 1024), IDESC_O,
                           (jp | kk) != 0);
-            umma_commit(bar(BAR_V_EMPTY + rv.stage));
+            if (one) umma_commit(bar(BAR_V_EMPTY + rv.stage));
             rv.next(V_STAGES);
             ++jp;
             prog = true;
           }
           if (jp == nbp) {
-            umma_commit(bar(BAR_O_FULL + slot));
+            if (one) umma_commit(bar(BAR_O_FULL + slot));
             for (int j = 0; j < nbp; ++j) ppar ^= 1u << (slot * MAX_BLOCKS + j);  // each block's barrier completed once
             ++ip;
             jp = 0;
@@ -382,8 +384,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         // ---- S = Q K^T of unit is
         if (is < n_local && is <= ip + 1) {
           const int slot = is & 1;
-          if (!s_open && mbar_test(bar(BAR_Q_FULL + rq.stage), rq.phase) &&
-              mbar_test(bar(BAR_R_FREE + slot), ((is >> 1) & 1) ^ 1u)) {
+          if (!s_open && mbar_test_warp(bar(BAR_Q_FULL + rq.stage), rq.phase) &&
+              mbar_test_warp(bar(BAR_R_FREE + slot), ((is >> 1) & 1) ^ 1u)) {
             s_open = true;
             js = 0;
             nbs = (a.tiles[unit_of(is) / a.Hkv].n_keys + KBLK - 1) / KBLK;
@@ -396,26 +398,27 @@ __global__ void __launch_bounds__(THREADS, 1)
             // 64 * run rows: one N = 64 * run MMA per 16-element step once all of them are in
             const int run = min(nbs - js, K_STAGES - rk.stage);
             bool landed = true;
-            for (int t = 0; t < run && landed; ++t) landed = mbar_test(bar(BAR_K_FULL + rk.stage + t), rk.phase);
+            for (int t = 0; t < run && landed; ++t) landed = mbar_test_warp(bar(BAR_K_FULL + rk.stage + t), rk.phase);
             if (!landed) break;
             tc_fence_after();
             const uint64_t qd = umma_desc_sw128(sQ + rq.stage * Q_BYTES);
             const uint64_t kd = umma_desc_sw128(sK + rk.stage * KV_HALF);
             const uint32_t idesc = umma_idesc_f16(TILE_M, run * KBLK);
+            if (one)
 #pragma unroll
-            for (int ks = 0; ks < HEAD_DIM / 16; ++ks)  // 16 elements = 32 bytes per step; Q halves 16 KB apart
-              umma_f16(tmem + slot * SLOT_COLS + js * KBLK, qd + ((ks >> 2) * Q_HALF + (ks & 3) * 32) / 16,
+              for (int ks = 0; ks < HEAD_DIM / 16; ++ks)  // 16 elements = 32 bytes per step; Q halves 16 KB apart
+                umma_f16(tmem + slot * SLOT_COLS + js * KBLK, qd + ((ks >> 2) * Q_HALF + (ks & 3) * 32) / 16,
                        kd + ((ks >> 2) * K_STAGES * KV_HALF + (ks & 3) * 32) / 16, idesc, ks > 0);
             for (int t = 0; t < run; ++t) {
-              umma_commit(bar(BAR_K_EMPTY + rk.stage));
+              if (one) umma_commit(bar(BAR_K_EMPTY + rk.stage));
               rk.next(K_STAGES);
             }
             js += run;
             prog = true;
           }
           if (s_open && js == nbs) {
-            umma_commit(bar(BAR_S_FULL + slot));
-            umma_commit(bar(BAR_Q_EMPTY + rq.stage));
+            if (one) umma_commit(bar(BAR_S_FULL + slot));
+            if (one) umma_commit(bar(BAR_Q_EMPTY + rq.stage));
             rq.next(Q_STAGES);
             ++is;
             s_open = false;
@@ -426,16 +429,17 @@ __global__ void __launch_bounds__(THREADS, 1)
         } else if (++idle % IDLE_CHECK == 0) {
           const uint64_t now = globaltimer_ns();
           if (idle == IDLE_CHECK) idle_since = now;  // the first check of this idle stretch
-          if ((ld_volatile(a.err) & DEV_ERR_TIMEOUT) || now - idle_since > WAIT_TIMEOUT_NS) {
-            atomicOr(a.err, DEV_ERR_TIMEOUT);
+          if (__any_sync(0xffffffffu,
+                         (ld_volatile(a.err) & DEV_ERR_TIMEOUT) || now - idle_since > WAIT_TIMEOUT_NS)) {
+            if (one) atomicOr(a.err, DEV_ERR_TIMEOUT);
             ok = false;
             break;
           }
         }
       }
       // every MMA this thread issued is complete once the drain barrier flips
-      umma_commit(bar(BAR_DRAIN));
-      mbar_wait(bar(BAR_DRAIN), 0, a.err, ok ? WAIT_TIMEOUT_NS : 100000000ull);
+      if (one) umma_commit(bar(BAR_DRAIN));
+      mbar_wait_warp(bar(BAR_DRAIN), 0, a.err, ok ? WAIT_TIMEOUT_NS : 100000000ull);
     }
   } else {
     // ======================= softmax + epilogue: warpgroup `slot` = warps 2 + 4 slot .. 5 + 4 slot,
@@ -670,12 +674,13 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
+    {
+      const bool one = elect_one();
       // ======================= TMA producer: Q; pass A's K blocks; pass B's K and V blocks chunk by chunk
       Ring rq, rk, rv;
       uint32_t armed = 0, armed_par = 0;
       auto arm = [&](int b, uint32_t par, uint32_t bytes) {
-        mbar_arrive_expect_tx(bar(b), bytes);
+        if (one) mbar_arrive_expect_tx(bar(b), bytes);
         armed |= 1u << b;
         armed_par = (armed_par & ~(1u << b)) | (par << b);
       };
@@ -702,20 +707,20 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
         Ring& r = st.kv ? rv : rk;
         const int stages = st.kv ? lt::V_STAGES : lt::K_STAGES;
         const int full0 = st.kv ? lt::B_V_FULL : lt::B_K_FULL, empty0 = st.kv ? lt::B_V_EMPTY : lt::B_K_EMPTY;
-        if (!mbar_wait(bar(empty0 + r.stage), r.phase ^ 1u, a.err, WAIT_TIMEOUT_NS)) return false;
+        if (!mbar_wait_warp(bar(empty0 + r.stage), r.phase ^ 1u, a.err, WAIT_TIMEOUT_NS)) return false;
         // half h of the stage: K halves lie K_STAGES * 8 KB apart (half-major K ring), V halves 8 KB apart
         const uint32_t dst = st.kv ? sV + r.stage * KV_BYTES : sK + r.stage * KV_HALF;
         const uint32_t hstride = st.kv ? KV_HALF : lt::K_STAGES * KV_HALF;
         const uint32_t fb = bar(full0 + r.stage);
         if (j * KBLK < ceil64(tp->m)) {
           arm(full0 + r.stage, r.phase, KV_BYTES);
-          for (int h = 0; h < 2; ++h) tma_load_2d(dst + h * hstride, &tm_pool, fb, h * 64, st.pool_row + j * KBLK);
+          for (int h = 0; one && h < 2; ++h) tma_load_2d(dst + h * hstride, &tm_pool, fb, h * 64, st.pool_row + j * KBLK);
         } else {
           const int groups = min(KBLK, tp->n_keys - j * KBLK) / GROUP_ROWS;
           arm(full0 + r.stage, r.phase, groups * GROUP_BYTES);
           if (groups * GROUP_ROWS == KBLK && st.k + KBLK <= seg_len(st.sv)) {
             // the whole block is 64 consecutive tokens of one pair: one 64-row box per half
-            for (int h = 0; h < 2; ++h)
+            for (int h = 0; one && h < 2; ++h)
               tma_load_2d(dst + h * hstride, &tm_kv64, fb, st.col0 + h * 64, tp->tok_begin + seg_start(st.sv) + st.k);
             st.k += KBLK;
             if (st.k >= seg_len(st.sv) && st.si + 1 < ATTN_TC_MAX_SEGS) {
@@ -726,7 +731,7 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
             for (int q = 0; q < groups;) {
               // two groups at once when both are 16 consecutive visible tokens of this pair
               const int n = (q + 2 <= groups && st.k + 2 * GROUP_ROWS <= seg_len(st.sv)) ? 2 : 1;
-              for (int h = 0; h < 2; ++h)
+              for (int h = 0; one && h < 2; ++h)
                 tma_load_2d(dst + q * GROUP_ROWS * 128 + h * hstride, n == 2 ? &tm_kv32 : &tm_kv, fb,
                             st.col0 + h * 64, tp->tok_begin + seg_start(st.sv) + st.k);
               st.k += n * GROUP_ROWS;
@@ -748,12 +753,12 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
         const int g = u % a.Hkv;
         const int nb = blocks_of(tp->n_keys);
         if (i + 1 < n_local) prefetch_tile(a.tiles + unit_of(i + 1) / a.Hkv);
-        if (!mbar_wait(bar(lt::B_Q_EMPTY + rq.stage), rq.phase ^ 1u, a.err, WAIT_TIMEOUT_NS)) {
+        if (!mbar_wait_warp(bar(lt::B_Q_EMPTY + rq.stage), rq.phase ^ 1u, a.err, WAIT_TIMEOUT_NS)) {
           ok = false;
           break;
         }
         arm(lt::B_Q_FULL + rq.stage, rq.phase, Q_BYTES);
-        for (int h = 0; h < 2; ++h)
+        for (int h = 0; one && h < 2; ++h)
           tma_load_3d(sQ + rq.stage * Q_BYTES + h * Q_HALF, &tm_q, bar(lt::B_Q_FULL + rq.stage), h * 64,
                       tp->tok_begin, g * G);
         rq.next(lt::Q_STAGES);
@@ -767,16 +772,17 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
       }
       if (!ok) {
         for (int b = 0; b < 32; ++b)
-          if (armed & (1u << b)) mbar_wait(bar(b), (armed_par >> b) & 1u, a.err, 100000000ull);
+          if (armed & (1u << b)) mbar_wait_warp(bar(b), (armed_par >> b) & 1u, a.err, 100000000ull);
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
+      const bool one = elect_one();
       // ======================= MMA issuer
       Ring rq, rk, rv, rp;
       uint32_t cc = 0;  // S chunks issued (both passes, all units): buffer cc & 1
       bool ok = true;
-      auto wait = [&](int b, uint32_t par) { return ok = ok && mbar_wait(bar(b), par, a.err, WAIT_TIMEOUT_NS); };
+      auto wait = [&](int b, uint32_t par) { return ok = ok && mbar_wait_warp(bar(b), par, a.err, WAIT_TIMEOUT_NS); };
       // S of key chunk c (its one or two 64-key blocks from the K ring) into buffer cc & 1
       auto issue_s = [&](int c, int nb) -> bool {
         const uint32_t buf = cc & 1u;
@@ -792,17 +798,18 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
           tc_fence_after();
           const uint64_t kd = umma_desc_sw128(sK + rk.stage * KV_HALF);
           const uint32_t idesc = umma_idesc_f16(TILE_M, run * KBLK);
+          if (one)
 #pragma unroll
-          for (int ks = 0; ks < HEAD_DIM / 16; ++ks)
-            umma_f16(tmem + lt::S_COL + lt::CH * buf + (j - 2 * c) * KBLK, qd + ((ks >> 2) * Q_HALF + (ks & 3) * 32) / 16,
+            for (int ks = 0; ks < HEAD_DIM / 16; ++ks)
+              umma_f16(tmem + lt::S_COL + lt::CH * buf + (j - 2 * c) * KBLK, qd + ((ks >> 2) * Q_HALF + (ks & 3) * 32) / 16,
                      kd + ((ks >> 2) * lt::K_STAGES * KV_HALF + (ks & 3) * 32) / 16, idesc, ks > 0);
           for (int t = 0; t < run; ++t) {
-            umma_commit(bar(lt::B_K_EMPTY + rk.stage));
+            if (one) umma_commit(bar(lt::B_K_EMPTY + rk.stage));
             rk.next(lt::K_STAGES);
           }
           j += run;
         }
-        umma_commit(bar(lt::B_S_FULL + buf));
+        if (one) umma_commit(bar(lt::B_S_FULL + buf));
         ++cc;
         return true;
       };
@@ -822,21 +829,21 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
             const int steps = min(KBLK, n_keys - j * KBLK) / 16;
             const uint32_t pcol = tmem + lt::P_COL + 32 * rp.stage;  // 16 keys = 8 columns per step
             const uint64_t vd = umma_desc_sw128_mn(sV + rv.stage * KV_BYTES, KV_HALF, 1024);
-            for (int kk = 0; kk < steps; ++kk)
+            for (int kk = 0; one && kk < steps; ++kk)
               umma_f16_ts(tmem + lt::O_COL, pcol + 8 * kk, vd + (kk * 2048) / 16, IDESC_O, (j | kk) != 0);
-            umma_commit(bar(lt::B_P_EMPTY + rp.stage));
-            umma_commit(bar(lt::B_V_EMPTY + rv.stage));
+            if (one) umma_commit(bar(lt::B_P_EMPTY + rp.stage));
+            if (one) umma_commit(bar(lt::B_V_EMPTY + rv.stage));
             rp.next(lt::P_STAGES);
             rv.next(lt::V_STAGES);
           }
         }
         if (!ok) break;
-        umma_commit(bar(lt::B_O_FULL));
-        umma_commit(bar(lt::B_Q_EMPTY + rq.stage));
+        if (one) umma_commit(bar(lt::B_O_FULL));
+        if (one) umma_commit(bar(lt::B_Q_EMPTY + rq.stage));
         rq.next(lt::Q_STAGES);
       }
-      umma_commit(bar(lt::B_DRAIN));
-      mbar_wait(bar(lt::B_DRAIN), 0, a.err, ok ? WAIT_TIMEOUT_NS : 100000000ull);
+      if (one) umma_commit(bar(lt::B_DRAIN));
+      mbar_wait_warp(bar(lt::B_DRAIN), 0, a.err, ok ? WAIT_TIMEOUT_NS : 100000000ull);
     }
   } else {
     // ======================= softmax + epilogue: warps 2..5 -> TMEM lane quarters 2, 3, 0, 1

@@ -105,16 +105,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   auto end_k = [&](int s) { return STATS ? true : s % G == G - 1; };
 
   if (warp == 0) {
-    if (lane == 0) {
+    {
+      const bool one = elect_one();
       Ring rq, rk;
       uint32_t armed = 0, armed_par = 0;  // bit per barrier: ever armed / parity of the last arm
       auto load = [&](Ring& r, int full, int empty, uint32_t base, int col, int row) -> bool {
-        if (!mbar_wait(bar(empty + r.stage), r.phase ^ 1u, err, WAIT_TIMEOUT_NS)) return false;
+        if (!mbar_wait_warp(bar(empty + r.stage), r.phase ^ 1u, err, WAIT_TIMEOUT_NS)) return false;
         const int b = full + r.stage;
-        mbar_arrive_expect_tx(bar(b), T_BYTES);
+        if (one) mbar_arrive_expect_tx(bar(b), T_BYTES);
         armed |= 1u << b;
         armed_par = (armed_par & ~(1u << b)) | (r.phase << b);
-        for (int h = 0; h < 2; ++h)
+        for (int h = 0; one && h < 2; ++h)
           tma_load_2d(base + r.stage * T_BYTES + h * T_HALF, &tm, bar(b), col + h * 64, row);
         return true;
       };
@@ -136,11 +137,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       }
       if (!ok) {  // every copy this thread started lands before the CTA can exit
         for (int b = 0; b < 32; ++b)
-          if (armed & (1u << b)) mbar_wait(bar(b), (armed_par >> b) & 1u, err, 100000000ull);
+          if (armed & (1u << b)) mbar_wait_warp(bar(b), (armed_par >> b) & 1u, err, 100000000ull);
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
+      const bool one = elect_one();
       Ring rq, rk, rs;
       constexpr uint32_t idesc = umma_idesc_f16(TILE, TILE);
       bool ok = true;
@@ -148,32 +150,34 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const SelUnit u = units[STATS ? w / Hq : w];
         const int n = steps_of(u);
         for (int s = 0; s < n && ok; ++s) {
-          ok = (!new_q(s) || mbar_wait(bar(B_QF + rq.stage), rq.phase, err, WAIT_TIMEOUT_NS)) &&
-               (!new_k(s) || mbar_wait(bar(B_KF + rk.stage), rk.phase, err, WAIT_TIMEOUT_NS)) &&
-               mbar_wait(bar(B_SE + rs.stage), rs.phase ^ 1u, err, WAIT_TIMEOUT_NS);
+          ok = (!new_q(s) || mbar_wait_warp(bar(B_QF + rq.stage), rq.phase, err, WAIT_TIMEOUT_NS)) &&
+               (!new_k(s) || mbar_wait_warp(bar(B_KF + rk.stage), rk.phase, err, WAIT_TIMEOUT_NS)) &&
+               mbar_wait_warp(bar(B_SE + rs.stage), rs.phase ^ 1u, err, WAIT_TIMEOUT_NS);
           if (!ok) break;
           tc_fence_after();
           const uint64_t qd = umma_desc_sw128(s0 + rq.stage * T_BYTES);
           const uint64_t kd = umma_desc_sw128(s0 + OFF_K + rk.stage * T_BYTES);
+          if (one) {
 #pragma unroll
-          for (int ks = 0; ks < HEAD_DIM / 16; ++ks) {  // 16 elements = 32 bytes a step; halves 16 KB apart
-            const uint64_t off = ((ks >> 2) * T_HALF + (ks & 3) * 32) / 16;
-            umma_f16(tmem + rs.stage * TILE, qd + off, kd + off, idesc, ks > 0);
+            for (int ks = 0; ks < HEAD_DIM / 16; ++ks) {  // 16 elements = 32 bytes a step; halves 16 KB apart
+              const uint64_t off = ((ks >> 2) * T_HALF + (ks & 3) * 32) / 16;
+              umma_f16(tmem + rs.stage * TILE, qd + off, kd + off, idesc, ks > 0);
+            }
+            umma_commit(bar(B_SF + rs.stage));
           }
-          umma_commit(bar(B_SF + rs.stage));
           rs.next(S_BUFS);
           if (end_q(s, n)) {
-            umma_commit(bar(B_QE + rq.stage));
+            if (one) umma_commit(bar(B_QE + rq.stage));
             rq.next(Q_STAGES);
           }
           if (end_k(s)) {
-            umma_commit(bar(B_KE + rk.stage));
+            if (one) umma_commit(bar(B_KE + rk.stage));
             rk.next(K_STAGES);
           }
         }
       }
-      umma_commit(bar(B_DRAIN));  // every MMA this thread issued is complete once it flips
-      mbar_wait(bar(B_DRAIN), 0, err, ok ? WAIT_TIMEOUT_NS : 100000000ull);
+      if (one) umma_commit(bar(B_DRAIN));  // every MMA this thread issued is complete once it flips
+      mbar_wait_warp(bar(B_DRAIN), 0, err, ok ? WAIT_TIMEOUT_NS : 100000000ull);
     }
   } else {
     const int quarter = warp & 3, part = (warp - 2) >> 2;
