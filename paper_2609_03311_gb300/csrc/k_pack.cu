@@ -19,10 +19,10 @@ constexpr int INPUT_ERRORS = DEV_ERR_UNKNOWN_DOC | DEV_ERR_INCOMPLETE | DEV_ERR_
                              DEV_ERR_POSITION;
 
 constexpr int ORDER_THREADS = 1024, ORDER_WARPS = ORDER_THREADS / 32;
-constexpr int ORDER_CTAS = 8;  // CTAs of the cluster for large batches
+constexpr int ORDER_CTAS = 8;         // CTAs of the cluster for large batches
+constexpr int ORDER_ONE_CTA = 4096;   // pairs that one CTA orders by itself (4,000: 17 us, as eight CTAs take)
 constexpr int DIGIT_BITS = 10;
 constexpr int ORDER_SMEM = ORDER_WARPS * (1 << DIGIT_BITS) * 4;  // a digit histogram per warp: 128 KB
-constexpr int AHEAD = 8;                                          // pairs a lane looks at together
 
 // Block-wide exclusive scan of one value per thread; *total gets the sum.
 __device__ int32_t block_scan(int32_t v, int32_t* warp_sums, int32_t* total) {
@@ -58,13 +58,26 @@ __device__ int32_t block_scan(int32_t v, int32_t* warp_sums, int32_t* total) {
 // sector per lane, and one SM takes about one sector a clock: seven such accesses a pair cost
 // one CTA 64 us at 20,000 pairs, eight CTAs 26 us.  One warp walking all pairs took 740 us,
 // with the other three kernels 778.
+template <int CTAS>
 __global__ void __launch_bounds__(ORDER_THREADS) k_pack_order(PackArgs a, int doc_bits) {
+  constexpr int AHEAD = CTAS > 1 ? 4 : 2;  // pairs a lane looks at together
   extern __shared__ int32_t hist[];  // [warp][digit]
   __shared__ int32_t digit_count[1 << DIGIT_BITS], warp_sums[32], cta_total;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = a.n_pairs;
-  const int rank = static_cast<int>(cluster_ctarank()), ctas = static_cast<int>(gridDim.x);  // one cluster
+  constexpr int ctas = CTAS;
+  const int rank = CTAS > 1 ? static_cast<int>(cluster_ctarank()) : 0;
+  // all threads of the cluster meet; what they wrote to global memory is visible after it
+  auto meet = [] {
+    if constexpr (CTAS > 1) {
+      __threadfence();
+      cluster_sync();
+    } else {
+      __syncthreads();
+    }
+  };
   // value `at` of CTA r's shared memory
   auto peer = [&](const int32_t* at, int r) {
+    if constexpr (CTAS == 1) return *at;
     int32_t v;
     asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(mapa_shared(smem_u32(at), r)) : "memory");
     return v;
@@ -101,8 +114,7 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_pack_order(PackArgs a, int do
     }
   }
   if (flags) atomicOr(a.err, flags);
-  __threadfence();
-  cluster_sync();
+  meet();
   if (ld_volatile(a.err) & INPUT_ERRORS) return;  // the same word for the whole cluster
 
   // ---- stable sort by doc id; the order goes to perm, by way of sorted_slot
@@ -133,19 +145,25 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_pack_order(PackArgs a, int do
     __syncthreads();
     if (tid < n_digits) {
       int32_t count = 0;
+#pragma unroll 8
       for (int w = 0; w < ORDER_WARPS; ++w) count += hist[w * n_digits + tid];
       digit_count[tid] = count;
     }
-    cluster_sync();
+    meet();
     int32_t all = 0, before = 0, total;  // of this digit: in the batch, in the CTAs before this one
-    if (tid < n_digits)
-      for (int r = 0; r < ctas; ++r) {
-        const int32_t c = peer(&digit_count[tid], r);
-        all += c;
-        before += r < rank ? c : 0;
+    if (tid < n_digits) {
+      int32_t c[CTAS];
+#pragma unroll
+      for (int r = 0; r < CTAS; ++r) c[r] = peer(&digit_count[tid], r);
+#pragma unroll
+      for (int r = 0; r < CTAS; ++r) {
+        all += c[r];
+        before += r < rank ? c[r] : 0;
       }
+    }
     int32_t run = block_scan(all, warp_sums, &total) + before;
     if (tid < n_digits)
+#pragma unroll 8
       for (int w = 0; w < ORDER_WARPS; ++w) {
         const int32_t c = hist[w * n_digits + tid];
         hist[w * n_digits + tid] = run;
@@ -177,8 +195,7 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_pack_order(PackArgs a, int do
         __syncwarp();
       }
     }
-    __threadfence();
-    cluster_sync();  // the pass's order is complete, and digit_count read, before either changes
+    meet();  // the pass's order is complete, and digit_count read, before either changes
     src = dst;
   }
 
@@ -194,10 +211,16 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_pack_order(PackArgs a, int do
     sum += len;
   }
   block_scan(sum, warp_sums, &total);
-  if (tid == 0) cta_total = total;
-  cluster_sync();
   int32_t carry = 0;
-  for (int r = 0; r < rank; ++r) carry += peer(&cta_total, r);
+  if constexpr (CTAS > 1) {
+    if (tid == 0) cta_total = total;
+    cluster_sync();
+    int32_t c[CTAS];
+#pragma unroll
+    for (int r = 0; r < CTAS; ++r) c[r] = peer(&cta_total, r);
+#pragma unroll
+    for (int r = 0; r < CTAS; ++r) carry += r < rank ? c[r] : 0;
+  }
   for (int s0 = lo; s0 < hi; s0 += ORDER_THREADS) {
     const int s = s0 + tid;  // written by this thread above
     const int32_t len = s < hi ? a.tok_off[s] : 0;
@@ -206,7 +229,7 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_pack_order(PackArgs a, int do
     carry += total;
   }
   if (tid == 0 && rank == ctas - 1) a.tok_off[n] = carry;
-  cluster_sync();  // no CTA leaves while another may read its total
+  if constexpr (CTAS > 1) cluster_sync();  // no CTA leaves while another may read its total
 }
 
 // One warp per sorted pair.
@@ -233,27 +256,31 @@ __global__ void k_pack_tokens(PackArgs a) {
 }  // namespace
 
 cudaError_t pack_setup() {
-  return cudaFuncSetAttribute(k_pack_order, cudaFuncAttributeMaxDynamicSharedMemorySize, ORDER_SMEM);
+  const cudaError_t e = cudaFuncSetAttribute(k_pack_order<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, ORDER_SMEM);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_pack_order<ORDER_CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, ORDER_SMEM);
 }
 
 cudaError_t launch_pack_order(const PackArgs& a, cudaStream_t st) {
   if (a.n_pairs <= 0) return cudaSuccess;
   int doc_bits = 1;
   while (doc_bits < 31 && (a.max_doc_id >> doc_bits)) ++doc_bits;
-  // eight CTAs above 512 pairs; below, one CTA has it done before the cluster's barriers pay
-  const unsigned ctas = a.n_pairs > 512 ? ORDER_CTAS : 1;
+  if (a.n_pairs <= ORDER_ONE_CTA) {
+    k_pack_order<1><<<1, ORDER_THREADS, ORDER_SMEM, st>>>(a, doc_bits);
+    return cudaGetLastError();
+  }
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(ctas);
+  cfg.gridDim = dim3(ORDER_CTAS);
   cfg.blockDim = dim3(ORDER_THREADS);
   cfg.dynamicSmemBytes = ORDER_SMEM;
   cfg.stream = st;
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = ctas;
+  at.val.clusterDim.x = ORDER_CTAS;
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_pack_order, a, doc_bits);
+  return cudaLaunchKernelEx(&cfg, k_pack_order<ORDER_CTAS>, a, doc_bits);
 }
 
 cudaError_t launch_pack_tokens(const PackArgs& a, cudaStream_t st) {
