@@ -61,6 +61,16 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
 
 __device__ __forceinline__ int ld_volatile(const int* p) { return *reinterpret_cast<const volatile int*>(p); }
 
+// ------------------------------------------------- dependent launches
+// The kernels of a pass are launched with programmatic stream serialization (launch_dependent):
+// a kernel's blocks may start, and set up barriers, tensor memory and whatever does not depend
+// on earlier kernels, as soon as every block of the kernel before has called pdl_trigger() and
+// there is room.  pdl_wait() returns when the kernel before has completed and its writes are
+// visible; every block calls it before it touches anything another kernel of the pass writes or
+// reads, and before it ends, so that completion carries over from kernel to kernel.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");

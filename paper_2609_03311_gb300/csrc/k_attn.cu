@@ -242,6 +242,8 @@ __global__ void __launch_bounds__(THREADS, DOPR_ATTN_MIN_BLOCKS) k_attn(const __
     fence_mbar_init();
   }
   __syncthreads();
+  pdl_trigger();
+  pdl_wait();
   if (m > 0) {
     if (tid == 0) {
       const int64_t base = a.slot_row[item.slot];
@@ -368,8 +370,7 @@ cudaError_t attn_setup() {
 cudaError_t launch_attention(const CUtensorMap& tm_pool, const AttnArgs& a, cudaStream_t st) {
   if (a.n_items <= 0) return cudaSuccess;
   dim3 grid(a.n_items, a.Hkv);
-  k_attn<<<grid, THREADS, attn_smem_bytes(a.mpad_cap), st>>>(tm_pool, a);
-  return cudaGetLastError();
+  return launch_dependent(k_attn, grid, THREADS, attn_smem_bytes(a.mpad_cap), st, tm_pool, a);
 }
 
 }  // namespace dopr

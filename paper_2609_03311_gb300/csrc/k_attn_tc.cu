@@ -223,6 +223,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
+  pdl_wait();
 
   if (warp == 0) {
     {
@@ -672,6 +674,8 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
+  pdl_wait();
 
   if (warp == 0) {
     {
@@ -1022,8 +1026,7 @@ cudaError_t launch_attention_tc(const CUtensorMap& tm_q, const CUtensorMap& tm_k
                                 int num_sms, cudaStream_t st) {
   if (a.n_units <= 0) return cudaSuccess;
   const int grid = a.n_units < num_sms ? a.n_units : num_sms;
-  k_attn_tc<<<grid, THREADS, SMEM_BYTES, st>>>(tm_q, tm_kv, tm_kv32, tm_kv64, tm_pool, a);
-  return cudaGetLastError();
+  return launch_dependent(k_attn_tc, grid, THREADS, SMEM_BYTES, st, tm_q, tm_kv, tm_kv32, tm_kv64, tm_pool, a);
 }
 
 cudaError_t launch_attention_tc_long(const CUtensorMap& tm_q, const CUtensorMap& tm_kv, const CUtensorMap& tm_kv32,
@@ -1031,8 +1034,7 @@ cudaError_t launch_attention_tc_long(const CUtensorMap& tm_q, const CUtensorMap&
                                      int num_sms, cudaStream_t st) {
   if (a.n_units <= 0) return cudaSuccess;
   const int grid = a.n_units < num_sms ? a.n_units : num_sms;
-  k_attn_tc_long<<<grid, lt::THREADS, lt::SMEM_BYTES, st>>>(tm_q, tm_kv, tm_kv32, tm_kv64, tm_pool, a);
-  return cudaGetLastError();
+  return launch_dependent(k_attn_tc_long, grid, lt::THREADS, lt::SMEM_BYTES, st, tm_q, tm_kv, tm_kv32, tm_kv64, tm_pool, a);
 }
 
 }  // namespace dopr

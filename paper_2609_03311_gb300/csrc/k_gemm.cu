@@ -530,6 +530,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   cluster_sync();  // both CTAs' barriers exist before either addresses the other's
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_trigger();
+  pdl_wait();
   {
     // the MMAs write both CTAs' TMEM at the leader's address: both allocations must agree
     uint32_t other;
@@ -713,6 +715,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   cluster_sync();  // both CTAs' barriers exist before either addresses the other's
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_trigger();
+  if (warp != 0) pdl_wait();  // the producer starts on the weights first
   {
     uint32_t other;  // as in k_gemm_pair: both allocations must agree
     asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(other) : "r"(mapa_shared(smem_u32(tmem_slot), rank ^ 1u)));
@@ -728,22 +732,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
+    // SwiGLU weights hold gate and up in alternating blocks of 128 rows: rank 0 takes gate rows, rank 1 up rows
+    auto weight_row = [&](int nb) {
+      const int o = nb * (BNT / 2);
+      return EPI == EPI_SWIGLU ? (o / 128) * 256 + o % 128 + static_cast<int>(rank) * 128
+                               : nb * BNT + static_cast<int>(rank) * (BNT / 2);
+    };
+    auto load_weights = [&](int s, int brow, int ks) {  // k-blocks past K are filled with zeros and count as copied
+      if (leader) mbar_arrive_expect_tx(full_bar(s), 2 * stage_bytes);
+      tma_load_3d_pair(sB + s * KB * b_blk, &tmB, mapa_shared(full_bar(s), 0), 0, brow, ks * KB);
+    };
+    // the first stages' weights, which no kernel writes, go out while the kernel before still runs
+    int ahead = 0;
+    if (pair < total)
+      for (; ahead < min(stages, k_steps); ++ahead)
+        if (one) load_weights(ahead, weight_row(pair / m_tiles), ahead);
+    pdl_wait();
     for (int t = pair; t < total && ok; t += n_pairs) {
       const int nb = t / m_tiles, row = (t % m_tiles) * 2 * R + static_cast<int>(rank) * R;
-      // SwiGLU weights hold gate and up in alternating blocks of 128 rows: rank 0 takes gate rows, rank 1 up rows
-      const int o = nb * (BNT / 2);
-      const int brow = EPI == EPI_SWIGLU ? (o / 128) * 256 + o % 128 + static_cast<int>(rank) * 128
-                                         : nb * BNT + static_cast<int>(rank) * (BNT / 2);
+      const int brow = weight_row(nb);
       for (int ks = 0; ks < k_steps; ++ks) {
         ok = wait_all_lanes(empty_bar(stage), phase ^ 1u, p);
         if (!ok) break;
         if (one) {
-          // k-blocks past K are filled with zeros and count as copied
-          if (leader) mbar_arrive_expect_tx(full_bar(stage), 2 * stage_bytes);
-          const uint32_t fb = mapa_shared(full_bar(stage), 0);
-          tma_load_3d_pair(sB + stage * KB * b_blk, &tmB, fb, 0, brow, ks * KB);
-          tma_load_3d_pair(sA + stage * KB * a_blk, &tmA, fb, 0, row, ks * KB);
+          if (ahead == 0) load_weights(stage, brow, ks);
+          tma_load_3d_pair(sA + stage * KB * a_blk, &tmA, mapa_shared(full_bar(stage), 0), 0, row, ks * KB);
         }
+        if (ahead > 0) --ahead;
         if (++stage == stages) {
           stage = 0;
           phase ^= 1u;
@@ -847,20 +862,17 @@ cudaError_t set_smem() {
 }
 
 template <int EPI>
-void launch_epi(const GemmOperandA& A, const GemmOperandB& B, const GemmParams& p, const GemmPlan& g, int num_sms,
+cudaError_t launch_epi(const GemmOperandA& A, const GemmOperandB& B, const GemmParams& p, const GemmPlan& g, int num_sms,
                 cudaStream_t st) {
   const int tiles = ((p.M + 2 * g.rows - 1) / (2 * g.rows)) * (p.N / g.cols);
   const int grid = 2 * (tiles < num_sms / 2 ? tiles : num_sms / 2 > 0 ? num_sms / 2 : 1);
   if (!g.few) {
-    k_gemm_pair<EPI><<<grid, THREADS, PAIR_SMEM_BYTES, st>>>(A.wide, B.wide, p);
-    return;
+    return launch_dependent(k_gemm_pair<EPI>, grid, THREADS, PAIR_SMEM_BYTES, st, A.wide, B.wide, p);
   }
   const CUtensorMap& ta = A.few[g.rows == 32 ? 0 : g.rows == 64 ? 1 : 2];
   const CUtensorMap& tb = B.few[g.cols == 128][GEMM_FEW_KB(g.rows) == 4];
-  few_kernel<EPI>(g.rows, g.cols, [&](auto* k) {
-    k<<<grid, THREADS, FEW_SMEM_BYTES, st>>>(ta, tb, p);
-    return 0;
-  });
+  return few_kernel<EPI>(g.rows, g.cols,
+                         [&](auto* k) { return launch_dependent(k, grid, THREADS, FEW_SMEM_BYTES, st, ta, tb, p); });
 }
 
 }  // namespace
@@ -910,20 +922,11 @@ cudaError_t launch_gemm(int epi, const GemmOperandA& A, const GemmOperandB& B, c
   p.timeout_ns = WAIT_TIMEOUT_NS;
   const GemmPlan g = gemm_plan(epi, p.M, p.N, p.K, num_sms);
   switch (epi) {
-    case EPI_STORE:
-      launch_epi<EPI_STORE>(A, B, p, g, num_sms, st);
-      break;
-    case EPI_RESID_ADD:
-      launch_epi<EPI_RESID_ADD>(A, B, p, g, num_sms, st);
-      break;
-    case EPI_SWIGLU:
-      launch_epi<EPI_SWIGLU>(A, B, p, g, num_sms, st);
-      break;
-    default:
-      launch_epi<EPI_QKV>(A, B, p, g, num_sms, st);
-      break;
+    case EPI_STORE: return launch_epi<EPI_STORE>(A, B, p, g, num_sms, st);
+    case EPI_RESID_ADD: return launch_epi<EPI_RESID_ADD>(A, B, p, g, num_sms, st);
+    case EPI_SWIGLU: return launch_epi<EPI_SWIGLU>(A, B, p, g, num_sms, st);
+    default: return launch_epi<EPI_QKV>(A, B, p, g, num_sms, st);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace dopr

@@ -41,6 +41,8 @@ constexpr int ROW_WARPS = 4, EMBED_AHEAD = 8;
 __global__ void __launch_bounds__(ROW_WARPS * 32)
     k_embed(const int32_t* __restrict__ tok_id, int T, const bf16* __restrict__ embed, const bf16* __restrict__ gain,
             int H, float eps, float* __restrict__ r, f16* __restrict__ xn, float* __restrict__ ss_out, Extents ext) {
+  pdl_trigger();
+  pdl_wait();
   const int row = blockIdx.x * ROW_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= T) return;
   const int64_t id = tok_id[row];
@@ -115,6 +117,8 @@ __global__ void __launch_bounds__(SCORE_THREADS)
             const int32_t* __restrict__ perm, const bf16* __restrict__ gain, const bf16* __restrict__ head, float eps,
             float* __restrict__ scores, Extents ext) {
   __shared__ float red[SCORE_THREADS / 32];
+  pdl_trigger();
+  pdl_wait();
   const int s = p_begin + blockIdx.x;
   const int64_t row = compact ? s - p_begin : tok_off[s + 1] - 1 - tok0;
   if (!index_ok(ext.err, row, ext.rows)) return;  // uniform across the block
@@ -175,6 +179,8 @@ __global__ void __launch_bounds__(MLP_THREADS)
                 float* __restrict__ part, Extents ext) {
   __shared__ float hn[MLP_PAIRS][MLP_CHUNK];
   __shared__ float red[MLP_WARPS][MLP_PAIRS];
+  pdl_trigger();
+  pdl_wait();
   const int s0 = p_begin + blockIdx.x * MLP_PAIRS, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   static_assert(MLP_WARPS == MLP_PAIRS, "a warp stages a pair");
   // this warp's pair: its row and norm factor (pairs past p_end stage zeros)
@@ -255,6 +261,8 @@ __global__ void __launch_bounds__(MLP_THREADS)
 // One warp per pair: its splits' sums in order, and b2.
 __global__ void k_score_mlp_sum(const float* __restrict__ part, int splits, int n, const int32_t* __restrict__ perm, float b2,
                                 float* __restrict__ scores, int* err) {
+  pdl_trigger();
+  pdl_wait();
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (i >= n) return;
   float t = 0.f;
@@ -273,6 +281,8 @@ __global__ void __launch_bounds__(GATHER_THREADS)
     k_gather_score_rows(const float* __restrict__ r, const float* __restrict__ ss, int H, int parts,
                         const int32_t* __restrict__ tok_off, int tok0, int p_begin, float* __restrict__ dst_r,
                         float* __restrict__ dst_ss, Extents ext) {
+  pdl_trigger();
+  pdl_wait();
   const int i = blockIdx.x;
   const int64_t row = tok_off[p_begin + i + 1] - 1 - tok0;
   if (!index_ok(ext.err, row, ext.rows) || !index_ok(ext.err, i, ext.rows)) return;
@@ -321,6 +331,8 @@ __global__ void k_prefix_store(const f16* __restrict__ qkv, int ld_qkv, int T, i
                                const int32_t* __restrict__ tok_pair, const int32_t* __restrict__ tok_pos,
                                const int32_t* __restrict__ pair_slot, const int64_t* __restrict__ slot_row,
                                const int32_t* __restrict__ slot_m, int layer, f16* __restrict__ pool, Extents ext) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= static_cast<int64_t>(T) * Hkv * 2) return;
@@ -353,8 +365,8 @@ __global__ void k_wait_timeout_probe(int* err, uint64_t timeout_ns) {
 cudaError_t launch_embed(const int32_t* tok_id, int T, const bf16* embed, const bf16* gain, int H, float eps, float* r,
                          f16* xn, float* ss, const Extents& ext, cudaStream_t st) {
   if (T <= 0) return cudaSuccess;
-  k_embed<<<(T + ROW_WARPS - 1) / ROW_WARPS, ROW_WARPS * 32, 0, st>>>(tok_id, T, embed, gain, H, eps, r, xn, ss, ext);
-  return cudaGetLastError();
+  return launch_dependent(k_embed, (T + ROW_WARPS - 1) / ROW_WARPS, ROW_WARPS * 32, 0, st, tok_id, T, embed, gain, H, eps,
+                          r, xn, ss, ext);
 }
 
 cudaError_t launch_bf16_to_f16(void* buf, int64_t n, int* range, cudaStream_t st) {
@@ -369,9 +381,8 @@ cudaError_t launch_score(const float* r, int H, const int32_t* tok_off, int tok0
                          const int32_t* perm, const bf16* gain, const bf16* head, float eps, float* scores,
                          const Extents& ext, cudaStream_t st) {
   if (p_end <= p_begin) return cudaSuccess;
-  k_score<<<p_end - p_begin, SCORE_THREADS, 0, st>>>(r, H, tok_off, tok0, p_begin, compact, perm, gain, head, eps, scores,
-                                                     ext);
-  return cudaGetLastError();
+  return launch_dependent(k_score, p_end - p_begin, SCORE_THREADS, 0, st, r, H, tok_off, tok0, p_begin, compact, perm, gain,
+                          head, eps, scores, ext);
 }
 
 int mlp_splits(int width) {
@@ -386,21 +397,19 @@ cudaError_t launch_score_mlp(const float* r, int H, const int32_t* tok_off, int 
   if (p_end <= p_begin) return cudaSuccess;
   const int n = p_end - p_begin, splits = mlp_splits(width);
   const int passes = (width + MLP_PASS * splits - 1) / (MLP_PASS * splits);
-  k_score_mlp<<<dim3((n + MLP_PAIRS - 1) / MLP_PAIRS, splits), MLP_THREADS, 0, st>>>(
-      r, H, tok_off, tok0, p_begin, p_end, compact, gain, eps, width, act, w1, b1, w2, passes, part, ext);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_dependent(k_score_mlp, dim3((n + MLP_PAIRS - 1) / MLP_PAIRS, splits), MLP_THREADS, 0, st, r, H,
+                                         tok_off, tok0, p_begin, p_end, compact, gain, eps, width, act, w1, b1, w2, passes,
+                                         part, ext);
   if (e != cudaSuccess) return e;
-  k_score_mlp_sum<<<(n + 3) / 4, 128, 0, st>>>(part, splits, n, perm + p_begin, b2, scores, ext.err);
-  return cudaGetLastError();
+  return launch_dependent(k_score_mlp_sum, (n + 3) / 4, 128, 0, st, part, splits, n, perm + p_begin, b2, scores, ext.err);
 }
 
 cudaError_t launch_gather_score_rows(const float* r, const float* ss, int H, int parts, const int32_t* tok_off,
                                      int tok0, int p_begin, int p_end, float* dst_r, float* dst_ss,
                                      const Extents& ext, cudaStream_t st) {
   if (p_end <= p_begin) return cudaSuccess;
-  k_gather_score_rows<<<p_end - p_begin, GATHER_THREADS, 0, st>>>(r, ss, H, parts, tok_off, tok0, p_begin, dst_r, dst_ss,
-                                                                  ext);
-  return cudaGetLastError();
+  return launch_dependent(k_gather_score_rows, p_end - p_begin, GATHER_THREADS, 0, st, r, ss, H, parts, tok_off, tok0, p_begin,
+                          dst_r, dst_ss, ext);
 }
 
 cudaError_t launch_store_transpose(const bf16* k, const bf16* v, int m, int Hkv, f16* dk, f16* dv, int* range,
@@ -418,9 +427,8 @@ cudaError_t launch_prefix_store(const f16* qkv, int ld_qkv, int T, int t0, int H
                                 const int32_t* slot_m, int layer, f16* pool, const Extents& ext, cudaStream_t st) {
   const int64_t threads = static_cast<int64_t>(T) * Hkv * 2 * 32;
   if (threads <= 0) return cudaSuccess;
-  k_prefix_store<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, st>>>(
-      qkv, ld_qkv, T, t0, Hq, Hkv, tok_pair, tok_pos, pair_slot, slot_row, slot_m, layer, pool, ext);
-  return cudaGetLastError();
+  return launch_dependent(k_prefix_store, static_cast<unsigned>((threads + 255) / 256), 256, 0, st, qkv, ld_qkv, T, t0, Hq, Hkv,
+                          tok_pair, tok_pos, pair_slot, slot_row, slot_m, layer, pool, ext);
 }
 
 cudaError_t launch_wait_timeout_probe(int* err, uint64_t timeout_ns, cudaStream_t st) {

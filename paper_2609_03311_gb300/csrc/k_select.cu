@@ -86,6 +86,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
+  pdl_wait();
 
   struct Ring {
     int stage = 0;
@@ -313,6 +315,8 @@ __global__ void __launch_bounds__(32 * COL_WARPS)
     k_sal_colstat(const int32_t* __restrict__ tok_pair, const int32_t* __restrict__ tok_off, int t0, int p0, int n_rows,
                   const int64_t* __restrict__ a_off, const float* __restrict__ A, int top_p, float* __restrict__ u,
                   Extents ext) {
+  pdl_trigger();
+  pdl_wait();
   const int t = blockIdx.x * COL_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (t >= n_rows) return;
   const int p = tok_pair[t0 + t];
@@ -387,6 +391,8 @@ __global__ void __launch_bounds__(TOPK_THREADS) k_sal_topk(const int32_t* __rest
                                                            int32_t* __restrict__ positions) {
   static_assert(SEL_MAX_N == 2 * TOPK_THREADS, "two positions a thread");
   __shared__ int warp_sums[32];
+  pdl_trigger();
+  pdl_wait();
   const int p = p0 + blockIdx.x;
   const int ts = tok_off[p] - t0, n = tok_off[p + 1] - tok_off[p];
   const int k = min(K, n);
@@ -423,6 +429,8 @@ __global__ void __launch_bounds__(TOPK_THREADS) k_sal_topk(const int32_t* __rest
 __global__ void k_sal_gather(const float* __restrict__ r, int H, const int32_t* __restrict__ tok_off, int t0,
                              int p0, int n_docs, const int32_t* __restrict__ positions, int K,
                              const bf16* __restrict__ gain, float eps, bf16* __restrict__ x, Extents ext) {
+  pdl_trigger();
+  pdl_wait();
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (w >= n_docs * K) return;
   const int p = p0 + w / K, j = w % K;
@@ -466,38 +474,27 @@ cudaError_t select_setup() {
 cudaError_t launch_select(const CUtensorMap& tm_rows, const SelectArgs& a, int num_sms, cudaStream_t st) {
   if (a.n_rows <= 0) return cudaSuccess;
   const int64_t stat_units = static_cast<int64_t>(a.n_row_tiles) * a.Hq;
-  k_sal_tc<true><<<static_cast<int>(stat_units < num_sms ? stat_units : num_sms), TC_THREADS, TC_SMEM, st>>>(
-      tm_rows, a.row_tiles, a.n_row_tiles, a.Hq, a.Hkv, a.n_rows, a.stats, nullptr, a.ext);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_dependent(k_sal_tc<true>, static_cast<int>(stat_units < num_sms ? stat_units : num_sms), TC_THREADS,
+                                   TC_SMEM, st, tm_rows, a.row_tiles, a.n_row_tiles, a.Hq, a.Hkv, a.n_rows, a.stats, nullptr,
+                                   a.ext);
   if (e != cudaSuccess) return e;
-  k_sal_tc<false><<<a.n_tiles < num_sms ? a.n_tiles : num_sms, TC_THREADS, TC_SMEM, st>>>(
-      tm_rows, a.row_tiles + a.n_row_tiles, a.n_tiles, a.Hq, a.Hkv, a.n_rows, a.stats, a.A, a.ext);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  e = launch_dependent(k_sal_tc<false>, a.n_tiles < num_sms ? a.n_tiles : num_sms, TC_THREADS, TC_SMEM, st, tm_rows,
+                       a.row_tiles + a.n_row_tiles, a.n_tiles, a.Hq, a.Hkv, a.n_rows, a.stats, a.A, a.ext);
+  if (e != cudaSuccess) return e;
   // registers for the longest document's columns (64 entries a lane at 2,048 tokens)
-  const int blocks = (a.n_rows + COL_WARPS - 1) / COL_WARPS;
-  auto colstat = [&](auto kernel) {
-    kernel<<<blocks, 32 * COL_WARPS, 0, st>>>(a.tok_pair, a.tok_off, a.t0, a.p0, a.n_rows, a.a_off, a.A, a.top_p, a.u,
-                                              a.ext);
-  };
-  if (a.max_n <= 512)
-    colstat(k_sal_colstat<16>);
-  else if (a.max_n <= 1024)
-    colstat(k_sal_colstat<32>);
-  else
-    colstat(k_sal_colstat<64>);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_sal_topk<<<a.n_docs, TOPK_THREADS, 0, st>>>(a.tok_off, a.t0, a.p0, a.u, a.top_k, a.positions);
-  return cudaGetLastError();
+  auto* colstat = a.max_n <= 512 ? k_sal_colstat<16> : a.max_n <= 1024 ? k_sal_colstat<32> : k_sal_colstat<64>;
+  e = launch_dependent(colstat, (a.n_rows + COL_WARPS - 1) / COL_WARPS, 32 * COL_WARPS, 0, st, a.tok_pair, a.tok_off, a.t0,
+                       a.p0, a.n_rows, a.a_off, a.A, a.top_p, a.u, a.ext);
+  if (e != cudaSuccess) return e;
+  return launch_dependent(k_sal_topk, a.n_docs, TOPK_THREADS, 0, st, a.tok_off, a.t0, a.p0, a.u, a.top_k, a.positions);
 }
 
 cudaError_t launch_select_gather(const SelectArgs& a, const float* r, int H, const bf16* gain, float eps,
                                  cudaStream_t st) {
   const int64_t threads = static_cast<int64_t>(a.n_docs) * a.top_k * 32;
   if (threads <= 0) return cudaSuccess;
-  k_sal_gather<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, st>>>(r, H, a.tok_off, a.t0, a.p0, a.n_docs,
-                                                                             a.positions, a.top_k, gain, eps, a.x,
-                                                                             a.ext);
-  return cudaGetLastError();
+  return launch_dependent(k_sal_gather, static_cast<unsigned>((threads + 255) / 256), 256, 0, st, r, H, a.tok_off, a.t0, a.p0,
+                          a.n_docs, a.positions, a.top_k, gain, eps, a.x, a.ext);
 }
 
 }  // namespace dopr
