@@ -144,17 +144,17 @@ bool kind_is_global(int32_t k) {
 void free_store(Store* s) {
   dev_free(s->pool); dev_free(s->d_slot_of); dev_free(s->d_slot_m); dev_free(s->d_slot_row); dev_free(s->d_slot_ok);
   dev_free(s->d_range);
+  host_free(s->h_err);
 }
 
 void free_workspace(Workspace& w) {
   dev_free(w.r); dev_free(w.xn); dev_free(w.qkv); dev_free(w.o); dev_free(w.act);
   dev_free(w.ss_e); dev_free(w.ss_a); dev_free(w.ss_m); dev_free(w.r_s); dev_free(w.ss_s);
-  dev_free(w.q_off); dev_free(w.q_tok); dev_free(w.doc_ids); dev_free(w.scores);
+  dev_free(w.in);
   dev_free(w.pair_slot); dev_free(w.perm); dev_free(w.sorted_slot); dev_free(w.tok_off);
   dev_free(w.tok_id); dev_free(w.tok_pos); dev_free(w.tok_pair);
-  dev_free(w.items); dev_free(w.tiles); dev_free(w.err); dev_free(w.ss_chunks);
-  host_free(w.h_tok_off); host_free(w.h_sorted_slot); host_free(w.h_err); host_free(w.h_items);
-  host_free(w.h_tiles);
+  dev_free(w.items); dev_free(w.err); dev_free(w.ss_count); dev_free(w.ss_chunks);
+  host_free(w.h_tok_off); host_free(w.h_sorted_slot); host_free(w.h_in); host_free(w.h_err); host_free(w.h_items);
   dev_free(w.sel_A); dev_free(w.sel_a_off); dev_free(w.sel_u); dev_free(w.sel_pos); dev_free(w.sel_x);
   dev_free(w.sel_units); dev_free(w.sel_stats);
   if (w.sel_empty) {
@@ -205,10 +205,9 @@ dopr_status alloc_chunk_buffers(Model* m, int cap) {
   STATUS_TRY(dev_alloc(&w.r_s, (size_t)cap * c.hidden));
   STATUS_TRY(dev_alloc(&w.ss_s, sums));
   const size_t few_groups = (size_t)GEMM_FEW_MAX_ROWS / 32 * (c.hidden / 128);
-  w.err_bytes = sizeof(int) * (64 + few_groups);
-  STATUS_TRY(dev_alloc(&w.err, 64 + few_groups));
+  w.n_ss_count = (int)few_groups;
+  STATUS_TRY(dev_alloc(&w.ss_count, few_groups));
   STATUS_TRY(dev_alloc(&w.ss_chunks, few_groups * 1024));
-  STATUS_TRY(host_alloc(&w.h_err, 1));
   const bool ok = make_gemm_operand_a(&w.tm_xn, w.xn, c.hidden, cap) &&
                   make_gemm_operand_a(&w.tm_o, w.o, m->o_dim, cap) && make_gemm_operand_a(&w.tm_act, w.act, c.ffn, cap);
   if (!ok) return fail(DOPR_ERR_CUDA, "cuTensorMapEncodeTiled failed for activation buffers");
@@ -229,34 +228,50 @@ dopr_status grow_dev(T** p, int64_t& cap, int64_t need) {
   return DOPR_OK;
 }
 
+template <typename T>
+dopr_status grow_host(T** p, int64_t& cap, int64_t need) {
+  if (need <= cap) return DOPR_OK;
+  const int64_t n = std::max<int64_t>(need, 2 * cap);
+  host_free(*p);
+  cap = 0;
+  STATUS_TRY(host_alloc(p, (size_t)n));
+  cap = n;
+  return DOPR_OK;
+}
+
+// Grow a buffer of `need` bytes, on the device or pinned on the host.
+template <typename T>
+dopr_status grow_bytes(T** p, int64_t& cap, int64_t need, bool pinned) {
+  uint8_t* b = reinterpret_cast<uint8_t*>(*p);
+  const dopr_status s = pinned ? grow_host(&b, cap, need) : grow_dev(&b, cap, need);
+  *p = reinterpret_cast<T*>(b);
+  return s;
+}
+
 // Grow the per-call buffers.
-dopr_status ensure_call_buffers(Model* m, int64_t n_pairs, int64_t n_tokens, int64_t n_qtokens) {
+dopr_status ensure_call_buffers(Model* m, int64_t n_pairs, int64_t n_tokens) {
   Workspace& w = m->ws;
   if (n_pairs > w.pair_cap) {
     const int64_t cap = std::max<int64_t>(n_pairs, 2 * w.pair_cap);
-    dev_free(w.q_off); dev_free(w.doc_ids); dev_free(w.scores); dev_free(w.pair_slot); dev_free(w.perm);
-    dev_free(w.sorted_slot); dev_free(w.tok_off); dev_free(w.items);
-    w.pair_cap = w.item_cap = 0;  // stays 0 if the growth fails, so no later call uses a freed buffer
-    STATUS_TRY(dev_alloc(&w.q_off, cap + 1));
-    STATUS_TRY(dev_alloc(&w.doc_ids, cap));
-    STATUS_TRY(dev_alloc(&w.scores, cap));
+    dev_free(w.pair_slot); dev_free(w.perm); dev_free(w.sorted_slot); dev_free(w.tok_off); dev_free(w.err);
+    w.scores = nullptr;
+    w.pair_cap = 0;  // stays 0 if the growth fails, so no later call uses a freed buffer
     STATUS_TRY(dev_alloc(&w.pair_slot, cap));
     STATUS_TRY(dev_alloc(&w.perm, cap));
     STATUS_TRY(dev_alloc(&w.sorted_slot, cap));
     STATUS_TRY(dev_alloc(&w.tok_off, cap + 1));
-    STATUS_TRY(dev_alloc(&w.items, 2 * (cap + 1024)));
+    STATUS_TRY(dev_alloc(&w.err, RESULT_HEAD + cap));
+    w.scores = reinterpret_cast<float*>(w.err + RESULT_HEAD);
     w.pair_cap = cap;
-    w.item_cap = 2 * (cap + 1024);
   }
   if (n_pairs > w.h_pair_cap) {
     const int64_t cap = std::max<int64_t>(n_pairs, 2 * w.h_pair_cap);
-    host_free(w.h_tok_off); host_free(w.h_sorted_slot); host_free(w.h_items);
-    w.h_pair_cap = w.h_item_cap = 0;
+    host_free(w.h_tok_off); host_free(w.h_sorted_slot); host_free(w.h_err);
+    w.h_pair_cap = 0;
     STATUS_TRY(host_alloc(&w.h_tok_off, cap + 1));
     STATUS_TRY(host_alloc(&w.h_sorted_slot, cap));
-    STATUS_TRY(host_alloc(&w.h_items, 2 * (cap + 1024)));
+    STATUS_TRY(host_alloc(&w.h_err, RESULT_HEAD + cap));
     w.h_pair_cap = cap;
-    w.h_item_cap = 2 * (cap + 1024);
   }
   if (n_tokens > w.tok_cap) {
     const int64_t cap = std::max<int64_t>(n_tokens, 2 * w.tok_cap);
@@ -267,22 +282,41 @@ dopr_status ensure_call_buffers(Model* m, int64_t n_pairs, int64_t n_tokens, int
     STATUS_TRY(dev_alloc(&w.tok_pair, cap));
     w.tok_cap = cap;
   }
-  if (n_tokens > w.tile_cap) {  // a tile holds at least one token
-    const int64_t cap = std::max<int64_t>(n_tokens, 2 * w.tile_cap);
-    dev_free(w.tiles);
-    host_free(w.h_tiles);
-    w.tile_cap = 0;
-    STATUS_TRY(dev_alloc(&w.tiles, cap));
-    STATUS_TRY(host_alloc(&w.h_tiles, cap));
-    w.tile_cap = cap;
+  // the plan: at most two items a pair (and the call's runs) and a tile a token
+  const int64_t items = 2 * (w.pair_cap + 1024);
+  if (n_tokens > 0 && w.item_cap < items) w.item_cap = items;
+  const int64_t plan = w.item_cap * (int64_t)sizeof(AttnItem) + w.tok_cap * (int64_t)sizeof(AttnTile);
+  if (n_tokens > 0 && (plan > w.plan_cap || plan > w.h_plan_cap)) {
+    w.tiles = nullptr;
+    STATUS_TRY(grow_bytes(&w.items, w.plan_cap, plan, false));
+    STATUS_TRY(grow_bytes(&w.h_items, w.h_plan_cap, plan, true));
   }
-  if (n_qtokens > w.qtok_cap) {
-    const int64_t cap = std::max<int64_t>(n_qtokens, 2 * w.qtok_cap);
-    dev_free(w.q_tok);
-    w.qtok_cap = 0;
-    STATUS_TRY(dev_alloc(&w.q_tok, cap));
-    w.qtok_cap = cap;
+  return DOPR_OK;
+}
+
+// A host call's inputs as one block: query offsets, document ids, query tokens.
+struct InputBlock {
+  int64_t docs, tokens, bytes;  // where the document ids and the tokens begin; all of it
+  InputBlock(int64_t n, int64_t nq) {
+    docs = ((n + 1) * (int64_t)sizeof(int32_t) + 15) / 16 * 16;
+    tokens = docs + n * (int64_t)sizeof(int64_t);
+    bytes = tokens + std::max<int64_t>(nq, 1) * (int64_t)sizeof(int32_t);
   }
+};
+// Copy them to the device with one transfer from pinned memory; the pointers of the copies.
+dopr_status upload_inputs(Workspace& w, int32_t n, const int32_t* qo, const int32_t* qt, const int64_t* doc,
+                          cudaStream_t st, const int32_t** dqo, const int32_t** dqt, const int64_t** ddoc) {
+  const int64_t nq = qo[n];
+  const InputBlock b(n, nq);
+  STATUS_TRY(grow_dev(&w.in, w.in_cap, b.bytes));
+  STATUS_TRY(grow_host(&w.h_in, w.h_in_cap, b.bytes));
+  memcpy(w.h_in, qo, sizeof(int32_t) * (n + 1));
+  memcpy(w.h_in + b.docs, doc, sizeof(int64_t) * n);
+  if (nq > 0) memcpy(w.h_in + b.tokens, qt, sizeof(int32_t) * nq);
+  CUDA_TRY(cudaMemcpyAsync(w.in, w.h_in, (size_t)b.bytes, cudaMemcpyHostToDevice, st));
+  *dqo = reinterpret_cast<const int32_t*>(w.in);
+  *ddoc = reinterpret_cast<const int64_t*>(w.in + b.docs);
+  *dqt = reinterpret_cast<const int32_t*>(w.in + b.tokens);
   return DOPR_OK;
 }
 
@@ -397,6 +431,11 @@ PackArgs pack_args(Model* m, Store* s, int32_t n, const int32_t* dqo, const int3
   a.tok_pos = w.tok_pos;
   a.tok_pair = w.tok_pair;
   a.err = w.err;
+  a.h_err = w.h_err;
+  a.h_tok_off = w.h_tok_off;
+  a.h_sorted_slot = w.h_sorted_slot;
+  a.zero = w.ss_count;
+  a.n_zero = w.n_ss_count;
   return a;
 }
 
@@ -494,18 +533,18 @@ struct AttnPlanner {
     plan.n_litems = (int32_t)litems.size();
     plan.n_tiles = (int32_t)tiles.size();
     plan.n_ltiles = (int32_t)ltiles.size();
-    if (n_items + plan.n_litems > w.item_cap || n_items + plan.n_litems > w.h_item_cap ||
-        plan.n_tiles + plan.n_ltiles > w.tile_cap)
+    const int64_t n_all = (int64_t)n_items + plan.n_litems, n_tiles = (int64_t)tiles.size() + ltiles.size();
+    const int64_t first_tile = n_all * (int64_t)sizeof(AttnItem);  // both records are whole 16-byte units
+    const int64_t bytes = first_tile + n_tiles * (int64_t)sizeof(AttnTile);
+    static_assert(sizeof(AttnItem) % 16 == 0 && sizeof(AttnTile) % 16 == 0, "the tiles follow the items");
+    if (n_all > w.item_cap || bytes > w.plan_cap || bytes > w.h_plan_cap)
       return fail(DOPR_ERR_UNSUPPORTED, "attention plan exceeds its buffers");
+    AttnTile* h_tiles = reinterpret_cast<AttnTile*>(reinterpret_cast<uint8_t*>(w.h_items) + first_tile);
+    w.tiles = reinterpret_cast<AttnTile*>(reinterpret_cast<uint8_t*>(w.items) + first_tile);
     std::copy(litems.begin(), litems.end(), w.h_items + n_items);
-    std::copy(tiles.begin(), tiles.end(), w.h_tiles);
-    std::copy(ltiles.begin(), ltiles.end(), w.h_tiles + tiles.size());
-    if (n_items + plan.n_litems > 0)
-      CUDA_TRY(cudaMemcpyAsync(w.items, w.h_items, sizeof(AttnItem) * (n_items + plan.n_litems),
-                               cudaMemcpyHostToDevice, st));
-    if (plan.n_tiles + plan.n_ltiles > 0)
-      CUDA_TRY(cudaMemcpyAsync(w.tiles, w.h_tiles, sizeof(AttnTile) * (plan.n_tiles + plan.n_ltiles),
-                               cudaMemcpyHostToDevice, st));
+    std::copy(tiles.begin(), tiles.end(), h_tiles);
+    std::copy(ltiles.begin(), ltiles.end(), h_tiles + tiles.size());
+    if (bytes > 0) CUDA_TRY(cudaMemcpyAsync(w.items, w.h_items, (size_t)bytes, cudaMemcpyHostToDevice, st));
     return DOPR_OK;
   }
 };
@@ -515,17 +554,14 @@ struct AttnPlanner {
 dopr_status run_packer(Model* m, Store* s, int32_t n, const int32_t* dqo, const int32_t* dqt, const int64_t* ddoc,
                        cudaStream_t st, Plan& plan) {
   Workspace& w = m->ws;
-  CUDA_TRY(cudaMemsetAsync(w.err, 0, w.err_bytes, st));
   PackArgs a = pack_args(m, s, n, dqo, dqt, ddoc);
+  // the kernel clears the error word and the chunk counts, and writes what is read here
   CUDA_TRY(prof_launch(m, K_PACK, 1, 0.0, 24.0 * n, st, [&] { return launch_pack_order(a, st); }));
-  CUDA_TRY(cudaMemcpyAsync(w.h_tok_off, w.tok_off, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(w.h_sorted_slot, w.sorted_slot, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(w.h_err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   STATUS_TRY(map_device_error(*w.h_err));
   plan.n_tokens = w.h_tok_off[n];
   // token buffers sized from the packed total, then packer part 2
-  STATUS_TRY(ensure_call_buffers(m, n, plan.n_tokens, 0));
+  STATUS_TRY(ensure_call_buffers(m, n, plan.n_tokens));
   a = pack_args(m, s, n, dqo, dqt, ddoc);
   CUDA_TRY(prof_launch(m, K_PACK, 1, 0.0, 16.0 * plan.n_tokens, st, [&] { return launch_pack_tokens(a, st); }));
   // chunks of whole pairs, then attention items (runs of one doc, <= ATTN_MAX_PAIRS),
@@ -642,7 +678,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
     base.eps = c.rms_eps;
     base.err = w.err;
     base.ss_chunks = w.ss_chunks;
-    base.ss_count = w.err + 64;
+    base.ss_count = w.ss_count;
     const int32_t np = s1 - s0;
     double last_keys = 0.0;  // keys seen by the score-token rows alone
     for (int32_t sp = s0; sp < s1; ++sp)
@@ -1190,7 +1226,8 @@ dopr_status dopr_store_create(const dopr_model_config* cfg, int64_t max_doc_id, 
     guard(fail(DOPR_ERR_CUDA, "kernel attribute setup failed: %s", cudaGetErrorString(cudaGetLastError())));
   if (st == DOPR_OK && guard(dev_alloc(&s->pool, (size_t)std::max<int64_t>(s->pool_bytes, 256))) &&
       guard(dev_alloc(&s->d_slot_of, nd)) && guard(dev_alloc(&s->d_slot_m, nd)) &&
-      guard(dev_alloc(&s->d_slot_row, nd)) && guard(dev_alloc(&s->d_slot_ok, nd)) && guard(dev_alloc(&s->d_range, 1))) {
+      guard(dev_alloc(&s->d_slot_row, nd)) && guard(dev_alloc(&s->d_slot_ok, nd)) && guard(dev_alloc(&s->d_range, 1)) &&
+      guard(host_alloc(&s->h_err, 1))) {
     if (cudaMemset(s->d_slot_of, 0xFF, nd * sizeof(int32_t)) != cudaSuccess ||
         cudaMemset(s->d_slot_ok, 0, nd) != cudaSuccess || cudaMemset(s->d_slot_m, 0, nd * sizeof(int32_t)) ||
         cudaMemset(s->pool, 0, (size_t)std::max<int64_t>(s->pool_bytes, 256)) != cudaSuccess)
@@ -1297,7 +1334,7 @@ dopr_status dopr_build_prefixes(dopr_model* m, dopr_store* s, int32_t n_docs, co
     if (x_offsets[d + 1] > x_offsets[d]) pd.push_back(d);
   const int32_t n = (int32_t)pd.size();
   if (n > 0) {
-    STATUS_TRY(ensure_call_buffers(m, n, rows, 0));
+    STATUS_TRY(ensure_call_buffers(m, n, rows));
     std::vector<int32_t> tok_id(rows), tok_pos(rows), tok_pair(rows);
     w.h_tok_off[0] = 0;
     for (int32_t p = 0; p < n; ++p) {
@@ -1349,7 +1386,8 @@ dopr_status dopr_build_prefixes(dopr_model* m, dopr_store* s, int32_t n_docs, co
       }
       dx = stage;
     }
-    CUDA_TRY(cudaMemsetAsync(w.err, 0, w.err_bytes, st));
+    CUDA_TRY(cudaMemsetAsync(w.err, 0, sizeof(int), st));
+    CUDA_TRY(cudaMemsetAsync(w.ss_count, 0, sizeof(int) * w.n_ss_count, st));
     BuildArgs b{dx, (int64_t)rows};
     const dopr_status rs = run_layers(m, s, plan, nullptr, st, &b);
     cudaError_t e = cudaMemcpyAsync(w.h_err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -1399,7 +1437,7 @@ dopr_status dopr_select_prefix_inputs(dopr_model* m, int32_t n_docs, const int32
     STATUS_TRY(dopr_store_create(&c, 0, 256, &empty));
     w.sel_empty = empty;
   }
-  dopr_status rs = ensure_call_buffers(m, n_docs, T, 0);
+  dopr_status rs = ensure_call_buffers(m, n_docs, T);
   if (rs != DOPR_OK) return rs;
   std::vector<int32_t> tok_pos(T), tok_pair(T);
   for (int32_t d = 0; d < n_docs; ++d) {
@@ -1473,7 +1511,8 @@ dopr_status dopr_select_prefix_inputs(dopr_model* m, int32_t n_docs, const int32
   CUDA_TRY(cudaMemcpyAsync(w.sel_units, units.data(), sizeof(SelUnit) * units.size(), cudaMemcpyHostToDevice, st));
   SelectState sel{top_k, top_p, w.sel_A, a_max, w.sel_a_off, w.sel_u, w.sel_pos, w.sel_x, w.sel_units, w.sel_stats,
                   std::move(chunks)};
-  cudaError_t e = cudaMemsetAsync(w.err, 0, w.err_bytes, st);
+  cudaError_t e = cudaMemsetAsync(w.err, 0, sizeof(int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w.ss_count, 0, sizeof(int) * w.n_ss_count, st);
   rs = e == cudaSuccess ? run_layers(m, w.sel_empty, plan, nullptr, st, nullptr, &sel)
                          : fail(DOPR_ERR_CUDA, "memset failed");
   if (rs == DOPR_OK) {
@@ -1543,29 +1582,25 @@ dopr_status dopr_score(dopr_model* m, dopr_store* s, int32_t n, const int32_t* q
   if (!io_on_device) {
     if (n > 0 && q_offsets[n] > 0 && !q_tokens) return fail(DOPR_ERR_INVALID_ARG, "q_tokens is NULL");
     STATUS_TRY(validate_host_inputs(m, s, n, q_offsets, q_tokens, doc_ids));
-    const int64_t nq = q_offsets[n];
-    STATUS_TRY(ensure_call_buffers(m, n, 0, std::max<int64_t>(nq, 1)));
-    CUDA_TRY(cudaMemcpyAsync(w.q_off, q_offsets, sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, st));
-    if (nq > 0) CUDA_TRY(cudaMemcpyAsync(w.q_tok, q_tokens, sizeof(int32_t) * nq, cudaMemcpyHostToDevice, st));
-    CUDA_TRY(cudaMemcpyAsync(w.doc_ids, doc_ids, sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
-    dqo = w.q_off;
-    dqt = w.q_tok;
-    ddoc = w.doc_ids;
+    STATUS_TRY(ensure_call_buffers(m, n, 0));
+    STATUS_TRY(upload_inputs(w, n, q_offsets, q_tokens, doc_ids, st, &dqo, &dqt, &ddoc));
   } else {
-    STATUS_TRY(ensure_call_buffers(m, n, 0, 0));
+    STATUS_TRY(ensure_call_buffers(m, n, 0));
   }
   Plan plan;
   STATUS_TRY(run_packer(m, s, n, dqo, dqt, ddoc, st, plan));
   // scores land in the workspace and reach the caller only once the device error
   // word is known to be clear: a failed call writes nothing
   STATUS_TRY(run_layers(m, s, plan, w.scores, st));
-  CUDA_TRY(cudaMemcpyAsync(w.h_err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  // one copy and one wait: the scores reach a host caller with the error word, a device caller
+  // through a kernel that reads the word first
+  if (io_on_device) CUDA_TRY(launch_commit_scores(w.err, w.scores, scores, n, st));
+  const size_t bytes = sizeof(int) * (io_on_device ? 1 : RESULT_HEAD + (size_t)n);
+  CUDA_TRY(cudaMemcpyAsync(w.h_err, w.err, bytes, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   prof_collect(m);
   STATUS_TRY(map_device_error(*w.h_err));
-  CUDA_TRY(cudaMemcpyAsync(scores, w.scores, sizeof(float) * n,
-                           io_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaStreamSynchronize(st));
+  if (!io_on_device) memcpy(scores, w.h_err + RESULT_HEAD, sizeof(float) * n);
   return DOPR_OK;
 }
 
@@ -1583,14 +1618,13 @@ dopr_status dopr_debug_pack_plan(dopr_model* m, dopr_store* s, int32_t n, const 
   STATUS_TRY(validate_host_inputs(m, s, n, q_offsets, q_tokens, doc_ids));
   CUDA_TRY(cudaSetDevice(m->device));
   Workspace& w = m->ws;
-  const int64_t nq = q_offsets[n];
-  STATUS_TRY(ensure_call_buffers(m, n, 0, std::max<int64_t>(nq, 1)));
+  STATUS_TRY(ensure_call_buffers(m, n, 0));
   cudaStream_t st = 0;
-  CUDA_TRY(cudaMemcpy(w.q_off, q_offsets, sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice));
-  if (nq > 0) CUDA_TRY(cudaMemcpy(w.q_tok, q_tokens, sizeof(int32_t) * nq, cudaMemcpyHostToDevice));
-  CUDA_TRY(cudaMemcpy(w.doc_ids, doc_ids, sizeof(int64_t) * n, cudaMemcpyHostToDevice));
+  const int32_t *dqo, *dqt;
+  const int64_t* ddoc;
+  STATUS_TRY(upload_inputs(w, n, q_offsets, q_tokens, doc_ids, st, &dqo, &dqt, &ddoc));
   Plan plan;
-  STATUS_TRY(run_packer(m, s, n, w.q_off, w.q_tok, w.doc_ids, st, plan));
+  STATUS_TRY(run_packer(m, s, n, dqo, dqt, ddoc, st, plan));
   const int64_t T = plan.n_tokens;
   CUDA_TRY(cudaStreamSynchronize(st));
   CUDA_TRY(cudaMemcpy(perm, w.perm, sizeof(int32_t) * n, cudaMemcpyDeviceToHost));

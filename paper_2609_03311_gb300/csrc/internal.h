@@ -82,6 +82,7 @@ struct Store {
   int32_t max_m = 0;
   CUtensorMap tm_pool{};
   bool tm_pool_ok = false;
+  int* h_err = nullptr;  // pinned: the ordering entry point's error word
 };
 
 // GEMM epilogues.
@@ -113,6 +114,8 @@ struct SelUnit {
   int64_t a_off;
 };
 
+constexpr int RESULT_HEAD = 64;  // ints before the scores of a result block
+
 struct Workspace {
   int chunk_cap = 0;  // tokens per chunk
   float* r = nullptr;          // [chunk][H] fp32 residual stream
@@ -127,11 +130,8 @@ struct Workspace {
   float* ss_s = nullptr;       // [chunk][2H/256] their attention-norm partial sums
   GemmOperandA tm_xn, tm_o, tm_act;
   // per call, grown on demand
-  int64_t pair_cap = 0, tok_cap = 0, qtok_cap = 0, item_cap = 0;
-  int32_t* q_off = nullptr;
-  int32_t* q_tok = nullptr;
-  int64_t* doc_ids = nullptr;
-  float* scores = nullptr;
+  int64_t pair_cap = 0, tok_cap = 0, in_cap = 0, item_cap = 0;
+  uint8_t* in = nullptr;  // a host call's inputs in one block (InputBlock)
   int32_t* pair_slot = nullptr;
   int32_t* perm = nullptr;
   int32_t* sorted_slot = nullptr;
@@ -139,20 +139,24 @@ struct Workspace {
   int32_t* tok_id = nullptr;
   int32_t* tok_pos = nullptr;
   int32_t* tok_pair = nullptr;
-  AttnItem* items = nullptr;     // all items of the call, then the mma.sync kernel's items
-  AttnTile* tiles = nullptr;     // tensor-core attention tiles of the call
-  int64_t tile_cap = 0;
-  // the call's device error word, then the few-row GEMMs' chunk counts (cleared with it)
+  // the attention plan in one block: all items of the call, the mma.sync kernel's items, then
+  // (`tiles` points there once the plan is made) the tensor-core tiles
+  AttnItem* items = nullptr;
+  AttnTile* tiles = nullptr;
+  int64_t plan_cap = 0;  // bytes
+  // the call's device error word (RESULT_HEAD ints), then its scores
   int* err = nullptr;
-  size_t err_bytes = 0;
+  float* scores = nullptr;
+  int* ss_count = nullptr;     // the few-row GEMMs' chunk counts, 0 when a pass starts
+  int n_ss_count = 0;
   float* ss_chunks = nullptr;  // [GEMM_FEW_MAX_ROWS / 32][H/128][1024]
   // pinned host staging
   int32_t* h_tok_off = nullptr;
   int32_t* h_sorted_slot = nullptr;
-  int* h_err = nullptr;
-  AttnItem* h_items = nullptr;
-  AttnTile* h_tiles = nullptr;
-  int64_t h_pair_cap = 0, h_item_cap = 0;
+  uint8_t* h_in = nullptr;
+  int* h_err = nullptr;      // the result block's copy
+  AttnItem* h_items = nullptr;  // the plan block's
+  int64_t h_pair_cap = 0, h_in_cap = 0, h_plan_cap = 0;
   // key token selection (dopr_select_prefix_inputs), grown on demand and kept
   Store* sel_empty = nullptr;  // a store of one empty document: a valid pool map for the attention kernels
   float* sel_A = nullptr;      // per-document attention matrices of the largest chunk (sum of n^2)
@@ -375,7 +379,14 @@ struct PackArgs {
   int32_t* tok_id;
   int32_t* tok_pos;
   int32_t* tok_pair;
-  int* err;
+  int* err;           // set to 0 first
+  // pinned host copies that the ordering kernel writes itself: the error word after validation,
+  // the offsets and slots (null: not wanted); and ints it clears
+  int* h_err;
+  int32_t* h_tok_off;
+  int32_t* h_sorted_slot;
+  int* zero;
+  int n_zero;
 };
 // Shared memory of the ordering kernel, once per device (dopr_store_create).
 cudaError_t pack_setup();
@@ -384,6 +395,8 @@ cudaError_t pack_setup();
 cudaError_t launch_pack_order(const PackArgs& a, cudaStream_t st);
 // Second part, once the token buffers are sized: token ids, positions, pair index.
 cudaError_t launch_pack_tokens(const PackArgs& a, cudaStream_t st);
+// out[0, n) = scores[0, n) unless the call's error word is set.
+cudaError_t launch_commit_scores(const int* err, const float* scores, float* out, int n, cudaStream_t st);
 
 // Sets the message dopr_last_error() returns on this thread.
 void set_last_error_message(const std::string& msg);

@@ -6,7 +6,8 @@
 // adjacent: a stable sort on doc_id (ties keep input order), then
 // lays every pair's [query tokens ; score token] end to end in that order
 // with RoPE positions m_doc + j.  Steps:
-//   1. k_pack_order, one cluster: validate pairs and look up store slots, sort by doc id
+//   1. k_pack_order, one cluster (which also leaves what the host plans with in pinned memory, so
+//      that no copies follow it): validate pairs and look up store slots, sort by doc id
 //      (radix, 10 bits a pass), exclusive scan of per-pair token counts (packed token offsets);
 //   2. k_pack_tokens (after the host has sized the token buffers): token ids / positions.
 #include "device_common.cuh"
@@ -83,6 +84,12 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_pack_order(PackArgs a, int do
     return v;
   };
 
+  if (rank == 0) {
+    for (int i = tid; i < a.n_zero; i += ORDER_THREADS) a.zero[i] = 0;
+    if (tid == 0) *a.err = 0;
+  }
+  meet();
+
   // ---- validate: every pair's slot, or the batch's errors
   int flags = 0;
   for (int p0 = rank * ORDER_THREADS + tid; p0 < n; p0 += ctas * ORDER_THREADS * AHEAD) {
@@ -115,7 +122,9 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_pack_order(PackArgs a, int do
   }
   if (flags) atomicOr(a.err, flags);
   meet();
-  if (ld_volatile(a.err) & INPUT_ERRORS) return;  // the same word for the whole cluster
+  const int found = ld_volatile(a.err);  // the same word for the whole cluster
+  if (rank == 0 && tid == 0) *a.h_err = found;
+  if (found & INPUT_ERRORS) return;
 
   // ---- stable sort by doc id; the order goes to perm, by way of sorted_slot
   const int passes = (doc_bits + DIGIT_BITS - 1) / DIGIT_BITS, bits = (doc_bits + passes - 1) / passes;
@@ -205,7 +214,9 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_pack_order(PackArgs a, int do
   int32_t sum = 0, total;
   for (int s = lo + tid; s < hi; s += ORDER_THREADS) {
     const int p = __ldcg(a.perm + s);
-    a.sorted_slot[s] = __ldcg(a.pair_slot + p);
+    const int slot = __ldcg(a.pair_slot + p);
+    a.sorted_slot[s] = slot;
+    if (a.h_sorted_slot) a.h_sorted_slot[s] = slot;
     const int len = a.q_off[p + 1] - a.q_off[p] + 1;
     a.tok_off[s] = len;
     sum += len;
@@ -225,10 +236,16 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_pack_order(PackArgs a, int do
     const int s = s0 + tid;  // written by this thread above
     const int32_t len = s < hi ? a.tok_off[s] : 0;
     const int32_t at = carry + block_scan(len, warp_sums, &total);
-    if (s < hi) a.tok_off[s] = at;
+    if (s < hi) {
+      a.tok_off[s] = at;
+      if (a.h_tok_off) a.h_tok_off[s] = at;
+    }
     carry += total;
   }
-  if (tid == 0 && rank == ctas - 1) a.tok_off[n] = carry;
+  if (tid == 0 && rank == ctas - 1) {
+    a.tok_off[n] = carry;
+    if (a.h_tok_off) a.h_tok_off[n] = carry;
+  }
   if constexpr (CTAS > 1) cluster_sync();  // no CTA leaves while another may read its total
 }
 
@@ -253,7 +270,19 @@ __global__ void k_pack_tokens(PackArgs a) {
   }
 }
 
+__global__ void k_commit_scores(const int* err, const float* __restrict__ scores, float* __restrict__ out, int n) {
+  pdl_trigger();
+  pdl_wait();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n && ld_volatile(err) == 0) out[i] = scores[i];
+}
+
 }  // namespace
+
+cudaError_t launch_commit_scores(const int* err, const float* scores, float* out, int n, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  return launch_dependent(k_commit_scores, (n + 255) / 256, 256, 0, st, err, scores, out, n);
+}
 
 cudaError_t pack_setup() {
   const cudaError_t e = cudaFuncSetAttribute(k_pack_order<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, ORDER_SMEM);

@@ -136,15 +136,13 @@ extern "C" dopr_status dopr_pack_order_noalloc(const dopr_store* store, int32_t 
   a.perm = perm;
   a.sorted_slot = scratch + NOALLOC_MAX_PAIRS;
   a.tok_off = tok_off;
-  a.err = err;
-  int h_err = 0;
-  e = cudaMemsetAsync(err, 0, sizeof(int32_t), stream);  // the error word must start at zero
-  if (e == cudaSuccess) e = launch_pack_order(a, stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h_err, err, sizeof(int32_t), cudaMemcpyDeviceToHost, stream);
+  a.err = err;  // cleared and copied to the store's pinned word by the kernel
+  a.h_err = store->h_err;
+  e = launch_pack_order(a, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) {
     set_last_error_message(std::string("CUDA error: ") + cudaGetErrorString(e));
     return DOPR_ERR_CUDA;
   }
-  return device_error_status(h_err);
+  return device_error_status(*store->h_err);
 }
