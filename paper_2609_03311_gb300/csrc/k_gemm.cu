@@ -56,7 +56,7 @@ static_assert(GEMM_B_BOX == BM, "each CTA of a pair stages 128 of a tile's 256 B
 constexpr int A_BYTES = BM * BK * 2;  // 16 KiB
 constexpr int THREADS = 320;
 constexpr int EPI_WARPS = 8;
-constexpr int XPOSE_WORDS = 32 * 33;  // per epilogue warp: 32 rows x 32 words, padded row stride 33
+constexpr int XPOSE_WORDS = 32 * 32;  // per epilogue warp: 32 rows x 32 words, 16-byte chunks swizzled by the row
 constexpr int XPOSE_BYTES = EPI_WARPS * XPOSE_WORDS * 4;
 constexpr int BAR_BYTES = 256;
 
@@ -139,12 +139,28 @@ __device__ __forceinline__ void publish_square_sums(const GemmParams& p, int row
   store_square_sums(p, row0, lane, group, sum);
 }
 
-// The warp's 32 rows x 32 words sit in `xs` (row-per-lane layout, stride 33).
+// Four words (a 16-byte chunk) of a row in a warp's transpose buffer: chunk c of row r lies at
+// c ^ s(r) with s a permutation of r & 7 that sends neighbours 4 apart, so that a lane writing its
+// own row, eight lanes reading one row and two times four lanes reading the same half of two
+// neighbouring rows all move whole 16-byte chunks without bank conflicts.
+__device__ __forceinline__ uint4* xs_chunk(uint32_t* xs, int r, int c) {
+  return reinterpret_cast<uint4*>(xs + r * 32 + ((c ^ ((r & 1) << 2 | (r >> 1 & 3))) << 2));
+}
+__device__ __forceinline__ void xs_put_row(uint32_t* xs, int lane, const uint32_t (&v)[32]) {
+#pragma unroll
+  for (int c = 0; c < 8; ++c) *xs_chunk(xs, lane, c) = make_uint4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+}
+__device__ __forceinline__ float4 xs_get(uint32_t* xs, int r, int c) {
+  const uint4 w = *xs_chunk(xs, r, c);
+  return make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
+}
+
+// The warp's 32 rows x 32 words sit in `xs` (row-per-lane layout, xs_chunk).
 // Write the first WORDS words of each row out transposed: with 32 words lane L covers rows
 // i*4 + L/8 (i = 0..7) and words (L%8)*4 .. +3, i.e. 8 lanes per 128-byte row segment
 // (16 words: 4 lanes per 64-byte segment).  dst(r, w) is where word w of row r goes.
 template <int WORDS, typename RowPtr>
-__device__ __forceinline__ void store_words_transposed(const uint32_t* xs, int lane, int row0, int M, RowPtr dst) {
+__device__ __forceinline__ void store_words_transposed(uint32_t* xs, int lane, int row0, int M, RowPtr dst) {
   constexpr int LANES = WORDS / 4;  // lanes to a row segment
   static_assert(WORDS == 32 || WORDS == 16, "row segments of 128 or 64 bytes");
 #pragma unroll
@@ -152,11 +168,7 @@ __device__ __forceinline__ void store_words_transposed(const uint32_t* xs, int l
     const int r = i * (32 / LANES) + lane / LANES;
     const int w = (lane % LANES) * 4;
     if (row0 + r < M) {
-      uint4 v;
-      v.x = xs[r * 33 + w + 0];
-      v.y = xs[r * 33 + w + 1];
-      v.z = xs[r * 33 + w + 2];
-      v.w = xs[r * 33 + w + 3];
+      const uint4 v = *xs_chunk(xs, r, w >> 2);
       *reinterpret_cast<uint4*>(dst(r, w)) = v;
     }
   }
@@ -166,7 +178,7 @@ __device__ __forceinline__ void store_words_transposed(const uint32_t* xs, int l
 // the tile's main loop still runs, so its load latency is off the epilogue's path.
 struct EpiPre {
   float scale;  // this thread's row: the consumer row scale (QKV, SwiGLU) or the previous norm factor
-  int pos[8];   // QKV: positions of the 8 rows a lane rotates in the transposed layout
+  int pos[4];   // QKV: positions of the 4 rows a lane rotates in the transposed layout
 };
 
 template <int EPI, int BNT>
@@ -182,7 +194,7 @@ __device__ __forceinline__ void epilogue_prefetch(const GemmParams& p, int row0,
   if constexpr (EPI == EPI_QKV) {
     if (nb * BNT + (BNT == 256 ? part * 128 : 0) < p.q_cols + p.k_cols)
 #pragma unroll
-      for (int i = 0; i < 8; ++i) pre.pos[i] = p.tok_pos[min(row0 + i * 4 + (lane >> 3), p.M - 1)];
+      for (int i = 0; i < 4; ++i) pre.pos[i] = p.tok_pos[min(row0 + i * 8 + (lane >> 2), p.M - 1)];
   }
 }
 
@@ -205,88 +217,91 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
       const int hc = nb * BNT + hh * 128;      // first output column of this head
       const bool rope = (EPI == EPI_QKV) && hc < p.q_cols + p.k_cols;
       if (rope) {
+        // The rotation runs in the transposed layout, 16 frequencies at a time: lane L owns rows
+        // i*8 + L/4 and frequencies w4 .. w4+3 of the 16, so RoPE-table reads and the stores are
+        // contiguous 4-lane row segments.  The (cos, sin) of the next 16 are fetched while these
+        // are rotated (rows past M read position 0's entries and are not stored).
+        constexpr int STEPS = ONE ? 2 : 4;
+        const int f0 = ONE ? part * 32 : 0, w4 = (lane & 3) * 4;
+        float4 c01[4], c23[4];
+        auto fetch_rope = [&](int f) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4* cs = reinterpret_cast<const float4*>(p.rope + static_cast<int64_t>(pre.pos[i]) * 64 + f + w4);
+            c01[i] = __ldg(cs);
+            c23[i] = __ldg(cs + 1);
+          }
+        };
+        fetch_rope(f0);
         // per-head RMSNorm of the row-scaled values: sum of squares in the row layout
         float ss = 0.f;
-#pragma unroll 1
-        for (int c = 0; c < 128; c += 32) {
-          uint32_t v[32];
+#pragma unroll
+        for (int c = 0; c < 128; c += 64) {
+          uint32_t v[32], w[32];
           tmem_ld32(taddr + hh * 128 + c, v);
+          tmem_ld32(taddr + hh * 128 + c + 32, w);
           tmem_ld_wait();
 #pragma unroll
           for (int j = 0; j < 32; ++j) ss += __uint_as_float(v[j]) * __uint_as_float(v[j]);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) ss += __uint_as_float(w[j]) * __uint_as_float(w[j]);
         }
         const float inv_row = rs * rsqrtf(ss * rs * rs * (1.f / 128.f) + p.eps);
         const bf16* wgt = hc < p.q_cols ? p.q_norm : p.k_norm;
-        // the rotation runs in the transposed layout: lane L owns rows i*4 + L/8 and
-        // columns w4 .. w4+3 of each 32-column chunk, so RoPE-table reads and the
-        // stores are contiguous 8-lane row segments
-        const int w4 = (lane & 7) * 4;
-        float inv_i[8];
+        float inv_i[4];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) inv_i[i] = __shfl_sync(0xffffffffu, inv_row, i * 4 + (lane >> 3));
-#pragma unroll 1
-        for (int c = ONE ? part * 32 : 0; c < (ONE ? part * 32 + 32 : 64); c += 32) {
-          // the rows' (cos, sin) for frequencies c+w4 .. +3 (rows past M read position
-          // 0's entries and are not stored), ahead of the accumulator reads below
-          float4 c01[8], c23[8];
+        for (int i = 0; i < 4; ++i) inv_i[i] = __shfl_sync(0xffffffffu, inv_row, i * 8 + (lane >> 2));
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const float4* cs = reinterpret_cast<const float4*>(p.rope + static_cast<int64_t>(pre.pos[i]) * 64 + c + w4);
-            c01[i] = cs[0];
-            c23[i] = cs[1];
-          }
+        for (int s = 0; s < STEPS; ++s) {
+          const int f = f0 + 16 * s;
+          uint32_t v[32];  // the row's 16 elements of the first half of the head, then those 64 further on
+          tmem_ld16x2(taddr + hh * 128 + f, taddr + hh * 128 + 64 + f, v);
+          tmem_ld_wait();
+          xs_put_row(xs, lane, v);
+          __syncwarp();
           float g1[4], g2[4];
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            g1[k] = __bfloat162float(wgt[c + w4 + k]);
-            g2[k] = __bfloat162float(wgt[64 + c + w4 + k]);
+            g1[k] = __bfloat162float(wgt[f + w4 + k]);
+            g2[k] = __bfloat162float(wgt[64 + f + w4 + k]);
           }
-          float4 x1[8], x2[8];
+          uint2 o1[4], o2[4];
 #pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            uint32_t v[32];
-            tmem_ld32(taddr + hh * 128 + half * 64 + c, v);
-            tmem_ld_wait();
+          for (int i = 0; i < 4; ++i) {
+            const int r = i * 8 + (lane >> 2);
+            const float4 x1 = xs_get(xs, r, lane & 3), x2 = xs_get(xs, r, 4 + (lane & 3));
+            const float cosv[4] = {c01[i].x, c01[i].z, c23[i].x, c23[i].z};
+            const float sinv[4] = {c01[i].y, c01[i].w, c23[i].y, c23[i].w};
+            const float a[4] = {x1.x, x1.y, x1.z, x1.w}, b[4] = {x2.x, x2.y, x2.z, x2.w};
+            float y1[4], y2[4];
+            bool out_of_range = false;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) xs[lane * 33 + j] = v[j];
-            __syncwarp();
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int r = i * 4 + (lane >> 3);
-              const float4 t = make_float4(__uint_as_float(xs[r * 33 + w4]), __uint_as_float(xs[r * 33 + w4 + 1]),
-                                           __uint_as_float(xs[r * 33 + w4 + 2]), __uint_as_float(xs[r * 33 + w4 + 3]));
-              if (half == 0)
-                x1[i] = t;
-              else
-                x2[i] = t;
+            for (int k = 0; k < 4; ++k) {
+              const float u = a[k] * inv_i[i] * g1[k], w = b[k] * inv_i[i] * g2[k];
+              y1[k] = u * cosv[k] - w * sinv[k];
+              y2[k] = w * cosv[k] + u * sinv[k];
+              out_of_range |= !(fp16_ok(y1[k]) && fp16_ok(y2[k]));
             }
-            __syncwarp();
+            bad |= out_of_range && row0 + r < p.M;
+            o1[i] = make_uint2(pack_f16x2(y1[0], y1[1]), pack_f16x2(y1[2], y1[3]));
+            o2[i] = make_uint2(pack_f16x2(y2[0], y2[1]), pack_f16x2(y2[2], y2[3]));
           }
+          if (s + 1 < STEPS) fetch_rope(f + 16);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int r = i * 4 + (lane >> 3);
+          for (int i = 0; i < 4; ++i) {
+            const int r = i * 8 + (lane >> 2);
             if (row0 + r < p.M) {
-              const float cosv[4] = {c01[i].x, c01[i].z, c23[i].x, c23[i].z};
-              const float sinv[4] = {c01[i].y, c01[i].w, c23[i].y, c23[i].w};
-              const float a[4] = {x1[i].x, x1[i].y, x1[i].z, x1[i].w}, b[4] = {x2[i].x, x2[i].y, x2[i].z, x2[i].w};
-              float y1[4], y2[4];
-#pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                const float u = a[k] * inv_i[i] * g1[k], w = b[k] * inv_i[i] * g2[k];
-                y1[k] = u * cosv[k] - w * sinv[k];
-                y2[k] = w * cosv[k] + u * sinv[k];
-                bad |= !(fp16_ok(y1[k]) && fp16_ok(y2[k]));
-              }
-              f16* orow = out + static_cast<int64_t>(row0 + r) * p.ld_out + hc + c + w4;
-              *reinterpret_cast<uint2*>(orow) = make_uint2(pack_f16x2(y1[0], y1[1]), pack_f16x2(y1[2], y1[3]));
-              *reinterpret_cast<uint2*>(orow + 64) = make_uint2(pack_f16x2(y2[0], y2[1]), pack_f16x2(y2[2], y2[3]));
+              f16* orow = out + static_cast<int64_t>(row0 + r) * p.ld_out + hc + f + w4;
+              *reinterpret_cast<uint2*>(orow) = o1[i];
+              *reinterpret_cast<uint2*>(orow + 64) = o2[i];
             }
           }
+          __syncwarp();
         }
       } else {
 #pragma unroll 1
         for (int c = ONE ? part * 64 : 0; c < (ONE ? part * 64 + 64 : 128); c += 64) {
-          uint32_t a[32], b[32];
+          uint32_t a[32], b[32], o[32];
           tmem_ld32(taddr + hh * 128 + c, a);
           tmem_ld32(taddr + hh * 128 + c + 32, b);
           tmem_ld_wait();
@@ -295,9 +310,10 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
             const float a0 = __uint_as_float(a[j]) * rs, a1 = __uint_as_float(a[j + 1]) * rs;
             const float b0 = __uint_as_float(b[j]) * rs, b1 = __uint_as_float(b[j + 1]) * rs;
             bad |= live && !(fp16_ok(a0) && fp16_ok(a1) && fp16_ok(b0) && fp16_ok(b1));
-            xs[lane * 33 + j / 2] = pack_f16x2(a0, a1);
-            xs[lane * 33 + 16 + j / 2] = pack_f16x2(b0, b1);
+            o[j / 2] = pack_f16x2(a0, a1);
+            o[16 + j / 2] = pack_f16x2(b0, b1);
           }
+          xs_put_row(xs, lane, o);
           __syncwarp();
           store_words_transposed<32>(xs, lane, row0, p.M, [&](int r, int wd) {
             return out + static_cast<int64_t>(row0 + r) * p.ld_out + hc + c + 2 * wd;
@@ -312,6 +328,9 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
     // residual values of chunk c+1 are loaded while chunk c is processed.
     float* res = reinterpret_cast<float*>(p.out);
     const int w4 = (lane & 7) * 4;
+    // this lane's chunk of row i*4 + lane/8 lies at cpos ^ 2 (i & 1) of the transpose buffer's row
+    const int cpos = (lane & 7) ^ ((lane >> 3 & 1) << 2 | lane >> 4);
+    uint32_t* xrow = xs + (lane >> 3) * 32;
     float ss[8], prev[8];
     // each lane fetched its own row's previous norm factor; the row layout below takes them by shuffle
 #pragma unroll
@@ -338,8 +357,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
       uint32_t v[32];
       tmem_ld32(taddr + c, v);
       tmem_ld_wait();
-#pragma unroll
-      for (int j = 0; j < 32; ++j) xs[lane * 33 + j] = v[j];
+      xs_put_row(xs, lane, v);
       __syncwarp();
       const int col = nb * BNT + c + w4;
       if (BNT < 256) {  // a chunk's sums stand alone here
@@ -358,10 +376,11 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
         const int r = i * 4 + (lane >> 3);
         if (row0 + r < p.M) {
           float4 x = cur[i];
-          x.x += __uint_as_float(xs[r * 33 + w4 + 0]);
-          x.y += __uint_as_float(xs[r * 33 + w4 + 1]);
-          x.z += __uint_as_float(xs[r * 33 + w4 + 2]);
-          x.w += __uint_as_float(xs[r * 33 + w4 + 3]);
+          const float4 d = *reinterpret_cast<const float4*>(xrow + i * 128 + ((cpos ^ (i & 1) << 1) << 2));
+          x.x += d.x;
+          x.y += d.y;
+          x.z += d.z;
+          x.w += d.w;
           *rrow(i, c) = x;
           if (p.xn_out) {
             ss[i] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
@@ -395,11 +414,17 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
         tmem_ld32(taddr + OUTS + c + 32 * half, u);
         tmem_ld_wait();
 #pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-          const float a0 = silu_f(__uint_as_float(g[j]) * rs) * (__uint_as_float(u[j]) * rs);
-          const float a1 = silu_f(__uint_as_float(g[j + 1]) * rs) * (__uint_as_float(u[j + 1]) * rs);
-          bad |= live && !(fp16_ok(a0) && fp16_ok(a1));
-          xs[lane * 33 + 16 * half + j / 2] = pack_f16x2(a0, a1);
+        for (int c4 = 0; c4 < 4; ++c4) {  // eight outputs: one 16-byte chunk
+          uint32_t o[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int j = c4 * 8 + 2 * k;
+            const float a0 = silu_f(__uint_as_float(g[j]) * rs) * (__uint_as_float(u[j]) * rs);
+            const float a1 = silu_f(__uint_as_float(g[j + 1]) * rs) * (__uint_as_float(u[j + 1]) * rs);
+            bad |= live && !(fp16_ok(a0) && fp16_ok(a1));
+            o[k] = pack_f16x2(a0, a1);
+          }
+          *xs_chunk(xs, lane, 4 * half + c4) = make_uint4(o[0], o[1], o[2], o[3]);
         }
       }
       __syncwarp();
