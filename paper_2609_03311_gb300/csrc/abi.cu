@@ -995,7 +995,8 @@ static bool make_tmap_k_blocks(CUtensorMap* map, const void* base, uint64_t k, u
 
 bool make_gemm_operand_a(GemmOperandA* a, const void* base, uint64_t k, uint64_t rows) {
   bool ok = make_tmap_16b_2d(&a->wide, base, k, rows, k * 2, GEMM_BK, GEMM_BM, true, true);
-  for (int i = 0; i < 3; ++i) ok = ok && make_tmap_k_blocks(&a->few[i], base, k, rows, 32u << i, GEMM_FEW_KB(32 << i));
+  for (int i = 0; i < 4; ++i)
+    ok = ok && make_tmap_k_blocks(&a->few[i], base, k, rows, 32u * (i + 1), GEMM_FEW_KB(32 * (i + 1)));
   return ok;
 }
 

@@ -96,7 +96,7 @@ __host__ __device__ constexpr int GEMM_FEW_KB(int rows) { return rows == 32 ? 4 
 // Tensor maps of a GEMM operand (fp16, 128-byte swizzle): `wide` 2-D boxes of 64 elements x 128
 // rows; `few` 3-D (64 elements, rows, k-blocks of 64) boxes of 64 x R rows x GEMM_FEW_KB(R).
 struct GemmOperandA {
-  CUtensorMap wide{}, few[3]{};  // R = 32, 64, 128
+  CUtensorMap wide{}, few[4]{};  // R = 32, 64, 96, 128
 };
 struct GemmOperandB {
   CUtensorMap wide{}, few[2][2]{};  // [64 or 128 tile columns: 32 or 64 rows a CTA][2 or 4 k-blocks]
@@ -276,7 +276,7 @@ struct GemmParams {
 };
 cudaError_t gemm_setup();
 // The tile a launch of M rows takes: wide (k_gemm_pair, 2 x 128 rows, 256 columns) or, for few
-// rows, 2 x 32, 64 or 128 rows and 64 or 128 columns (k_gemm_few).
+// rows, 2 x 32, 64, 96 or 128 rows and 64 or 128 columns (k_gemm_few).
 struct GemmPlan {
   bool few;
   int rows, cols;  // A rows per CTA of the pair, columns

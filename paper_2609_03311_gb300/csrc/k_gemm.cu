@@ -669,7 +669,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 
 // ============================================================================
 // Few rows (the last layer's score rows, small batches): the pair kernel with narrower tiles,
-// 64 or 128 columns, and R = 32, 64 or 128 A rows per CTA instead of 128.
+// 64 or 128 columns, and R = 32, 64, 96 or 128 A rows per CTA instead of 128.
 //
 // With few rows a launch is bound by streaming the weights, and 256-column tiles leave most
 // SMs without a tile (O and down of the 8B shape: 16 tiles on 32 of 152 SMs) while each SM
@@ -870,14 +870,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 template <int EPI, typename F>
 auto few_kernel(int rows, int cols, F&& f) {
   if constexpr (EPI == EPI_RESID_ADD || EPI == EPI_SWIGLU)
-    if (cols == 64) return rows == 32 ? f(k_gemm_few<EPI, 64, 32>) : rows == 64 ? f(k_gemm_few<EPI, 64, 64>) : f(k_gemm_few<EPI, 64, 128>);
-  return rows == 32 ? f(k_gemm_few<EPI, 128, 32>) : rows == 64 ? f(k_gemm_few<EPI, 128, 64>) : f(k_gemm_few<EPI, 128, 128>);
+    if (cols == 64)
+      return rows == 32   ? f(k_gemm_few<EPI, 64, 32>)
+             : rows == 64 ? f(k_gemm_few<EPI, 64, 64>)
+             : rows == 96 ? f(k_gemm_few<EPI, 64, 96>)
+                          : f(k_gemm_few<EPI, 64, 128>);
+  return rows == 32   ? f(k_gemm_few<EPI, 128, 32>)
+         : rows == 64 ? f(k_gemm_few<EPI, 128, 64>)
+         : rows == 96 ? f(k_gemm_few<EPI, 128, 96>)
+                      : f(k_gemm_few<EPI, 128, 128>);
 }
 
 template <int EPI>
 cudaError_t set_smem() {
   cudaError_t e = cudaFuncSetAttribute(k_gemm_pair<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, PAIR_SMEM_BYTES);
-  for (int rows = 32; rows <= BM; rows *= 2)
+  for (int rows = 32; rows <= BM; rows += 32)
     for (int cols = 64; cols <= 128; cols *= 2)
       if (e == cudaSuccess)
         e = few_kernel<EPI>(rows, cols, [](auto* k) {
@@ -894,7 +901,7 @@ cudaError_t launch_epi(const GemmOperandA& A, const GemmOperandB& B, const GemmP
   if (!g.few) {
     return launch_dependent(k_gemm_pair<EPI>, grid, THREADS, PAIR_SMEM_BYTES, st, A.wide, B.wide, p);
   }
-  const CUtensorMap& ta = A.few[g.rows == 32 ? 0 : g.rows == 64 ? 1 : 2];
+  const CUtensorMap& ta = A.few[g.rows / 32 - 1];
   const CUtensorMap& tb = B.few[g.cols == 128][GEMM_FEW_KB(g.rows) == 4];
   return few_kernel<EPI>(g.rows, g.cols,
                          [&](auto* k) { return launch_dependent(k, grid, THREADS, FEW_SMEM_BYTES, st, ta, tb, p); });
@@ -931,7 +938,7 @@ GemmPlan gemm_plan(int epi, int M, int N, int K, int num_sms) {
   const int cols[2] = {128, 64};
   for (int n : cols) {
     if (N % n || (n == 64 && epi != EPI_RESID_ADD && epi != EPI_SWIGLU)) continue;
-    for (int R = 32; R <= BM; R *= 2)
+    for (int R = 32; R <= BM; R += 32)
       if (clocks(R, n) < least) {
         least = clocks(R, n);
         best = GemmPlan{true, R, n};
