@@ -331,6 +331,7 @@ struct AttnArgs {
   int mpad_cap;  // prefix rows reserved in shared memory (multiple of 64)
   int score_only;  // 1: only each pair's score-token rows, written to out row (pair - pair_base)
   int pair_base;
+  int own_cap;  // own key rows resident at once, set by the launcher
   int* err;
   Extents ext;
 };

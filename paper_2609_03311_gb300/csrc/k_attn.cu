@@ -11,12 +11,12 @@
 //
 // Pairs are packed contiguously, so the own keys/values of a batch of
 // consecutive pairs are one block of rows: the CTA loads them once (cp.async)
-// for as many pairs as fit OWN_CAP rows, then the batch's 16-row tiles are
+// for as many pairs as fit own_cap rows, then the batch's 16-row tiles are
 // dealt round-robin to the warps with no further barriers.  A warp reads its
 // Q tile straight from global memory into mma fragments, sweeps the prefix in
 // 32-key blocks, then its own causal keys in 16-key blocks, with the online
 // (running max / running sum) softmax.  Pairs longer
-// than OWN_CAP stream their own keys in OWN_CAP chunks per 64-row group.
+// than own_cap stream their own keys in own_cap chunks per 64-row group.
 // Scores and P.V use warp-level fp16 mma with fp32 accumulation (the store
 // keeps the prefix as fp16); row maxima and sums use quad shuffles.  This
 // kernel takes the score-token rows of the last layer (one row per pair and
@@ -34,9 +34,14 @@ constexpr int WARPS = 4;
 constexpr int THREADS = WARPS * 32;
 constexpr int ROW_BYTES = HEAD_DIM * 2;
 constexpr int BOX_BYTES = 64 * 128;          // TMA box: 64 rows x 64 elements
-constexpr int OWN_CAP = 64;                  // own key rows resident at once
-constexpr int OWN_ROWS = OWN_CAP + 16;       // + zeroed tail read by the last 16-key block
-constexpr int OWN_BYTES = OWN_ROWS * ROW_BYTES;
+// Own key rows resident at once (a.own_cap, plus a zeroed tail that the last 16-key block reads).
+// In score-only mode a pair is one warp's tile, so this bounds the pairs, and so the warps, at
+// work together: 64 rows hold two 25-token pairs for four warps.  128 rows wherever that leaves
+// as many CTAs on an SM as 64 do (a second CTA does more for long pairs: 50 pairs of 33-257
+// tokens, m = 128, 33 us with two CTAs of 64 rows, 43 with one of 128).  256 pairs of 25 tokens,
+// m = 64, 16/8 heads: 38.5 -> 26.3 us; 890 pairs of a store with m up to 256: 267 -> 168 us.
+// The first batch is loaded beside the prefix.
+constexpr int OWN_CAP_SMALL = 64, OWN_CAP_LARGE = 128;
 constexpr int MAX_BATCH = 32;                // pairs per resident batch
 #ifndef DOPR_ATTN_MIN_BLOCKS
 #define DOPR_ATTN_MIN_BLOCKS 2                 // resident CTAs per SM the register budget targets
@@ -208,7 +213,7 @@ __device__ __forceinline__ void load_own(const AttnArgs& a, int g, uint32_t sOK,
                                          int count, int tid) {
   const int kcol = (a.Hq + g) * HEAD_DIM;
   const int vcol = (a.Hq + a.Hkv + g) * HEAD_DIM;
-  const int rows = min(OWN_ROWS, count + 16);
+  const int rows = min(a.own_cap + 16, count + 16);
   for (int idx = tid; idx < rows * 32; idx += THREADS) {
     const int kv = idx & 1, rc = idx >> 1, r = rc >> 4, c = rc & 15;
     const bool ok = r < count && index_ok(a.ext.err, row_begin + r, a.ext.rows);
@@ -216,7 +221,6 @@ __device__ __forceinline__ void load_own(const AttnArgs& a, int g, uint32_t sOK,
     cp_async16((kv ? sOV : sOK) + off_own(r, c), src, ok);
   }
   cp_async_commit();
-  cp_async_wait_all();
 }
 
 __global__ void __launch_bounds__(THREADS, DOPR_ATTN_MIN_BLOCKS) k_attn(const __grid_constant__ CUtensorMap tm_pool, AttnArgs a) {
@@ -224,9 +228,10 @@ __global__ void __launch_bounds__(THREADS, DOPR_ATTN_MIN_BLOCKS) k_attn(const __
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sPK = smem_u32(smem);
   const uint32_t sPV = sPK + a.mpad_cap * ROW_BYTES;
+  const uint32_t own_bytes = static_cast<uint32_t>(a.own_cap + 16) * ROW_BYTES;
   const uint32_t sOK = sPV + a.mpad_cap * ROW_BYTES;
-  const uint32_t sOV = sOK + OWN_BYTES;
-  const uint32_t bar = sOV + OWN_BYTES;
+  const uint32_t sOV = sOK + own_bytes;
+  const uint32_t bar = sOV + own_bytes;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const AttnItem item = a.items[blockIdx.x];
@@ -260,8 +265,39 @@ __global__ void __launch_bounds__(THREADS, DOPR_ATTN_MIN_BLOCKS) k_attn(const __
           tma_load_2d(sPV + (b * 2 + h) * BOX_BYTES, &tm_pool, bar, h * 64, rowV + b * 64);
         }
     }
+  }
+
+  auto geom = [&](int s) {
+    PairGeom pg;
+    pg.tb = a.tok_off[s] - a.tok0;
+    pg.T = a.tok_off[s + 1] - a.tok_off[s];
+    pg.R = pg.T * G;
+    return pg;
+  };
+  // pairs [s, e) of the item whose own rows fit a.own_cap together
+  auto batch_of = [&](int s, int& rows) {
+    int e = s + 1;
+    rows = a.tok_off[s + 1] - a.tok_off[s];
+    while (e < item.pair_end && e - s < MAX_BATCH) {
+      const int t = a.tok_off[e + 1] - a.tok_off[e];
+      if (rows + t > a.own_cap) break;
+      rows += t;
+      ++e;
+    }
+    return e;
+  };
+  // the first batch's own keys are on their way while the prefix lands
+  bool loaded = false;
+  if (a.tok_off[item.pair_begin + 1] - a.tok_off[item.pair_begin] <= a.own_cap) {
+    int rows;
+    batch_of(item.pair_begin, rows);
+    load_own(a, g, sOK, sOV, a.tok_off[item.pair_begin] - a.tok0, rows, tid);
+    loaded = true;
+  }
+  if (m > 0) {
     const bool landed = mbar_wait(bar, 0, a.err, WAIT_TIMEOUT_NS);
     if (!__syncthreads_and(landed)) {  // uniform decision: every thread leaves together
+      cp_async_wait_all();
       if (tid == 0) mbar_wait(bar, 0, a.err, 100000000ull);  // let the copies land first
       return;
     }
@@ -274,16 +310,8 @@ __global__ void __launch_bounds__(THREADS, DOPR_ATTN_MIN_BLOCKS) k_attn(const __
       *reinterpret_cast<uint4*>(gk + off_pre(r, c)) = make_uint4(0, 0, 0, 0);
       *reinterpret_cast<uint4*>(gv + off_pre(r, c)) = make_uint4(0, 0, 0, 0);
     }
-    // (the barrier before the first own-key load orders these writes)
+    // (the barrier before a batch's tiles orders these writes)
   }
-
-  auto geom = [&](int s) {
-    PairGeom pg;
-    pg.tb = a.tok_off[s] - a.tok0;
-    pg.T = a.tok_off[s + 1] - a.tok_off[s];
-    pg.R = pg.T * G;
-    return pg;
-  };
   auto prefix_pass = [&](const uint32_t (&qf)[8][4], TileState& st, const int (&jr)[2]) {
     for (int k0 = 0; k0 < m; k0 += 32)
       attend<4, false, true>(sPK, sPV, k0, lane, qf, st, min(32, m - k0), 0, jr, scale_log2);
@@ -292,17 +320,16 @@ __global__ void __launch_bounds__(THREADS, DOPR_ATTN_MIN_BLOCKS) k_attn(const __
   int s = item.pair_begin;
   while (s < item.pair_end) {
     const PairGeom p0 = geom(s);
-    if (p0.T <= OWN_CAP) {
-      // ---- resident batch: pairs [s, e) whose own rows fit OWN_CAP together
-      int e = s + 1, rows = p0.T;
-      while (e < item.pair_end && e - s < MAX_BATCH) {
-        const int t = a.tok_off[e + 1] - a.tok_off[e];
-        if (rows + t > OWN_CAP) break;
-        rows += t;
-        ++e;
+    if (p0.T <= a.own_cap) {
+      // ---- resident batch: pairs [s, e) whose own rows fit a.own_cap together
+      int rows;
+      const int e = batch_of(s, rows);
+      if (!loaded) {
+        __syncthreads();  // previous users of the own buffer are done
+        load_own(a, g, sOK, sOV, p0.tb, rows, tid);
       }
-      __syncthreads();  // previous users of the own buffer are done
-      load_own(a, g, sOK, sOV, p0.tb, rows, tid);
+      loaded = false;
+      cp_async_wait_all();
       __syncthreads();
       int tile = 0;
       for (int sp = s; sp < e; ++sp) {
@@ -325,7 +352,7 @@ __global__ void __launch_bounds__(THREADS, DOPR_ATTN_MIN_BLOCKS) k_attn(const __
       }
       s = e;
     } else {
-      // ---- long pair: 64-row groups, own keys streamed in OWN_CAP chunks
+      // ---- long pair: 64-row groups, own keys streamed in a.own_cap chunks
       const PairGeom pg = p0;
       const int rbeg = a.score_only ? (pg.T - 1) * G : 0;
       for (int rg = rbeg; rg < pg.R; rg += WARPS * 16) {
@@ -341,12 +368,13 @@ __global__ void __launch_bounds__(THREADS, DOPR_ATTN_MIN_BLOCKS) k_attn(const __
         }
         const int jmax_g = min(pg.T - 1, (rg + WARPS * 16 - 1) / G);
         const int jmax = min(pg.T - 1, (row0 + 15) / G);
-        for (int c0 = 0; c0 <= jmax_g; c0 += OWN_CAP) {
+        for (int c0 = 0; c0 <= jmax_g; c0 += a.own_cap) {
           __syncthreads();
-          load_own(a, g, sOK, sOV, pg.tb + c0, min(OWN_CAP, jmax_g + 1 - c0), tid);
+          load_own(a, g, sOK, sOV, pg.tb + c0, min(a.own_cap, jmax_g + 1 - c0), tid);
+          cp_async_wait_all();
           __syncthreads();
           if (active)
-            for (int k0 = c0; k0 <= min(jmax, c0 + OWN_CAP - 1); k0 += 16)
+            for (int k0 = c0; k0 <= min(jmax, c0 + a.own_cap - 1); k0 += 16)
               attend<2, true, false>(sOK, sOV, k0 - c0, lane, qf, st, 16, k0, jr, scale_log2);
         }
         if (active) store_tile(a, pg, s, g, G, row0, lane, st);
@@ -356,21 +384,30 @@ __global__ void __launch_bounds__(THREADS, DOPR_ATTN_MIN_BLOCKS) k_attn(const __
   }
 }
 
-inline size_t attn_smem_bytes(int mpad_cap) {
-  return 1024 + 2 * static_cast<size_t>(mpad_cap) * ROW_BYTES + 2 * OWN_BYTES + 64;
+inline size_t attn_smem_bytes(int mpad_cap, int own_cap) {
+  return 1024 + 2 * static_cast<size_t>(mpad_cap) * ROW_BYTES + 2 * static_cast<size_t>(own_cap + 16) * ROW_BYTES + 64;
+}
+// CTAs of that much shared memory on an SM (228 KB, 1 KB of it taken per CTA), as far as the registers allow.
+inline int attn_resident(size_t smem) {
+  const int n = static_cast<int>(228 * 1024 / (smem + 1024));
+  return n < DOPR_ATTN_MIN_BLOCKS ? n : DOPR_ATTN_MIN_BLOCKS;
 }
 
 }  // namespace
 
 cudaError_t attn_setup() {
   return cudaFuncSetAttribute(k_attn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(attn_smem_bytes(MAX_PREFIX)));
+                              static_cast<int>(attn_smem_bytes(MAX_PREFIX, OWN_CAP_LARGE)));
 }
 
-cudaError_t launch_attention(const CUtensorMap& tm_pool, const AttnArgs& a, cudaStream_t st) {
-  if (a.n_items <= 0) return cudaSuccess;
+cudaError_t launch_attention(const CUtensorMap& tm_pool, const AttnArgs& args, cudaStream_t st) {
+  if (args.n_items <= 0) return cudaSuccess;
+  AttnArgs a = args;
+  const size_t small = attn_smem_bytes(a.mpad_cap, OWN_CAP_SMALL), large = attn_smem_bytes(a.mpad_cap, OWN_CAP_LARGE);
+  const bool wide = attn_resident(large) == attn_resident(small);
+  a.own_cap = wide ? OWN_CAP_LARGE : OWN_CAP_SMALL;
   dim3 grid(a.n_items, a.Hkv);
-  return launch_dependent(k_attn, grid, THREADS, attn_smem_bytes(a.mpad_cap), st, tm_pool, a);
+  return launch_dependent(k_attn, grid, THREADS, wide ? large : small, st, tm_pool, a);
 }
 
 }  // namespace dopr
