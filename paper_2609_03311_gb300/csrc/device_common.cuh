@@ -29,6 +29,11 @@ enum : int {
 // fp16); NaN compares false.  Epilogues that write fp16 operands OR the negation
 // into a per-thread flag and report it once per tile (report_range).
 __device__ __forceinline__ bool fp16_ok(float x) { return fabsf(x) <= 65504.f; }
+// The same over many values: `most` collects the largest magnitude (NaN once a value was NaN), one
+// instruction a value; fp16_ok(most) at the end tells whether all were in range.
+__device__ __forceinline__ void track_range(float& most, float x) {
+  asm("max.NaN.f32 %0, %0, %1;" : "+f"(most) : "f"(fabsf(x)));
+}
 __device__ __forceinline__ void report_range(int* err, bool bad) {
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0 && err) atomicOr(err, DEV_ERR_RANGE);
 }
@@ -352,9 +357,11 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     }
   }
 }
-// Arrive (release, cluster scope) on a barrier given by its shared::cluster address.
+// Arrive on a barrier given by its shared::cluster address, for a hand-over of tensor memory: the
+// reads are complete (tcgen05.wait::ld) and no other memory is passed on, so the release need
+// not reach past this CTA (at cluster scope it waited for the warp's global stores, 1,300 clocks).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // 2-D tile load into this CTA's shared memory whose completion counts on a barrier of
 // either CTA of the pair (bar: shared::cluster address).

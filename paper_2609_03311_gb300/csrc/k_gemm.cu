@@ -200,11 +200,12 @@ __device__ __forceinline__ void epilogue_prefetch(const GemmParams& p, int row0,
 
 // BNT: columns of the tile, 256 (k_gemm_pair) or 64 / 128 (k_gemm_few).  The arithmetic on a row
 // is the same for every BNT, operation for operation.
-template <int EPI, int BNT>
+// release(): called by the whole warp once it has read its last accumulator value.
+template <int EPI, int BNT, typename Release>
 __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t taddr, int row0, int nb, int part,
-                                              int lane, uint32_t* xs, const EpiPre& pre) {
+                                              int lane, uint32_t* xs, const EpiPre& pre, Release release) {
   // row0: first row of this warp; lane = row - row0 = TMEM lane
-  bool bad = false;  // a value written as fp16 is not finite or beyond 65504 (reported once per tile)
+  float most = 0.f;  // the largest magnitude written as fp16 (track_range; reported once per tile)
   // this lane's row exists (rows past M hold whatever the operand buffers held there; never stored)
   const bool live = row0 + lane < p.M;
   if constexpr (EPI == EPI_STORE || EPI == EPI_QKV) {
@@ -236,15 +237,12 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
         // per-head RMSNorm of the row-scaled values: sum of squares in the row layout
         float ss = 0.f;
 #pragma unroll
-        for (int c = 0; c < 128; c += 64) {
-          uint32_t v[32], w[32];
+        for (int c = 0; c < 128; c += 32) {
+          uint32_t v[32];
           tmem_ld32(taddr + hh * 128 + c, v);
-          tmem_ld32(taddr + hh * 128 + c + 32, w);
           tmem_ld_wait();
 #pragma unroll
           for (int j = 0; j < 32; ++j) ss += __uint_as_float(v[j]) * __uint_as_float(v[j]);
-#pragma unroll
-          for (int j = 0; j < 32; ++j) ss += __uint_as_float(w[j]) * __uint_as_float(w[j]);
         }
         const float inv_row = rs * rsqrtf(ss * rs * rs * (1.f / 128.f) + p.eps);
         const bf16* wgt = hc < p.q_cols ? p.q_norm : p.k_norm;
@@ -257,6 +255,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
           uint32_t v[32];  // the row's 16 elements of the first half of the head, then those 64 further on
           tmem_ld16x2(taddr + hh * 128 + f, taddr + hh * 128 + 64 + f, v);
           tmem_ld_wait();
+          if (s + 1 == STEPS) release();
           xs_put_row(xs, lane, v);
           __syncwarp();
           float g1[4], g2[4];
@@ -274,15 +273,16 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
             const float sinv[4] = {c01[i].y, c01[i].w, c23[i].y, c23[i].w};
             const float a[4] = {x1.x, x1.y, x1.z, x1.w}, b[4] = {x2.x, x2.y, x2.z, x2.w};
             float y1[4], y2[4];
-            bool out_of_range = false;
+            float row_most = 0.f;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
               const float u = a[k] * inv_i[i] * g1[k], w = b[k] * inv_i[i] * g2[k];
               y1[k] = u * cosv[k] - w * sinv[k];
               y2[k] = w * cosv[k] + u * sinv[k];
-              out_of_range |= !(fp16_ok(y1[k]) && fp16_ok(y2[k]));
+              track_range(row_most, y1[k]);
+              track_range(row_most, y2[k]);
             }
-            bad |= out_of_range && row0 + r < p.M;
+            if (row0 + r < p.M) track_range(most, row_most);
             o1[i] = make_uint2(pack_f16x2(y1[0], y1[1]), pack_f16x2(y1[2], y1[3]));
             o2[i] = make_uint2(pack_f16x2(y2[0], y2[1]), pack_f16x2(y2[2], y2[3]));
           }
@@ -305,14 +305,20 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
           tmem_ld32(taddr + hh * 128 + c, a);
           tmem_ld32(taddr + hh * 128 + c + 32, b);
           tmem_ld_wait();
+          if (c + 64 == (ONE ? part * 64 + 64 : 128)) release();
+          float row_most = 0.f;
 #pragma unroll
           for (int j = 0; j < 32; j += 2) {
             const float a0 = __uint_as_float(a[j]) * rs, a1 = __uint_as_float(a[j + 1]) * rs;
             const float b0 = __uint_as_float(b[j]) * rs, b1 = __uint_as_float(b[j + 1]) * rs;
-            bad |= live && !(fp16_ok(a0) && fp16_ok(a1) && fp16_ok(b0) && fp16_ok(b1));
+            track_range(row_most, a0);
+            track_range(row_most, a1);
+            track_range(row_most, b0);
+            track_range(row_most, b1);
             o[j / 2] = pack_f16x2(a0, a1);
             o[16 + j / 2] = pack_f16x2(b0, b1);
           }
+          if (live) track_range(most, row_most);
           xs_put_row(xs, lane, o);
           __syncwarp();
           store_words_transposed<32>(xs, lane, row0, p.M, [&](int r, int wd) {
@@ -357,6 +363,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
       uint32_t v[32];
       tmem_ld32(taddr + c, v);
       tmem_ld_wait();
+      if (c + 32 == cend) release();
       xs_put_row(xs, lane, v);
       __syncwarp();
       const int col = nb * BNT + c + w4;
@@ -386,7 +393,10 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
             ss[i] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
             const float sc = prev[i];
             const float n0 = x.x * g4.x * sc, n1 = x.y * g4.y * sc, n2 = x.z * g4.z * sc, n3 = x.w * g4.w * sc;
-            bad |= !(fp16_ok(n0) && fp16_ok(n1) && fp16_ok(n2) && fp16_ok(n3));
+            track_range(most, n0);
+            track_range(most, n1);
+            track_range(most, n2);
+            track_range(most, n3);
             uint2 o;
             o.x = pack_f16x2(n0, n1);
             o.y = pack_f16x2(n2, n3);
@@ -405,7 +415,9 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
     const float rs = pre.scale;
     constexpr int OUTS = BNT / 2;                  // outputs of the tile
     constexpr int MINE = OUTS >= 64 ? OUTS / 2 : 32;  // of this warp (with 32 in all, part 0 takes them)
-    if (part * MINE < OUTS) {
+    if (part * MINE >= OUTS) {
+      release();
+    } else {
       const int c = part * MINE;
 #pragma unroll
       for (int half = 0; half < MINE / 32; ++half) {
@@ -413,6 +425,8 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
         tmem_ld32(taddr + c + 32 * half, g);
         tmem_ld32(taddr + OUTS + c + 32 * half, u);
         tmem_ld_wait();
+        if (half + 1 == MINE / 32) release();
+        float row_most = 0.f;
 #pragma unroll
         for (int c4 = 0; c4 < 4; ++c4) {  // eight outputs: one 16-byte chunk
           uint32_t o[4];
@@ -421,11 +435,13 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
             const int j = c4 * 8 + 2 * k;
             const float a0 = silu_f(__uint_as_float(g[j]) * rs) * (__uint_as_float(u[j]) * rs);
             const float a1 = silu_f(__uint_as_float(g[j + 1]) * rs) * (__uint_as_float(u[j + 1]) * rs);
-            bad |= live && !(fp16_ok(a0) && fp16_ok(a1));
+            track_range(row_most, a0);
+            track_range(row_most, a1);
             o[k] = pack_f16x2(a0, a1);
           }
           *xs_chunk(xs, lane, 4 * half + c4) = make_uint4(o[0], o[1], o[2], o[3]);
         }
+        if (live) track_range(most, row_most);
       }
       __syncwarp();
       store_words_transposed<MINE / 2>(xs, lane, row0, p.M, [&](int r, int wd) {
@@ -434,7 +450,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
       __syncwarp();
     }
   }
-  report_range(p.err, bad);
+  report_range(p.err, !fp16_ok(most));
 }
 
 // ============================================================================
@@ -497,6 +513,12 @@ __device__ __forceinline__ void pair_tile_coords(int t, int m_tiles, int n_tiles
 // A bounded wait of the whole warp: all lanes go on or give up together.
 __device__ __forceinline__ bool wait_all_lanes(uint32_t bar, uint32_t parity, const GemmParams& p) {
   return __all_sync(0xffffffffu, mbar_wait_cluster(bar, parity, p.err, p.timeout_ns)) != 0;
+}
+// An epilogue warp has read its part of an accumulator: tell the leader.
+__device__ __forceinline__ void free_accumulator(uint32_t tempty_bar, int lane) {
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty_bar, 0));
 }
 // A producer that gave up: its copies in flight land within microseconds; give them that long
 // before the CTA can reach its exit (no barrier to wait on: they count on the leader's).
@@ -650,10 +672,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       if (!mbar_wait_cluster(tfull_bar(acc), acc_phase, p.err, p.timeout_ns)) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BN;
-      epilogue_tile<EPI, BN>(p, taddr, row0, nb, part, lane, xs, pre);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
+      epilogue_tile<EPI, BN>(p, taddr, row0, nb, part, lane, xs, pre, [&] { free_accumulator(tempty_bar(acc), lane); });
     }
   }
 
@@ -849,10 +868,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       if (!mbar_wait_cluster(tfull_bar(acc), (local / PAIR_ACCS) & 1, p.err, p.timeout_ns)) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BNT;
-      if (mine) epilogue_tile<EPI, BNT>(p, taddr, row0, nb, part, lane, xs, pre);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
+      if (mine)
+        epilogue_tile<EPI, BNT>(p, taddr, row0, nb, part, lane, xs, pre, [&] { free_accumulator(tempty_bar(acc), lane); });
+      else
+        free_accumulator(tempty_bar(acc), lane);
     }
   }
 
