@@ -179,12 +179,39 @@ __device__ __forceinline__ void store_words_transposed(uint32_t* xs, int lane, i
 struct EpiPre {
   float scale;  // this thread's row: the consumer row scale (QKV, SwiGLU) or the previous norm factor
   int pos[4];   // QKV: positions of the 4 rows a lane rotates in the transposed layout
+  float4 res[2][8];  // residual add: the lane's values of the warp's first two 32-column chunks
+  uint2 gain;        // and the next norm's gains of the lane's four columns of the first
 };
+
+__device__ __forceinline__ void bf16x4_floats(uint2 w, float (&v)[4]) {
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.x));
+  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.y));
+  v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+}
+
+// The residual values of lane L, rows i*4 + L/8 of the warp, columns col + (L%8)*4..+3.
+__device__ __forceinline__ float4* residual_at(const GemmParams& p, int row0, int i, int col, int lane) {
+  return reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) +
+                                   static_cast<int64_t>(row0 + i * 4 + (lane >> 3)) * p.ld_out + col + (lane & 7) * 4);
+}
+__device__ __forceinline__ void load_residual(const GemmParams& p, int row0, int col, int lane, float4 (&res)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    res[i] = row0 + i * 4 + (lane >> 3) < p.M ? *residual_at(p, row0, i, col, lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+__device__ __forceinline__ uint2 load_gain(const GemmParams& p, int col, int lane) {
+  return p.xn_out ? __ldg(reinterpret_cast<const uint2*>(p.xn_gain + col + (lane & 7) * 4)) : make_uint2(0u, 0u);
+}
 
 template <int EPI, int BNT>
 __device__ __forceinline__ void epilogue_prefetch(const GemmParams& p, int row0, int nb, int part, int lane,
                                                   EpiPre& pre) {
   if constexpr (EPI == EPI_RESID_ADD) {
+    const int col = nb * BNT + part * (BNT / 2);
+    load_residual(p, row0, col, lane, pre.res[0]);
+    if (BNT > 64) load_residual(p, row0, col + 32, lane, pre.res[1]);
+    pre.gain = load_gain(p, col, lane);
     pre.scale = p.xn_out ? norm_factor(p.ss_pre, p.ss_pre_parts, p, row0 + lane) : 1.f;
   } else if constexpr (EPI == EPI_STORE) {
     pre.scale = 1.f;
@@ -203,7 +230,7 @@ __device__ __forceinline__ void epilogue_prefetch(const GemmParams& p, int row0,
 // release(): called by the whole warp once it has read its last accumulator value.
 template <int EPI, int BNT, typename Release>
 __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t taddr, int row0, int nb, int part,
-                                              int lane, uint32_t* xs, const EpiPre& pre, Release release) {
+                                              int lane, uint32_t* xs, EpiPre& pre, Release release) {
   // row0: first row of this warp; lane = row - row0 = TMEM lane
   float most = 0.f;  // the largest magnitude written as fp16 (track_range; reported once per tile)
   // this lane's row exists (rows past M hold whatever the operand buffers held there; never stored)
@@ -252,6 +279,8 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
 #pragma unroll
         for (int s = 0; s < STEPS; ++s) {
           const int f = f0 + 16 * s;
+          const uint2 gw[2] = {__ldg(reinterpret_cast<const uint2*>(wgt + f + w4)),
+                               __ldg(reinterpret_cast<const uint2*>(wgt + 64 + f + w4))};
           uint32_t v[32];  // the row's 16 elements of the first half of the head, then those 64 further on
           tmem_ld16x2(taddr + hh * 128 + f, taddr + hh * 128 + 64 + f, v);
           tmem_ld_wait();
@@ -259,12 +288,8 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
           xs_put_row(xs, lane, v);
           __syncwarp();
           float g1[4], g2[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            g1[k] = __bfloat162float(wgt[f + w4 + k]);
-            g2[k] = __bfloat162float(wgt[64 + f + w4 + k]);
-          }
-          uint2 o1[4], o2[4];
+          bf16x4_floats(gw[0], g1);
+          bf16x4_floats(gw[1], g2);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int r = i * 8 + (lane >> 2);
@@ -283,19 +308,13 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
               track_range(row_most, y2[k]);
             }
             if (row0 + r < p.M) track_range(most, row_most);
-            o1[i] = make_uint2(pack_f16x2(y1[0], y1[1]), pack_f16x2(y1[2], y1[3]));
-            o2[i] = make_uint2(pack_f16x2(y2[0], y2[1]), pack_f16x2(y2[2], y2[3]));
-          }
-          if (s + 1 < STEPS) fetch_rope(f + 16);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int r = i * 8 + (lane >> 2);
             if (row0 + r < p.M) {
               f16* orow = out + static_cast<int64_t>(row0 + r) * p.ld_out + hc + f + w4;
-              *reinterpret_cast<uint2*>(orow) = o1[i];
-              *reinterpret_cast<uint2*>(orow + 64) = o2[i];
+              *reinterpret_cast<uint2*>(orow) = make_uint2(pack_f16x2(y1[0], y1[1]), pack_f16x2(y1[2], y1[3]));
+              *reinterpret_cast<uint2*>(orow + 64) = make_uint2(pack_f16x2(y2[0], y2[1]), pack_f16x2(y2[2], y2[3]));
             }
           }
+          if (s + 1 < STEPS) fetch_rope(f + 16);
           __syncwarp();
         }
       } else {
@@ -330,9 +349,9 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
     }
   } else if constexpr (EPI == EPI_RESID_ADD) {
     // r += C, then (optionally) the next RMSNorm's operand f16(r * g * rs_pre) and partial sums of r^2.
-    // Lane L owns rows i*4 + L/8 (i = 0..7) and columns (L%8)*4..+3 of each 32-column chunk; the
-    // residual values of chunk c+1 are loaded while chunk c is processed.
-    float* res = reinterpret_cast<float*>(p.out);
+    // Lane L owns rows i*4 + L/8 (i = 0..7) and columns (L%8)*4..+3 of each 32-column chunk.  The
+    // residual values are fetched two chunks ahead (the first two before the main loop ends):
+    // one ahead, a chunk took their latency, 2,200 clocks.
     const int w4 = (lane & 7) * 4;
     // this lane's chunk of row i*4 + lane/8 lies at cpos ^ 2 (i & 1) of the transpose buffer's row
     const int cpos = (lane & 7) ^ ((lane >> 3 & 1) << 2 | lane >> 4);
@@ -344,26 +363,15 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
       ss[i] = 0.f;
       prev[i] = __shfl_sync(0xffffffffu, pre.scale, i * 4 + (lane >> 3));
     }
-    auto rrow = [&](int i, int c) {
-      return reinterpret_cast<float4*>(res + static_cast<int64_t>(row0 + i * 4 + (lane >> 3)) * p.ld_out + nb * BNT +
-                                       c + w4);
-    };
-    const int cbeg = part * (BNT / 2), cend = cbeg + BNT / 2;  // this warp's half of the columns
-    float4 cur[8];
+    constexpr int CHUNKS = BNT / 64;  // 32-column chunks of this warp's half of the columns
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      cur[i] = (row0 + i * 4 + (lane >> 3) < p.M) ? *rrow(i, cbeg) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-    for (int c = cbeg; c < cend; c += 32) {
-      float4 nxt[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        nxt[i] = (c + 32 < cend && row0 + i * 4 + (lane >> 3) < p.M) ? *rrow(i, c + 32)
-                                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int q = 0; q < CHUNKS; ++q) {
+      const int c = part * (BNT / 2) + 32 * q;
+      float4(&res)[8] = pre.res[q & 1];
       uint32_t v[32];
       tmem_ld32(taddr + c, v);
       tmem_ld_wait();
-      if (c + 32 == cend) release();
+      if (q + 1 == CHUNKS) release();
       xs_put_row(xs, lane, v);
       __syncwarp();
       const int col = nb * BNT + c + w4;
@@ -371,28 +379,24 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
 #pragma unroll
         for (int i = 0; i < 8; ++i) ss[i] = 0.f;
       }
-      float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (p.xn_out) {
-        const uint2 gw = *reinterpret_cast<const uint2*>(p.xn_gain + col);
-        const float2 g01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gw.x));
-        const float2 g23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gw.y));
-        g4 = make_float4(g01.x, g01.y, g23.x, g23.y);
-      }
+      float g[4];
+      bf16x4_floats(pre.gain, g);
+      if (q + 1 < CHUNKS) pre.gain = load_gain(p, nb * BNT + c + 32, lane);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int r = i * 4 + (lane >> 3);
         if (row0 + r < p.M) {
-          float4 x = cur[i];
+          float4 x = res[i];
           const float4 d = *reinterpret_cast<const float4*>(xrow + i * 128 + ((cpos ^ (i & 1) << 1) << 2));
           x.x += d.x;
           x.y += d.y;
           x.z += d.z;
           x.w += d.w;
-          *rrow(i, c) = x;
+          *residual_at(p, row0, i, nb * BNT + c, lane) = x;
           if (p.xn_out) {
             ss[i] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
             const float sc = prev[i];
-            const float n0 = x.x * g4.x * sc, n1 = x.y * g4.y * sc, n2 = x.z * g4.z * sc, n3 = x.w * g4.w * sc;
+            const float n0 = x.x * g[0] * sc, n1 = x.y * g[1] * sc, n2 = x.z * g[2] * sc, n3 = x.w * g[3] * sc;
             track_range(most, n0);
             track_range(most, n1);
             track_range(most, n2);
@@ -403,8 +407,8 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
             *reinterpret_cast<uint2*>(p.xn_out + static_cast<int64_t>(row0 + r) * p.ld_out + col) = o;
           }
         }
-        cur[i] = nxt[i];
       }
+      if (q + 2 < CHUNKS) load_residual(p, row0, nb * BNT + c + 64, lane, res);
       __syncwarp();
       if (BNT < 256 && p.ss_out)
         publish_square_sums(p, row0, lane, (nb * BNT + c) / 128, (nb * BNT + c) / 32 % 4, ss);
