@@ -731,7 +731,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   const uint32_t drain_bar = bar0 + 8u * (2 * FEW_MAX_STAGES + 4);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * FEW_MAX_STAGES + 5);
   constexpr uint32_t TMEM_COLS = PAIR_ACCS * BNT;
-  constexpr uint32_t IDESC = umma_idesc_f16(PAIR_BM, BNT);
+  // With at most 64 rows a CTA the residual launches take M = 128 MMAs, 64 rows a CTA: each reads
+  // half as much of A (48 -> 32 clocks of shared memory at 64 columns).  A CTA's rows are then
+  // TMEM lanes 0..63 for the tile's first half of the columns and 64..127 for its second.
+  constexpr bool SHORT = EPI == EPI_RESID_ADD && BNT == 64 && R <= 64;
+  constexpr uint32_t IDESC = umma_idesc_f16(SHORT ? BM : PAIR_BM, BNT);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
@@ -864,16 +868,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     uint32_t* xs = xpose + (warp - 2) * XPOSE_WORDS;
     int local = 0;
     for (int t = pair; t < total; t += n_pairs, ++local) {
-      const int nb = t / m_tiles, row0 = (t % m_tiles) * 2 * R + static_cast<int>(rank) * R + quarter * 32;
-      const bool mine = quarter * 32 < R && row0 < p.M;  // a quarter with rows of the tile (R is a multiple of 32)
+      const int block = SHORT ? quarter & 1 : quarter;   // the 32 rows of this lane quarter,
+      const int cols = SHORT ? quarter >> 1 : part;      // and this warp's half of the columns
+      const int nb = t / m_tiles, row0 = (t % m_tiles) * 2 * R + static_cast<int>(rank) * R + block * 32;
+      // a warp with rows of the tile (R is a multiple of 32)
+      const bool mine = block * 32 < R && row0 < p.M && !(SHORT && part != 0);
       const int acc = local % PAIR_ACCS;
       EpiPre pre;
-      if (mine) epilogue_prefetch<EPI, BNT>(p, row0, nb, part, lane, pre);
+      if (mine) epilogue_prefetch<EPI, BNT>(p, row0, nb, cols, lane, pre);
       if (!mbar_wait_cluster(tfull_bar(acc), (local / PAIR_ACCS) & 1, p.err, p.timeout_ns)) break;
       tc_fence_after();
-      const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BNT;
+      // (epilogue_tile adds the half's first column, which here is a lane offset)
+      const uint32_t taddr =
+          tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BNT - (SHORT ? cols * (BNT / 2) : 0);
       if (mine)
-        epilogue_tile<EPI, BNT>(p, taddr, row0, nb, part, lane, xs, pre, [&] { free_accumulator(tempty_bar(acc), lane); });
+        epilogue_tile<EPI, BNT>(p, taddr, row0, nb, cols, lane, xs, pre, [&] { free_accumulator(tempty_bar(acc), lane); });
       else
         free_accumulator(tempty_bar(acc), lane);
     }
@@ -942,17 +951,19 @@ cudaError_t gemm_setup() {
 
 // The clocks a CTA pair needs for a 64-wide k-block of a tile of 2 R rows and n columns: its SMs
 // take in R + n / 2 operand rows of 128 bytes at about 64 bytes a clock, and the four MMAs take
-// 512 at n = 256 but 288 at 128 and 192 at 64 (each reads 128 A rows a CTA, whatever R is).
+// 512 at n = 256 but 288 at 128 and 192 at 64 (each reads 128 A rows a CTA, whatever R is; the
+// residual launches' 64-row MMAs 128).
 // Every tile adds a start and an epilogue that is not hidden, about 2,000 clocks.  The tile
 // with the least clocks over the launch's rounds is taken; the wide one unless a narrow one
 // saves a tenth (its L2 reuse is better).  Measured (cold cache, wide / taken): N 4,096
-// K 12,288, 25 rows 63.7 / 30.5 us, 180 rows 66.0 / 42.2 us; N 4,096 K 4,096, 25 rows
-// 28.0 / 14.5 us; gate/up N 24,576 K 4,096, 25 rows 59.0 / 47.6 us.
+// K 12,288, 25 rows 63.7 / 26 us, 180 rows 66.0 / 37 us; N 4,096 K 4,096, 25 rows
+// 28.0 / 13 us; gate/up N 24,576 K 4,096, 25 rows 59.0 / 39 us.
 GemmPlan gemm_plan(int epi, int M, int N, int K, int num_sms) {
   const int64_t pairs = num_sms / 2 > 0 ? num_sms / 2 : 1;
   auto clocks = [&](int R, int n) {
     const int64_t tiles = static_cast<int64_t>((M + 2 * R - 1) / (2 * R)) * (N / n);
-    const int64_t in = 2 * (R + n / 2), mma = n == BN ? 2 * BN : 96 + 3 * n / 2;
+    const bool half_m = epi == EPI_RESID_ADD && n == 64 && R <= 64;
+    const int64_t in = 2 * (R + n / 2), mma = n == BN ? 2 * BN : half_m ? 128 : 96 + 3 * n / 2;
     return (tiles + pairs - 1) / pairs * (K / BK * (in > mma ? in : mma) + 2000);
   };
   GemmPlan best{false, BM, BN};
