@@ -127,13 +127,15 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-// Maximum of the 32 values whose mask bit is set (-inf when none).
+// Maximum of the 32 values whose mask bit is set (-inf when none).  WHOLE: every bit is (the
+// caller's warp agrees, see whole_chunk), so the selections are left out; same value.
+template <bool WHOLE>
 __device__ __forceinline__ float masked_max32(const uint32_t (&v)[32], uint32_t mask) {
   float t[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
-    const float a = (mask >> (2 * i)) & 1u ? __uint_as_float(v[2 * i]) : -INFINITY;
-    const float b = (mask >> (2 * i + 1)) & 1u ? __uint_as_float(v[2 * i + 1]) : -INFINITY;
+    const float a = WHOLE || ((mask >> (2 * i)) & 1u) ? __uint_as_float(v[2 * i]) : -INFINITY;
+    const float b = WHOLE || ((mask >> (2 * i + 1)) & 1u) ? __uint_as_float(v[2 * i + 1]) : -INFINITY;
     t[i] = fmaxf(a, b);
   }
 #pragma unroll
@@ -147,12 +149,13 @@ __device__ __forceinline__ float masked_max32(const uint32_t (&v)[32], uint32_t 
 // as fp16 pairs (key 2i in the low half of pk[i]) for a TMEM store.  Returns
 // sum + the two 16-column partial sums, each a fixed pairwise tree, added in
 // column order.
+template <bool WHOLE>
 __device__ __forceinline__ float exp_pack(uint32_t (&v)[32], uint32_t mask, float scale_log2, float mxs, float sum,
                                           uint32_t (&pk)[16]) {
 #pragma unroll
   for (int e = 0; e < 32; ++e) {
     const float x = ex2_approx(fmaf(__uint_as_float(v[e]), scale_log2, -mxs));
-    v[e] = __float_as_uint((mask >> e) & 1u ? x : 0.f);
+    v[e] = __float_as_uint(WHOLE || ((mask >> e) & 1u) ? x : 0.f);
   }
 #pragma unroll
   for (int i = 0; i < 16; ++i) pk[i] = pack_f16x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
@@ -169,6 +172,11 @@ __device__ __forceinline__ float exp_pack(uint32_t (&v)[32], uint32_t mask, floa
   }
   return sum;
 }
+
+// Does every row of the warp see all 32 columns of a chunk?  In long tiles most do, and half of the
+// instructions on a score were its mask (4 documents of 777-2,048 tokens 171 -> 158 us); in the short
+// kernel few do and the vote cost 3 %.
+__device__ __forceinline__ bool whole_chunk(uint32_t mask) { return __all_sync(0xffffffffu, mask == 0xffffffffu) != 0; }
 
 __global__ void __launch_bounds__(THREADS, 1)
     k_attn_tc(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kv,
@@ -493,7 +501,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         uint32_t v[32];
         tmem_ld32(trow + c0, v);
         tmem_ld_wait();
-        mx = fmaxf(mx, masked_max32(v, vis_mask(c0)));
+        mx = fmaxf(mx, masked_max32<false>(v, vis_mask(c0)));
       }
       const float mxs = (mx == -INFINITY) ? 0.f : mx * scale_log2;
       // ---- pass 2: P = 2^((s - max) * scale) per 64-key block, as fp16 into TMEM
@@ -509,7 +517,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             uint32_t v[32];
             tmem_ld32(trow + cb, v);
             tmem_ld_wait();
-            sum = exp_pack(v, vis_mask(cb), scale_log2, mxs, sum, pk);
+            sum = exp_pack<false>(v, vis_mask(cb), scale_log2, mxs, sum, pk);
           } else {
 #pragma unroll
             for (int q = 0; q < 16; ++q) pk[q] = 0u;
@@ -902,8 +910,14 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
           tmem_ld32(sb, v0);
           tmem_ld32(sb + 32, v1);
           tmem_ld_wait();
-          mx = fmaxf(mx, masked_max32(v0, vis_mask(c0)));
-          mx = fmaxf(mx, masked_max32(v1, vis_mask(c0 + 32)));
+          const uint32_t m0 = vis_mask(c0), m1 = vis_mask(c0 + 32);
+          if (whole_chunk(m0 & m1)) {
+            mx = fmaxf(mx, masked_max32<true>(v0, m0));
+            mx = fmaxf(mx, masked_max32<true>(v1, m1));
+          } else {
+            mx = fmaxf(mx, masked_max32<false>(v0, m0));
+            mx = fmaxf(mx, masked_max32<false>(v1, m1));
+          }
         }
         tc_fence_before();
         __syncwarp();
@@ -932,9 +946,11 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
           tmem_ld32(sb, v0);
           tmem_ld32(sb + 32, v1);
           tmem_ld_wait();
-          sum = exp_pack(v0, vis_mask(cb), scale_log2, mxs, sum, pk);
+          const uint32_t m0 = vis_mask(cb), m1 = vis_mask(cb + 32);
+          const bool whole = whole_chunk(m0 & m1);
+          sum = whole ? exp_pack<true>(v0, m0, scale_log2, mxs, sum, pk) : exp_pack<false>(v0, m0, scale_log2, mxs, sum, pk);
           tmem_st16(lane_base + lt::P_COL + 32 * rp.stage, pk);
-          sum = exp_pack(v1, vis_mask(cb + 32), scale_log2, mxs, sum, pk);
+          sum = whole ? exp_pack<true>(v1, m1, scale_log2, mxs, sum, pk) : exp_pack<false>(v1, m1, scale_log2, mxs, sum, pk);
           tmem_st16(lane_base + lt::P_COL + 32 * rp.stage + 16, pk);
           tmem_st_wait();
           tc_fence_before();

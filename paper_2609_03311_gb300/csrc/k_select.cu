@@ -329,26 +329,29 @@ __global__ void __launch_bounds__(32 * COL_WARPS)
 #pragma unroll
   for (int q = 0; q < NV; ++q) v[q] = q * 32 + lane < cnt ? __float_as_uint(col[q * 32 + lane]) : 0u;
   uint32_t thr = 0;
-  int above = 0;  // entries larger than thr
+  int above = 0;      // entries larger than thr
+  bool split = false;  // exactly k entries are not below thr: the search is over
   if (k < cnt) {
 #pragma unroll 1
-    for (int b = 30; b >= 0; --b) {
+    for (int b = 30; b >= 0 && !split; --b) {
       const uint32_t cand = thr | (1u << b);
       int c = 0;
 #pragma unroll
       for (int q = 0; q < NV; ++q) c += v[q] >= cand;
-      if (static_cast<int>(__reduce_add_sync(0xffffffffu, c)) >= k) thr = cand;
+      c = static_cast<int>(__reduce_add_sync(0xffffffffu, c));
+      if (c >= k) thr = cand;
+      split = c == k;
     }
   }
   float sum = 0.f;
 #pragma unroll
   for (int q = 0; q < NV; ++q)
-    if (v[q] > thr || k == cnt) {
+    if (v[q] > thr || k == cnt || (split && v[q] == thr)) {
       sum += __uint_as_float(v[q]);
       ++above;
     }
   sum = warp_sum(sum);
-  if (k < cnt) sum += static_cast<float>(k - static_cast<int>(__reduce_add_sync(0xffffffffu, above))) * __uint_as_float(thr);
+  if (k < cnt && !split) sum += static_cast<float>(k - static_cast<int>(__reduce_add_sync(0xffffffffu, above))) * __uint_as_float(thr);
   if (lane == 0) u[t] = sum / static_cast<float>(k);
 }
 
@@ -411,6 +414,10 @@ __global__ void __launch_bounds__(TOPK_THREADS) k_sal_topk(const int32_t* __rest
     const uint32_t cand = thr | (1u << b);
     const int c = __syncthreads_count(in[0] && key[0] >= cand) + __syncthreads_count(in[1] && key[1] >= cand);
     if (c >= k) thr = cand;
+    if (c == k) {  // the k largest are those not below thr (which is above 0): no ties to share out
+      --thr;
+      break;
+    }
   }
   int n_above, n_ties, n_all;
   const bool gt0 = in[0] && key[0] > thr, gt1 = in[1] && key[1] > thr;
