@@ -639,6 +639,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
   const int mpad = ((s->max_m + 63) / 64) * 64;
   const int sms = m->num_sms;
   const bool scoring = !build && !sel;
+  auto gemm_launches = [&](int epi, int M, int N, int K) { return gemm_plan(epi, M, N, K, sms).wide_rows > 0 ? 2 : 1; };
   auto gemm_cost = [](double M, double N, double K, double out_bytes) {
     return std::make_pair(2.0 * M * N * K, (M * K + N * K) * 2.0 + out_bytes);
   };
@@ -739,7 +740,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
       pq.k_norm = m->k_norm + (size_t)l * HEAD_DIM;
       pq.q_cols = Hq * HEAD_DIM;
       pq.k_cols = Hkv * HEAD_DIM;
-      CUDA_TRY(prof_launch(m, K_GEMM_QKV, 1, qkv.first, qkv.second, st,
+      CUDA_TRY(prof_launch(m, K_GEMM_QKV, gemm_launches(EPI_QKV, Tc, m->qkv_dim, H), qkv.first, qkv.second, st,
                            [&] { return launch_gemm(EPI_QKV, w.tm_xn, m->tm_qkv[l], pq, sms, st); }));
       if (build) {  // this layer's keys and values are the document's stored prefix states
         CUDA_TRY(prof_launch(m, K_PREFIX_STORE, 1, 0.0, T * 2.0 * Hkv * HEAD_DIM * 2 * 2, st, [&] {
@@ -840,7 +841,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
       po.ss_out_parts = parts;
       po.ss_pre = ss_pre;
       po.ss_pre_parts = ss_pre_parts;
-      CUDA_TRY(prof_launch(m, K_GEMM_O, 1, last ? op_last.first : op.first, last ? op_last.second : op.second, st,
+      CUDA_TRY(prof_launch(m, K_GEMM_O, gemm_launches(EPI_RESID_ADD, rows, H, m->o_dim), last ? op_last.first : op.first, last ? op_last.second : op.second, st,
                            [&] { return launch_gemm(EPI_RESID_ADD, w.tm_o, m->tm_o[l], po, sms, st); }));
       GemmParams pg = base;  // gate/up + MLP-norm row scale + SwiGLU
       pg.M = rows;
@@ -852,7 +853,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
       pg.ss_parts = parts;
       pg.ss_pre = ss_pre;
       pg.ss_pre_parts = ss_pre_parts;
-      CUDA_TRY(prof_launch(m, K_GEMM_GATE_UP, 1, last ? gu_last.first : gu.first, last ? gu_last.second : gu.second,
+      CUDA_TRY(prof_launch(m, K_GEMM_GATE_UP, gemm_launches(EPI_SWIGLU, rows, 2 * F, H), last ? gu_last.first : gu.first, last ? gu_last.second : gu.second,
                            st, [&] { return launch_gemm(EPI_SWIGLU, w.tm_xn, m->tm_gu[l], pg, sms, st); }));
       GemmParams pd = base;  // down projection + residual, emits the next attention norm's operand
       pd.M = rows;
@@ -868,7 +869,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
         pd.ss_pre = w.ss_m;  // the MLP norm of this layer
         pd.ss_pre_parts = parts;
       }
-      CUDA_TRY(prof_launch(m, K_GEMM_DOWN, 1, last ? dn_last.first : dn.first, last ? dn_last.second : dn.second, st,
+      CUDA_TRY(prof_launch(m, K_GEMM_DOWN, gemm_launches(EPI_RESID_ADD, rows, H, F), last ? dn_last.first : dn.first, last ? dn_last.second : dn.second, st,
                            [&] { return launch_gemm(EPI_RESID_ADD, w.tm_act, m->tm_down[l], pd, sms, st); }));
     }
     if (scoring) {

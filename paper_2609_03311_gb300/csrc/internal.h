@@ -271,6 +271,9 @@ struct GemmParams {
   const bf16* q_norm;
   const bf16* k_norm;
   int q_cols, k_cols;
+  // k_gemm_few: rows [row_begin, M) only; beside: the launch before is the wide one of the same
+  // product's first rows, which is waited for at the end alone
+  int row_begin, beside;
   int* err;
   uint64_t timeout_ns;
 };
@@ -280,6 +283,7 @@ cudaError_t gemm_setup();
 struct GemmPlan {
   bool few;
   int rows, cols;  // A rows per CTA of the pair, columns
+  int wide_rows;   // > 0: that many rows in wide tiles, the others in `rows` x `cols` tiles beside them
 };
 GemmPlan gemm_plan(int epi, int M, int N, int K, int num_sms);
 // C[M][N] = A[M][K] * B[N][K]^T followed by the epilogue `epi`.

@@ -119,7 +119,7 @@ __device__ __forceinline__ void store_square_sums(const GemmParams& p, int row0,
 // waits.
 __device__ __forceinline__ void publish_square_sums(const GemmParams& p, int row0, int lane, int group, int chunk,
                                                     const float (&ss)[8]) {
-  const int64_t at = static_cast<int64_t>(row0 / 32) * p.ss_out_parts + group;
+  const int64_t at = static_cast<int64_t>((row0 - p.row_begin) / 32) * p.ss_out_parts + group;
   float* mine = p.ss_chunks + ((at * 4 + chunk) * 8) * 32 + lane;
 #pragma unroll
   for (int i = 0; i < 8; ++i) __stcg(mine + i * 32, ss[i]);
@@ -581,8 +581,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   cluster_sync();  // both CTAs' barriers exist before either addresses the other's
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_trigger();
+  // in this order: a few-row launch beside this one (GemmParams::beside) may take it that whatever
+  // this kernel waited for is done
   pdl_wait();
+  pdl_trigger();
   {
     // the MMAs write both CTAs' TMEM at the leader's address: both allocations must agree
     uint32_t other;
@@ -741,7 +743,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  const int m_tiles = (p.M + 2 * R - 1) / (2 * R), k_blocks = p.K / BK, k_steps = (k_blocks + KB - 1) / KB;
+  const int m_tiles = (p.M - p.row_begin + 2 * R - 1) / (2 * R);
+  const int k_blocks = p.K / BK, k_steps = (k_blocks + KB - 1) / KB;
   int total = m_tiles * (p.N / BNT);
 
   if (threadIdx.x == 0) {
@@ -768,7 +771,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_trigger();
-  if (warp != 0) pdl_wait();  // the producer starts on the weights first
+  // (the producer starts on the weights first; beside the wide launch of the same product there is
+  // nothing to wait for but that launch itself, at the end)
+  if (warp != 0 && !p.beside) pdl_wait();
   {
     uint32_t other;  // as in k_gemm_pair: both allocations must agree
     asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(other) : "r"(mapa_shared(smem_u32(tmem_slot), rank ^ 1u)));
@@ -799,9 +804,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     if (pair < total)
       for (; ahead < min(stages, k_steps); ++ahead)
         if (one) load_weights(ahead, weight_row(pair / m_tiles), ahead);
-    pdl_wait();
+    if (!p.beside) pdl_wait();
     for (int t = pair; t < total && ok; t += n_pairs) {
-      const int nb = t / m_tiles, row = (t % m_tiles) * 2 * R + static_cast<int>(rank) * R;
+      const int nb = t / m_tiles, row = p.row_begin + (t % m_tiles) * 2 * R + static_cast<int>(rank) * R;
       const int brow = weight_row(nb);
       for (int ks = 0; ks < k_steps; ++ks) {
         ok = wait_all_lanes(empty_bar(stage), phase ^ 1u, p);
@@ -870,7 +875,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     for (int t = pair; t < total; t += n_pairs, ++local) {
       const int block = SHORT ? quarter & 1 : quarter;   // the 32 rows of this lane quarter,
       const int cols = SHORT ? quarter >> 1 : part;      // and this warp's half of the columns
-      const int nb = t / m_tiles, row0 = (t % m_tiles) * 2 * R + static_cast<int>(rank) * R + block * 32;
+      const int nb = t / m_tiles;
+      const int row0 = p.row_begin + (t % m_tiles) * 2 * R + static_cast<int>(rank) * R + block * 32;
       // a warp with rows of the tile (R is a multiple of 32)
       const bool mine = block * 32 < R && row0 < p.M && !(SHORT && part != 0);
       const int acc = local % PAIR_ACCS;
@@ -888,6 +894,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     }
   }
 
+  if (p.beside) pdl_wait();  // completion carries over: the next kernel waits for this one only
   tc_fence_before();
   __syncthreads();
   cluster_sync();  // neither CTA leaves while the other may still address its barriers or TMEM
@@ -928,7 +935,7 @@ cudaError_t set_smem() {
 template <int EPI>
 cudaError_t launch_epi(const GemmOperandA& A, const GemmOperandB& B, const GemmParams& p, const GemmPlan& g, int num_sms,
                 cudaStream_t st) {
-  const int tiles = ((p.M + 2 * g.rows - 1) / (2 * g.rows)) * (p.N / g.cols);
+  const int tiles = ((p.M - p.row_begin + 2 * g.rows - 1) / (2 * g.rows)) * (p.N / g.cols);
   const int grid = 2 * (tiles < num_sms / 2 ? tiles : num_sms / 2 > 0 ? num_sms / 2 : 1);
   if (!g.few) {
     return launch_dependent(k_gemm_pair<EPI>, grid, THREADS, PAIR_SMEM_BYTES, st, A.wide, B.wide, p);
@@ -958,27 +965,73 @@ cudaError_t gemm_setup() {
 // saves a tenth (its L2 reuse is better).  Measured (cold cache, wide / taken): N 4,096
 // K 12,288, 25 rows 63.7 / 26 us, 180 rows 66.0 / 37 us; N 4,096 K 4,096, 25 rows
 // 28.0 / 13 us; gate/up N 24,576 K 4,096, 25 rows 59.0 / 39 us.
-GemmPlan gemm_plan(int epi, int M, int N, int K, int num_sms) {
-  const int64_t pairs = num_sms / 2 > 0 ? num_sms / 2 : 1;
-  auto clocks = [&](int R, int n) {
-    const int64_t tiles = static_cast<int64_t>((M + 2 * R - 1) / (2 * R)) * (N / n);
-    const bool half_m = epi == EPI_RESID_ADD && n == 64 && R <= 64;
-    const int64_t in = 2 * (R + n / 2), mma = n == BN ? 2 * BN : half_m ? 128 : 96 + 3 * n / 2;
-    return (tiles + pairs - 1) / pairs * (K / BK * (in > mma ? in : mma) + 2000);
-  };
-  GemmPlan best{false, BM, BN};
-  if (M > GEMM_FEW_MAX_ROWS) return best;
-  int64_t least = clocks(BM, BN) * 9 / 10;
+namespace {
+int64_t block_clocks(int epi, int R, int n) {
+  const bool half_m = epi == EPI_RESID_ADD && n == 64 && R <= 64;
+  const int64_t in = 2 * (R + n / 2), mma = n == BN ? 2 * BN : half_m ? 128 : 96 + 3 * n / 2;
+  return in > mma ? in : mma;
+}
+int64_t rounds(int M, int N, int R, int n, int64_t pairs) {
+  return (static_cast<int64_t>((M + 2 * R - 1) / (2 * R)) * (N / n) + pairs - 1) / pairs;
+}
+// The few-row plan of M <= GEMM_FEW_MAX_ROWS rows with the least clocks, if below `least` (which is updated).
+bool few_plan(int epi, int M, int N, int K, int64_t pairs, int64_t tile_clocks, int64_t& least, GemmPlan& plan) {
+  bool found = false;
   const int cols[2] = {128, 64};
   for (int n : cols) {
     if (N % n || (n == 64 && epi != EPI_RESID_ADD && epi != EPI_SWIGLU)) continue;
-    for (int R = 32; R <= BM; R += 32)
-      if (clocks(R, n) < least) {
-        least = clocks(R, n);
-        best = GemmPlan{true, R, n};
+    for (int R = 32; R <= BM; R += 32) {
+      const int64_t c = rounds(M, N, R, n, pairs) * (K / BK * block_clocks(epi, R, n) + tile_clocks);
+      if (c < least) {
+        least = c;
+        plan = GemmPlan{true, R, n, 0};
+        found = true;
       }
+    }
+  }
+  return found;
+}
+}  // namespace
+
+GemmPlan gemm_plan(int epi, int M, int N, int K, int num_sms) {
+  const int64_t pairs = num_sms / 2 > 0 ? num_sms / 2 : 1;
+  GemmPlan best{false, BM, BN, 0};
+  const int64_t wide = rounds(M, N, BM, BN, pairs);
+  if (M <= GEMM_FEW_MAX_ROWS) {
+    int64_t least = wide * (K / BK * block_clocks(epi, BM, BN) + 2000) * 9 / 10;
+    few_plan(epi, M, N, K, pairs, 2000, least, best);
+    if (best.few) return best;
+  }
+  // A last round that few tiles share: where the rows beyond the rounds before it make a single
+  // round of narrow tiles, they go to a few-row launch beside the wide one.  It has a start and an
+  // end of its own, about 6,000 clocks.  N 4,096, K 12,288: 3,800 rows are 240 tiles, 3.2 rounds of
+  // 76 pairs, of which 3,584 rows are 2.95 and the other 216 go beside them: 3 rounds instead of 4.
+  // Prefix build and scoring (4,096 and 2,432 rows a product, 8B width): 2,196 -> 2,102 us.
+  int64_t least = wide * (K / BK) * 2 * BN * 98 / 100;
+  const int m_tiles = (M + PAIR_BM - 1) / PAIR_BM;
+  for (int mt = m_tiles - 1; mt > 0 && M - mt * PAIR_BM <= GEMM_FEW_MAX_ROWS; --mt) {
+    const int rest = M - mt * PAIR_BM;
+    const int64_t base = rounds(mt * PAIR_BM, N, BM, BN, pairs) * (K / BK) * 2 * BN + 6000;
+    int64_t few = least - base;
+    GemmPlan p;
+    if (few > 0 && few_plan(epi, rest, N, K, pairs, 0, few, p) && rounds(rest, N, p.rows, p.cols, pairs) == 1) {
+      least = base + few;
+      best = p;
+      best.few = false;
+      best.wide_rows = mt * PAIR_BM;
+    }
   }
   return best;
+}
+
+static cudaError_t launch_one(int epi, const GemmOperandA& A, const GemmOperandB& B, const GemmParams& p, const GemmPlan& g,
+                              int num_sms, cudaStream_t st) {
+  switch (epi) {
+    case EPI_STORE: return launch_epi<EPI_STORE>(A, B, p, g, num_sms, st);
+    case EPI_RESID_ADD: return launch_epi<EPI_RESID_ADD>(A, B, p, g, num_sms, st);
+    case EPI_SWIGLU: return launch_epi<EPI_SWIGLU>(A, B, p, g, num_sms, st);
+    default: return launch_epi<EPI_QKV>(A, B, p, g, num_sms, st);
+  }
 }
 
 cudaError_t launch_gemm(int epi, const GemmOperandA& A, const GemmOperandB& B, const GemmParams& params, int num_sms,
@@ -987,12 +1040,16 @@ cudaError_t launch_gemm(int epi, const GemmOperandA& A, const GemmOperandB& B, c
   GemmParams p = params;
   p.timeout_ns = WAIT_TIMEOUT_NS;
   const GemmPlan g = gemm_plan(epi, p.M, p.N, p.K, num_sms);
-  switch (epi) {
-    case EPI_STORE: return launch_epi<EPI_STORE>(A, B, p, g, num_sms, st);
-    case EPI_RESID_ADD: return launch_epi<EPI_RESID_ADD>(A, B, p, g, num_sms, st);
-    case EPI_SWIGLU: return launch_epi<EPI_SWIGLU>(A, B, p, g, num_sms, st);
-    default: return launch_epi<EPI_QKV>(A, B, p, g, num_sms, st);
+  if (g.wide_rows > 0) {  // the first rows wide, the rest beside them
+    p.M = g.wide_rows;
+    const cudaError_t e = launch_one(epi, A, B, p, GemmPlan{false, BM, BN, 0}, num_sms, st);
+    if (e != cudaSuccess) return e;
+    p.M = params.M;
+    p.row_begin = g.wide_rows;
+    p.beside = 1;
+    return launch_one(epi, A, B, p, GemmPlan{true, g.rows, g.cols, 0}, num_sms, st);
   }
+  return launch_one(epi, A, B, p, g, num_sms, st);
 }
 
 }  // namespace dopr

