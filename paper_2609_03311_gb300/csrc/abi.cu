@@ -181,7 +181,7 @@ dopr_status build_weight_maps(Model* m) {
   for (int l = 0; l < L; ++l) {
     const bool ok = make_gemm_operand_b(&m->tm_qkv[l], m->w_qkv + (size_t)l * m->qkv_dim * H, H, m->qkv_dim) &&
                     make_gemm_operand_b(&m->tm_o[l], m->w_o + (size_t)l * H * m->o_dim, m->o_dim, H) &&
-                    make_gemm_operand_b(&m->tm_gu[l], m->w_gu + (size_t)l * 2 * F * H, H, 2 * F) &&
+                    make_gemm_operand_b(&m->tm_gu[l], m->w_gu + (size_t)l * 2 * F * H, H, 2 * F, true) &&
                     make_gemm_operand_b(&m->tm_down[l], m->w_down + (size_t)l * H * F, F, H);
     if (!ok) return fail(DOPR_ERR_CUDA, "cuTensorMapEncodeTiled failed for layer %d weights", l);
   }
@@ -994,6 +994,20 @@ static bool make_tmap_k_blocks(CUtensorMap* map, const void* base, uint64_t k, u
   return r == CUDA_SUCCESS;
 }
 
+// Gate/up weights [rows / 256][gate, up][128][k] as the 5-D tensor (64 elements, 128 rows, gate or up, blocks, k / 64).
+static bool make_tmap_gate_up(CUtensorMap* map, const void* base, uint64_t k, uint64_t rows, uint32_t box_blocks) {
+  auto fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[5] = {GEMM_BK, 128, 2, rows / 256, k / GEMM_BK};
+  cuuint64_t strides[4] = {k * 2, 128 * k * 2, 256 * k * 2, GEMM_BK * 2};
+  cuuint32_t box[5] = {GEMM_BK, 32, 2, 1, box_blocks};
+  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
 bool make_gemm_operand_a(GemmOperandA* a, const void* base, uint64_t k, uint64_t rows) {
   bool ok = make_tmap_16b_2d(&a->wide, base, k, rows, k * 2, GEMM_BK, GEMM_BM, true, true);
   for (int i = 0; i < 4; ++i)
@@ -1001,10 +1015,11 @@ bool make_gemm_operand_a(GemmOperandA* a, const void* base, uint64_t k, uint64_t
   return ok;
 }
 
-bool make_gemm_operand_b(GemmOperandB* b, const void* base, uint64_t k, uint64_t rows) {
+bool make_gemm_operand_b(GemmOperandB* b, const void* base, uint64_t k, uint64_t rows, bool gate_up) {
   bool ok = make_tmap_16b_2d(&b->wide, base, k, rows, k * 2, GEMM_BK, GEMM_B_BOX, true, true);
   for (int n = 0; n < 2; ++n)
     for (int kb = 0; kb < 2; ++kb) ok = ok && make_tmap_k_blocks(&b->few[n][kb], base, k, rows, 32u << n, 2u << kb);
+  for (int kb = 0; kb < 2 && gate_up; ++kb) ok = ok && make_tmap_gate_up(&b->gate_up[kb], base, k, rows, 2u << kb);
   return ok;
 }
 
@@ -1689,7 +1704,7 @@ dopr_status dopr_debug_gemm(int32_t M, int32_t N, int32_t K, const void* A, cons
   if (gemm_setup() != cudaSuccess) return fail(DOPR_ERR_CUDA, "gemm setup failed");
   GemmOperandA ta;
   GemmOperandB tb;
-  if (!make_gemm_operand_a(&ta, A, K, M) || !make_gemm_operand_b(&tb, B, K, N))
+  if (!make_gemm_operand_a(&ta, A, K, M) || !make_gemm_operand_b(&tb, B, K, N, epilogue == EPI_SWIGLU))
     return fail(DOPR_ERR_CUDA, "cuTensorMapEncodeTiled failed (pointers must be 16-byte aligned)");
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);

@@ -100,9 +100,16 @@ struct GemmOperandA {
 };
 struct GemmOperandB {
   CUtensorMap wide{}, few[2][2]{};  // [64 or 128 tile columns: 32 or 64 rows a CTA][2 or 4 k-blocks]
+  // Of gate/up weights (blocks of 128 gate rows and 128 up rows), 5-D (64 elements, row of the block, gate or up,
+  // block, k-blocks of 64): boxes of 32 gate rows, then the 32 up rows of the same outputs
+  CUtensorMap gate_up[2]{};  // [2 or 4 k-blocks]
 };
+// k_gemm_few launches of at most 64 rows a CTA whose MMAs take 64 rows of each CTA instead of 128
+__host__ __device__ constexpr bool gemm_half_m(int epi, int rows, int cols) {
+  return rows <= 64 && ((epi == EPI_RESID_ADD && cols == 64) || (epi == EPI_SWIGLU && cols == 128));
+}
 bool make_gemm_operand_a(GemmOperandA* a, const void* base, uint64_t k, uint64_t rows);
-bool make_gemm_operand_b(GemmOperandB* b, const void* base, uint64_t k, uint64_t rows);
+bool make_gemm_operand_b(GemmOperandB* b, const void* base, uint64_t k, uint64_t rows, bool gate_up = false);
 
 // Key token selection (k_select.cu).
 constexpr int SEL_MAX_N = 2048;  // longest document the selection takes

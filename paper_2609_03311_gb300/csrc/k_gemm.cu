@@ -228,7 +228,8 @@ __device__ __forceinline__ void epilogue_prefetch(const GemmParams& p, int row0,
 // BNT: columns of the tile, 256 (k_gemm_pair) or 64 / 128 (k_gemm_few).  The arithmetic on a row
 // is the same for every BNT, operation for operation.
 // release(): called by the whole warp once it has read its last accumulator value.
-template <int EPI, int BNT, typename Release>
+// HALF: the MMAs took 64 rows of each CTA (gemm_half_m), so that a lane holds half the tile's columns.
+template <int EPI, int BNT, bool HALF, typename Release>
 __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t taddr, int row0, int nb, int part,
                                               int lane, uint32_t* xs, EpiPre& pre, Release release) {
   // row0: first row of this warp; lane = row - row0 = TMEM lane
@@ -427,7 +428,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
       for (int half = 0; half < MINE / 32; ++half) {
         uint32_t g[32], u[32];
         tmem_ld32(taddr + c + 32 * half, g);
-        tmem_ld32(taddr + OUTS + c + 32 * half, u);
+        tmem_ld32(taddr + (HALF ? MINE : OUTS) + c + 32 * half, u);
         tmem_ld_wait();
         if (half + 1 == MINE / 32) release();
         float row_most = 0.f;
@@ -678,7 +679,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       if (!mbar_wait_cluster(tfull_bar(acc), acc_phase, p.err, p.timeout_ns)) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BN;
-      epilogue_tile<EPI, BN>(p, taddr, row0, nb, part, lane, xs, pre, [&] { free_accumulator(tempty_bar(acc), lane); });
+      epilogue_tile<EPI, BN, false>(p, taddr, row0, nb, part, lane, xs, pre, [&] { free_accumulator(tempty_bar(acc), lane); });
     }
   }
 
@@ -733,10 +734,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   const uint32_t drain_bar = bar0 + 8u * (2 * FEW_MAX_STAGES + 4);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * FEW_MAX_STAGES + 5);
   constexpr uint32_t TMEM_COLS = PAIR_ACCS * BNT;
-  // With at most 64 rows a CTA the residual launches take M = 128 MMAs, 64 rows a CTA: each reads
-  // half as much of A (48 -> 32 clocks of shared memory at 64 columns).  A CTA's rows are then
-  // TMEM lanes 0..63 for the tile's first half of the columns and 64..127 for its second.
-  constexpr bool SHORT = EPI == EPI_RESID_ADD && BNT == 64 && R <= 64;
+  // With at most 64 rows a CTA the residual and gate/up launches take M = 128 MMAs, 64 rows a CTA:
+  // each reads half as much of A (48 -> 32 clocks of shared memory at 64 columns).  A CTA's rows are
+  // then TMEM lanes 0..63 for the tile's first half of the columns and 64..127 for its second; for
+  // gate and up of an output to share a lane, each CTA stages 32 gate rows and their 32 up rows.
+  // Cold cache, 25 rows: gate/up N 24,576 K 4,096 (201 MB of weights, 29.7 us at the copy's rate)
+  // 40.3 -> 36.3 us.
+  constexpr bool SHORT = gemm_half_m(EPI, R, BNT);
+  constexpr bool MIXED = SHORT && EPI == EPI_SWIGLU;
   constexpr uint32_t IDESC = umma_idesc_f16(SHORT ? BM : PAIR_BM, BNT);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -792,12 +797,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     // SwiGLU weights hold gate and up in alternating blocks of 128 rows: rank 0 takes gate rows, rank 1 up rows
     auto weight_row = [&](int nb) {
       const int o = nb * (BNT / 2);
+      if constexpr (MIXED) return o + static_cast<int>(rank) * 32;
       return EPI == EPI_SWIGLU ? (o / 128) * 256 + o % 128 + static_cast<int>(rank) * 128
                                : nb * BNT + static_cast<int>(rank) * (BNT / 2);
     };
     auto load_weights = [&](int s, int brow, int ks) {  // k-blocks past K are filled with zeros and count as copied
       if (leader) mbar_arrive_expect_tx(full_bar(s), 2 * stage_bytes);
-      tma_load_3d_pair(sB + s * KB * b_blk, &tmB, mapa_shared(full_bar(s), 0), 0, brow, ks * KB);
+      if constexpr (MIXED)  // brow: the CTA's first output
+        tma_load_5d_pair(sB + s * KB * b_blk, &tmB, mapa_shared(full_bar(s), 0), 0, brow % 128, 0, brow / 128, ks * KB);
+      else
+        tma_load_3d_pair(sB + s * KB * b_blk, &tmB, mapa_shared(full_bar(s), 0), 0, brow, ks * KB);
     };
     // the first stages' weights, which no kernel writes, go out while the kernel before still runs
     int ahead = 0;
@@ -886,9 +895,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       tc_fence_after();
       // (epilogue_tile adds the half's first column, which here is a lane offset)
       const uint32_t taddr =
-          tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BNT - (SHORT ? cols * (BNT / 2) : 0);
+          tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BNT - (SHORT ? cols * 32 : 0);
       if (mine)
-        epilogue_tile<EPI, BNT>(p, taddr, row0, nb, cols, lane, xs, pre, [&] { free_accumulator(tempty_bar(acc), lane); });
+        epilogue_tile<EPI, BNT, SHORT>(p, taddr, row0, nb, cols, lane, xs, pre, [&] { free_accumulator(tempty_bar(acc), lane); });
       else
         free_accumulator(tempty_bar(acc), lane);
     }
@@ -941,7 +950,9 @@ cudaError_t launch_epi(const GemmOperandA& A, const GemmOperandB& B, const GemmP
     return launch_dependent(k_gemm_pair<EPI>, grid, THREADS, PAIR_SMEM_BYTES, st, A.wide, B.wide, p);
   }
   const CUtensorMap& ta = A.few[g.rows / 32 - 1];
-  const CUtensorMap& tb = B.few[g.cols == 128][GEMM_FEW_KB(g.rows) == 4];
+  const int four = GEMM_FEW_KB(g.rows) == 4;
+  const CUtensorMap& tb =
+      EPI == EPI_SWIGLU && gemm_half_m(EPI, g.rows, g.cols) ? B.gate_up[four] : B.few[g.cols == 128][four];
   return few_kernel<EPI>(g.rows, g.cols,
                          [&](auto* k) { return launch_dependent(k, grid, THREADS, FEW_SMEM_BYTES, st, ta, tb, p); });
 }
@@ -958,17 +969,16 @@ cudaError_t gemm_setup() {
 
 // The clocks a CTA pair needs for a 64-wide k-block of a tile of 2 R rows and n columns: its SMs
 // take in R + n / 2 operand rows of 128 bytes at about 64 bytes a clock, and the four MMAs take
-// 512 at n = 256 but 288 at 128 and 192 at 64 (each reads 128 A rows a CTA, whatever R is; the
-// residual launches' 64-row MMAs 128).
+// 512 at n = 256 but 288 at 128 and 192 at 64 (each reads 128 A rows a CTA, whatever R is; 64-row
+// MMAs, gemm_half_m, 128 at 64 columns and 192 at 128).
 // Every tile adds a start and an epilogue that is not hidden, about 2,000 clocks.  The tile
 // with the least clocks over the launch's rounds is taken; the wide one unless a narrow one
 // saves a tenth (its L2 reuse is better).  Measured (cold cache, wide / taken): N 4,096
 // K 12,288, 25 rows 63.7 / 26 us, 180 rows 66.0 / 37 us; N 4,096 K 4,096, 25 rows
-// 28.0 / 13 us; gate/up N 24,576 K 4,096, 25 rows 59.0 / 39 us.
+// 28.0 / 13 us; gate/up N 24,576 K 4,096, 25 rows 59.0 / 36 us.
 namespace {
 int64_t block_clocks(int epi, int R, int n) {
-  const bool half_m = epi == EPI_RESID_ADD && n == 64 && R <= 64;
-  const int64_t in = 2 * (R + n / 2), mma = n == BN ? 2 * BN : half_m ? 128 : 96 + 3 * n / 2;
+  const int64_t in = 2 * (R + n / 2), mma = n == BN ? 2 * BN : gemm_half_m(epi, R, n) ? 64 + n : 96 + 3 * n / 2;
   return in > mma ? in : mma;
 }
 int64_t rounds(int M, int N, int R, int n, int64_t pairs) {
@@ -1006,9 +1016,9 @@ GemmPlan gemm_plan(int epi, int M, int N, int K, int num_sms) {
   // round of narrow tiles, they go to a few-row launch beside the wide one.  It has a start and an
   // end of its own, about 6,000 clocks.  N 4,096, K 12,288: 3,800 rows are 240 tiles, 3.2 rounds of
   // 76 pairs, of which 3,584 rows are 2.95 and the other 216 go beside them: 3 rounds instead of 4.
-  // Against the same library without it, whole
-  // calls: prefix build and scoring (8B width) 2,138 -> 2,100 us, selection of long documents (4B width, 5,650 rows a
-  // product) 2,183 -> 2,136, uncompressed scoring 2,654 -> 2,640.
+  // Against the same library without it, whole calls: prefix build and scoring (8B width) 2,138 ->
+  // 2,100 us, selection of long documents (4B width, 5,650 rows a product) 2,183 -> 2,136,
+  // uncompressed scoring 2,654 -> 2,640.
   int64_t least = wide * (K / BK) * 2 * BN * 98 / 100;
   const int m_tiles = (M + PAIR_BM - 1) / PAIR_BM;
   for (int mt = m_tiles - 1; mt > 0 && M - mt * PAIR_BM <= GEMM_FEW_MAX_ROWS; --mt) {

@@ -373,7 +373,8 @@ def test_bounded_wait_gives_up_and_context_survives():
     assert torch.allclose(out.float(), (A.float() @ B.float().T), rtol=1e-2, atol=1e-1)
 
 
-@pytest.mark.parametrize("N,K", [(256, 64), (512, 320), (1024, 3072), (2560, 1024), (4096, 2048)])
+@pytest.mark.parametrize("N,K", [(256, 64), (512, 320), (1024, 3072), (2560, 1024), (4096, 2048),
+                                 (9728, 320)])  # 9,728: gate/up takes 128-column tiles of 64 rows a CTA too
 def test_gemm_few_rows_match_wide_tiles_bit_for_bit(N, K):
     # Launches of few rows take narrow tiles (64 or 128 columns, 32 to 128 rows a CTA), chosen by size; more than
     # 1,024 rows always take the wide ones.  A row's K order is the same in all, so its result is too.  K = 320 is not
