@@ -445,3 +445,22 @@ def test_gemm_rows_beside_the_wide_tiles(M, N, K):
     ref = _ref_gemm(A, B) + R.double()
     scale = (A.double().abs() @ B.double().abs().T) + R.double().abs()
     assert torch.all((got.double() - ref).abs() <= 1e-5 * scale + 1e-6)
+
+
+@pytest.mark.parametrize("heads,hidden,ffn", [((2, 1), 256, 512), ((4, 2), 256, 512), ((16, 8), 4096, 2048)])
+def test_large_batches_match_their_parts_bit_for_bit(heads, hidden, ffn):
+    # More than 1,024 tokens take the wide tiles.  Two q heads and one kv head leave a tile of one rotated and one plain
+    # head; hidden 4,096 puts the last rows of O and down, with their sums of squares, into a launch beside the wide one.
+    # Parts of the batch take few-row tiles throughout.
+    shape = synth.ModelShape("wide-2l", n_layers=2, hidden=hidden, n_q_heads=heads[0], n_kv_heads=heads[1],
+                             head_dim=128, ffn=ffn, vocab=300)
+    rig = Rig(shape, {0: 64, 1: 17}, seed=21)
+    pairs = synth.random_pairs(40, 2, 24, 48, shape.vocab, seed=21)
+    qo, qt, di = pairs["q_offsets"], pairs["q_tokens"], pairs["doc_ids"]
+    lens = np.diff(qo)
+    assert lens.sum() + 40 > 1024 + 64
+    base = rig.score(pairs)
+    for sel in (np.arange(0, 40, 2), np.arange(30, 40), np.array([3])):
+        part = {"q_offsets": np.concatenate([[0], np.cumsum(lens[sel])]).astype(np.int32),
+                "q_tokens": np.concatenate([qt[qo[p]:qo[p + 1]] for p in sel]).astype(np.int32), "doc_ids": di[sel]}
+        np.testing.assert_array_equal(rig.score(part), base[sel])
