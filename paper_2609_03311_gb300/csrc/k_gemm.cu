@@ -995,10 +995,10 @@ cudaError_t gemm_setup() {
 // 512 at n = 256 but 288 at 128 and 192 at 64 (each reads 128 A rows a CTA, whatever R is; 64-row
 // MMAs, gemm_half_m, 128 at 64 columns and 192 at 128).
 // Every tile adds a start and an epilogue that is not hidden, about 2,000 clocks.  The tile
-// with the least clocks over the launch's rounds is taken; the wide one unless a narrow one
-// saves a tenth (its L2 reuse is better).  Measured (cold cache, wide / taken): N 4,096
-// K 12,288, 25 rows 63.7 / 26 us, 180 rows 66.0 / 37 us; N 4,096 K 4,096, 25 rows
-// 28.0 / 13 us; gate/up N 24,576 K 4,096, 25 rows 59.0 / 36 us.
+// with the least clocks over the launch's rounds is taken, the wide one of two equal ones.
+// Measured (cold cache, wide / taken): N 4,096 K 12,288, 25 rows 63.7 / 26 us, 180 rows
+// 66.0 / 37 us; N 4,096 K 4,096, 25 rows 28.0 / 13 us; gate/up N 24,576 K 4,096, 25 rows
+// 59.0 / 36 us, 180 rows (estimates 3 % apart) 50.1 / 46.4 us.
 namespace {
 int64_t block_clocks(int epi, int R, int n) {
   const int64_t in = 2 * (R + n / 2), mma = n == BN ? 2 * BN : gemm_half_m(epi, R, n) ? 64 + n : 96 + 3 * n / 2;
@@ -1031,7 +1031,7 @@ GemmPlan gemm_plan(int epi, int M, int N, int K, int num_sms) {
   GemmPlan best{false, BM, BN, 0};
   const int64_t wide = rounds(M, N, BM, BN, pairs);
   if (M <= GEMM_FEW_MAX_ROWS) {
-    int64_t least = wide * (K / BK * block_clocks(epi, BM, BN) + 2000) * 9 / 10;
+    int64_t least = wide * (K / BK * block_clocks(epi, BM, BN) + 2000);
     few_plan(epi, M, N, K, pairs, 2000, least, best);
     if (best.few) return best;
   }
