@@ -73,6 +73,10 @@ __device__ __forceinline__ int ld_volatile(const int* p) { return *reinterpret_c
 // there is room.  pdl_wait() returns when the kernel before has completed and its writes are
 // visible; every block calls it before it touches anything another kernel of the pass writes or
 // reads, and before it ends, so that completion carries over from kernel to kernel.
+// A resident kernel thus sees memory change: what a kernel of the pass writes is read through
+// plain pointers (never __ldg or const __restrict__, whose loads may go through the non-coherent
+// path and be moved above the wait); those are for weights, gains, the RoPE table and whatever
+// was copied or finished before the first dependent launch.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

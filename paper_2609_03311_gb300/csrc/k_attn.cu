@@ -164,10 +164,10 @@ __device__ __forceinline__ void load_q(const AttnArgs& a, const PairGeom& pg, in
 #pragma unroll
   for (int ks = 0; ks < 8; ++ks) {
     const int w = ks * 8 + t;  // 32-bit word index of columns 16ks + 2t
-    qf[ks][0] = qa ? __ldg(qa + w) : 0u;
-    qf[ks][1] = qb ? __ldg(qb + w) : 0u;
-    qf[ks][2] = qa ? __ldg(qa + w + 4) : 0u;
-    qf[ks][3] = qb ? __ldg(qb + w + 4) : 0u;
+    qf[ks][0] = qa ? qa[w] : 0u;
+    qf[ks][1] = qb ? qb[w] : 0u;
+    qf[ks][2] = qa ? qa[w + 4] : 0u;
+    qf[ks][3] = qb ? qb[w + 4] : 0u;
   }
 }
 

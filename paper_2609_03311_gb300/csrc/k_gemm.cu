@@ -79,7 +79,7 @@ __device__ __forceinline__ float norm_factor(const float* ss, int parts, const G
       float4 v[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q)
-        v[q] = i + 4 * q < parts ? __ldg(reinterpret_cast<const float4*>(s + i) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[q] = i + 4 * q < parts ? reinterpret_cast<const float4*>(s + i)[q] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int q = 0; q < 8; ++q)
         if (i + 4 * q < parts) {

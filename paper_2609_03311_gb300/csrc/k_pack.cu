@@ -270,7 +270,7 @@ __global__ void k_pack_tokens(PackArgs a) {
   }
 }
 
-__global__ void k_commit_scores(const int* err, const float* __restrict__ scores, float* __restrict__ out, int n) {
+__global__ void k_commit_scores(const int* err, const float* scores, float* __restrict__ out, int n) {
   pdl_trigger();
   pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;

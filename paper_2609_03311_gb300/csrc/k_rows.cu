@@ -39,7 +39,7 @@ __device__ __forceinline__ void bf16x4_to_float(const bf16* p, float (&v)[4]) {
 // 25 rows 9.7 -> 7.6 us, 3,800 rows 29.3 -> 26.1 us, 32,768 rows 171 -> 158 us.
 constexpr int ROW_WARPS = 4, EMBED_AHEAD = 8;
 __global__ void __launch_bounds__(ROW_WARPS * 32)
-    k_embed(const int32_t* __restrict__ tok_id, int T, const bf16* __restrict__ embed, const bf16* __restrict__ gain,
+    k_embed(const int32_t* tok_id, int T, const bf16* __restrict__ embed, const bf16* __restrict__ gain,
             int H, float eps, float* __restrict__ r, f16* __restrict__ xn, float* __restrict__ ss_out, Extents ext) {
   pdl_trigger();
   pdl_wait();
@@ -113,7 +113,7 @@ __global__ void k_bf16_to_f16(uint32_t* __restrict__ buf, int64_t n_words, int* 
 // walked it in 192 dependent loads, 37-40 us; a block in four rounds, 6 us).
 constexpr int SCORE_THREADS = 256;
 __global__ void __launch_bounds__(SCORE_THREADS)
-    k_score(const float* __restrict__ r, int H, const int32_t* __restrict__ tok_off, int tok0, int p_begin, int compact,
+    k_score(const float* r, int H, const int32_t* __restrict__ tok_off, int tok0, int p_begin, int compact,
             const int32_t* __restrict__ perm, const bf16* __restrict__ gain, const bf16* __restrict__ head, float eps,
             float* __restrict__ scores, Extents ext) {
   __shared__ float red[SCORE_THREADS / 32];
@@ -173,7 +173,7 @@ __device__ __forceinline__ float head_act(float z, int act) {
   }
 }
 __global__ void __launch_bounds__(MLP_THREADS)
-    k_score_mlp(const float* __restrict__ r, int H, const int32_t* __restrict__ tok_off, int tok0, int p_begin,
+    k_score_mlp(const float* r, int H, const int32_t* __restrict__ tok_off, int tok0, int p_begin,
                 int p_end, int compact, const bf16* __restrict__ gain, float eps, int width, int act,
                 const bf16* __restrict__ w1, const bf16* __restrict__ b1, const bf16* __restrict__ w2, int passes,
                 float* __restrict__ part, Extents ext) {
@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(MLP_THREADS)
   }
 }
 // One warp per pair: its splits' sums in order, and b2.
-__global__ void k_score_mlp_sum(const float* __restrict__ part, int splits, int n, const int32_t* __restrict__ perm, float b2,
+__global__ void k_score_mlp_sum(const float* part, int splits, int n, const int32_t* __restrict__ perm, float b2,
                                 float* __restrict__ scores, int* err) {
   pdl_trigger();
   pdl_wait();
@@ -278,7 +278,7 @@ __global__ void k_score_mlp_sum(const float* __restrict__ part, int splits, int 
 // 4.5 us at 1-100 pairs of 4,096 elements: a latency, like the score head's).
 constexpr int GATHER_THREADS = 256;
 __global__ void __launch_bounds__(GATHER_THREADS)
-    k_gather_score_rows(const float* __restrict__ r, const float* __restrict__ ss, int H, int parts,
+    k_gather_score_rows(const float* r, const float* ss, int H, int parts,
                         const int32_t* __restrict__ tok_off, int tok0, int p_begin, float* __restrict__ dst_r,
                         float* __restrict__ dst_ss, Extents ext) {
   pdl_trigger();
@@ -327,7 +327,7 @@ __global__ void k_store_transpose(const uint4* __restrict__ k, const uint4* __re
 // raw value of every kv head from the packed QKV buffer into its document's block of
 // the store pool, in the layout dopr_store_put writes: per layer, K then V, per kv
 // head, m rows of 128.  One warp per (token, kv head, K|V), 8 bytes a lane.
-__global__ void k_prefix_store(const f16* __restrict__ qkv, int ld_qkv, int T, int t0, int Hq, int Hkv,
+__global__ void k_prefix_store(const f16* qkv, int ld_qkv, int T, int t0, int Hq, int Hkv,
                                const int32_t* __restrict__ tok_pair, const int32_t* __restrict__ tok_pos,
                                const int32_t* __restrict__ pair_slot, const int64_t* __restrict__ slot_row,
                                const int32_t* __restrict__ slot_m, int layer, f16* __restrict__ pool, Extents ext) {

@@ -61,7 +61,7 @@ __device__ __forceinline__ float ex2_approx(float x) {
 template <bool STATS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_sal_tc(const __grid_constant__ CUtensorMap tm, const SelUnit* __restrict__ units, int n_units, int Hq, int Hkv,
-             int n_rows, float2* __restrict__ stats, float* __restrict__ A, Extents ext) {
+             int n_rows, float2* stats, float* __restrict__ A, Extents ext) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t s0 = smem_u32(smem);
@@ -313,7 +313,7 @@ constexpr int COL_WARPS = 8;
 template <int NV>
 __global__ void __launch_bounds__(32 * COL_WARPS)
     k_sal_colstat(const int32_t* __restrict__ tok_pair, const int32_t* __restrict__ tok_off, int t0, int p0, int n_rows,
-                  const int64_t* __restrict__ a_off, const float* __restrict__ A, int top_p, float* __restrict__ u,
+                  const int64_t* __restrict__ a_off, const float* A, int top_p, float* __restrict__ u,
                   Extents ext) {
   pdl_trigger();
   pdl_wait();
@@ -390,7 +390,7 @@ __device__ __forceinline__ int block_scan(int c, int* warp_sums, int* total) {
 // floats do, then two scans pick the ties and place the positions (8 us; a bitonic sort of
 // 2,048 keys and a serial compaction took 33-40 us).
 __global__ void __launch_bounds__(TOPK_THREADS) k_sal_topk(const int32_t* __restrict__ tok_off, int t0, int p0,
-                                                           const float* __restrict__ u, int K,
+                                                           const float* u, int K,
                                                            int32_t* __restrict__ positions) {
   static_assert(SEL_MAX_N == 2 * TOPK_THREADS, "two positions a thread");
   __shared__ int warp_sums[32];
@@ -433,8 +433,8 @@ __global__ void __launch_bounds__(TOPK_THREADS) k_sal_topk(const int32_t* __rest
 }
 
 // One warp per (document, selected slot): x = bf16(RMSNorm(r_row) * g_final), zeros for -1.
-__global__ void k_sal_gather(const float* __restrict__ r, int H, const int32_t* __restrict__ tok_off, int t0,
-                             int p0, int n_docs, const int32_t* __restrict__ positions, int K,
+__global__ void k_sal_gather(const float* r, int H, const int32_t* __restrict__ tok_off, int t0,
+                             int p0, int n_docs, const int32_t* positions, int K,
                              const bf16* __restrict__ gain, float eps, bf16* __restrict__ x, Extents ext) {
   pdl_trigger();
   pdl_wait();

@@ -1,0 +1,75 @@
+"""Rules of the dependent launches, checked on the CUDA sources (no GPU needed).
+
+A kernel launched with programmatic stream serialization is resident while the kernels before it still write.  What
+such a kernel reads through the non-coherent path (``__ldg``, ``const ... __restrict__`` parameters) must not change
+while it is resident, and the compiler may move those loads above ``pdl_wait()``: they are for data that no kernel of a
+pass writes."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_03311_gb300", "csrc")
+SOURCES = sorted(f for f in os.listdir(CSRC) if f.endswith(".cu"))
+
+# weights and gains; tables of the store; what is copied to the device, or finished before a wait of the host, ahead of
+# the first dependent launch (packed offsets and order, a build's or selection's token records, score tiles)
+CONSTANT = {"embed", "gain", "head", "w1", "b1", "w2", "slot_row", "slot_m", "tok_off", "perm", "tok_pair", "tok_pos",
+            "pair_slot", "units", "a_off"}
+CONSTANT_LDG = ("xn_gain", "cs", "wgt")  # the next norm's gains, the RoPE table's entries, the q/k norm gains
+
+
+def _source(name):
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def _block(text, start):
+    """The brace-delimited block that begins at or after `start`."""
+    i = text.index("{", start)
+    depth = 0
+    for j in range(i, len(text)):
+        depth += (text[j] == "{") - (text[j] == "}")
+        if depth == 0:
+            return text[i:j + 1]
+    raise AssertionError("unbalanced braces")
+
+
+def _kernels(text):
+    """(name, parameter list, body) of every __global__ function defined in the text."""
+    for m in re.finditer(r"__global__\b", text):
+        sig = re.compile(r"(\bk_\w+)\s*\(").search(text, m.end())
+        depth, i = 1, sig.end()
+        while depth:
+            depth += (text[i] == "(") - (text[i] == ")")
+            i += 1
+        yield sig.group(1), text[sig.end():i - 1], _block(text, i)
+
+
+def _call_args(text, name):
+    for m in re.finditer(r"\b%s\s*\(" % name, text):
+        depth, i = 1, m.end()
+        while depth:
+            depth += (text[i] == "(") - (text[i] == ")")
+            i += 1
+        yield text[m.end():i - 1]
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_non_coherent_loads_are_of_constant_data(name):
+    text = _source(name)
+    for arg in _call_args(text, "__ldg"):
+        assert any(re.search(r"\b%s\b" % c, arg) for c in CONSTANT_LDG), f"{name}: __ldg({arg})"
+    for kernel, params, body in _kernels(text):
+        if "pdl_wait()" not in body:
+            continue
+        for p in params.split(","):
+            if re.search(r"\bconst\b", p) and "__restrict__" in p:
+                assert p.split()[-1] in CONSTANT, f"{name}: {kernel} reads {p.split()[-1]} through the non-coherent path"
+
+
+def test_the_rule_sees_the_dependent_kernels():
+    found = {k for s in SOURCES for k, _, body in _kernels(_source(s)) if "pdl_wait()" in body}
+    assert {"k_embed", "k_gemm_pair", "k_gemm_few", "k_attn", "k_attn_tc", "k_attn_tc_long", "k_sal_tc", "k_sal_colstat",
+            "k_sal_topk", "k_sal_gather", "k_score", "k_score_mlp", "k_score_mlp_sum", "k_gather_score_rows",
+            "k_prefix_store", "k_commit_scores"} <= found
