@@ -152,7 +152,9 @@ __device__ __forceinline__ bool elect_one() {
   return ok != 0;
 }
 
-// The same by a whole converged warp: all lanes go on or give up together.
+// The same by a whole converged warp: all lanes go on or give up together.  Whoever goes on to
+// work the whole warp does (tensor memory accesses, shuffles) waits this way: with lanes that gave
+// up by themselves at the time limit the others would wait for them without one.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* err, uint64_t timeout_ns) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, timeout_ns)) != 0;
 }

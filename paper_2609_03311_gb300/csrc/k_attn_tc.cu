@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       auto chunk_live = [&](int c0) { return c0 < m || (c0 <= whi && c0 + 31 >= wlo); };
       auto vis_mask = [&](int c0) { return bits_in(-c0, m - c0) | bits_in(olo - c0, ohi + 1 - c0); };
 
-      if (!mbar_wait(bar(BAR_S_FULL + slot), par, a.err, WAIT_TIMEOUT_NS)) break;
+      if (!mbar_wait_warp(bar(BAR_S_FULL + slot), par, a.err, WAIT_TIMEOUT_NS)) break;
       tc_fence_after();
       // ---- pass 1: the row maximum over the visible keys
       float mx = -INFINITY;
@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       // ---- epilogue: O / sum -> fp16 at (token, q head g * G + hh), 64 columns at a
       // time through this warp's staging lines (128 bytes per row, 16-byte chunks
       // swizzled by the row), each store instruction writing four 128-byte row pieces
-      if (!mbar_wait(bar(BAR_O_FULL + slot), par, a.err, WAIT_TIMEOUT_NS)) break;
+      if (!mbar_wait_warp(bar(BAR_O_FULL + slot), par, a.err, WAIT_TIMEOUT_NS)) break;
       tc_fence_after();
       const float inv = sum > 0.f ? 1.f / sum : 0.f;
       bool bad = false;  // a stored output value not finite or beyond fp16's range
@@ -899,7 +899,7 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
       float mx = -INFINITY;
       for (int c = 0; c < nc && ok; ++c) {
         const uint32_t buf = cc & 1u;
-        if (!mbar_wait(bar(lt::B_S_FULL + buf), (cc >> 1) & 1u, a.err, WAIT_TIMEOUT_NS)) {
+        if (!mbar_wait_warp(bar(lt::B_S_FULL + buf), (cc >> 1) & 1u, a.err, WAIT_TIMEOUT_NS)) {
           ok = false;
           break;
         }
@@ -930,13 +930,13 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
       float sum = 0.f;
       for (int c = 0; c < nc && ok; ++c) {
         const uint32_t buf = cc & 1u;
-        if (!mbar_wait(bar(lt::B_S_FULL + buf), (cc >> 1) & 1u, a.err, WAIT_TIMEOUT_NS)) {
+        if (!mbar_wait_warp(bar(lt::B_S_FULL + buf), (cc >> 1) & 1u, a.err, WAIT_TIMEOUT_NS)) {
           ok = false;
           break;
         }
         tc_fence_after();
         for (int j = 2 * c; j < min(nb, 2 * c + 2); ++j) {
-          if (!mbar_wait(bar(lt::B_P_EMPTY + rp.stage), rp.phase ^ 1u, a.err, WAIT_TIMEOUT_NS)) {
+          if (!mbar_wait_warp(bar(lt::B_P_EMPTY + rp.stage), rp.phase ^ 1u, a.err, WAIT_TIMEOUT_NS)) {
             ok = false;
             break;
           }
@@ -966,7 +966,7 @@ __global__ void __launch_bounds__(lt::THREADS, 1)
       }
       if (!ok) break;
       // ---- epilogue: O / sum -> fp16, 64 columns at a time through this warp's staging lines
-      if (!mbar_wait(bar(lt::B_O_FULL), static_cast<uint32_t>(i) & 1u, a.err, WAIT_TIMEOUT_NS)) break;
+      if (!mbar_wait_warp(bar(lt::B_O_FULL), static_cast<uint32_t>(i) & 1u, a.err, WAIT_TIMEOUT_NS)) break;
       tc_fence_after();
       const float inv = sum > 0.f ? 1.f / sum : 0.f;
       bool bad = false;  // a stored output value not finite or beyond fp16's range

@@ -683,7 +683,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       }
       // All MMAs this thread issued are complete once drain_bar flips.
       if (one) umma_commit_pair_mc(drain_bar, 1);
-      mbar_wait(drain_bar, 0, p.err, ok ? p.timeout_ns : 100000000ull);
+      mbar_wait_warp(drain_bar, 0, p.err, ok ? p.timeout_ns : 100000000ull);
     }
   } else {
     // ---------------- epilogue warps 2..9 (both CTAs) on this CTA's 128 rows of the tile
@@ -699,7 +699,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       const uint32_t acc_phase = (local / PAIR_ACCS) & 1;
       EpiPre pre;
       epilogue_prefetch<EPI, BN>(p, row0, nb, part, lane, pre);
-      if (!mbar_wait_cluster(tfull_bar(acc), acc_phase, p.err, p.timeout_ns)) break;
+      if (!wait_all_lanes(tfull_bar(acc), acc_phase, p)) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BN;
       epilogue_tile<EPI, BN, false>(p, taddr, row0, nb, part, lane, xs, pre, [&] { free_accumulator(tempty_bar(acc), lane); });
@@ -896,7 +896,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
         if (ok && one) umma_commit_pair_mc(tfull_bar(acc), 3);
       }
       if (one) umma_commit_pair_mc(drain_bar, 1);
-      mbar_wait(drain_bar, 0, p.err, ok ? p.timeout_ns : 100000000ull);
+      mbar_wait_warp(drain_bar, 0, p.err, ok ? p.timeout_ns : 100000000ull);
     }
   } else {
     // ---------------- epilogue warps 2..9 (both CTAs) on this CTA's R rows of the tile
@@ -914,7 +914,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       const int acc = local % PAIR_ACCS;
       EpiPre pre;
       if (mine) epilogue_prefetch<EPI, BNT>(p, row0, nb, cols, lane, pre);
-      if (!mbar_wait_cluster(tfull_bar(acc), (local / PAIR_ACCS) & 1, p.err, p.timeout_ns)) break;
+      if (!wait_all_lanes(tfull_bar(acc), (local / PAIR_ACCS) & 1, p)) break;
       tc_fence_after();
       // (epilogue_tile adds the half's first column, which here is a lane offset)
       const uint32_t taddr =

@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const int ct = STATS ? s : u.ct;
         const int nvis = pos - (ct * TILE + part * 32) + 1;  // visible columns among this thread's 32, if in 1..31
         const float2 nst = !STATS && s + 1 < n ? stat_at(s + 1) : st;
-        if (!mbar_wait(bar(B_SF + rs.stage), rs.phase, err, WAIT_TIMEOUT_NS)) {
+        if (!mbar_wait_warp(bar(B_SF + rs.stage), rs.phase, err, WAIT_TIMEOUT_NS)) {
           ok = false;
           break;
         }
@@ -259,12 +259,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       if (!ok) break;
       if constexpr (STATS) {
         // the four parts of a row meet in shared memory; part 0 writes the result
-        if (!mbar_wait(bar(B_RE), unit_par ^ 1u, err, WAIT_TIMEOUT_NS)) break;
+        if (!mbar_wait_warp(bar(B_RE), unit_par ^ 1u, err, WAIT_TIMEOUT_NS)) break;
         red[part * TILE + r] = make_float2(mx, sum);
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(B_RF));
         if (part == 0) {
-          if (!mbar_wait(bar(B_RF), unit_par, err, WAIT_TIMEOUT_NS)) break;
+          if (!mbar_wait_warp(bar(B_RF), unit_par, err, WAIT_TIMEOUT_NS)) break;
           float2 x[PARTS];
 #pragma unroll
           for (int p = 0; p < PARTS; ++p) x[p] = red[p * TILE + r];

@@ -1,4 +1,4 @@
-"""Rules of the dependent launches, checked on the CUDA sources (no GPU needed).
+"""Rules of the dependent launches and of the bounded waits, checked on the CUDA sources (no GPU needed).
 
 A kernel launched with programmatic stream serialization is resident while the kernels before it still write.  What
 such a kernel reads through the non-coherent path (``__ldg``, ``const ... __restrict__`` parameters) must not change
@@ -73,3 +73,12 @@ def test_the_rule_sees_the_dependent_kernels():
     assert {"k_embed", "k_gemm_pair", "k_gemm_few", "k_attn", "k_attn_tc", "k_attn_tc_long", "k_sal_tc", "k_sal_colstat",
             "k_sal_topk", "k_sal_gather", "k_score", "k_score_mlp", "k_score_mlp_sum", "k_gather_score_rows",
             "k_prefix_store", "k_commit_scores"} <= found
+
+
+def test_waits_before_work_of_the_whole_warp_are_the_whole_warps():
+    # A lane that gives up by itself at the time limit leaves the others in a shuffle or a tensor memory access that
+    # waits for it.  Single-lane waits stay where the block meets right after (k_attn) and in the one-thread probe.
+    for name in SOURCES:
+        single = list(_call_args(_source(name), "mbar_wait")) + list(_call_args(_source(name), "mbar_wait_cluster"))
+        allowed = {"k_attn.cu": 2, "k_rows.cu": 1, "k_gemm.cu": 1}.get(name, 0)  # k_gemm: inside wait_all_lanes
+        assert len(single) == allowed, (name, single)
