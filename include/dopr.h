@@ -322,10 +322,10 @@ DOPR_API dopr_status dopr_debug_gemm(int32_t M, int32_t N, int32_t K, const void
                             int32_t epilogue, void *cuda_stream);
 
 /*
- * Runs one test kernel whose bounded wait on a barrier that nothing
- * completes must give up after about timeout_ms milliseconds.  Returns
- * DOPR_ERR_TIMEOUT when the kernel reported the expired wait (the expected
- * result), DOPR_OK if it did not.  Used to check the timeout path of the
+ * Runs one test kernel whose bounded waits, one on a barrier that nothing
+ * completes and one at a gate that nothing opens, must give up after about
+ * timeout_ms milliseconds.  Returns DOPR_ERR_TIMEOUT when the kernel reported
+ * both waits as expired (the expected result), DOPR_OK if it did not.  Used to check the timeout path of the
  * device waits without hanging the GPU.
  */
 DOPR_API dopr_status dopr_debug_wait_timeout(int32_t timeout_ms);

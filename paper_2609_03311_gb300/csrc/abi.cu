@@ -205,8 +205,8 @@ dopr_status alloc_chunk_buffers(Model* m, int cap) {
   STATUS_TRY(dev_alloc(&w.r_s, (size_t)cap * c.hidden));
   STATUS_TRY(dev_alloc(&w.ss_s, sums));
   const size_t few_groups = (size_t)GEMM_FEW_MAX_ROWS / 32 * (c.hidden / 128);
-  w.n_ss_count = (int)few_groups;
-  STATUS_TRY(dev_alloc(&w.ss_count, few_groups));
+  w.n_ss_count = (int)few_groups + 1;  // and the gate word
+  STATUS_TRY(dev_alloc(&w.ss_count, few_groups + 1));
   STATUS_TRY(dev_alloc(&w.ss_chunks, few_groups * 1024));
   const bool ok = make_gemm_operand_a(&w.tm_xn, w.xn, c.hidden, cap) &&
                   make_gemm_operand_a(&w.tm_o, w.o, m->o_dim, cap) && make_gemm_operand_a(&w.tm_act, w.act, c.ffn, cap);
@@ -639,7 +639,14 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
   const int mpad = ((s->max_m + 63) / 64) * 64;
   const int sms = m->num_sms;
   const bool scoring = !build && !sel;
-  auto gemm_launches = [&](int epi, int M, int N, int K) { return gemm_plan(epi, M, N, K, sms).wide_rows > 0 ? 2 : 1; };
+  // one projection: its launch, or two of a split product (gemm_plan)
+  int products = 0;
+  auto project = [&](KernelKind kind, int epi, const GemmOperandA& a, const GemmOperandB& b, GemmParams& p,
+                     const std::pair<double, double>& cost) {
+    p.gate_number = ++products;
+    const int launches = gemm_plan(epi, p.M, p.N, p.K, sms).wide_rows > 0 ? 2 : 1;
+    return prof_launch(m, kind, launches, cost.first, cost.second, st, [&] { return launch_gemm(epi, a, b, p, sms, st); });
+  };
   auto gemm_cost = [](double M, double N, double K, double out_bytes) {
     return std::make_pair(2.0 * M * N * K, (M * K + N * K) * 2.0 + out_bytes);
   };
@@ -680,6 +687,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
     base.err = w.err;
     base.ss_chunks = w.ss_chunks;
     base.ss_count = w.ss_count;
+    base.gate = w.ss_count + w.n_ss_count - 1;
     const int32_t np = s1 - s0;
     double last_keys = 0.0;  // keys seen by the score-token rows alone
     for (int32_t sp = s0; sp < s1; ++sp)
@@ -740,8 +748,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
       pq.k_norm = m->k_norm + (size_t)l * HEAD_DIM;
       pq.q_cols = Hq * HEAD_DIM;
       pq.k_cols = Hkv * HEAD_DIM;
-      CUDA_TRY(prof_launch(m, K_GEMM_QKV, gemm_launches(EPI_QKV, Tc, m->qkv_dim, H), qkv.first, qkv.second, st,
-                           [&] { return launch_gemm(EPI_QKV, w.tm_xn, m->tm_qkv[l], pq, sms, st); }));
+      CUDA_TRY(project(K_GEMM_QKV, EPI_QKV, w.tm_xn, m->tm_qkv[l], pq, qkv));
       if (build) {  // this layer's keys and values are the document's stored prefix states
         CUDA_TRY(prof_launch(m, K_PREFIX_STORE, 1, 0.0, T * 2.0 * Hkv * HEAD_DIM * 2 * 2, st, [&] {
           return launch_prefix_store(w.qkv, m->qkv_dim, Tc, t0, Hq, Hkv, w.tok_pair, w.tok_pos, w.sorted_slot,
@@ -841,8 +848,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
       po.ss_out_parts = parts;
       po.ss_pre = ss_pre;
       po.ss_pre_parts = ss_pre_parts;
-      CUDA_TRY(prof_launch(m, K_GEMM_O, gemm_launches(EPI_RESID_ADD, rows, H, m->o_dim), last ? op_last.first : op.first, last ? op_last.second : op.second, st,
-                           [&] { return launch_gemm(EPI_RESID_ADD, w.tm_o, m->tm_o[l], po, sms, st); }));
+      CUDA_TRY(project(K_GEMM_O, EPI_RESID_ADD, w.tm_o, m->tm_o[l], po, last ? op_last : op));
       GemmParams pg = base;  // gate/up + MLP-norm row scale + SwiGLU
       pg.M = rows;
       pg.N = 2 * F;
@@ -853,8 +859,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
       pg.ss_parts = parts;
       pg.ss_pre = ss_pre;
       pg.ss_pre_parts = ss_pre_parts;
-      CUDA_TRY(prof_launch(m, K_GEMM_GATE_UP, gemm_launches(EPI_SWIGLU, rows, 2 * F, H), last ? gu_last.first : gu.first, last ? gu_last.second : gu.second,
-                           st, [&] { return launch_gemm(EPI_SWIGLU, w.tm_xn, m->tm_gu[l], pg, sms, st); }));
+      CUDA_TRY(project(K_GEMM_GATE_UP, EPI_SWIGLU, w.tm_xn, m->tm_gu[l], pg, last ? gu_last : gu));
       GemmParams pd = base;  // down projection + residual, emits the next attention norm's operand
       pd.M = rows;
       pd.N = H;
@@ -869,8 +874,7 @@ dopr_status run_layers(Model* m, Store* s, const Plan& plan, float* d_scores, cu
         pd.ss_pre = w.ss_m;  // the MLP norm of this layer
         pd.ss_pre_parts = parts;
       }
-      CUDA_TRY(prof_launch(m, K_GEMM_DOWN, gemm_launches(EPI_RESID_ADD, rows, H, F), last ? dn_last.first : dn.first, last ? dn_last.second : dn.second, st,
-                           [&] { return launch_gemm(EPI_RESID_ADD, w.tm_act, m->tm_down[l], pd, sms, st); }));
+      CUDA_TRY(project(K_GEMM_DOWN, EPI_RESID_ADD, w.tm_act, m->tm_down[l], pd, last ? dn_last : dn));
     }
     if (scoring) {
       if (m->mlp_width > 0) {
@@ -1710,9 +1714,11 @@ dopr_status dopr_debug_gemm(int32_t M, int32_t N, int32_t K, const void* A, cons
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  int* err = nullptr;
-  CUDA_TRY(cudaMalloc(&err, sizeof(int)));
-  cudaMemsetAsync(err, 0, sizeof(int), st);
+  int* err = nullptr;  // and the gate word
+  CUDA_TRY(cudaMalloc(&err, 64 * sizeof(int)));
+  // (whatever wrote A and B on this stream is complete before the memset, and so before a launch
+  // that copies from B ahead of its wait)
+  cudaMemsetAsync(err, 0, 64 * sizeof(int), st);
   GemmParams gp{};
   gp.M = M;
   gp.N = N;
@@ -1720,6 +1726,8 @@ dopr_status dopr_debug_gemm(int32_t M, int32_t N, int32_t K, const void* A, cons
   gp.out = out;
   gp.ld_out = epilogue == EPI_SWIGLU ? N / 2 : N;
   gp.err = err;
+  gp.gate = err + 32;
+  gp.gate_number = 1;
   cudaError_t e = launch_gemm(epilogue, ta, tb, gp, sms, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   int h = 0;
@@ -1754,15 +1762,15 @@ dopr_status dopr_debug_wait_timeout(int32_t timeout_ms) {
   g_last_error.clear();
   if (timeout_ms <= 0 || timeout_ms > 10000) return fail(DOPR_ERR_INVALID_ARG, "timeout_ms in (0, 10000]");
   int* err = nullptr;
-  CUDA_TRY(cudaMalloc(&err, sizeof(int)));
-  cudaMemset(err, 0, sizeof(int));
+  CUDA_TRY(cudaMalloc(&err, 3 * sizeof(int)));
+  cudaMemset(err, 0, 3 * sizeof(int));
   cudaError_t e = launch_wait_timeout_probe(err, (uint64_t)timeout_ms * 1000000ull, 0);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
-  int h = 0;
-  if (e == cudaSuccess) e = cudaMemcpy(&h, err, sizeof(int), cudaMemcpyDeviceToHost);
+  int h[3] = {};
+  if (e == cudaSuccess) e = cudaMemcpy(h, err, sizeof(h), cudaMemcpyDeviceToHost);
   cudaFree(err);
   if (e != cudaSuccess) return fail(DOPR_ERR_CUDA, "probe failed: %s", cudaGetErrorString(e));
-  return map_device_error(h);
+  return map_device_error(h[0] & h[1]);  // both waits gave up
 }
 
 }  // extern "C"

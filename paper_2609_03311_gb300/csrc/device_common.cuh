@@ -77,6 +77,12 @@ __device__ __forceinline__ int ld_volatile(const int* p) { return *reinterpret_c
 // plain pointers (never __ldg or const __restrict__, whose loads may go through the non-coherent
 // path and be moved above the wait); those are for weights, gains, the RoPE table and whatever
 // was copied or finished before the first dependent launch.
+//
+// One kernel does not wait so at its start: the few-row GEMM that runs beside the wide one of the
+// same product (GemmParams::beside) would wait for that launch to end.  It reads only what the
+// wide launch waited for, and a gate hands that on: a thread of the wide launch that has returned
+// from its own pdl_wait() opens the gate with a release, every warp beside passes it with an
+// acquire before it reads, and the copying warp adds a fence to the proxy that its copies read by.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -139,6 +145,34 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
     }
   }
 }
+
+// The gate: a word that its opener sets to the launch's number (0 is none).
+__device__ __forceinline__ void gate_open(int* gate, int number) {
+  asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(gate), "r"(number) : "memory");
+}
+// A converged warp passes the gate: lane 0 acquires, the other lanes' accesses follow by the
+// warp's barrier.  Bounded like mbar_wait; false in all lanes when it gave up.
+__device__ __forceinline__ bool gate_wait_warp(const int* gate, int number, int* err, uint64_t timeout_ns) {
+  bool ok = true;
+  if ((threadIdx.x & 31) == 0) {
+    const uint64_t t0 = globaltimer_ns();
+    for (;;) {
+      int v;
+      asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(gate) : "memory");
+      if (v == number) break;
+      if ((ld_volatile(err) & DEV_ERR_TIMEOUT) || globaltimer_ns() - t0 > timeout_ns) {
+        atomicOr(err, DEV_ERR_TIMEOUT);
+        ok = false;
+        break;
+      }
+    }
+  }
+  __syncwarp();
+  return __all_sync(0xffffffffu, ok) != 0;
+}
+// Ahead of copies (async proxy) of global memory that other threads wrote with plain stores and
+// this one has acquired.
+__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
 // True in one lane of the (converged) warp.  Code that only this lane runs, inside a loop the
 // whole warp runs, leaves the loop's state warp-uniform.

@@ -154,7 +154,7 @@ struct Workspace {
   // the call's device error word (RESULT_HEAD ints), then its scores
   int* err = nullptr;
   float* scores = nullptr;
-  int* ss_count = nullptr;     // the few-row GEMMs' chunk counts, 0 when a pass starts
+  int* ss_count = nullptr;     // the few-row GEMMs' chunk counts, then their gate word; 0 when a pass starts
   int n_ss_count = 0;
   float* ss_chunks = nullptr;  // [GEMM_FEW_MAX_ROWS / 32][H/128][1024]
   // pinned host staging
@@ -279,8 +279,11 @@ struct GemmParams {
   const bf16* k_norm;
   int q_cols, k_cols;
   // k_gemm_few: rows [row_begin, M) only; beside: the launch before is the wide one of the same
-  // product's first rows, which is waited for at the end alone
+  // product's first rows, which is waited for at the end alone.  The wide one opens the gate
+  // (gate_open, device_common.cuh) with the product's number in its pass, from 1 on
   int row_begin, beside;
+  int* gate;
+  int gate_number;
   int* err;
   uint64_t timeout_ns;
 };

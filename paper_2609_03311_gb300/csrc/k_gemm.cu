@@ -605,9 +605,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   cluster_sync();  // both CTAs' barriers exist before either addresses the other's
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  // in this order: a few-row launch beside this one (GemmParams::beside) may take it that whatever
-  // this kernel waited for is done
+  // in this order: a few-row launch beside this one (GemmParams::beside) starts once this kernel's
+  // blocks have triggered, and the gate hands it what this kernel waited for
   pdl_wait();
+  if (p.gate && blockIdx.x == 0 && threadIdx.x == 0) gate_open(p.gate, p.gate_number);
   pdl_trigger();
   {
     // the MMAs write both CTAs' TMEM at the leader's address: both allocations must agree
@@ -799,9 +800,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_trigger();
-  // (the producer starts on the weights first; beside the wide launch of the same product there is
-  // nothing to wait for but that launch itself, at the end)
-  if (warp != 0 && !p.beside) pdl_wait();
+  // (the producer starts on the weights first)
+  auto wait_for_inputs = [&] {
+    if (!p.beside)
+      pdl_wait();
+    else if (gate_wait_warp(p.gate, p.gate_number, p.err, p.timeout_ns))
+      fence_proxy_async_global();
+    else
+      total = 0;  // gave up: no tile runs
+  };
+  if (warp != 0) wait_for_inputs();
   {
     uint32_t other;  // as in k_gemm_pair: both allocations must agree
     asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(other) : "r"(mapa_shared(smem_u32(tmem_slot), rank ^ 1u)));
@@ -836,7 +844,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     if (pair < total)
       for (; ahead < min(stages, k_steps); ++ahead)
         if (one) load_weights(ahead, weight_row(pair / m_tiles), ahead);
-    if (!p.beside) pdl_wait();
+    wait_for_inputs();
+    if (total == 0 && ahead > 0) ok = false;  // gave up with weights on their way
     for (int t = pair; t < total && ok; t += n_pairs) {
       const int nb = t / m_tiles, row = p.row_begin + (t % m_tiles) * 2 * R + static_cast<int>(rank) * R;
       const int brow = weight_row(nb);
@@ -1081,9 +1090,10 @@ cudaError_t launch_gemm(int epi, const GemmOperandA& A, const GemmOperandB& B, c
     if (e != cudaSuccess) return e;
     p.M = params.M;
     p.row_begin = g.wide_rows;
-    p.beside = 1;
+    p.beside = p.gate != nullptr;  // without a gate it waits for the wide launch like any other kernel
     return launch_one(epi, A, B, p, GemmPlan{true, g.rows, g.cols, 0}, num_sms, st);
   }
+  p.gate = nullptr;
   return launch_one(epi, A, B, p, g, num_sms, st);
 }
 

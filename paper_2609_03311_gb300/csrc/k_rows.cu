@@ -347,8 +347,13 @@ __global__ void k_prefix_store(const f16* qkv, int ld_qkv, int T, int t0, int Hq
   reinterpret_cast<uint2*>(pool + row * HEAD_DIM)[lane] = src[lane];
 }
 
-// Test kernel: one bounded wait on an mbarrier that is never completed.
+// Test kernel: a bounded wait on an mbarrier that is never completed (block 0, error word err[0])
+// and one at a gate that is never opened (block 1, err[1]; the gate is err[2]).
 __global__ void k_wait_timeout_probe(int* err, uint64_t timeout_ns) {
+  if (blockIdx.x == 1) {
+    gate_wait_warp(err + 2, 1, err + 1, timeout_ns);
+    return;
+  }
   __shared__ uint64_t bar;
   const uint32_t b = smem_u32(&bar);
   if (threadIdx.x == 0) {
@@ -432,7 +437,7 @@ cudaError_t launch_prefix_store(const f16* qkv, int ld_qkv, int T, int t0, int H
 }
 
 cudaError_t launch_wait_timeout_probe(int* err, uint64_t timeout_ns, cudaStream_t st) {
-  k_wait_timeout_probe<<<1, 32, 0, st>>>(err, timeout_ns);
+  k_wait_timeout_probe<<<2, 32, 0, st>>>(err, timeout_ns);
   return cudaGetLastError();
 }
 

@@ -82,3 +82,17 @@ def test_waits_before_work_of_the_whole_warp_are_the_whole_warps():
         single = list(_call_args(_source(name), "mbar_wait")) + list(_call_args(_source(name), "mbar_wait_cluster"))
         allowed = {"k_attn.cu": 2, "k_rows.cu": 1, "k_gemm.cu": 1}.get(name, 0)  # k_gemm: inside wait_all_lanes
         assert len(single) == allowed, (name, single)
+
+
+def test_the_few_row_launch_beside_a_wide_one_passes_its_gate_before_it_reads():
+    # The launch beside does not wait for the kernel before it until its end; what that kernel waited for reaches it
+    # through the gate: a release after the wide launch's wait, an acquire and a proxy fence before the first read.
+    bodies = {k: body for k, _, body in _kernels(_source("k_gemm.cu"))}
+    wide, few = bodies["k_gemm_pair"], bodies["k_gemm_few"]
+    assert wide.index("pdl_wait()") < wide.index("gate_open(") < wide.index("pdl_trigger()")
+    wait = _block(few, few.index("auto wait_for_inputs"))
+    assert "gate_wait_warp(" in wait and "fence_proxy_async_global()" in wait and "pdl_wait()" in wait
+    assert few.count("pdl_wait()") == wait.count("pdl_wait()") + 1  # the other one carries completion over, at the end
+    first, producer = few.index("if (warp != 0) wait_for_inputs();"), few.index("if (warp == 0) {")
+    second = few.index("wait_for_inputs();", producer)
+    assert second < few.index("&tmA, mapa_shared") and first < few.index("epilogue_prefetch<")
