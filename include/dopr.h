@@ -354,8 +354,9 @@ DOPR_API dopr_status dopr_debug_wait_timeout(int32_t timeout_ms);
  * process exits.  The first call on a device looks the array's device address
  * up (cudaGetSymbolAddress) with that device current; make that first call
  * before any stream capture.  Every call shares the one array: calls that
- * overlap on the GPU (other streams, other host threads) race and must be
- * serialised by the caller.  The call runs on cuda_stream (NULL = default)
+ * overlap on the GPU (on different streams) race and must be serialised by
+ * the caller; host threads may call on one stream, each call returns its own
+ * status.  The call runs on cuda_stream (NULL = default)
  * and returns after its results are written (it synchronises the stream).
  * Errors: INVALID_ARG, UNKNOWN_DOC, INCOMPLETE, UNSUPPORTED, CUDA.
  */

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -82,8 +83,12 @@ struct Store {
   int32_t max_m = 0;
   CUtensorMap tm_pool{};
   bool tm_pool_ok = false;
-  int* h_err = nullptr;  // pinned: the ordering entry point's error word
+  // pinned error words of the ordering entry point: a call takes one (a bit of h_err_taken) for as
+  // long as it runs, since calls of several host threads may wait on one stream
+  int* h_err = nullptr;  // [STORE_ERR_WORDS]
+  mutable std::atomic<uint64_t> h_err_taken{0};
 };
+constexpr int STORE_ERR_WORDS = 64;
 
 // GEMM epilogues.
 enum GemmEpi : int { EPI_STORE = 0, EPI_RESID_ADD = 1, EPI_SWIGLU = 2, EPI_QKV = 3 };
@@ -395,8 +400,8 @@ struct PackArgs {
   int32_t* tok_pos;
   int32_t* tok_pair;
   int* err;           // set to 0 first
-  // pinned host copies that the ordering kernel writes itself: the error word after validation,
-  // the offsets and slots (null: not wanted); and ints it clears
+  // pinned host copies that the ordering kernel writes itself (null: not wanted): the error word
+  // after validation, the offsets and slots; and ints it clears
   int* h_err;
   int32_t* h_tok_off;
   int32_t* h_sorted_slot;

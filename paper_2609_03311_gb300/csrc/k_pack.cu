@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_pack_order(PackArgs a, int do
   if (flags) atomicOr(a.err, flags);
   meet();
   const int found = ld_volatile(a.err);  // the same word for the whole cluster
-  if (rank == 0 && tid == 0) *a.h_err = found;
+  if (rank == 0 && tid == 0 && a.h_err) *a.h_err = found;
   if (found & INPUT_ERRORS) return;
 
   // ---- stable sort by doc id; the order goes to perm, by way of sorted_slot

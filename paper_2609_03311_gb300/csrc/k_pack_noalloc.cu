@@ -78,6 +78,31 @@ dopr_status device_error_status(int e) {
   return DOPR_OK;
 }
 
+// A pinned error word of the store for the length of one call; null when all are taken.
+class ErrorWord {
+ public:
+  explicit ErrorWord(const Store& s) : taken_(s.h_err_taken) {
+    uint64_t t = taken_.load();
+    while (~t) {
+      const uint64_t free = ~t & (t + 1);  // the lowest clear bit
+      if (taken_.compare_exchange_weak(t, t | free)) {
+        bit_ = free;
+        word_ = s.h_err + __builtin_ctzll(free);
+        return;
+      }
+    }
+  }
+  ~ErrorWord() { taken_ &= ~bit_; }
+  ErrorWord(const ErrorWord&) = delete;
+  ErrorWord& operator=(const ErrorWord&) = delete;
+  int* word() const { return word_; }
+
+ private:
+  std::atomic<uint64_t>& taken_;
+  uint64_t bit_ = 0;
+  int* word_ = nullptr;
+};
+
 }  // namespace
 }  // namespace dopr
 
@@ -136,13 +161,17 @@ extern "C" dopr_status dopr_pack_order_noalloc(const dopr_store* store, int32_t 
   a.perm = perm;
   a.sorted_slot = scratch + NOALLOC_MAX_PAIRS;
   a.tok_off = tok_off;
-  a.err = err;  // cleared and copied to the store's pinned word by the kernel
-  a.h_err = store->h_err;
+  // cleared by the kernel and copied by it to this call's pinned word; without one, by a copy
+  const ErrorWord word(*store);
+  int found = 0;
+  a.err = err;
+  a.h_err = word.word();
   e = launch_pack_order(a, stream);
+  if (e == cudaSuccess && !a.h_err) e = cudaMemcpyAsync(&found, err, sizeof(int), cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) {
     set_last_error_message(std::string("CUDA error: ") + cudaGetErrorString(e));
     return DOPR_ERR_CUDA;
   }
-  return device_error_status(*store->h_err);
+  return device_error_status(a.h_err ? *a.h_err : found);
 }

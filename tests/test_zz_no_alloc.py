@@ -93,3 +93,37 @@ def test_noalloc_limits_and_errors(rig):
     perm, tok_off = _noalloc(store, qo2, docs2)
     np.testing.assert_array_equal(perm, want["perm"])
     np.testing.assert_array_equal(tok_off, want["tok_off"])
+
+
+def test_noalloc_status_is_the_calls_own_with_threads_on_one_stream(rig):
+    # Calls of several threads on one stream do not overlap on the GPU; each must return its own status although the
+    # next call's kernel may be done before the first thread looks.
+    import threading
+
+    cfg, model, store, doc_m = rig
+    stream = torch.cuda.Stream()
+    qo, _, docs = _batch(doc_m, 300, 8)
+    bad = docs.copy()
+    bad[17] = 5  # not stored
+    wrong = []
+
+    def work(ids, want):
+        perm = torch.zeros(300, dtype=torch.int32, device="cuda")
+        tok_off = torch.zeros(301, dtype=torch.int32, device="cuda")
+        q, d = torch.tensor(qo, device="cuda"), torch.tensor(ids, device="cuda")
+        torch.cuda.synchronize()
+        for _ in range(2000):
+            try:
+                dopr.pack_order_noalloc(store, q, d, perm, tok_off, stream=stream)
+                got = dopr.OK
+            except dopr.DoprError as e:
+                got = e.status
+            if got != want:
+                wrong.append((want, got))
+
+    threads = [threading.Thread(target=work, args=a) for a in ((docs, dopr.OK), (bad, dopr.ERR_UNKNOWN_DOC)) * 2]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong, (len(wrong), wrong[:4])
