@@ -322,6 +322,18 @@ DOPR_API dopr_status dopr_debug_gemm(int32_t M, int32_t N, int32_t K, const void
                             int32_t epilogue, void *cuda_stream);
 
 /*
+ * The launch or launches a projection of M rows takes on num_sms SMs (host
+ * arithmetic only: usable without a GPU), for testing.  epilogue as in
+ * dopr_debug_gemm, or 3 for the QKV projection.
+ *   out [4] int32: {1 when few-row tiles take every row, rows per CTA of the
+ *       pair, columns, W}; W > 0: the first W rows in wide tiles, the others
+ *       in few-row tiles of that size by a launch beside.
+ * Errors: INVALID_ARG, UNSUPPORTED (K % 64, N % 256).
+ */
+DOPR_API dopr_status dopr_debug_gemm_plan(int32_t epilogue, int32_t M, int32_t N, int32_t K, int32_t num_sms,
+                                          int32_t *out);
+
+/*
  * Runs one test kernel whose bounded waits, one on a barrier that nothing
  * completes and one at a gate that nothing opens, must give up after about
  * timeout_ms milliseconds.  Returns DOPR_ERR_TIMEOUT when the kernel reported

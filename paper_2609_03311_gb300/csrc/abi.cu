@@ -1737,6 +1737,19 @@ dopr_status dopr_debug_gemm(int32_t M, int32_t N, int32_t K, const void* A, cons
   return map_device_error(h);
 }
 
+dopr_status dopr_debug_gemm_plan(int32_t epilogue, int32_t M, int32_t N, int32_t K, int32_t num_sms, int32_t* out) {
+  g_last_error.clear();
+  if (epilogue < 0 || epilogue > EPI_QKV || M <= 0 || N <= 0 || K <= 0 || num_sms <= 0 || !out)
+    return fail(DOPR_ERR_INVALID_ARG, "bad gemm plan args");
+  if (K % GEMM_BK || N % GEMM_BN) return fail(DOPR_ERR_UNSUPPORTED, "K % 64 and N % 256 must be 0");
+  const GemmPlan g = gemm_plan(epilogue, M, N, K, num_sms);
+  out[0] = g.few;
+  out[1] = g.rows;
+  out[2] = g.cols;
+  out[3] = g.wide_rows;
+  return DOPR_OK;
+}
+
 dopr_status dopr_profile_enable(dopr_model* m, int32_t enable) {
   g_last_error.clear();
   if (!m) return fail(DOPR_ERR_INVALID_ARG, "model is NULL");

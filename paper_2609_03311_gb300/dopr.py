@@ -25,7 +25,7 @@ STATUS_NAMES = ["OK", "INVALID_ARG", "UNKNOWN_DOC", "INCOMPLETE", "OUT_OF_MEMORY
 (W_EMBED, W_ATTN_NORM, W_Q, W_K, W_V, W_Q_NORM, W_K_NORM, W_O, W_MLP_NORM, W_GATE, W_UP, W_DOWN, W_FINAL_NORM,
  W_SCORE_HEAD) = range(14)
 
-EPI_STORE, EPI_RESID_ADD, EPI_SWIGLU = 0, 1, 2
+EPI_STORE, EPI_RESID_ADD, EPI_SWIGLU, EPI_QKV = 0, 1, 2, 3  # EPI_QKV: gemm_plan only
 
 
 class DoprError(RuntimeError):
@@ -72,6 +72,7 @@ def load():
         "dopr_score": ([P, P, i32, P, P, P, P, P, i32], i32),
         "dopr_debug_pack_plan": ([P, P, i32, P, P, P, P, P, P, P, P], i32),
         "dopr_debug_gemm": ([i32, i32, i32, P, P, P, i32, P], i32),
+        "dopr_debug_gemm_plan": ([i32, i32, i32, i32, i32, P], i32),
         "dopr_debug_wait_timeout": ([i32], i32),
         "dopr_pack_order_noalloc": ([P, i32, P, P, P, P, P], i32),
         "dopr_profile_enable": ([P, i32], i32),
@@ -317,6 +318,14 @@ def gemm(A: torch.Tensor, B: torch.Tensor, epilogue: int = EPI_STORE, out: torch
     st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     _check(load().dopr_debug_gemm(M, N, K, _ptr(A), _ptr(B), _ptr(out), epilogue, st))
     return out
+
+
+def gemm_plan(epilogue: int, M: int, N: int, K: int, num_sms: int = 152) -> dict:
+    """The tiles a projection of M rows takes (host-only, no GPU): few (narrow tiles take every row), rows per CTA and
+    cols of the narrow tile, wide_rows (rows in wide tiles when the others go to a narrow launch beside them, else 0)."""
+    out = (ctypes.c_int32 * 4)()
+    _check(load().dopr_debug_gemm_plan(int(epilogue), int(M), int(N), int(K), int(num_sms), out))
+    return {"few": bool(out[0]), "rows": out[1], "cols": out[2], "wide_rows": out[3]}
 
 
 def pack_order_noalloc(store: Store, q_offsets: torch.Tensor, doc_ids: torch.Tensor, perm: torch.Tensor,

@@ -373,12 +373,16 @@ def test_bounded_wait_gives_up_and_context_survives():
     assert torch.allclose(out.float(), (A.float() @ B.float().T), rtol=1e-2, atol=1e-1)
 
 
+def _plan(epi, M, N, K):
+    return dopr.gemm_plan(epi, M, N, K, torch.cuda.get_device_properties(0).multi_processor_count)
+
+
 @pytest.mark.parametrize("N,K", [(256, 64), (512, 320), (1024, 3072), (2560, 1024), (4096, 2048),
                                  (9728, 320)])  # 9,728: gate/up takes 128-column tiles of 64 rows a CTA too
 def test_gemm_few_rows_match_wide_tiles_bit_for_bit(N, K):
-    # Launches of few rows take narrow tiles (64 or 128 columns, 32 to 128 rows a CTA), chosen by size; more than
-    # 1,024 rows always take the wide ones.  A row's K order is the same in all, so its result is too.  K = 320 is not
-    # a whole number of the narrow kernel's 128- or 256-element stages.
+    # Launches of few rows take narrow tiles (64 or 128 columns, 32 to 128 rows a CTA), chosen by size; these 1,300 rows
+    # all take the wide ones.  A row's K order is the same in all, so its result is too.  K = 320 is not a whole number
+    # of the narrow kernel's 128- or 256-element stages.
     g = torch.Generator(device="cuda").manual_seed(N + K)
     A = torch.randn(1300, K, device="cuda", generator=g).to(torch.float16)
     B = (0.05 * torch.randn(N, K, device="cuda", generator=g)).to(torch.float16)
@@ -387,8 +391,9 @@ def test_gemm_few_rows_match_wide_tiles_bit_for_bit(N, K):
     def run(M, epi):
         return dopr.gemm(A[:M].contiguous(), B, epi, out=R[:M].clone() if epi == dopr.EPI_RESID_ADD else None)
 
-    # (with N = 4,096 the 1,300 rows are themselves 1,024 in wide tiles and the rest in a few-row launch beside them)
     for epi in (dopr.EPI_STORE, dopr.EPI_RESID_ADD, dopr.EPI_SWIGLU):
+        plan = _plan(epi, 1300, N, K)
+        assert not plan["few"] and plan["wide_rows"] == 0 and _plan(epi, 33, N, K)["few"]
         wide = run(1300, epi)
         for M in (1, 31, 32, 33, 64, 65, 127, 128, 129, 255, 256, 257, 640, 1023, 1024):
             assert torch.equal(run(M, epi), wide[:M]), (epi, M)
@@ -429,38 +434,60 @@ def test_pack_order_at_digit_and_block_edges(max_doc, ids):
     store.close()
 
 
-@pytest.mark.parametrize("M,N,K", [(1300, 4096, 2048), (1025, 2560, 1024), (2432, 4096, 1024), (5650, 2560, 1024)])
+@pytest.mark.parametrize("M,N,K", [(1300, 4096, 4096), (1450, 4096, 4096), (2432, 4096, 4096), (3800, 4096, 4096),
+                                   (5650, 2560, 4096)])
 def test_gemm_rows_beside_the_wide_tiles(M, N, K):
     # Sizes whose last round of wide tiles is nearly empty: its rows go to a few-row launch that starts beside the wide
-    # one.  Both sides of the boundary against the same product of fewer rows and against the reference.
+    # one (32, 64, 96 and 128 rows a CTA, 64 and 128 columns among these).  Both sides of the boundary against the same
+    # product of fewer rows, which is not split, and against the reference.
     g = torch.Generator(device="cuda").manual_seed(M)
     A = torch.randn(M, K, device="cuda", generator=g).to(torch.float16)
     B = (0.05 * torch.randn(N, K, device="cuda", generator=g)).to(torch.float16)
     R = torch.randn(M, N, device="cuda", generator=g)
-    got = dopr.gemm(A, B, dopr.EPI_RESID_ADD, out=R.clone())
-    for lo in range(0, M, 1024):  # 1,024 rows and fewer are never split
-        hi = min(M, lo + 1024)
-        part = dopr.gemm(A[lo:hi].contiguous(), B, dopr.EPI_RESID_ADD, out=R[lo:hi].clone())
-        assert torch.equal(got[lo:hi], part), lo
+
+    def run(lo, hi, epi):
+        return dopr.gemm(A[lo:hi].contiguous(), B, epi, out=R[lo:hi].clone() if epi == dopr.EPI_RESID_ADD else None)
+
+    for epi in (dopr.EPI_STORE, dopr.EPI_SWIGLU, dopr.EPI_RESID_ADD):
+        assert 0 < _plan(epi, M, N, K)["wide_rows"] < M
+        got = run(0, M, epi)
+        for lo in range(0, M, 512):
+            hi = min(M, lo + 512)
+            assert _plan(epi, hi - lo, N, K)["wide_rows"] == 0
+            assert torch.equal(got[lo:hi], run(lo, hi, epi)), (epi, lo)
     ref = _ref_gemm(A, B) + R.double()
     scale = (A.double().abs() @ B.double().abs().T) + R.double().abs()
-    assert torch.all((got.double() - ref).abs() <= 1e-5 * scale + 1e-6)
+    assert torch.all((got.double() - ref).abs() <= 1e-5 * scale + 1e-6)  # got: the residual sum
 
 
-@pytest.mark.parametrize("heads,hidden,ffn", [((2, 1), 256, 512), ((4, 2), 256, 512), ((16, 8), 4096, 2048)])
-def test_large_batches_match_their_parts_bit_for_bit(heads, hidden, ffn):
+@pytest.mark.parametrize("heads,hidden,ffn,n_pairs", [((2, 1), 256, 512, 40), ((4, 2), 256, 512, 40),
+                                                      ((16, 8), 4096, 2048, 40), ((32, 8), 4096, 4096, 33)])
+def test_large_batches_match_their_parts_bit_for_bit(heads, hidden, ffn, n_pairs):
     # More than 1,024 tokens take the wide tiles.  Two q heads and one kv head leave a tile of one rotated and one plain
-    # head; hidden 4,096 puts the last rows of O and down, with their sums of squares, into a launch beside the wide one.
-    # Parts of the batch take few-row tiles throughout.
+    # head.  Hidden 4,096 splits products: at K 2,048 (ffn) QKV and gate/up, with 32 heads and ffn 4,096 the first
+    # layer's O and down, whose last rows' sums of squares and next norm's operand then come from the launch beside.
+    # Parts of the batch take few-row tiles or unsplit wide ones.
     shape = synth.ModelShape("wide-2l", n_layers=2, hidden=hidden, n_q_heads=heads[0], n_kv_heads=heads[1],
                              head_dim=128, ffn=ffn, vocab=300)
     rig = Rig(shape, {0: 64, 1: 17}, seed=21)
-    pairs = synth.random_pairs(40, 2, 24, 48, shape.vocab, seed=21)
+    pairs = synth.random_pairs(n_pairs, 2, 24, 48, shape.vocab, seed=21)
     qo, qt, di = pairs["q_offsets"], pairs["q_tokens"], pairs["doc_ids"]
     lens = np.diff(qo)
-    assert lens.sum() + 40 > 1024 + 64
+    T = int(lens.sum()) + n_pairs
+    assert T > 1024 + 64
+    dopr.profile_enable(rig.model, False)  # clears the launch counts
     base = rig.score(pairs)
-    for sel in (np.arange(0, 40, 2), np.arange(30, 40), np.array([3])):
+    launches = {k: v["launches"] for k, v in dopr.profile_read(rig.model).items()}
+    split = {"gemm_qkv": (dopr.EPI_QKV, (heads[0] + 2 * heads[1]) * 128, hidden, 2),  # of both layers
+             "gemm_o": (dopr.EPI_RESID_ADD, hidden, heads[0] * 128, 1),  # the last layer's has a row a pair
+             "gemm_gate_up": (dopr.EPI_SWIGLU, 2 * ffn, hidden, 1),
+             "gemm_down": (dopr.EPI_RESID_ADD, hidden, ffn, 1)}
+    split = {k: layers if _plan(epi, T, N, K)["wide_rows"] else 0 for k, (epi, N, K, layers) in split.items()}
+    assert {k: launches[k] - 2 for k in split} == split
+    if hidden == 4096:
+        want = ("gemm_qkv", "gemm_gate_up") if ffn == 2048 else ("gemm_o", "gemm_gate_up", "gemm_down")
+        assert {k for k, n in split.items() if n} == set(want)
+    for sel in (np.arange(0, n_pairs, 2), np.arange(n_pairs - 10, n_pairs), np.array([3])):
         part = {"q_offsets": np.concatenate([[0], np.cumsum(lens[sel])]).astype(np.int32),
                 "q_tokens": np.concatenate([qt[qo[p]:qo[p + 1]] for p in sel]).astype(np.int32), "doc_ids": di[sel]}
         np.testing.assert_array_equal(rig.score(part), base[sel])
