@@ -441,42 +441,39 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
   } else {  // EPI_SWIGLU: the tile's first half of the columns gate, its second half up of the same outputs
     f16* out = reinterpret_cast<f16*>(p.out);
     const float rs = pre.scale;
-    constexpr int OUTS = BNT / 2;                  // outputs of the tile
-    constexpr int MINE = OUTS >= 64 ? OUTS / 2 : 32;  // of this warp (with 32 in all, part 0 takes them)
-    if (part * MINE >= OUTS) {
-      release();
-    } else {
-      const int c = part * MINE;
+    constexpr int OUTS = BNT / 2;   // outputs of the tile
+    constexpr int MINE = OUTS / 2;  // of this warp
+    static_assert(BNT >= 128, "two chunks of 32 outputs or more");
+    const int c = part * MINE;
 #pragma unroll
-      for (int half = 0; half < MINE / 32; ++half) {
-        uint32_t g[32], u[32];
-        tmem_ld32(taddr + c + 32 * half, g);
-        tmem_ld32(taddr + (HALF ? MINE : OUTS) + c + 32 * half, u);
-        tmem_ld_wait();
-        if (half + 1 == MINE / 32) release();
-        float row_most = 0.f;
+    for (int half = 0; half < MINE / 32; ++half) {
+      uint32_t g[32], u[32];
+      tmem_ld32(taddr + c + 32 * half, g);
+      tmem_ld32(taddr + (HALF ? MINE : OUTS) + c + 32 * half, u);
+      tmem_ld_wait();
+      if (half + 1 == MINE / 32) release();
+      float row_most = 0.f;
 #pragma unroll
-        for (int c4 = 0; c4 < 4; ++c4) {  // eight outputs: one 16-byte chunk
-          uint32_t o[4];
+      for (int c4 = 0; c4 < 4; ++c4) {  // eight outputs: one 16-byte chunk
+        uint32_t o[4];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int j = c4 * 8 + 2 * k;
-            const float a0 = silu_f(__uint_as_float(g[j]) * rs) * (__uint_as_float(u[j]) * rs);
-            const float a1 = silu_f(__uint_as_float(g[j + 1]) * rs) * (__uint_as_float(u[j + 1]) * rs);
-            track_range(row_most, a0);
-            track_range(row_most, a1);
-            o[k] = pack_f16x2(a0, a1);
-          }
-          *xs_chunk(xs, lane, 4 * half + c4) = make_uint4(o[0], o[1], o[2], o[3]);
+        for (int k = 0; k < 4; ++k) {
+          const int j = c4 * 8 + 2 * k;
+          const float a0 = silu_f(__uint_as_float(g[j]) * rs) * (__uint_as_float(u[j]) * rs);
+          const float a1 = silu_f(__uint_as_float(g[j + 1]) * rs) * (__uint_as_float(u[j + 1]) * rs);
+          track_range(row_most, a0);
+          track_range(row_most, a1);
+          o[k] = pack_f16x2(a0, a1);
         }
-        if (live) track_range(most, row_most);
+        *xs_chunk(xs, lane, 4 * half + c4) = make_uint4(o[0], o[1], o[2], o[3]);
       }
-      __syncwarp();
-      store_words_transposed<MINE / 2>(xs, lane, row0, p.M, [&](int r, int wd) {
-        return out + static_cast<int64_t>(row0 + r) * p.ld_out + nb * OUTS + c + 2 * wd;
-      });
-      __syncwarp();
+      if (live) track_range(most, row_most);
     }
+    __syncwarp();
+    store_words_transposed<MINE / 2>(xs, lane, row0, p.M, [&](int r, int wd) {
+      return out + static_cast<int64_t>(row0 + r) * p.ld_out + nb * OUTS + c + 2 * wd;
+    });
+    __syncwarp();
   }
   report_range(p.err, !fp16_ok(most));
 }
@@ -949,12 +946,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 // f(kernel) for the few-rows kernel of a plan.
 template <int EPI, typename F>
 auto few_kernel(int rows, int cols, F&& f) {
-  if constexpr (EPI == EPI_RESID_ADD || EPI == EPI_SWIGLU)
+  if constexpr (EPI == EPI_RESID_ADD)
     if (cols == 64)
       return rows == 32   ? f(k_gemm_few<EPI, 64, 32>)
              : rows == 64 ? f(k_gemm_few<EPI, 64, 64>)
-             : rows == 96 ? f(k_gemm_few<EPI, 64, 96>)
-                          : f(k_gemm_few<EPI, 64, 128>);
+                          : f(k_gemm_few<EPI, 64, 96>);
   return rows == 32   ? f(k_gemm_few<EPI, 128, 32>)
          : rows == 64 ? f(k_gemm_few<EPI, 128, 64>)
          : rows == 96 ? f(k_gemm_few<EPI, 128, 96>)
@@ -1019,10 +1015,13 @@ int64_t rounds(int M, int N, int R, int n, int64_t pairs) {
 // The few-row plan of M <= GEMM_FEW_MAX_ROWS rows with the least clocks, if below `least` (which is updated).
 bool few_plan(int epi, int M, int N, int K, int64_t pairs, int64_t tile_clocks, int64_t& least, GemmPlan& plan) {
   bool found = false;
+  // 64 columns for the residual launches alone, and of at most 96 rows a CTA: gate/up tiles of 128
+  // columns take no more clocks than any of 64 that has as many rounds (64-row MMAs up to 64 rows,
+  // the same operand bytes as 64 x 128 or 96 x 128 beyond), and 128 x 64 no fewer than 96 x 128
   const int cols[2] = {128, 64};
   for (int n : cols) {
-    if (N % n || (n == 64 && epi != EPI_RESID_ADD && epi != EPI_SWIGLU)) continue;
-    for (int R = 32; R <= BM; R += 32) {
+    if (N % n || (n == 64 && epi != EPI_RESID_ADD)) continue;
+    for (int R = 32; R <= (n == 64 ? 96 : BM); R += 32) {
       const int64_t c = rounds(M, N, R, n, pairs) * (K / BK * block_clocks(epi, R, n) + tile_clocks);
       if (c < least) {
         least = c;

@@ -25,7 +25,7 @@ def test_tiles_are_ones_that_a_kernel_exists_for(epi, N, K, sms):
         p = dopr.gemm_plan(epi, M, N, K, sms)
         if p["few"] or p["wide_rows"]:
             assert (p["rows"], p["cols"]) in {(r, 128) for r in (32, 64, 96, 128)} | \
-                ({(r, 64) for r in (32, 64, 96, 128)} if epi in (dopr.EPI_RESID_ADD, dopr.EPI_SWIGLU) else set())
+                ({(r, 64) for r in (32, 64, 96)} if epi == dopr.EPI_RESID_ADD else set())
         else:
             assert (p["rows"], p["cols"]) == (128, 256)
         rest = M - p["wide_rows"] if p["wide_rows"] else M if p["few"] else 0
