@@ -12,18 +12,20 @@
 //   warp 0      (both CTAs) TMA producer; the copies of both CTAs complete on
 //               the leader's full barrier of the stage;
 //   warp 1      allocates 512 TMEM columns in both CTAs (two accumulators of
-//               256 columns); in the leader one thread issues the MMAs and
+//               256 columns); in the leader one lane issues the MMAs and
 //               commits stage releases and accumulator-ready barriers to both
-//               CTAs (multicast);
+//               CTAs (multicast), the whole warp running the loop;
 //   warps 2..9  (both CTAs) epilogue on the CTA's 128 rows of the tile:
 //               tcgen05.ld the finished accumulator (one TMEM lane quarter =
 //               32 rows per warp, one row per thread; two warps per quarter,
-//               each taking half of the tile's 256 columns), apply the
-//               epilogue in that row-per-thread layout, then transpose 32x32-
-//               word chunks through padded shared memory so every global
-//               access is a 128-byte row segment written by 8 consecutive
-//               lanes; finally tell the leader the accumulator is free, so the
-//               next tile's MMAs overlap the epilogue.
+//               each taking half of the tile's 256 columns, or for two rotated
+//               heads half of the frequencies), tell the leader that the
+//               accumulator is free after its last read, so the next tile's
+//               MMAs overlap the rest, and bring 32x32-word chunks through
+//               shared memory (16-byte chunks swizzled by the row) from the
+//               row-per-thread layout into one where consecutive lanes hold a
+//               row segment: 8 lanes 128 bytes of a row, in the QKV rotation
+//               4 lanes 32 bytes of either half of a head.
 // Tiles are visited in L2 groups (pair_tile_order): blocks of activation rows (up to
 // 48 MiB: 4,096 rows at K = 4,096) that stay in L2 while the weight tiles stream past
 // them, or, for the residual-epilogue launches, blocks of weight columns while the
@@ -35,8 +37,8 @@
 //   RMSNorm(r) * g = rs * (r (.) g) with rs = rsqrt(mean(r^2) + eps).  The
 //   residual-add epilogue writes r' = r + C, the next GEMM's operand
 //   f16(r' (.) g_next * rs_pre) -- rs_pre is the row's previous norm factor,
-//   which keeps the operand near unit scale -- and, per row and 256-column
-//   tile, the partial sum of r'^2.  The consuming GEMM sums those partials
+//   which keeps the operand near unit scale -- and, per row and 128 columns,
+//   the partial sum of r'^2.  The consuming GEMM sums those partials
 //   (in a fixed order) and scales its accumulator rows by rs / rs_pre.
 //   QKV epilogue: row scale, then per 128-column q/k head RMSNorm with the
 //   q/k gain and rotate-half RoPE at the token's position (pairs i, i+64),
@@ -254,7 +256,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tadd
         // The rotation runs in the transposed layout, 16 frequencies at a time: lane L owns rows
         // i*8 + L/4 and frequencies w4 .. w4+3 of the 16, so RoPE-table reads and the stores are
         // contiguous 4-lane row segments.  The (cos, sin) of the next 16 are fetched while these
-        // are rotated (rows past M read position 0's entries and are not stored).
+        // are rotated (rows past M read the last row's entries and are not stored).
         const int w4 = (lane & 3) * 4;
         float4 c01[4], c23[4];
         auto fetch_rope = [&](int f) {
@@ -721,10 +723,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 // With few rows a launch is bound by streaming the weights, and 256-column tiles leave most
 // SMs without a tile (O and down of the 8B shape: 16 tiles on 32 of 152 SMs) while each SM
 // takes in operand bytes at no more than about 64 bytes a clock, of which half or more were A
-// rows that hold nothing.  Narrow tiles put 4 times as many SMs to work, and a CTA copies only
-// its R rows (the MMA still runs 128 rows a CTA; what it reads past the R rows is other shared
-// memory, in tile rows that are never stored).  A stage is KB 64-wide k-blocks, so that each
-// operand is one copy of at least 8 KB a stage (a 3-D map: 64 elements, rows, k-blocks).
+// rows that hold nothing.  Narrow tiles put 2 or 4 times as many SMs to work, and a CTA copies only
+// its R rows (the MMAs run 128 rows a CTA, or 64 where SHORT below holds; what they read past the R
+// rows is other shared memory, in tile rows that are never stored).  A stage is KB 64-wide k-blocks,
+// so that each operand is one copy of at least 8 KB a stage (a 3-D map: 64 elements, rows, k-blocks;
+// gate and up rows together a 5-D one).
 // The K order of a row's MMAs is the wide tiles', so its result is the same bit for bit.
 constexpr int FEW_RING = 192 * 1024;
 constexpr int FEW_MAX_STAGES = 12;
