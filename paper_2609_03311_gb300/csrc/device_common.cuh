@@ -82,7 +82,7 @@ __device__ __forceinline__ int ld_volatile(const int* p) { return *reinterpret_c
 // same product (GemmParams::beside) would wait for that launch to end.  It reads only what the
 // wide launch waited for, and a gate hands that on: a thread of the wide launch that has returned
 // from its own pdl_wait() opens the gate with a release, every warp beside passes it with an
-// acquire before it reads, and the copying warp adds a fence to the proxy that its copies read by.
+// acquire before it reads, and a fence to the proxy that copies read by follows.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

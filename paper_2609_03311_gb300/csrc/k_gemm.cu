@@ -607,7 +607,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   // in this order: a few-row launch beside this one (GemmParams::beside) starts once this kernel's
   // blocks have triggered, and the gate hands it what this kernel waited for
   pdl_wait();
-  if (p.gate && blockIdx.x == 0 && threadIdx.x == 0) gate_open(p.gate, p.gate_number);
+  if (p.gate && blockIdx.x == 0 && threadIdx.x == THREADS - 32) gate_open(p.gate, p.gate_number);  // an epilogue warp's
   pdl_trigger();
   {
     // the MMAs write both CTAs' TMEM at the leader's address: both allocations must agree
@@ -794,22 +794,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     tmem_alloc_pair(smem_u32(tmem_slot), TMEM_COLS);
     tmem_relinquish_pair();
   }
+  // during the set-up, which hides the acquire's latency
+  const bool gate_passed = !p.beside || gate_wait_warp(p.gate, p.gate_number, p.err, p.timeout_ns);
+  if (p.beside) fence_proxy_async_global();
   tc_fence_before();
   __syncthreads();
   cluster_sync();  // both CTAs' barriers exist before either addresses the other's
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_trigger();
-  // (the producer starts on the weights first)
-  auto wait_for_inputs = [&] {
-    if (!p.beside)
-      pdl_wait();
-    else if (gate_wait_warp(p.gate, p.gate_number, p.err, p.timeout_ns))
-      fence_proxy_async_global();
-    else
-      total = 0;  // gave up: no tile runs
-  };
-  if (warp != 0) wait_for_inputs();
+  // (the producer starts on the weights first; beside the wide launch of the same product the gate
+  // stands for this wait)
+  if (warp != 0 && !p.beside) pdl_wait();
+  if (!gate_passed) total = 0;  // gave up: no tile runs
   {
     uint32_t other;  // as in k_gemm_pair: both allocations must agree
     asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(other) : "r"(mapa_shared(smem_u32(tmem_slot), rank ^ 1u)));
@@ -844,8 +841,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     if (pair < total)
       for (; ahead < min(stages, k_steps); ++ahead)
         if (one) load_weights(ahead, weight_row(pair / m_tiles), ahead);
-    wait_for_inputs();
-    if (total == 0 && ahead > 0) ok = false;  // gave up with weights on their way
+    if (!p.beside) pdl_wait();
     for (int t = pair; t < total && ok; t += n_pairs) {
       const int nb = t / m_tiles, row = p.row_begin + (t % m_tiles) * 2 * R + static_cast<int>(rank) * R;
       const int brow = weight_row(nb);
@@ -1050,9 +1046,10 @@ GemmPlan gemm_plan(int epi, int M, int N, int K, int num_sms) {
   // round of narrow tiles, they go to a few-row launch beside the wide one.  It has a start and an
   // end of its own, about 6,000 clocks.  N 4,096, K 12,288: 3,800 rows are 240 tiles, 3.2 rounds of
   // 76 pairs, of which 3,584 rows are 2.95 and the other 216 go beside them: 3 rounds instead of 4.
-  // Against the same library without it, whole calls: prefix build and scoring (8B width) 2,138 ->
-  // 2,100 us, selection of long documents (4B width, 5,650 rows a product) 2,183 -> 2,136,
-  // uncompressed scoring 2,654 -> 2,640.
+  // Against the same library without it, whole calls: prefix build and scoring (8B width) 2,134 ->
+  // 2,114 us, selection of long documents (4B width, 5,650 rows a product) 2,186 -> 2,136,
+  // uncompressed scoring 2,665 either way; the call of these 3,800 rows, under the power cap
+  // throughout, 3,145 -> 3,164.
   int64_t least = wide * (K / BK) * 2 * BN * 98 / 100;
   const int m_tiles = (M + PAIR_BM - 1) / PAIR_BM;
   for (int mt = m_tiles - 1; mt > 0 && M - mt * PAIR_BM <= GEMM_FEW_MAX_ROWS; --mt) {

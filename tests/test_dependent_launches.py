@@ -90,9 +90,9 @@ def test_the_few_row_launch_beside_a_wide_one_passes_its_gate_before_it_reads():
     bodies = {k: body for k, _, body in _kernels(_source("k_gemm.cu"))}
     wide, few = bodies["k_gemm_pair"], bodies["k_gemm_few"]
     assert wide.index("pdl_wait()") < wide.index("gate_open(") < wide.index("pdl_trigger()")
-    wait = _block(few, few.index("auto wait_for_inputs"))
-    assert "gate_wait_warp(" in wait and "fence_proxy_async_global()" in wait and "pdl_wait()" in wait
-    assert few.count("pdl_wait()") == wait.count("pdl_wait()") + 1  # the other one carries completion over, at the end
-    first, producer = few.index("if (warp != 0) wait_for_inputs();"), few.index("if (warp == 0) {")
-    second = few.index("wait_for_inputs();", producer)
-    assert second < few.index("&tmA, mapa_shared") and first < few.index("epilogue_prefetch<")
+    passed = few.index("gate_wait_warp(")
+    assert passed < few.index("fence_proxy_async_global()") < few.index("__syncthreads()") < few.index("tma_load_")
+    assert passed < few.index("epilogue_prefetch<") and "if (!gate_passed) total = 0;" in few
+    # without a gate every warp waits for the kernel before, and a launch beside does so at its end
+    assert few.count("if (!p.beside) pdl_wait();") == 1 and few.count("if (warp != 0 && !p.beside) pdl_wait();") == 1
+    assert few.index("if (p.beside) pdl_wait();") > few.index("epilogue_tile<") and few.count("pdl_wait()") == 3
