@@ -96,7 +96,11 @@ constexpr int GEMM_BM = 128, GEMM_BN = 256, GEMM_BK = 64;
 // Rows of a B (weight) tensor-map box: each CTA of a pair stages 128 of a tile's 256 B rows.
 constexpr int GEMM_B_BOX = 128;
 constexpr int GEMM_SS_PER_TILE = 2;  // partial sums of squares a residual epilogue writes per row and n-tile
-constexpr int GEMM_FEW_MAX_ROWS = 1024;  // launches of more rows always take the wide tiles
+// Rows that a k_gemm_few launch takes at most: what the chunk-sum scratch (Workspace::ss_chunks) is
+// sized for.  It is not where narrow and wide tiles meet: with 2,304 here, whole calls of 28 layers
+// of hidden 1,024 (O and down have 4 tile columns) take 2,107 us for 2,419 at 1,107 tokens, 2,156 for
+// 2,478 at 1,517, 2,501 for 2,804 at 2,009 and 2,536 for 2,847 at 2,296, and as long at 82 and 4,100.
+constexpr int GEMM_FEW_MAX_ROWS = 1024;
 __host__ __device__ constexpr int GEMM_FEW_KB(int rows) { return rows == 32 ? 4 : 2; }  // 64-wide k-blocks to a stage of k_gemm_few
 // Tensor maps of a GEMM operand (fp16, 128-byte swizzle): `wide` 2-D boxes of 64 elements x 128
 // rows; `few` 3-D (64 elements, rows, k-blocks of 64) boxes of 64 x R rows x GEMM_FEW_KB(R).

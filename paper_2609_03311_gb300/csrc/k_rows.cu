@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(SCORE_THREADS)
 // elements of four W1 rows into all eight pairs (fp32), so a W1 element is read from L2 once
 // for eight pairs, and not once a pair, and each pass over a pair's hn serves 32 units.  The
 // sums over a CTA's units go to part[pair][split]; k_score_mlp_sum adds them in split order.
-// 50 pairs, 1,024 units, 2,560 elements: one CTA per pair 508 us, these 29 us.
+// 50 pairs, 1,024 units, 2,560 elements, cold cache: one CTA per pair 508 us, these 24 + 4 us.
 constexpr int MLP_WARPS = 8, MLP_PAIRS = 8, MLP_UNITS = 4, MLP_CHUNK = 1024;
 constexpr int MLP_THREADS = 32 * MLP_WARPS;
 constexpr int MLP_PASS = MLP_WARPS * MLP_UNITS;  // hidden units of one pass

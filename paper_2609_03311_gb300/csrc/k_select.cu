@@ -17,8 +17,8 @@
 // Both tensor-core kernels are bound by the softmax warps (an FMA, an ex2 and an add per
 // score), not by the MMAs or memory: S is computed twice rather than kept, since 16-32
 // heads of n x n scores would be 16-64 times the bytes of A-bar.  Both together, against
-// one CTA per row with scalar dot products: 32 documents of 512 tokens, 16 heads, 84 us
-// (4,402 before); 4 documents of 777-2,048 tokens, 32 heads, 143 us (8,751 before).
+// one CTA per row with scalar dot products: 32 documents of 512 tokens, 16 heads, 83 us
+// (4,402 before); 4 documents of 777-2,048 tokens, 32 heads, 140 us (8,751 before).
 #include <float.h>
 #include <math.h>
 
